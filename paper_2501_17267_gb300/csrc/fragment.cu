@@ -211,94 +211,114 @@ __global__ void __launch_bounds__(kWarps * 32) fragment_wave_kernel(const FragAr
     if (lane == 0) sp[centre] = ((words[h + l * (h + l * h)] >> br) & 1u) ? (int8_t)-1 : (int8_t)1;
 }
 
-// Exact zero-temperature fragment marginals (l <= 3): the centre spin of each fragment
+// Exact zero-temperature fragment marginals (l = 1 or 3): the centre spin of each fragment
 // is set by comparing the lowest cube energy over the cube's free spins with s_c = +1 and
-// with s_c = -1 (+1 on a tie).  One block per fragment; its threads split the 2^F states
-// of the F free spins into contiguous stretches of the Gray-code order (state g(n) =
-// n ^ (n >> 1)), each energy obtained from the previous one by the flipped spin's change.
-constexpr int kTropBlock = 256;
+// with s_c = -1 (+1 on a tie).
+//
+// The minima come from eliminating the spins plane by plane instead of enumerating all
+// 2^27 states.  With T(s) the lowest energy of plane 0 (and its bonds to plane 1) given
+// plane 1's nine spins s, T starts as plane 0's own energy of every state, and the nine z
+// bonds are taken in one at a time: for spin q with z bond J,
+//   T'(.., s_q, ..) = min(T(.., s_q, ..) + J, T(.., -s_q, ..) - J),
+// a min-plus butterfly over bit q of the 512 states (s_q is plane 0's spin before the step
+// and plane 1's after it).  Plane 2 likewise from above, and the two tables plus plane 1's
+// own energy give the two minima.  A state that contradicts a fixed spin starts at kBarred.
+// About 28 K additions and minima a cube instead of 2^27 energies: 232.4 ms -> 0.23 ms for
+// four L = 12 lattices (27 launches of 4.7 us and the energies).
+//
+// A warp owns a fragment: lane holds bits 4 .. 8 of a state (spin q of a plane is bit q,
+// q = dx + 3 dy, set meaning -1), its 16 registers bits 0 .. 3, so four butterflies stay in
+// registers and five are shuffles.
+constexpr int kTropWarps = 4;         // fragments per block
+constexpr int kBarred = 1 << 20;      // above any cube energy (54 bonds of |J| <= 2)
 
-__global__ void __launch_bounds__(kTropBlock) fragment_tropical_kernel(int8_t* spins, const uint2* const* j6_ptrs,
-                                                                       int L, int l, int wave)
+__global__ void __launch_bounds__(kTropWarps * 32) fragment_tropical_kernel(int8_t* spins, const uint2* const* j6_ptrs,
+                                                                            int L, int l, int wave)
 {
-    __shared__ int s_F, s_cf;
-    __shared__ int s_h[27], s_nn[27];
-    __shared__ int s_nj[27][6], s_nJ[27][6];
-    __shared__ int s_mp[kTropBlock / 32], s_mm[kTropBlock / 32];
-    const int inst = blockIdx.y, tid = threadIdx.x;
-    const int h = (l - 1) / 2, V = l * l * l, per = L / l;
-    const int frag = blockIdx.x;
+    constexpr unsigned kAll = 0xFFFFFFFFu;
+    const int inst = blockIdx.y, lane = threadIdx.x & 31;
+    const int per = L / l;
+    const int frag = blockIdx.x * kTropWarps + (int)(threadIdx.x >> 5);
+    if (frag >= per * per * per) return;  // the whole warp
     const int ca = wave % l, cb = (wave / l) % l, cc = wave / (l * l);
     const int cx = ca + l * (frag % per), cy = cb + l * ((frag / per) % per), cz = cc + l * (frag / (per * per));
     int8_t* __restrict__ sp = spins + (size_t)inst * L * L * L;
-    const uint2* __restrict__ j6 = j6_ptrs[inst];
-    auto site_of = [&](int q) {
-        const int dx = q % l, dy = (q / l) % l, dz = q / (l * l);
-        return ((cx + dx - h + L) % L) + L * (((cy + dy - h + L) % L) + L * ((cz + dz - h + L) % L));
+    const int centre = cx + L * (cy + L * cz);
+    if (l == 1) {  // no bonds inside the cube: a tie
+        if (lane == 0) sp[centre] = 1;
+        return;
+    }
+    // lane q < 27: cube site q, its value (0 = free) and its three forward bonds
+    int value = 0, Jx = 0, Jy = 0, Jz = 0;
+    if (lane < 27) {
+        const int dx = lane % 3, dy = (lane / 3) % 3, dz = lane / 9;
+        const int x = cx + dx - 1, y = cy + dy - 1, z = cz + dz - 1;
+        const int i = (x < 0 ? x + L : x >= L ? x - L : x) +
+                      L * ((y < 0 ? y + L : y >= L ? y - L : y) + L * (z < 0 ? z + L : z >= L ? z - L : z));
+        value = sp[i];
+        const uint2 rec = j6_ptrs[inst][i];
+        Jx = coupling(rec, 0);
+        Jy = coupling(rec, 2);
+        Jz = coupling(rec, 4);
+    }
+    const uint32_t fixed = __ballot_sync(kAll, value != 0), minus = __ballot_sync(kAll, value < 0);
+    auto sign = [&](int bit) { return ((lane >> (bit - 4)) & 1) ? -1 : 1; };  // of a spin held by the lane
+    // plane dz's own energy of the lane's 16 states (kBarred where a fixed spin disagrees)
+    auto plane_energy = [&](int dz, int (&T)[16]) {
+        const int b = 9 * dz;
+        const int J01 = __shfl_sync(kAll, Jx, b), J12 = __shfl_sync(kAll, Jx, b + 1);
+        const int J34 = __shfl_sync(kAll, Jx, b + 3), J45 = __shfl_sync(kAll, Jx, b + 4);
+        const int J67 = __shfl_sync(kAll, Jx, b + 6), J78 = __shfl_sync(kAll, Jx, b + 7);
+        const int J03 = __shfl_sync(kAll, Jy, b), J14 = __shfl_sync(kAll, Jy, b + 1);
+        const int J25 = __shfl_sync(kAll, Jy, b + 2), J36 = __shfl_sync(kAll, Jy, b + 3);
+        const int J47 = __shfl_sync(kAll, Jy, b + 4), J58 = __shfl_sync(kAll, Jy, b + 5);
+        const int s4 = sign(4), s5 = sign(5), s6 = sign(6), s7 = sign(7), s8 = sign(8);
+        const int high = J45 * s4 * s5 + J67 * s6 * s7 + J78 * s7 * s8 + J47 * s4 * s7 + J58 * s5 * s8;
+        const int h1 = J14 * s4, h2 = J25 * s5, h3 = J34 * s4 + J36 * s6;  // fields on spins 1, 2, 3
+        const uint32_t m = (fixed >> b) & 511u, v = (minus >> b) & 511u;
+        const bool lane_ok = ((((uint32_t)lane << 4) ^ v) & m & 0x1F0u) == 0u;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const int s0 = (e & 1) ? -1 : 1, s1 = (e & 2) ? -1 : 1, s2 = (e & 4) ? -1 : 1, s3 = (e & 8) ? -1 : 1;
+            const int E = high + s1 * h1 + s2 * h2 + s3 * h3 + s0 * s1 * J01 + s1 * s2 * J12 + s0 * s3 * J03;
+            T[e] = lane_ok && (((uint32_t)e ^ v) & m & 15u) == 0u ? E : kBarred;
+        }
     };
-    if (tid == 0) {
-        int idx[27];
-        int F = 0;
-        for (int q = 0; q < V; ++q) idx[q] = sp[site_of(q)] != 0 ? -1 : F++;
-        for (int k = 0; k < F; ++k) s_h[k] = 0, s_nn[k] = 0;
-        for (int q = 0; q < V; ++q) {  // bonds inside the cube, each once (+x, +y, +z)
-            const int dd[3] = {q % l, (q / l) % l, q / (l * l)};
-            const uint2 rec = j6[site_of(q)];
-            for (int d = 0; d < 3; ++d) {
-                const int step = d == 0 ? 1 : d == 1 ? l : l * l;
-                if (dd[d] + 1 >= l) continue;
-                const int r = q + step;
-                const int J = coupling(rec, 2 * d);
-                if (idx[q] >= 0 && idx[r] >= 0) {
-                    const int a = idx[q], b = idx[r];
-                    s_nj[a][s_nn[a]] = b, s_nJ[a][s_nn[a]++] = J;
-                    s_nj[b][s_nn[b]] = a, s_nJ[b][s_nn[b]++] = J;
-                } else if (idx[q] >= 0) {
-                    s_h[idx[q]] += J * sp[site_of(r)];
-                } else if (idx[r] >= 0) {
-                    s_h[idx[r]] += J * sp[site_of(q)];
-                }
+    // the nine z bonds of plane dz to the plane above it
+    auto eliminate = [&](int dz, int (&T)[16]) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int J = __shfl_sync(kAll, Jz, 9 * dz + q);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+                if (e & (1 << q)) continue;
+                const int up = T[e], dn = T[e | (1 << q)];
+                T[e] = min(up + J, dn - J);
+                T[e | (1 << q)] = min(dn + J, up - J);
             }
         }
-        s_F = F;
-        s_cf = idx[h + l * (h + l * h)];
-    }
-    __syncthreads();
-    const int F = s_F, cf = s_cf;
-    const uint32_t total = 1u << F;
-    const uint32_t seg = (total + kTropBlock - 1) / kTropBlock;
-    const uint32_t n0 = tid * seg, n1 = min(n0 + seg, total);
-    int mp = 0x7FFFFFFF, mm = 0x7FFFFFFF;
-    if (n0 < total) {
-        uint32_t st = n0 ^ (n0 >> 1);  // bit k set: free spin k is -1
-        auto sv = [&](int k) { return ((st >> k) & 1u) ? -1 : 1; };
-        int E = 0;
-        for (int k = 0; k < F; ++k) {
-            E += s_h[k] * sv(k);
-            for (int t = 0; t < s_nn[k]; ++t)
-                if (s_nj[k][t] > k) E += s_nJ[k][t] * sv(k) * sv(s_nj[k][t]);
-        }
-        if (sv(cf) > 0) mp = E; else mm = E;
-        for (uint32_t n = n0 + 1; n < n1; ++n) {
-            const int k = __ffs(n) - 1;  // the spin that flips from g(n - 1) to g(n)
-            int field = s_h[k];
-            for (int t = 0; t < s_nn[k]; ++t) field += s_nJ[k][t] * sv(s_nj[k][t]);
-            E -= 2 * sv(k) * field;
-            st ^= 1u << k;
-            if (sv(cf) > 0) mp = min(mp, E); else mm = min(mm, E);
-        }
-    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        mp = min(mp, __shfl_xor_sync(0xFFFFFFFFu, mp, o));
-        mm = min(mm, __shfl_xor_sync(0xFFFFFFFFu, mm, o));
-    }
-    if ((tid & 31) == 0) s_mp[tid >> 5] = mp, s_mm[tid >> 5] = mm;
-    __syncthreads();
-    if (tid == 0) {
-        for (int k = 1; k < kTropBlock / 32; ++k) mp = min(mp, s_mp[k]), mm = min(mm, s_mm[k]);
-        sp[cx + L * (cy + L * cz)] = mp <= mm ? (int8_t)1 : (int8_t)-1;
-    }
+        for (int q = 4; q < 9; ++q) {
+            const int J = __shfl_sync(kAll, Jz, 9 * dz + q);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) T[e] = min(T[e] + J, __shfl_xor_sync(kAll, T[e], 1 << (q - 4)) - J);
+        }
+    };
+    int U[16], V[16];
+    plane_energy(0, U);
+    eliminate(0, U);
+    plane_energy(2, V);
+    eliminate(1, V);
+    int W[16];
+    plane_energy(1, W);
+    int m = 0x7FFFFFFF;
+#pragma unroll
+    for (int e = 0; e < 16; ++e) m = min(m, U[e] + V[e] + W[e]);
+    // the centre is spin 4 of plane 1: bit 0 of the lane
+#pragma unroll
+    for (int o = 16; o > 1; o >>= 1) m = min(m, __shfl_xor_sync(kAll, m, o));
+    const int mm = __shfl_sync(kAll, m, 1);
+    if (lane == 0) sp[centre] = m <= mm ? (int8_t)1 : (int8_t)-1;
 }
 
 int32_t check(const char* what)
@@ -339,9 +359,9 @@ int32_t launch_fragment_tropical_waves(int8_t* spins, const uint2* const* j6_ptr
                                        cudaStream_t st)
 {
     const int per = L / l;
-    const dim3 grid(per * per * per, I);
+    const dim3 grid((per * per * per + kTropWarps - 1) / kTropWarps, I);
     for (int w = 0; w < l * l * l; ++w) {
-        fragment_tropical_kernel<<<grid, kTropBlock, 0, st>>>(spins, j6_ptrs, L, l, w);
+        fragment_tropical_kernel<<<grid, kTropWarps * 32, 0, st>>>(spins, j6_ptrs, L, l, w);
         const int32_t rc = check("fragment_tropical_kernel");
         if (rc != SG_OK) return rc;
     }

@@ -208,3 +208,14 @@ def test_tropical_fragments_match_oracle(sg, L, l):
     res = sg.fragment_tropical_run(inst, l, spins="host")
     ospins, oE = o.fragment_tropical(L, J3, l)
     assert np.array_equal(res["spins"], ospins) and res["E"] == oE
+
+
+@pytest.mark.gpu
+def test_tropical_fragments_with_general_couplings_match_oracle(sg):
+    """|J| <= 2 and absent bonds: the plane-by-plane minima against the enumeration."""
+    from paper_2501_17267_gb300 import workloads as wl
+    J3 = wl.random_couplings(5, 6)
+    inst = sg.Instance.from_couplings(6, J3, e_gs=-1)
+    res = sg.fragment_tropical_run(inst, 3, spins="host")
+    ospins, oE = o.fragment_tropical(6, J3, 3)
+    assert np.array_equal(res["spins"], ospins) and res["E"] == oE
