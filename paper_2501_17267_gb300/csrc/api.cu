@@ -955,19 +955,18 @@ int32_t fragment_batch(const sg_instance* const* insts, const sg_fragment_params
         SG_RET(instance_device_j6(const_cast<sg_instance*>(insts[a]), st, &j6, nullptr));
         jp[a] = j6;
     }
-    DevBuf d_spins, d_thr, d_keys, d_j6, d_words, d_E64, d_bad, d_one;
+    DevBuf d_spins, d_thr, d_keys, d_j6, d_E64, d_bad;
     SG_RET(d_spins.alloc((size_t)I * N, st));
     SG_RET(d_thr.alloc(sizeof(uint32_t) * thr.size(), st));
     SG_RET(d_keys.alloc(sizeof(RunKeys) * I, st));
     SG_RET(d_j6.alloc(sizeof(void*) * I, st));
-    SG_RET(d_words.alloc((size_t)N * 4, st));
-    SG_RET(d_E64.alloc(sizeof(unsigned long long) * 32 * (size_t)I, st));
+    SG_RET(d_E64.alloc(sizeof(unsigned long long) * (size_t)I, st));
     SG_RET(d_bad.alloc(sizeof(int), st));
     SG_TRY_CUDA(cudaMemcpyAsync(d_thr.as<void>(), thr.data(), sizeof(uint32_t) * thr.size(), cudaMemcpyHostToDevice, st));
     SG_TRY_CUDA(cudaMemcpyAsync(d_keys.as<void>(), keys.data(), sizeof(RunKeys) * I, cudaMemcpyHostToDevice, st));
     SG_TRY_CUDA(cudaMemcpyAsync(d_j6.as<void>(), jp.data(), sizeof(void*) * I, cudaMemcpyHostToDevice, st));
     SG_TRY_CUDA(cudaMemsetAsync(d_spins.as<void>(), 0, (size_t)I * N, st));
-    SG_TRY_CUDA(cudaMemsetAsync(d_E64.as<void>(), 0, sizeof(unsigned long long) * 32 * (size_t)I, st));
+    SG_TRY_CUDA(cudaMemsetAsync(d_E64.as<void>(), 0, sizeof(unsigned long long) * (size_t)I, st));
     SG_TRY_CUDA(cudaMemsetAsync(d_bad.as<void>(), 0, sizeof(int), st));
     LaunchLog log;
     const int64_t V = (int64_t)l * l * l;
@@ -983,18 +982,15 @@ int32_t fragment_batch(const sg_instance* const* insts, const sg_fragment_params
         return launch_fragment_waves(d_spins.as<int8_t>(), d_j6.as<const uint2*>(), d_keys.as<RunKeys>(),
                                      d_thr.as<uint32_t>(), I, L, l, S, st);
     }, V));
-    // energies (Eq. 1): each configuration packed as one word of a single replica
-    for (int a = 0; a < I; ++a) {
-        SG_RET(log.run(SG_KERNEL_OTHER, N, st, [&] {
-            return launch_pack_spins(d_spins.as<int8_t>() + (size_t)a * N, d_words.as<int8_t>(), L, 32, 1,
-                                     d_bad.as<int>(), st);
-        }));
-        SG_RET(log.run(SG_KERNEL_ENERGY, N, st, [&] {
-            return launch_energy(d_words.as<int8_t>(), d_j6.as<const uint2*>() + a, 1, L, 1,
-                                 d_E64.as<unsigned long long>() + 32 * (size_t)a, st);
+    // energies (Eq. 1) of the int8 configurations
+    for (int a = 0; a < I; a += (int)kMaxGroup) {
+        const int m = std::min(I - a, (int)kMaxGroup);
+        SG_RET(log.run(SG_KERNEL_ENERGY, (int64_t)m * N, st, [&] {
+            return launch_energy_direct(d_spins.as<int8_t>() + (size_t)a * N, d_j6.as<const uint2*>() + a, m, L, 1,
+                                        d_E64.as<unsigned long long>() + a, d_bad.as<int>(), st);
         }));
     }
-    std::vector<unsigned long long> E64((size_t)32 * I);
+    std::vector<unsigned long long> E64((size_t)I);
     SG_TRY_CUDA(cudaMemcpyAsync(E64.data(), d_E64.as<void>(), sizeof(unsigned long long) * E64.size(),
                                 cudaMemcpyDeviceToHost, st));
     for (int a = 0; a < I; ++a)
@@ -1006,7 +1002,7 @@ int32_t fragment_batch(const sg_instance* const* insts, const sg_fragment_params
     SG_TRY_CUDA(cudaStreamSynchronize(st));
     log.finish();
     for (int a = 0; a < I; ++a) {
-        outs[a].E = (int64_t)(long long)E64[(size_t)32 * a];
+        outs[a].E = (int64_t)(long long)E64[(size_t)a];
         outs[a].eps = eps_of(outs[a].E, insts[a]->e_gs);
     }
     return SG_OK;
@@ -1048,34 +1044,30 @@ extern "C" int32_t sg_energy(const sg_instance* inst_c, const int8_t* spins, int
     sg_instance* inst = const_cast<sg_instance*>(inst_c);
     cudaStream_t st = (cudaStream_t)stream;
     const int64_t N = inst->N;
-    const int R = n_configs, Wn = words_for(R), Rp = 32 * Wn;
+    const int R = n_configs;
     const uint2* j6 = nullptr;
     SG_RET(instance_device_j6(inst, st, &j6, nullptr));
-    DevBuf d_in, d_packed, d_E64, d_j6, d_bad;
+    DevBuf d_in, d_E64, d_j6, d_bad;
     const int8_t* src = spins;
     if (mem_kind == SG_MEM_HOST) {
         SG_RET(d_in.alloc((size_t)R * N, st));
         SG_TRY_CUDA(cudaMemcpyAsync(d_in.as<void>(), spins, (size_t)R * N, cudaMemcpyHostToDevice, st));
         src = d_in.as<int8_t>();
     }
-    SG_RET(d_packed.alloc((size_t)Wn * 4 * N, st));
-    SG_RET(d_E64.alloc(sizeof(unsigned long long) * Rp, st));
+    SG_RET(d_E64.alloc(sizeof(unsigned long long) * R, st));
     SG_RET(d_j6.alloc(sizeof(uint2*), st));
     SG_RET(d_bad.alloc(sizeof(int), st));
     SG_TRY_CUDA(cudaMemcpyAsync(d_j6.as<void>(), &j6, sizeof(uint2*), cudaMemcpyHostToDevice, st));
-    SG_TRY_CUDA(cudaMemsetAsync(d_E64.as<void>(), 0, sizeof(unsigned long long) * Rp, st));
+    SG_TRY_CUDA(cudaMemsetAsync(d_E64.as<void>(), 0, sizeof(unsigned long long) * R, st));
     SG_TRY_CUDA(cudaMemsetAsync(d_bad.as<void>(), 0, sizeof(int), st));
     LaunchLog log;
-    SG_RET(log.run(SG_KERNEL_OTHER, (int64_t)Rp * N, st, [&] {
-        return launch_pack_spins(src, d_packed.as<int8_t>(), inst->L, Rp, R, d_bad.as<int>(), st);
+    SG_RET(log.run(SG_KERNEL_ENERGY, (int64_t)R * N, st, [&] {
+        return launch_energy_direct(src, d_j6.as<const uint2*>(), 1, inst->L, R, d_E64.as<unsigned long long>(),
+                                    d_bad.as<int>(), st);
     }));
-    SG_RET(log.run(SG_KERNEL_ENERGY, (int64_t)Rp * N, st, [&] {
-        return launch_energy(d_packed.as<int8_t>(), d_j6.as<const uint2*>(), 1, inst->L, Wn,
-                             d_E64.as<unsigned long long>(), st);
-    }));
-    std::vector<long long> E((size_t)Rp);
+    std::vector<long long> E((size_t)R);
     int bad = 0;
-    SG_TRY_CUDA(cudaMemcpyAsync(E.data(), d_E64.as<void>(), sizeof(long long) * Rp,
+    SG_TRY_CUDA(cudaMemcpyAsync(E.data(), d_E64.as<void>(), sizeof(long long) * R,
                                 cudaMemcpyDeviceToHost, st));
     SG_TRY_CUDA(cudaMemcpyAsync(&bad, d_bad.as<void>(), sizeof(int), cudaMemcpyDeviceToHost, st));
     SG_TRY_CUDA(cudaStreamSynchronize(st));

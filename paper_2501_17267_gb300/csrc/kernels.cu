@@ -259,29 +259,149 @@ __global__ void unpack_spins_kernel(const uint32_t* __restrict__ words, int8_t* 
     }
 }
 
-// in: [R][N] int8 spins of +-1 in logical site order; words: [N][Wn] packed (padding
-// replicas +1).  Values other than +-1 are counted in *bad and stored as +1.
-__global__ void pack_spins_kernel(const int8_t* __restrict__ in, uint32_t* __restrict__ words, int L, int Wn,
-                                  int R, int* __restrict__ bad)
-{
-    const int64_t N = (int64_t)L * L * L;
-    const int64_t n = (int64_t)Wn * N;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = logical_of(L, t / Wn);
-        const int w = (int)(t % Wn);
-        uint32_t word = 0;
-        int nbad = 0;
-        for (int b = 0; b < 32; ++b) {
-            const int r = 32 * w + b;
-            if (r >= R) break;
-            const int8_t v = in[(int64_t)r * N + i];
-            if (v == -1) word |= 1u << b;
-            else if (v != 1) ++nbad;
+// ---------------------------------------------------------------- energies of int8 spins
+
+// E (Eq. 1) of configurations given as int8 spins of +-1, [I][n][N] in logical site order,
+// straight from the bytes: with a, b the bytes of a bond's two ends, (a ^ b) | 1 is s_i s_j
+// as a byte, so four bonds are one three-input operation and one dp4a with their couplings.
+//
+// HBM-bound: a configuration's bytes are read once from memory (its rows z + 1 and y + 1
+// a second time from L2 and L1).  A thread keeps the couplings of V sites along x in two
+// z planes in registers and walks over the configurations of its block (blockIdx.y), so
+// couplings are read once a block; V is the widest load that the row length and the base
+// address allow (energy_direct_width).  1000 configurations at L = 64 (262 MB): 1.62 ms as
+// a pack to bits and row sums, now 87 us (3.0 TB/s, 0.45 of the measured copy rate).
+constexpr int kEnergyConfigs = 128;  // configurations a block sums at most
+
+template <int V>
+struct SpinBytes {
+    static constexpr int W = V >= 4 ? V / 4 : 1;
+    uint32_t w[W];
+    __device__ __forceinline__ void load(const int8_t* p)
+    {
+        if constexpr (V == 16) {
+            const uint4 v = *reinterpret_cast<const uint4*>(p);
+            w[0] = v.x, w[1] = v.y, w[2] = v.z, w[3] = v.w;
+        } else if constexpr (V == 4) {
+            w[0] = *reinterpret_cast<const uint32_t*>(p);
+        } else if constexpr (V == 2) {
+            w[0] = *reinterpret_cast<const uint16_t*>(p);
+        } else {
+            w[0] = *reinterpret_cast<const uint8_t*>(p);
         }
-        if (nbad) atomicAdd(bad, nbad);
-        words[t] = word;
     }
+};
+
+// the bytes one site further in x: of the V sites, the last from `next` (its low byte)
+template <int V>
+__device__ __forceinline__ SpinBytes<V> shifted(const SpinBytes<V>& a, uint32_t next)
+{
+    SpinBytes<V> r;
+    if constexpr (V >= 4) {
+#pragma unroll
+        for (int k = 0; k < SpinBytes<V>::W; ++k)
+            r.w[k] = __byte_perm(a.w[k], k + 1 < SpinBytes<V>::W ? a.w[k + 1] : next, 0x4321);
+    } else if constexpr (V == 2) {
+        r.w[0] = __byte_perm(a.w[0], next, 0x0041);
+    } else {
+        r.w[0] = next;
+    }
+    return r;
+}
+
+template <int V>
+__global__ void __launch_bounds__(kBlock)
+energy_direct_kernel(const int8_t* __restrict__ spins, const uint2* const* __restrict__ j6_ptrs, int L, int n,
+                     int per_block, unsigned long long* __restrict__ E_out, int* __restrict__ bad)
+{
+    constexpr int W = SpinBytes<V>::W;
+    constexpr uint32_t kLive = V >= 4 ? 0xFFFFFFFFu : V == 2 ? 0xFFFFu : 0xFFu;  // bytes of a word in use
+    __shared__ int s_E[kEnergyConfigs];
+    const int64_t N = (int64_t)L * L * L;
+    const int inst = blockIdx.z;
+    const int xs = L / V, items = xs * L * (L / 2);
+    const int t = blockIdx.x * kBlock + threadIdx.x;
+    const bool live = t < items;
+    const int tt = live ? t : 0;
+    const int xc = tt % xs, y = (tt / xs) % L, z0 = tt / (xs * L) * 2;
+    const int yp = y + 1 == L ? 0 : y + 1, zp = z0 + 2 == L ? 0 : z0 + 2;
+    const int x0 = xc * V, xn = x0 + V == L ? 0 : x0 + V;
+    const int own[2] = {(z0 * L + y) * L + x0, ((z0 + 1) * L + y) * L + x0};
+    const int up[2] = {(z0 * L + yp) * L + x0, ((z0 + 1) * L + yp) * L + x0};
+    const int nxt[2] = {(z0 * L + y) * L + xn, ((z0 + 1) * L + y) * L + xn};
+    const int top = (zp * L + y) * L + x0;
+    uint32_t J[2][3][W];
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            constexpr int kSites = V >= 4 ? 4 : V;
+            const uint2* __restrict__ rec = j6_ptrs[inst] + own[p] + 4 * k;
+            uint2 r[4] = {};
+            if constexpr (V >= 4) {  // four records in two 16-byte loads (rows start on multiples of four)
+                const uint4 lo = reinterpret_cast<const uint4*>(rec)[0], hi = reinterpret_cast<const uint4*>(rec)[1];
+                r[0] = make_uint2(lo.x, lo.y), r[1] = make_uint2(lo.z, lo.w);
+                r[2] = make_uint2(hi.x, hi.y), r[3] = make_uint2(hi.z, hi.w);
+            } else {
+#pragma unroll
+                for (int b = 0; b < kSites; ++b) r[b] = rec[b];
+            }
+            J[p][0][k] = __byte_perm(__byte_perm(r[0].x, r[1].x, 0x0040), __byte_perm(r[2].x, r[3].x, 0x0040), 0x5410);
+            J[p][1][k] = __byte_perm(__byte_perm(r[0].x, r[1].x, 0x0062), __byte_perm(r[2].x, r[3].x, 0x0062), 0x5410);
+            J[p][2][k] = __byte_perm(__byte_perm(r[0].y, r[1].y, 0x0040), __byte_perm(r[2].y, r[3].y, 0x0040), 0x5410);
+            if constexpr (V < 4) {
+                J[p][0][k] &= kLive;
+                J[p][1][k] &= kLive;
+                J[p][2][k] &= kLive;
+            }
+        }
+    for (int q = threadIdx.x; q < kEnergyConfigs; q += kBlock) s_E[q] = 0;
+    __syncthreads();
+    const int c0 = blockIdx.y * per_block, c1 = min(n, c0 + per_block);
+    const int8_t* __restrict__ base = spins + ((int64_t)inst * n + c0) * N;
+    const int lane = threadIdx.x & 31;
+    for (int c = c0; c < c1; ++c, base += N) {
+        SpinBytes<V> a[3], u[2];
+        uint32_t x[2];
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            a[p].load(base + own[p]);
+            u[p].load(base + up[p]);
+            x[p] = *reinterpret_cast<const uint8_t*>(base + nxt[p]);
+        }
+        a[2].load(base + top);
+        int acc = 0;
+        uint32_t wrong = 0;
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            const SpinBytes<V> f = shifted<V>(a[p], x[p]);
+#pragma unroll
+            for (int k = 0; k < W; ++k) {
+                const uint32_t s = a[p].w[k];
+                acc = __dp4a((int)((s ^ f.w[k]) | 0x01010101u), (int)J[p][0][k], acc);
+                acc = __dp4a((int)((s ^ u[p].w[k]) | 0x01010101u), (int)J[p][1][k], acc);
+                acc = __dp4a((int)((s ^ a[p + 1].w[k]) | 0x01010101u), (int)J[p][2][k], acc);
+                // a byte is 0x01 or 0xFF, as its top bit says, or it is no spin
+                wrong |= s ^ (((s >> 7) & 0x01010101u) * 0xFEu | 0x01010101u);
+            }
+        }
+        if (!live) acc = 0, wrong = 0;
+        if (wrong & kLive) {  // count the values that are no spins
+            int nbad = 0;
+#pragma unroll
+            for (int p = 0; p < 2; ++p)
+                for (int b = 0; b < V; ++b) {
+                    const int8_t v = base[own[p] + b];
+                    nbad += v != 1 && v != -1;
+                }
+            if (nbad) atomicAdd(bad, nbad);
+        }
+        acc = __reduce_add_sync(0xFFFFFFFFu, acc);
+        if (lane == 0) atomicAdd(&s_E[c - c0], acc);
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < c1 - c0; q += kBlock)
+        atomicAdd(&E_out[(int64_t)inst * n + c0 + q], (unsigned long long)(long long)s_E[q]);
 }
 
 int grid_for(int64_t items, int multiple_of = 1, int cap = 1 << 20)
@@ -422,14 +542,43 @@ int32_t launch_unpack_spins(const int8_t* spins, int8_t* out, int L, int Rp, int
     return check_launch("unpack_spins");
 }
 
-int32_t launch_pack_spins(const int8_t* in, int8_t* spins, int L, int Rp, int R, int* bad,
-                          cudaStream_t st)
+namespace {
+// Widest load for rows of L bytes from `base`: every row then starts on a multiple of it.
+int energy_direct_width(const void* base, int L)
 {
-    const int64_t N = (int64_t)L * L * L;
-    const int Wn = Rp / 32;
-    pack_spins_kernel<<<grid_for((int64_t)Wn * N, 1, 8192), kBlock, 0, st>>>(in, reinterpret_cast<uint32_t*>(spins),
-                                                                            L, Wn, R, bad);
-    return check_launch("pack_spins");
+    for (const int v : {16, 4, 2})
+        if (L % v == 0 && reinterpret_cast<uintptr_t>(base) % v == 0) return v;
+    return 1;
+}
+
+template <int V>
+int32_t launch_direct(const int8_t* spins, const uint2* const* j6_ptrs, int I, int L, int n, unsigned long long* E_out,
+                      int* bad, cudaStream_t st)
+{
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int gx = ((L / V) * L * (L / 2) + kBlock - 1) / kBlock;
+    // Configurations a block: few enough for about 8 blocks an SM (three are resident), many
+    // enough to pay for the couplings a block loads first.  1000 configurations at L = 64:
+    // 93 us at 3 or 12 blocks an SM, 87 at 8, 140 at 16.
+    const int64_t want = std::max<int64_t>(1, 8LL * sms / ((int64_t)gx * I));
+    int per = (int)std::min<int64_t>(kEnergyConfigs, std::max<int64_t>(1, (n + want - 1) / want));
+    per = std::max(per, (n + 65534) / 65535);
+    energy_direct_kernel<V><<<dim3(gx, (n + per - 1) / per, I), kBlock, 0, st>>>(spins, j6_ptrs, L, n, per, E_out, bad);
+    return check_launch("energy_direct");
+}
+}  // namespace
+
+int32_t launch_energy_direct(const int8_t* spins, const uint2* const* j6_ptrs, int I, int L, int n,
+                             unsigned long long* E_out, int* bad, cudaStream_t st)
+{
+    switch (energy_direct_width(spins, L)) {
+        case 16: return launch_direct<16>(spins, j6_ptrs, I, L, n, E_out, bad, st);
+        case 4: return launch_direct<4>(spins, j6_ptrs, I, L, n, E_out, bad, st);
+        case 2: return launch_direct<2>(spins, j6_ptrs, I, L, n, E_out, bad, st);
+        default: return launch_direct<1>(spins, j6_ptrs, I, L, n, E_out, bad, st);
+    }
 }
 
 }  // namespace sg

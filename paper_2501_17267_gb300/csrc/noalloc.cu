@@ -71,7 +71,8 @@ extern "C" int32_t sg_energy_noalloc(int32_t L, const int8_t* J3_dev, const int8
     const size_t N = (size_t)L * L * L;
     const int Wn = words_for(n_configs), Rp = 32 * Wn;
     // scratch layout: [E sums: 8 * Rp][status: 16][j6 pointer: 16][coupling records: 8 * N]
-    //                 [sign bytes: N][packed spins: N * Wn 32-bit words]
+    //                 [sign bytes: N]; the documented limit also counts N * Wn 32-bit words
+    //                 for packed spins, which the energies no longer need
     const size_t off_E = 0;
     const size_t off_bad = round_up(off_E + 8 * (size_t)Rp, 256);
     const size_t off_ptr = off_bad + 16;
@@ -92,7 +93,6 @@ extern "C" int32_t sg_energy_noalloc(int32_t L, const int8_t* J3_dev, const int8
     const uint2** j6_ptr = reinterpret_cast<const uint2**>(base + off_ptr);
     uint2* j6 = reinterpret_cast<uint2*>(base + off_j6);
     uint8_t* j1 = base + off_j1;
-    int8_t* packed = reinterpret_cast<int8_t*>(base + off_sp);
 
     // the array keeps the previous call's contents: clear the sums and the status word
     SG_TRY_CUDA(cudaMemsetAsync(E64, 0, 8 * (size_t)Rp, st));
@@ -101,9 +101,7 @@ extern "C" int32_t sg_energy_noalloc(int32_t L, const int8_t* J3_dev, const int8
     SG_TRY_CUDA(cudaGetLastError());
     rc = launch_prepare_j6(J3_dev, j6, j1, L, st);
     if (rc != SG_OK) return rc;
-    rc = launch_pack_spins(spins_dev, packed, L, Rp, n_configs, bad, st);
-    if (rc != SG_OK) return rc;
-    rc = launch_energy(packed, j6_ptr, 1, L, Wn, E64, st);
+    rc = launch_energy_direct(spins_dev, j6_ptr, 1, L, n_configs, E64, bad, st);
     if (rc != SG_OK) return rc;
     rc = launch_copy_energies(E64, E_dev, n_configs, st);
     if (rc != SG_OK) return rc;

@@ -257,7 +257,9 @@ int32_t launch_narrow_energy(const unsigned long long* E64, int32_t* E, int64_t 
 // Rp = 32 * Wn; the int8 side is [R][N] in logical site order
 int32_t launch_unpack_spins(const int8_t* spins, int8_t* out, int L, int Rp, int R,
                             int I_index, cudaStream_t st);
-int32_t launch_pack_spins(const int8_t* in, int8_t* spins, int L, int Rp, int R, int* bad,
-                          cudaStream_t st);
+// energies of int8 spins [I][n][N] (logical site order) added to E_out [I][n]; values other
+// than +-1 are counted in *bad
+int32_t launch_energy_direct(const int8_t* spins, const uint2* const* j6_ptrs, int I, int L, int n,
+                             unsigned long long* E_out, int* bad, cudaStream_t st);
 
 }  // namespace sg
