@@ -433,16 +433,16 @@ int32_t run_sa_group(const std::vector<int>& members, const sg_instance* const* 
     // SA keeps no per-sweep energies: the energy of every replica is computed once,
     // from the final spins.
     SG_RET(log.run(SG_KERNEL_INIT, cells, st, [&] { return launch_init_spins(spins, kp, I, L, Wn, R, st); }));
-    // Small lattices with unit couplings: every sweep in one launch, a word per thread-block
+    // Unit couplings, where it is faster: every sweep in one launch, a word per thread-block
     // cluster (cluster.cu).  Knob SG_SA_CLUSTER = 0 / 1 disables or forces it.
     const char* ck = getenv("SG_SA_CLUSTER");
-    int threads = 256;
-    int C = unit_j && S > 0 && !(ck && atoi(ck) == 0) ? sa_cluster_blocks(I, L, Wn, (int64_t)I * (N / 2) * R, &threads)
-                                                      : 0;
-    if (ck && atoi(ck) == 1 && unit_j && S > 0 && C == 0) C = sa_cluster_blocks(I, L, Wn, 0, &threads);
+    int threads = 0;
+    const int C = unit_j && S > 0 && !(ck && atoi(ck) == 0) ? sa_cluster_blocks(I, L, Wn, ck && atoi(ck) == 1, &threads)
+                                                            : 0;
     if (C > 0) {
         SG_RET(log.run(SG_KERNEL_SWEEP_CHUNK, (int64_t)I * N * R * S, st, [&] {
-            return launch_sa_cluster(spins, j1p, kp, d_thr.as<uint32_t>(), I, L, Wn, R, S, C, threads, st);
+            return launch_sa_cluster(spins, j1p, kp, d_thr.as<uint32_t>(), d_flag.as<int>() + 1, I, L, Wn, R, S, C,
+                                     threads, st);
         }));
     } else if (S >= kGraphMinSweeps) {
         // the kernel reads row *base + c of the whole [S][kThrRow] table

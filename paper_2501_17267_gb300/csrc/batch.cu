@@ -587,10 +587,21 @@ int32_t run_sa_planes(const std::vector<int>& members, const sg_instance* const*
         }
         *words_total = wo;
     };
-    auto lpt_order = [](const std::vector<double>& work) {
+    // Longest first.  In the cluster form (wg = 0) the small lattices come after the others, for
+    // single blocks to take (n_cluster: the ones before them) -- where there are enough of them
+    // to give every block one; fewer are better off with a whole cluster each.
+    int n_cluster = 0;
+    auto lpt_order = [&](int wg, const std::vector<Plane>& planes, const std::vector<double>& work) {
         std::vector<int> order(work.size());
         for (size_t q = 0; q < order.size(); ++q) order[q] = (int)q;
         std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return work[x] > work[y]; });
+        n_cluster = (int)order.size();
+        if (wg == 0) {
+            auto small = [&](int x) { return planes[x].L <= kListAloneL; };
+            if (std::count_if(order.begin(), order.end(), small) >= sms)
+                n_cluster = (int)(std::stable_partition(order.begin(), order.end(), [&](int x) { return !small(x); }) -
+                                  order.begin());
+        }
         return order;
     };
     // planes of a launch sit in shared memory when the largest of them fits
@@ -611,7 +622,8 @@ int32_t run_sa_planes(const std::vector<int>& members, const sg_instance* const*
     auto concurrency = [&](int wg) { return wg == 0 ? std::max(1, sms / Ccl) : blocks_for(wg); };
     auto sweep_launch = [&](int wg, const Plane* d_pl, const int* d_ord, int n, unsigned* d_next,
                             cudaStream_t s) -> int32_t {
-        if (wg == 0) return launch_sa_cluster_planes(d_pl, d_ord, n, d_next, Ccl, max_L, s);
+        // d_next: two plane counters, then the status word of the cluster form's bounded waits
+        if (wg == 0) return launch_sa_cluster_planes(d_pl, d_ord, n_cluster, n, d_next, Ccl, max_L, s);
         return launch_sa_planes(wg, d_pl, d_ord, n, d_next, unit, blocks_for(wg), s, smem_for(wg));
     };
 
@@ -629,7 +641,7 @@ int32_t run_sa_planes(const std::vector<int>& members, const sg_instance* const*
         cudaGetDeviceProperties(&prop, dev);
         std::ostringstream ks;
         ks << prop.name << "/" << sms << "/" << (unit ? "u" : "g") << "/smem" << smem_for(1) / 1024 << "/c" << Ccl
-           << "/t4";
+           << "/t5";
         for (auto& m : mix)
             ks << "/" << std::get<0>(m.first) << "x" << std::get<1>(m.first) << "x" << std::get<2>(m.first) << "x" << m.second;
         key = ks.str();
@@ -673,17 +685,17 @@ int32_t run_sa_planes(const std::vector<int>& members, const sg_instance* const*
                     pl.s_end = std::min(pl.S, trial_sweeps);
                     trial_work += (double)pl.L * pl.L * pl.L * 32 * width(wg) * pl.s_end;
                 }
-                const std::vector<int> order = lpt_order(work);
+                const std::vector<int> order = lpt_order(wg, planes, work);
                 SG_B(d_pl.alloc(sizeof(Plane) * planes.size(), st));
                 SG_B(d_ord.alloc(sizeof(int) * order.size(), st));
-                SG_B(d_next.alloc(sizeof(unsigned), st));
+                SG_B(d_next.alloc(3 * sizeof(unsigned), st));
                 SG_TRY_CUDA(cudaMemcpyAsync(d_pl.p, planes.data(), sizeof(Plane) * planes.size(), cudaMemcpyHostToDevice, st));
                 SG_TRY_CUDA(cudaMemcpyAsync(d_ord.p, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice, st));
                 SG_B(launch_planes_init(width(wg), static_cast<Plane*>(d_pl.p), (int)planes.size(), st));
                 const int conc = concurrency(wg);
                 double t_best = 1e300;
                 for (int rep = 0; rep < 2; ++rep) {
-                    SG_TRY_CUDA(cudaMemsetAsync(d_next.p, 0, sizeof(unsigned), st));
+                    SG_TRY_CUDA(cudaMemsetAsync(d_next.p, 0, 3 * sizeof(unsigned), st));
                     SG_TRY_CUDA(cudaStreamSynchronize(st));
                     const auto t0 = std::chrono::steady_clock::now();
                     SG_B(sweep_launch(wg, static_cast<Plane*>(d_pl.p), static_cast<int*>(d_ord.p),
@@ -718,11 +730,11 @@ int32_t run_sa_planes(const std::vector<int>& members, const sg_instance* const*
     Buf d_sp, d_pl, d_ord, d_next, d_E, d_outs, d_stage;
     SG_B(d_sp.alloc(words * 4, st));
     make_planes(WGm, static_cast<uint32_t*>(d_sp.p), &planes, &work, &words);
-    const std::vector<int> order = lpt_order(work);
+    const std::vector<int> order = lpt_order(WG, planes, work);
     const int n = (int)planes.size();
     SG_B(d_pl.alloc(sizeof(Plane) * n, st));
     SG_B(d_ord.alloc(sizeof(int) * n, st));
-    SG_B(d_next.alloc(sizeof(unsigned), st));
+    SG_B(d_next.alloc(3 * sizeof(unsigned), st));
     SG_B(d_E.alloc(sizeof(unsigned long long) * (size_t)n * 32 * WGm, st));
     // spin outputs: device targets directly, host targets through one staging area
     std::vector<int8_t*> outp(I, nullptr);
@@ -765,7 +777,7 @@ int32_t run_sa_planes(const std::vector<int>& members, const sg_instance* const*
         return SG_ECUDA;
     }
     auto device_work = [&](cudaStream_t s) -> int32_t {
-        SG_TRY_CUDA(cudaMemsetAsync(d_next.p, 0, sizeof(unsigned), s));
+        SG_TRY_CUDA(cudaMemsetAsync(d_next.p, 0, 3 * sizeof(unsigned), s));
         SG_TRY_CUDA(cudaMemsetAsync(d_E.p, 0, sizeof(unsigned long long) * (size_t)n * 32 * WGm, s));
         SG_B(launch_planes_init(WGm, static_cast<Plane*>(d_pl.p), n, s));
         if (timed) SG_TRY_CUDA(cudaEventRecord(ev[0], s));
@@ -805,6 +817,8 @@ int32_t run_sa_planes(const std::vector<int>& members, const sg_instance* const*
     }
 
     std::vector<unsigned long long> E((size_t)n * 32 * WGm);
+    int status = 0;
+    SG_TRY_CUDA(cudaMemcpyAsync(&status, static_cast<unsigned*>(d_next.p) + 2, sizeof(int), cudaMemcpyDeviceToHost, st));
     SG_TRY_CUDA(cudaMemcpyAsync(E.data(), d_E.p, sizeof(unsigned long long) * E.size(), cudaMemcpyDeviceToHost, st));
     for (int a = 0; a < I; ++a) {
         const sg_sa_result& o = outs[members[a]];
@@ -814,6 +828,10 @@ int32_t run_sa_planes(const std::vector<int>& members, const sg_instance* const*
                                         cudaMemcpyDeviceToHost, st));
     }
     SG_TRY_CUDA(cudaStreamSynchronize(st));
+    if (status != 0) {
+        set_error("a bounded device-side wait gave up (status %d)", status);
+        return SG_ETIMEOUT;
+    }
     {
         int64_t attempts = 0, cells = 0;
         for (int a = 0; a < I; ++a) {

@@ -1,24 +1,29 @@
-// cluster.cu -- simulated annealing (App. D.1) of small lattices with many replicas:
-// one launch runs every sweep, each word of 32 replicas on its own thread-block cluster.
+// cluster.cu -- simulated annealing (App. D.1) with every sweep in one launch: each word of
+// 32 replicas on its own thread-block cluster.
 //
 // A half sweep of a small lattice is too little work to pay for a launch, and a whole
 // lattice per block (batch.cu) leaves most SMs idle when an instance has few words.
-// Here cluster (word w, instance) of C blocks splits the lattice into C slabs of L / C
-// z-planes; block r keeps slab r of word w in its shared memory for the whole run.  The
-// sites of one colour read only sites of the other colour: x and y neighbours lie in
-// the block's own slab, z neighbours across a slab boundary in the next block's slab,
-// read through distributed shared memory.  A cluster barrier separates half sweeps.
-// Every attempt draws the same counters as the row kernel (site, sweep, word), so the
-// results are bit-identical to it and to the oracle.
+// Here cluster (word, instance) of C blocks splits the lattice into C slabs of L / C
+// z-planes, block r keeping slab r of the word in its shared memory for the whole run
+// (slab.cuh: the updates, and how the blocks exchange their faces).  Every attempt draws
+// the same counters as the row kernel (site, sweep, word), so the results are
+// bit-identical to it and to the oracle.
+//
+// One row of thresholds serves a whole sweep, which says beforehand how much a half sweep
+// has to do: at beta > 1.4 every threshold that can matter is below 2^24, a draw can only
+// accept when its leading byte is 0, and the byte-by-byte compare falls away; at
+// beta > 5.6 the thresholds are all 0 and there is nothing to draw.
 #include <cooperative_groups.h>
 #include <stdint.h>
 #include <stdlib.h>
 
 #include <algorithm>
 #include <cstdint>
+#include <map>
+#include <mutex>
+#include <tuple>
 
-#include "metropolis.cuh"
-#include "philox.cuh"
+#include "slab.cuh"
 #include "sg_internal.h"
 
 namespace cg = cooperative_groups;
@@ -26,19 +31,14 @@ namespace cg = cooperative_groups;
 namespace sg {
 namespace {
 
-// Single runs: 256 or 512 threads a block, chosen with the cluster size (sa_cluster_blocks).
-// Batches (planes of up to L = 48 per cluster, tens of words per thread per half sweep):
-// 768 threads per block measured fastest on the 512-instance uneven batch -- 1.95 s per
-// step against 2.10 at 512, 1.97 at 1024 and 2.89 at 256 -- although at 85 registers a
-// thread spills about 100 bytes: more warps hide the update's dependencies better.
-constexpr int kListBlock = 768;
-constexpr int kTieCap = 32;  // queued tie entries per warp
+constexpr int kListBlock = 512;  // threads a block of the batch form
 
 struct ClusterArgs {
     uint32_t* spins;                // [I][N][Wn] words, storage order
     const uint8_t* const* j1_ptrs;  // per instance: [N] coupling sign bits (all |J| = 1)
     const RunKeys* keys;            // [I]
     const uint32_t* thr;            // [S][kThrRow]
+    int* status;                    // SG_ETIMEOUT when a bounded wait gave up
     int L, Wn, R, S, C;             // side, words, replicas, sweeps, blocks per cluster
     uint32_t Hmagic;                // ceil(2^32 / (L / 2))
 };
@@ -61,157 +61,159 @@ struct PlaneRun {
     uint32_t Hmagic;              // ceil(2^32 / (L / 2))
 };
 
-// Called by every thread of every block of the cluster; slab: dynamic shared memory of
-// at least (L / C) * L * L words.  Ends with the plane written back and a cluster barrier.
-template <int NT>
-__device__ __forceinline__ void anneal_plane(const PlaneRun& p, const int C, uint32_t* slab, uint4* s_ties,
-                                             int* s_tie_n)
+// Shared state of a block, two sweeps' tables by sweep parity.
+struct Shared {
+    slab::Planes planes[2];
+    slab::Geometry geo;
+    uint32_t row[2][kThrRow];
+    int mode[2];
+    uint64_t bar[2];  // by colour: the neighbours' face words of that colour have arrived
+    int fail[2];      // by colour: a wait for that barrier gave up (read one half sweep later)
+};
+
+// Called by every thread of every block of the cluster once the barriers are initialised;
+// phase: the barriers' phase bits, kept from plane to plane.  Ends with the plane written
+// back.  Returns false when a wait gave up.
+template <class S>
+__device__ __forceinline__ bool anneal_plane(const PlaneRun& p, const int C, unsigned char* smem, Shared& sh,
+                                             uint32_t& phase)
 {
     cg::cluster_group cluster = cg::this_cluster();
-    const int r = (int)cluster.block_rank();
-    const int w = p.w;
-    const int L = p.L, H = L >> 1, LL = L * L;
-    const int zc = L / C;              // z-planes per slab
-    const int slab_words = zc * LL;
-    const int z0 = r * zc;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const RunKeys key = p.key;
-    const uint8_t* __restrict__ j1 = p.j1;
-    uint32_t* __restrict__ g = p.g;
-    // slabs of the blocks above (z0 + zc) and below (z0 - 1), periodic in z
-    const uint32_t* up = cluster.map_shared_rank(slab, (r + 1) % C);
-    const uint32_t* dn = cluster.map_shared_rank(slab, (r + C - 1) % C);
-    const uint32_t valid = word_valid_bits(p.R, w);
-    uint4* ties = s_ties + warp * kTieCap * 2;
-    const int items = zc * L * H;  // sites of one colour in the slab
+    const int r = C > 1 ? (int)cluster.block_rank() : 0;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, warps = blockDim.x >> 5;
+    const slab::Geometry& geo = sh.geo;
+    if (tid == 0) sh.geo.init(p.L, C, r, warps, p.Hmagic);
+    __syncthreads();
+    uint32_t* w = reinterpret_cast<uint32_t*>(smem) + geo.LL;
+    uint8_t* sgn = smem + slab::Geometry::words(p.L, C) * 4;
+    slab::load_slab(geo, p.g, p.stride, p.j1, w, sgn);
 
-    // geometry of slab item q (site j of slab row rl) in a half sweep of colour `colour`:
-    // its slab position, its six neighbours' (z neighbours in another block's slab when
-    // `zup` / `zdn`), its logical index and its coupling sign bits
-    struct Site {
-        int is, nb[6];
-        bool zup, zdn;
-        uint32_t i, sbits;
+    // Thresholds of sweep `sw` into the tables of its parity, by the last warp (lane k holds
+    // the row's entry k): lane 3 j + m makes plane j of k = 2 + 2 m, lanes 24 .. 26 lz.
+    const int src = 2 + 2 * (lane % 3), bit = 24 + (lane / 3) % 8;
+    const int slot = lane / 3 * 4 + lane % 3;  // of Planes: tp[j] = {x, y, z, -}, then lz
+    auto set_tables = [&](int sw, uint32_t entry) {
+        const int b = sw & 1;
+        const uint32_t t = __shfl_sync(slab::kAll, entry, src);
+        const unsigned any = __ballot_sync(slab::kAll, t != 0u), lead = __ballot_sync(slab::kAll, t >> 24 != 0u);
+        const uint32_t low = (t & 0xFFFFFFu) ? ~0u : 0u;
+        if (lane < 27) reinterpret_cast<uint32_t*>(&sh.planes[b])[slot] = lane < 24 ? 0u - ((t >> bit) & 1u) : low;
+        if (lane < kThrRow) sh.row[b][lane] = entry;
+        if (lane == 0) sh.mode[b] = !any ? slab::kNoDraws : !lead ? slab::kTailOnly : slab::kCompare;
     };
-    auto site_of = [&](int q, int colour) {
-        Site t;
-        const int rl = H == 1 ? q : (int)__umulhi((uint32_t)q, p.Hmagic);
-        const int j = q - rl * H;
-        const int zl = rl / L, y = rl - zl * L;
-        const int z = z0 + zl;
-        const int par = (y + z + colour) & 1;
-        const int rowoff = rl * L;
-        const int pos = par * H + j;
-        t.is = rowoff + pos;
-        const int ho = rowoff + (1 - par) * H;
-        t.nb[0] = ho + (j + par == H ? 0 : j + par);
-        t.nb[1] = ho + (j + par == 0 ? H - 1 : j + par - 1);
-        t.nb[2] = t.is + (y + 1 == L ? -(L - 1) * L : L);
-        t.nb[3] = t.is + (y == 0 ? (L - 1) * L : -L);
-        t.zup = zl + 1 >= zc;
-        t.zdn = zl == 0;
-        t.nb[4] = t.zup ? y * L + pos : t.is + LL;
-        t.nb[5] = t.zdn ? (zc - 1) * LL + y * L + pos : t.is - LL;
-        t.i = (uint32_t)((z * L + y) * L + 2 * j + par);
-        t.sbits = j1[t.i];
-        return t;
+    auto entry_of = [&](int sw) {
+        return lane < kThrRow && sw < p.s_end ? p.thr[(size_t)sw * kThrRow + lane] : 0u;
     };
-    // this thread's first item of each colour, fixed for the run
-    Site first0, first1;
-    if (tid < items) {
-        first0 = site_of(tid, 0);
-        first1 = site_of(tid, 1);
+    uint32_t entry = 0;  // last warp: the next sweep's row, loaded a sweep ahead of its use
+    if (warp == warps - 1) {
+        set_tables(p.s_begin, entry_of(p.s_begin));
+        entry = entry_of(p.s_begin + 1);
     }
-    // The draws of this thread's first item of a half sweep depend only on its site and
-    // the sweep, so they are computed while the cluster barrier before it completes.
-    uint32_t A0[8];
-    auto draws_ahead = [&](int sw, int colour) {
-        if (sw < p.s_end && tid < items) mp::lead_planes((colour ? first1 : first0).i, (uint32_t)sw, (uint32_t)w, key, A0);
-    };
 
-    for (int q = tid; q < slab_words; q += NT) slab[q] = g[(size_t)(z0 * LL + q) * p.stride];
-    if (tid < NT / 32) s_tie_n[tid] = 0;
-    cluster.barrier_arrive();
-    draws_ahead(p.s_begin, 0);
-    cluster.barrier_wait();  // every slab loaded before any block reads its neighbours'
+    __syncthreads();  // the slab is in place
+    S s(geo, w, sgn, reinterpret_cast<const uint4*>(smem + slab::smem_queue_offset(p.L, C)));
+    s.draws.k0 = p.key.k0;
+    s.draws.k1 = p.key.k1;
+    s.word = (uint32_t)p.w;
+    s.valid = word_valid_bits(p.R, p.w);
+    const uint32_t up = (uint32_t)(r + 1 == C ? 0 : r + 1), dn = (uint32_t)(r == 0 ? C - 1 : r - 1);
+    uint32_t up_w = 0, dn_w = 0, up_bar = 0, dn_bar = 0;
+    if (C > 1) {
+        up_w = slab::cluster_addr(s.w0, up) - s.w0;
+        dn_w = slab::cluster_addr(s.w0, dn) - s.w0;
+        up_bar = slab::cluster_addr(slab::smem_addr(&sh.bar[0]), up);
+        dn_bar = slab::cluster_addr(slab::smem_addr(&sh.bar[0]), dn);
+        cluster.sync();  // every block has loaded its halos before a neighbour pushes into them
+    } else {
+        __syncthreads();
+    }
 
-    for (int sw = p.s_begin; sw < p.s_end; ++sw) {
-        const uint32_t* thr = p.thr + (size_t)sw * kThrRow;  // the sweep's thresholds, k = 0 .. 15
-        uint32_t tp[24], lz[3];  // its threshold planes: the same for every replica
-        {
-            const uint32_t t2 = thr[2], t4 = thr[4], t6 = thr[6];
-#pragma unroll
-            for (int m = 0; m < 24; ++m)
-                tp[m] = mp::threshold_plane_bit(m < 8 ? t2 : m < 16 ? t4 : t6, m % 8) ? ~0u : 0u;
-            lz[0] = (t2 & 0xFFFFFFu) ? ~0u : 0u;
-            lz[1] = (t4 & 0xFFFFFFu) ? ~0u : 0u;
-            lz[2] = (t6 & 0xFFFFFFu) ? ~0u : 0u;
+    uint32_t A[S::kItems][8];
+    bool ok = true;
+    s.draws.set_sweep((uint32_t)p.s_begin, s.word);
+    s.first_draws(A);
+    for (int sw = p.s_begin; sw < p.s_end && ok; ++sw) {
+        const int b = sw & 1;
+        const int mode = sh.mode[b];
+        s.sweep = (uint32_t)sw;
+        s.planes = slab::smem_addr(&sh.planes[b]);
+        s.thr = sh.row[b];
+        if (warp == warps - 1) {  // the other parity's tables were last read before the barrier that ended sweep sw - 1
+            set_tables(sw + 1, entry);
+            entry = entry_of(sw + 2);
         }
-        // one half sweep of colour `colour`; `fst`: this thread's first item of that colour
-        auto half = [&](const int colour, const Site& fst) {
-            for (int q = tid; q < items; q += NT) {
-                const Site t = q == tid ? fst : site_of(q, colour);
-                const uint32_t self = slab[t.is];
-                uint32_t n[6];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) n[k] = slab[t.nb[k]];
-                n[4] = t.zup ? up[t.nb[4]] : slab[t.nb[4]];
-                n[5] = t.zdn ? dn[t.nb[5]] : slab[t.nb[5]];
-                uint32_t S[6];
-                mp::unit_signs(t.sbits, S);
-                uint32_t A[8];
-                if (q == tid) {
-#pragma unroll
-                    for (int m = 0; m < 8; ++m) A[m] = A0[m];
-                } else {
-                    mp::lead_planes(t.i, (uint32_t)sw, (uint32_t)w, key, A);
-                }
-                uint32_t flip, tie, c0, c1, c2;
-                mp::update_word_unit(self, n, S, valid, tp, A, &flip, &tie, &c0, &c1, &c2);
-                tie &= (c1 & lz[2]) | (~c1 & ((c0 & lz[1]) | (~c0 & lz[0])));  // the others reject
-                if (tie) {
-                    const int p = atomicAdd(&s_tie_n[warp], 1);
-                    if (p < kTieCap) {
-                        ties[2 * p] = make_uint4(t.i, (uint32_t)t.is, 0u, tie);
-                        ties[2 * p + 1] = make_uint4(c0, c1, self ^ flip, 0u);
-                    } else {  // list full: decide here
-                        flip |= mp::resolve_tie_bits(tie, c0, c1, thr, 0, t.i, (uint32_t)sw, (uint32_t)w, key.k0,
-                                                     key.k1);
-                    }
-                }
-                if (flip) slab[t.is] = self ^ flip;
+        // the end of a half sweep: the faces pushed, the block met, the neighbours' faces here
+        auto finish = [&](int colour) {
+            __syncthreads();
+            if (C > 1) {
+                if (sh.fail[colour ^ 1]) return false;  // set before this barrier, the same for every thread
+                if (!slab::mbar_wait(&sh.bar[colour], (phase >> colour) & 1u)) sh.fail[colour] = 1;
+                phase ^= 1u << colour;
             }
-            // this warp's ties, decided by its lanes together (a word has at most one
-            // entry, and its owner stored the entry's word: a blind store)
-            __syncwarp();
-            const int nt = min(s_tie_n[warp], kTieCap);
-            for (int e = lane; e < nt; e += 32) {
-                const uint4 t = ties[2 * e], u = ties[2 * e + 1];
-                const uint32_t acc =
-                    mp::resolve_tie_bits(t.w, u.x, u.y, thr, 0, t.x, (uint32_t)sw, (uint32_t)w, key.k0, key.k1);
-                if (acc) slab[t.y] = u.z ^ acc;
-            }
-            __syncwarp();
-            if (lane == 0) s_tie_n[warp] = 0;
-            // the half sweep is complete in every slab once all blocks have arrived
-            cluster.barrier_arrive();
-            if (colour == 0) draws_ahead(sw, 1);
-            else draws_ahead(sw + 1, 0);
-            cluster.barrier_wait();
+            return true;
         };
-        half(0, first0);
-        half(1, first1);
+        auto expect = [&](int colour) {
+            if (C > 1 && tid == 0) slab::mbar_expect(&sh.bar[colour], (uint32_t)geo.LL * 4u);
+        };
+        if constexpr (S::kResident) {
+            expect(0);
+            if (mode == slab::kCompare) s.template half<0, slab::kCompare, false, false>(A, true);
+            else if (mode == slab::kTailOnly) s.template half<0, slab::kTailOnly, false, false>(A, true);
+            else s.template half<0, slab::kNoDraws, false, false>(A, false);
+            s.template push_faces<0>(C == 1, up_w, dn_w, up_bar, dn_bar);
+            if (!(ok = finish(0))) break;
+            const bool next = sh.mode[b ^ 1] != slab::kNoDraws;
+            expect(1);
+            if (mode == slab::kCompare) s.template half<1, slab::kCompare, false, false>(A, next);
+            else if (mode == slab::kTailOnly) s.template half<1, slab::kTailOnly, false, false>(A, next);
+            else s.template half<1, slab::kNoDraws, false, false>(A, next);
+            s.template push_faces<1>(C == 1, up_w, dn_w, up_bar + 8u, dn_bar + 8u);
+            ok = finish(1);
+        } else {
+            for (int colour = 0; colour < 2 && ok; ++colour) {
+                expect(colour);
+                if (mode == slab::kCompare) s.template half<slab::kCompare, false, false>(colour, A[0]);
+                else if (mode == slab::kTailOnly) s.template half<slab::kTailOnly, false, false>(colour, A[0]);
+                else {
+                    s.template half<slab::kNoDraws, false, false>(colour, A[0]);
+                    if (colour == 1 && sh.mode[b ^ 1] != slab::kNoDraws) s.first_draws(A);
+                }
+                s.push_faces(colour, C == 1, up_w, dn_w, up_bar + 8u * colour, dn_bar + 8u * colour);
+                ok = finish(colour);
+            }
+        }
     }
-    for (int q = tid; q < slab_words; q += NT) g[(size_t)(z0 * LL + q) * p.stride] = slab[q];
-    cluster.sync();  // no block goes on (or leaves) while another may still read its slab
+    if (C > 1) {
+        __syncthreads();
+        ok = ok && !sh.fail[0] && !sh.fail[1];
+    }
+    const int n = geo.zc * geo.LL;
+    uint32_t* dst = p.g + (size_t)geo.z0 * geo.LL * p.stride;
+    if (ok)
+        for (int q = tid; q < n; q += blockDim.x) dst[(size_t)q * p.stride] = w[q];
+    __syncthreads();
+    return ok;
 }
 
-template <int NT>
-__global__ void __launch_bounds__(NT) sa_cluster_kernel(const ClusterArgs a)
+__device__ __forceinline__ void init_shared(Shared& sh)
 {
-    extern __shared__ uint32_t slab[];  // [L / C][L][L] words of this block's slab, storage order
-    __shared__ uint4 s_ties[(NT / 32) * kTieCap * 2];  // per warp: {site, local, -, tie}, {c0, c1, word, -}
-    __shared__ int s_tie_n[NT / 32];
+    if (threadIdx.x == 0) {
+        slab::mbar_init(&sh.bar[0]);
+        slab::mbar_init(&sh.bar[1]);
+        slab::mbar_init_fence();
+        sh.fail[0] = sh.fail[1] = 0;
+    }
+    __syncthreads();
+}
+
+// S: slab::Sweeper, or slab::Resident when a block has a thread for each of its x pairs and a
+// warp to spare for the tables.
+template <class S>
+__global__ void __launch_bounds__(S::kResident ? slab::kMaxThreads + 32 : slab::kMaxThreads, 1)
+sa_cluster_kernel(const ClusterArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ Shared sh;
     const int w = blockIdx.y, inst = blockIdx.z;
     PlaneRun p;
     p.g = a.spins + (size_t)inst * a.L * a.L * a.L * a.Wn + w;
@@ -225,32 +227,30 @@ __global__ void __launch_bounds__(NT) sa_cluster_kernel(const ClusterArgs a)
     p.s_begin = 0;
     p.s_end = a.S;
     p.Hmagic = a.Hmagic;
-    anneal_plane<NT>(p, a.C, slab, s_ties, s_tie_n);
+    init_shared(sh);
+    uint32_t phase = 0;
+    if (!anneal_plane<S>(p, a.C, smem, sh, phase) && threadIdx.x == 0) atomicExch(a.status, SG_ETIMEOUT);
+    if (a.C > 1) cg::this_cluster().sync();  // no block leaves while another may still push to it
 }
 
-// Persistent form for batches (batch.cu's planes of one word, [N][1]): clusters take
-// planes from `order` (longest first) through the counter `next` until none is left;
-// every plane's side is a multiple of C.
-// (Registers are not capped: one block per SM without spills measured 8 % faster on the
-// uneven-batch workload than two per SM with a 128-register cap.)
+// Persistent form for batches (batch.cu's planes of one word, [N][1]).  Clusters take planes
+// order[0 .. n_cluster) through the counter next[0] until none is left (every side a multiple
+// of C), then each block by itself planes order[n_cluster .. n) through next[1]: a small
+// lattice does not fill a cluster, its half sweep being a chain of latencies, and four of them
+// side by side take little longer than one.  next[2]: status word.
 __global__ void __launch_bounds__(kListBlock, 1) sa_cluster_list_kernel(const Plane* __restrict__ planes,
-                                                                 const int* __restrict__ order, int n,
-                                                                 unsigned* __restrict__ next, int C)
+                                                                        const int* __restrict__ order, int n_cluster,
+                                                                        int n, unsigned* __restrict__ next, int C)
 {
-    extern __shared__ uint32_t slab[];
-    __shared__ uint4 s_ties[(kListBlock / 32) * kTieCap * 2];
-    __shared__ int s_tie_n[kListBlock / 32];
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ Shared sh;
     __shared__ int s_item;
     cg::cluster_group cluster = cg::this_cluster();
     const int r = (int)cluster.block_rank();
-    for (;;) {
-        if (r == 0 && threadIdx.x == 0) {  // claim the next plane for the whole cluster
-            const int it = (int)atomicAdd(next, 1u);
-            for (int k = 0; k < C; ++k) *cluster.map_shared_rank(&s_item, k) = it;
-        }
-        cluster.sync();
-        const int it = s_item;
-        if (it >= n) break;
+    init_shared(sh);
+    uint32_t phase = 0;
+    bool ok = true;
+    auto run = [&](int it, int blocks) {
         const Plane& q = planes[order[it]];
         PlaneRun p;
         p.g = q.spins;
@@ -262,99 +262,58 @@ __global__ void __launch_bounds__(kListBlock, 1) sa_cluster_list_kernel(const Pl
         p.w = q.w0;
         p.R = q.R;
         p.s_begin = q.s_begin;
-        p.s_end = q.s_end;
+        p.s_end = ok ? q.s_end : q.s_begin;  // after a wait gave up: no more sweeps
         p.Hmagic = q.Hmagic;
-        anneal_plane<kListBlock>(p, C, slab, s_ties, s_tie_n);  // ends with a cluster barrier
+        bool done;
+        switch (slab::resident_items(slab::pairs_of(q.L, blocks), kListBlock)) {
+            case 1: done = anneal_plane<slab::Resident<1>>(p, blocks, smem, sh, phase); break;
+            case 2: done = anneal_plane<slab::Resident<2>>(p, blocks, smem, sh, phase); break;
+            default: done = anneal_plane<slab::Sweeper>(p, blocks, smem, sh, phase); break;
+        }
+        if (!done) {
+            ok = false;
+            if (threadIdx.x == 0) atomicExch(reinterpret_cast<int*>(next + 2), SG_ETIMEOUT);
+        }
+    };
+    for (;;) {
+        if (r == 0 && threadIdx.x == 0) {  // claim the next plane for the whole cluster
+            const int it = (int)atomicAdd(next, 1u);
+            for (int k = 0; k < C; ++k) *cluster.map_shared_rank(&s_item, k) = it;
+        }
+        cluster.sync();
+        const int it = s_item;
+        if (it >= n_cluster) break;
+        run(it, C);
+        cluster.sync();  // s_item is read in every block before it is written again
     }
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_item = n_cluster + (int)atomicAdd(next + 1, 1u);
+        __syncthreads();
+        const int it = s_item;
+        if (it >= n) break;
+        run(it, 1);
+    }
+    cluster.sync();  // no block leaves while rank 0 may still write its s_item
 }
 
 }  // namespace
 
-// Blocks per cluster for an SA run of I instances of side L with Wn words, or 0 when the
-// run is better served by the row kernel: a divisor C <= 8 of L whose slab fits shared
-// memory, the largest for which all I * Wn clusters are resident at once (as the driver
-// reports for this kernel, so that the run is one wave).  Knob SG_SA_CLUSTER_C forces C.
-const void* sa_cluster_fn(int threads)
+// The driver's answer depends on nothing but these arguments and the device, and asking costs
+// tens of microseconds a shape: it is kept (one entry a kernel and shape, a few hundred at most).
+int resident_clusters(const void* fn, int C, size_t smem, int threads)
 {
-    return threads == 512 ? (const void*)sa_cluster_kernel<512> : (const void*)sa_cluster_kernel<256>;
-}
-
-int sa_cluster_blocks(int I, int L, int Wn, int64_t half_sweep_attempts, int* threads)
-{
-    *threads = 256;
-    if (half_sweep_attempts > ((int64_t)1 << 24)) return 0;  // long half sweeps: the row kernel
-    int dev = 0, smem = 0, sms = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t clusters = (int64_t)I * Wn;
-    const char* e = getenv("SG_SA_CLUSTER_C");
-    const int forced = e ? atoi(e) : 0;
-    const char* et = getenv("SG_SA_CLUSTER_THREADS");
-    const int forced_t = et ? atoi(et) : 0;
-    // For each block size, the largest C whose clusters are all resident at once (one wave);
-    // of the two, the one with fewer rounds of items a thread times blocks an SM runs (a
-    // half sweep's length), ties to 256 threads.  Measured at L = 16 with 1024 replicas:
-    // 512 threads at C = 4 (one block an SM) 3.80 ms a run against 3.93 for 256 threads at
-    // C = 8 (two blocks on most SMs); one cluster at L = 4: 1.98 ms with 256, 2.03 with 512.
-    int bestC = 0, bestT = 256;
-    int64_t best_cost = INT64_MAX;
-    for (const int t : {256, 512}) {
-        if (forced_t && t != forced_t) continue;
-        for (int C = 8; C >= 1; --C) {
-            if (L % C || (forced && C != forced)) continue;
-            const size_t bytes = (size_t)(L / C) * L * L * 4;
-            // static shared memory: t / 32 warps' tie queues (32 entries of 32 bytes) and more
-            if (bytes + (size_t)t * 32 + 4096 > (size_t)smem) continue;
-            if (!forced) {
-                if (bytes > 48 * 1024 && cudaFuncSetAttribute(sa_cluster_fn(t), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                              (int)bytes) != cudaSuccess) {
-                    cudaGetLastError();
-                    continue;
-                }
-                cudaLaunchConfig_t cfg{};
-                cfg.gridDim = dim3(C, (unsigned)std::min<int64_t>(clusters, 65535), 1);
-                cfg.blockDim = dim3(t, 1, 1);
-                cfg.dynamicSmemBytes = bytes;
-                cudaLaunchAttribute attr[1];
-                attr[0].id = cudaLaunchAttributeClusterDimension;
-                attr[0].val.clusterDim.x = C;
-                attr[0].val.clusterDim.y = 1;
-                attr[0].val.clusterDim.z = 1;
-                cfg.attrs = attr;
-                cfg.numAttrs = 1;
-                int active = 0;
-                if (cudaOccupancyMaxActiveClusters(&active, sa_cluster_fn(t), &cfg) != cudaSuccess) {
-                    cudaGetLastError();
-                    continue;
-                }
-                if (active < clusters) continue;
-            }
-            const int64_t items = (int64_t)(L / C) * L * (L / 2);  // sites of one colour a block
-            const int64_t rounds = (items + t - 1) / t;
-            const int64_t per_sm = (clusters * C + sms - 1) / sms;
-            const int64_t cost = rounds * per_sm;
-            if (cost < best_cost) {
-                best_cost = cost;
-                bestC = C;
-                bestT = t;
-            }
-            break;
-        }
-    }
-    *threads = bestT;
-    return bestC;
-}
-
-namespace {
-// Resident clusters of C blocks with `smem` bytes each for `fn`, or 0.
-int active_clusters(const void* fn, int C, size_t smem, int threads)
-{
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    static std::mutex mu;
+    static std::map<std::tuple<int, const void*, int, size_t, int>, int> known;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
+    const auto key = std::make_tuple(dev, fn, C, smem, threads);
+    std::lock_guard<std::mutex> lock(mu);
+    const auto it = known.find(key);
+    if (it != known.end()) return it->second;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(C, 1, 1);
     cfg.blockDim = dim3(threads, 1, 1);
@@ -367,11 +326,103 @@ int active_clusters(const void* fn, int C, size_t smem, int threads)
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int active = 0;
-    if (cudaOccupancyMaxActiveClusters(&active, fn, &cfg) != cudaSuccess) {
+    if (!allow_shared(fn) || cudaOccupancyMaxActiveClusters(&active, fn, &cfg) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
+    if (known.size() < 4096) known.emplace(key, active);
     return active;
+}
+
+// Lets `fn` use as much dynamic shared memory as a block can have beside its static one.  (The
+// limit is always the same one, so that launches from several threads do not lower it under one
+// another.)
+bool allow_shared(const void* fn)
+{
+    int dev = 0, most = 0;
+    cudaFuncAttributes at{};
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaFuncGetAttributes(&at, fn) != cudaSuccess ||
+        cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)at.sharedSizeBytes) !=
+            cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return true;
+}
+
+namespace {
+// The kernel for a block of at most `threads` threads, and its threads: the resident forms get
+// a warp more, for the tables.
+const void* sa_cluster_fn(int L, int C, int threads)
+{
+    switch (slab::resident_items(slab::pairs_of(L, C), threads)) {
+        case 1: return (const void*)sa_cluster_kernel<slab::Resident<1>>;
+        case 2: return (const void*)sa_cluster_kernel<slab::Resident<2>>;
+        default: return (const void*)sa_cluster_kernel<slab::Sweeper>;
+    }
+}
+int sa_block_threads(int L, int C, int threads)
+{
+    const int64_t pairs = slab::pairs_of(L, C);
+    return slab::resident_threads(pairs, threads) + (slab::resident_items(pairs, threads) ? 32 : 0);
+}
+}  // namespace
+
+// Blocks per cluster (and the threads to plan a block with) for an SA run of I instances of
+// side L with Wn words, or 0 when the row kernel should run it.  Candidates are the divisors
+// C <= 8 of L whose slab fits shared memory; clusters that are not resident at once (as the
+// driver reports for the kernel) run in waves.  A half sweep's cycles, fitted to measurements
+// on a GB300 (us at 2.07 GHz), times the waves:
+//   resident blocks  750 + 400 per warp of pairs an SM partition holds (L = 4 on one block of
+//                    one warp 0.53, L = 16 with 1024 replicas on C = 4 blocks of 16 warps 1.2)
+//   other blocks     2000 + 300 per warp of items (20 x L = 50 on C = 5 12.8, L = 64 on C = 8 20.6)
+//   row kernels      6500 + 490 per warp of items over the whole GPU (18.2 and 5.2 for the same)
+// The fewest cycles win, fewer blocks among equals; L = 16 with 1024 replicas takes C = 4 (2.4
+// ms a run of 1000 sweeps against 5.1 at C = 2), L = 4 one block (1.05 ms against 1.20 at
+// C = 2 and 1.25 at C = 4).  force: a cluster form whatever the row kernel would take.
+// Knobs: SG_SA_CLUSTER_C forces C, SG_SA_CLUSTER_THREADS the threads.
+int sa_cluster_blocks(int I, int L, int Wn, bool force, int* threads)
+{
+    *threads = slab::kMaxThreads;
+    int dev = 0, smem = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t clusters = (int64_t)I * Wn;
+    const char* e = getenv("SG_SA_CLUSTER_C");
+    const int forced = e ? atoi(e) : 0;
+    const char* et = getenv("SG_SA_CLUSTER_THREADS");
+    const int t = et && atoi(et) >= 32 && atoi(et) <= slab::kMaxThreads ? atoi(et) / 32 * 32 : slab::kMaxThreads;
+    *threads = t;
+    const double row_items = (double)clusters * L * L * (L / 2) / 32.0;  // warps of items a half sweep
+    double best = force || forced ? 1e300 : 0.95 * (6500.0 + 490.0 * row_items / (4.0 * sms));
+    int bestC = 0;
+    for (int C = 1; C <= 8; ++C) {
+        if (L % C || (forced && C != forced)) continue;
+        const int bt = sa_block_threads(L, C, t);
+        const size_t bytes = slab::smem_bytes(L, C, bt);
+        if (bytes + 2048 > (size_t)smem) continue;
+        const int64_t active = resident_clusters(sa_cluster_fn(L, C, t), C, bytes, bt);
+        if (active < 1) continue;
+        const int64_t pairs = slab::pairs_of(L, C);
+        const int64_t waves = (clusters + active - 1) / active;
+        const int64_t per_sm = (std::min(clusters, active) * C + sms - 1) / sms;  // blocks on the busiest SM
+        const double warps = std::max(1.0, (double)per_sm * (double)((pairs + 31) / 32) / 4.0);
+        const double cost = waves * (slab::resident_items(pairs, t) ? 750.0 + 400.0 * warps : 2000.0 + 300.0 * warps);
+        if (cost < best) {
+            best = cost;
+            bestC = C;
+        }
+    }
+    return bestC;
+}
+
+namespace {
+// Shared memory of a block of the batch form: its slab of the largest lattice, or a whole small one.
+size_t sa_list_smem(int max_L, int C)
+{
+    return std::max(slab::smem_bytes(max_L, C, kListBlock), slab::smem_bytes(std::min(max_L, kListAloneL), 1, kListBlock));
 }
 }  // namespace
 
@@ -384,24 +435,24 @@ int sa_cluster_list_blocks(const int* Ls, int n, int max_L)
         bool ok = true;
         for (int k = 0; k < n && ok; ++k) ok = Ls[k] % C == 0;
         if (!ok) continue;
-        const size_t bytes = (size_t)(max_L / C) * max_L * max_L * 4;
-        if (bytes + 12 * 1024 > (size_t)smem) continue;
-        if (active_clusters((const void*)sa_cluster_list_kernel, C, bytes, kListBlock) > 0) return C;
+        const size_t bytes = sa_list_smem(max_L, C);
+        if (bytes + 2048 > (size_t)smem) continue;
+        if (resident_clusters((const void*)sa_cluster_list_kernel, C, bytes, kListBlock) > 0) return C;
     }
     return 0;
 }
 
-int32_t launch_sa_cluster_planes(const Plane* d_planes, const int* d_order, int n, unsigned* d_next, int C,
-                                 int max_L, cudaStream_t st)
+int32_t launch_sa_cluster_planes(const Plane* d_planes, const int* d_order, int n_cluster, int n, unsigned* d_next,
+                                 int C, int max_L, cudaStream_t st)
 {
-    const size_t smem = (size_t)(max_L / C) * max_L * max_L * 4;
-    const int clusters = active_clusters((const void*)sa_cluster_list_kernel, C, smem, kListBlock);
+    const size_t smem = sa_list_smem(max_L, C);
+    const int clusters = resident_clusters((const void*)sa_cluster_list_kernel, C, smem, kListBlock);
     if (clusters < 1) {
         set_error("sa_cluster_list_kernel: no cluster of %d blocks with %zu bytes fits", C, smem);
         return SG_ECUDA;
     }
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(C * std::min(clusters, n), 1, 1);
+    cfg.gridDim = dim3(C * std::min(clusters, std::max(n_cluster, (n - n_cluster + C - 1) / C)), 1, 1);
     cfg.blockDim = dim3(kListBlock, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
@@ -412,7 +463,7 @@ int32_t launch_sa_cluster_planes(const Plane* d_planes, const int* d_order, int 
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, sa_cluster_list_kernel, d_planes, d_order, n, d_next, C);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, sa_cluster_list_kernel, d_planes, d_order, n_cluster, n, d_next, C);
     if (e != cudaSuccess) {
         cudaGetLastError();
         set_error("sa_cluster_list_kernel launch failed: %s", cudaGetErrorString(e));
@@ -422,10 +473,10 @@ int32_t launch_sa_cluster_planes(const Plane* d_planes, const int* d_order, int 
 }
 
 int32_t launch_sa_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const RunKeys* keys, const uint32_t* thr,
-                          int I, int L, int Wn, int R, int S, int C, int threads, cudaStream_t st)
+                          int* status, int I, int L, int Wn, int R, int S, int C, int threads, cudaStream_t st)
 {
-    if (threads != 256 && threads != 512) {
-        set_error("sa_cluster_kernel: %d threads a block (256 or 512)", threads);
+    if (threads < 32 || threads > slab::kMaxThreads || threads % 32) {
+        set_error("sa_cluster_kernel: %d threads a block (a multiple of 32 up to %d)", threads, slab::kMaxThreads);
         return SG_EINVAL;
     }
     ClusterArgs a{};
@@ -433,6 +484,7 @@ int32_t launch_sa_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const Ru
     a.j1_ptrs = j1_ptrs;
     a.keys = keys;
     a.thr = thr;
+    a.status = status;
     a.L = L;
     a.Wn = Wn;
     a.R = R;
@@ -440,11 +492,10 @@ int32_t launch_sa_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const Ru
     a.C = C;
     const int H = L / 2;
     a.Hmagic = H == 1 ? 0u : (uint32_t)((0x100000000ull + (uint64_t)H - 1) / (uint64_t)H);
-    const size_t smem = (size_t)(L / C) * L * L * 4;
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(sa_cluster_fn(threads), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-            cudaSuccess) {
-        cudaGetLastError();
+    const void* fn = sa_cluster_fn(L, C, threads);
+    threads = sa_block_threads(L, C, threads);
+    const size_t smem = slab::smem_bytes(L, C, threads);
+    if (smem > 48 * 1024 && !allow_shared(fn)) {
         set_error("sa_cluster_kernel: cannot use %zu bytes of shared memory", smem);
         return SG_ECUDA;
     }
@@ -460,8 +511,8 @@ int32_t launch_sa_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const Ru
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = threads == 512 ? cudaLaunchKernelEx(&cfg, sa_cluster_kernel<512>, a)
-                                         : cudaLaunchKernelEx(&cfg, sa_cluster_kernel<256>, a);
+    void* args[] = {&a};
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
     if (e != cudaSuccess) {
         cudaGetLastError();
         set_error("sa_cluster_kernel launch failed: %s", cudaGetErrorString(e));

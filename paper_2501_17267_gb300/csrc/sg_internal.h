@@ -190,19 +190,28 @@ int32_t launch_sweep_rows_pt(int8_t* spins, const uint2* const* j6_ptrs,
                              bool unit_j, int I, int L, int Wn, int K, uint32_t sweep, int colour,
                              const ExchangeArgs* xch, unsigned* done, bool* fused, cudaStream_t st,
                              const uint32_t* sweep_base = nullptr, int* status = nullptr, int sms = 0);
-// cluster.cu: SA of small lattices, all sweeps in one launch, one thread-block cluster of C
-// blocks per (word, instance); sa_cluster_blocks gives C and the threads a block (256 or
-// 512), or 0 when the row kernel should run instead (long half sweeps, slabs too large, or
-// more clusters than fit at once).
-int sa_cluster_blocks(int I, int L, int Wn, int64_t half_sweep_attempts, int* threads);
+// Clusters of C blocks with `smem` bytes of dynamic shared memory each that the device keeps
+// resident at once for kernel `fn` (0: none, or the shape is refused); allow_shared raises the
+// kernel's limit of dynamic shared memory to the most a block can have.
+int resident_clusters(const void* fn, int C, size_t smem, int threads);
+bool allow_shared(const void* fn);
+
+// cluster.cu: SA with all sweeps in one launch, one thread-block cluster of C blocks per
+// (word, instance); sa_cluster_blocks gives C and the threads to plan a block with, or 0 when
+// the row kernel should run instead (its estimate is shorter, unless `force`; slabs too large,
+// or more clusters than fit at once).
+int sa_cluster_blocks(int I, int L, int Wn, bool force, int* threads);
 int32_t launch_sa_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const RunKeys* keys,
-                          const uint32_t* thr /* [S][kThrRow] */, int I, int L, int Wn, int R, int S, int C,
-                          int threads, cudaStream_t st);
+                          const uint32_t* thr /* [S][kThrRow] */, int* status, int I, int L, int Wn, int R, int S,
+                          int C, int threads, cudaStream_t st);
 // The persistent cluster form for batches of one-word planes (batch.cu): C for planes of
 // sides Ls (every side a multiple of C, the slab of the largest fitting), or 0.
 int sa_cluster_list_blocks(const int* Ls, int n, int max_L);
-int32_t launch_sa_cluster_planes(const Plane* d_planes, const int* d_order, int n, unsigned* d_next, int C,
-                                 int max_L, cudaStream_t st);
+// Planes order[0 .. n_cluster) go to clusters, the others, of sides up to kListAloneL, to
+// single blocks; d_next: two zeroed counters and the status word.
+constexpr int kListAloneL = 16;
+int32_t launch_sa_cluster_planes(const Plane* d_planes, const int* d_order, int n_cluster, int n, unsigned* d_next,
+                                 int C, int max_L, cudaStream_t st);
 // fragment.cu: the fragment meta-heuristic's waves (one launch per wave) on [I][N] int8 spins
 // (0 = not fixed yet; all fixed on return), thr: [S][kThrRow] geometric schedule.
 int32_t launch_fragment_waves(int8_t* spins, const uint2* const* j6_ptrs, const RunKeys* keys, const uint32_t* thr,
