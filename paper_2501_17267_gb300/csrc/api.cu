@@ -612,11 +612,14 @@ int32_t run_pt_group(const std::vector<int>& members, const sg_instance* const* 
     size_t coop_smem = 0;
     std::vector<int> cplan;
     if (unit_j && Wn == 1 && S > 0 && pt_coop_wanted(I, L, K)) cplan = pt_coop_plan(I, L, K, &coop_blocks, &coop_smem);
-    const int Ccl = cplan.empty() && unit_j && Wn == 1 && S > 0 ? pt_cluster_blocks(I, L, K) : 0;
-    int Mh = 0, side_sms = 0;
-    const int Chy = cplan.empty() && Ccl == 0 && unit_j && Wn == 1 && S >= kGraphMinSweeps
-                        ? pt_cluster_split(I, L, K, &Mh, &side_sms)
-                        : 0;
+    double t_wave = 0, t_split = 0;
+    int Ccl = cplan.empty() && unit_j && Wn == 1 && S > 0 ? pt_cluster_blocks(I, L, K, &t_wave) : 0;
+    int Mh = 0, side_sms = 0, Chy = 0;
+    // (a split may beat one wave of smaller clusters: 16 instances at L = 48 take 8 blocks each
+    // for 15 of them rather than 6 for all)
+    if (cplan.empty() && unit_j && Wn == 1 && S >= kGraphMinSweeps && (Ccl == 0 || t_wave > 0))
+        Chy = pt_cluster_split(I, L, K, &Mh, &side_sms, &t_split);
+    if (Ccl > 0 && Chy > 0) (t_split < t_wave ? Ccl : Chy) = 0;
     if (!cplan.empty()) {
         DevBuf d_cflags, d_csums, d_cabort, d_carr, d_cpub, d_cplan;
         SG_RET(d_cflags.alloc(sizeof(int) * (size_t)coop_blocks, st));
@@ -630,7 +633,7 @@ int32_t run_pt_group(const std::vector<int>& members, const sg_instance* const* 
         const CoopScratch cs{d_cflags.as<int>(), d_csums.as<int>(), d_cabort.as<int>(), d_carr.as<int>(),
                              d_cpub.as<uint32_t>(), d_cplan.as<int>()};
         const ExchangeTablesDev xd{d_xtab.as<uint32_t>(), d_xoff.as<uint32_t>(), d_xlen.as<uint32_t>(),
-                                   d_xtail.as<uint32_t>()};
+                                   d_xtail.as<uint32_t>(), xt.tab.size()};
         const long long limit = wait_limit();
         for (int s0 = 0; s0 < S; s0 += kClusterChunkSweeps) {
             const int s1 = std::min(S, s0 + kClusterChunkSweeps);
@@ -640,15 +643,13 @@ int32_t run_pt_group(const std::vector<int>& members, const sg_instance* const* 
             }));
         }
     } else if (Ccl > 0) {
-        bool aligned = true;
-        for (int a = 0; a < I; ++a) aligned &= (reinterpret_cast<uintptr_t>(jp[I + a]) & 15u) == 0;
         const ExchangeTablesDev xd{d_xtab.as<uint32_t>(), d_xoff.as<uint32_t>(), d_xlen.as<uint32_t>(),
-                                   d_xtail.as<uint32_t>()};
+                                   d_xtail.as<uint32_t>(), xt.tab.size()};
         for (int s0 = 0; s0 < S; s0 += kClusterChunkSweeps) {
             const int s1 = std::min(S, s0 + kClusterChunkSweeps);
             SG_RET(log.run(SG_KERNEL_SWEEP_CHUNK, (int64_t)I * N * K * (s1 - s0), st, [&] {
                 return launch_pt_cluster(spins, j1p, kp, d_thr.as<uint32_t>(), perm, inv, E, acc, minE, xd,
-                                         d_flag.as<int>() + 1, I, L, K, Ccl, s0, s1, aligned, st);
+                                         d_flag.as<int>() + 1, I, L, K, Ccl, s0, s1, st);
             }));
         }
     } else if (Chy > 0) {
@@ -675,15 +676,13 @@ int32_t run_pt_group(const std::vector<int>& members, const sg_instance* const* 
         SG_TRY_CUDA(cudaStreamCreateWithPriority(&sd.side, cudaStreamNonBlocking, prio_hi));
         SG_TRY_CUDA(cudaEventRecord(sd.fork, st));
         SG_TRY_CUDA(cudaStreamWaitEvent(sd.side, sd.fork, 0));
-        bool aligned = true;
-        for (int a = 0; a < Mh; ++a) aligned &= (reinterpret_cast<uintptr_t>(jp[I + a]) & 15u) == 0;
         const ExchangeTablesDev xd{d_xtab.as<uint32_t>(), d_xoff.as<uint32_t>(), d_xlen.as<uint32_t>(),
-                                   d_xtail.as<uint32_t>()};
+                                   d_xtail.as<uint32_t>(), xt.tab.size()};
         for (int s0 = 0; s0 < S; s0 += kClusterChunkSweeps) {
             const int s1 = std::min(S, s0 + kClusterChunkSweeps);
             SG_RET(log.run(SG_KERNEL_SWEEP_CHUNK, (int64_t)Mh * N * K * (s1 - s0), sd.side, [&] {
                 return launch_pt_cluster(spins, j1p, kp, d_thr.as<uint32_t>(), perm, inv, E, acc, minE, xd,
-                                         d_flag.as<int>() + 1, Mh, L, K, Chy, s0, s1, aligned, sd.side);
+                                         d_flag.as<int>() + 1, Mh, L, K, Chy, s0, s1, sd.side);
             }));
         }
         const size_t o = (size_t)Mh;

@@ -3,24 +3,19 @@
 // shared memory for the whole chunk.
 //
 // Cluster `inst` of C blocks splits the L^3 lattice of its instance into C z-slabs of
-// L / C planes; block r keeps slab r (one 32-bit word of 32 slots per site, storage
-// order) and the slab's coupling sign bytes in shared memory.  Both are brought in at
-// the start of the launch by bulk asynchronous copies (cp.async.bulk, completion on an
-// mbarrier whose wait is bounded) and the spins are written back at the end; in
-// between, nothing but the exchange tables is read from global memory.  A half sweep
-// reads only sites of the other colour: x and y neighbours lie in the block's own slab,
-// z neighbours across a slab boundary in the next block's slab (distributed shared
-// memory).  A cluster barrier separates the two half sweeps of a sweep and the sweeps.
+// L / C planes, one 32-bit word of 32 slots per site (slab.cuh: the updates, and how the
+// blocks exchange their faces); the spins are written back at the end.
 //
 // Energies and the exchange.  Each bond joins a colour-0 and a colour-1 site, so the
 // colour-1 half sweep sums every slot's energy afresh (6 - 2c per site for unit
 // couplings, c the satisfied count after the update), in bit-sliced counters per
-// thread reduced through a warp bit transpose.  Every block adds its sums into block 0's
-// shared memory (distributed atomics, one buffer per sweep parity); after the barrier
-// that ends the sweep every block reads the totals and decides the exchange itself --
-// the same integer decisions from the same draws -- so its slot-to-rung map and its
-// threshold planes are ready for the next sweep without another barrier.  Block 0
-// clears a parity's buffer one sweep later, when every block has read it.
+// thread reduced through a warp bit transpose.  Every block pushes its 32 sums to every
+// block of the cluster (st.async, two buffers by sweep parity, each with its own
+// barrier), and every warp of every block decides the exchange itself -- the same integer
+// decisions from the same draws -- so that it can make its share of the next sweep's
+// threshold planes at once; one block barrier then starts the next sweep.  The exchange
+// thresholds are kept in shared memory where they fit, since a lookup of them lies on the
+// path of every sweep.
 //
 // Every attempt draws the same counters as the row kernel (site, sweep, word) and the
 // exchange the same counters as the stand-alone exchange (pair, sweep), so results are
@@ -30,10 +25,9 @@
 #include <stdlib.h>
 
 #include <algorithm>
+#include <atomic>
 
-#include "metropolis.cuh"
-#include "philox.cuh"
-#include "ptslab.cuh"
+#include "slab.cuh"
 #include "sg_internal.h"
 
 namespace cg = cooperative_groups;
@@ -41,10 +35,7 @@ namespace cg = cooperative_groups;
 namespace sg {
 namespace {
 
-using pts::kThreads;
-using pts::kWarps;
-// bounded waits: iterations of mbarrier.try_wait (each may suspend the thread briefly)
-constexpr int kWaitSpins = 1 << 22;
+constexpr int kThreads = slab::kMaxThreads;
 
 struct PtcArgs {
     uint32_t* spins;                // [I][N] words (slots 0..31 of a site), storage order
@@ -63,216 +54,244 @@ struct PtcArgs {
     int* status;                    // SG_ETIMEOUT when a bounded wait gave up
     int L, K, C, s_begin, s_end;
     const uint32_t* sweep_base;     // if set, sweeps run from *sweep_base + s_begin to *sweep_base + s_end
-    uint32_t Hmagic, Lmagic;        // ceil(2^32 / (L / 2)), ceil(2^32 / L)
-    int bulk;                       // slabs staged by bulk copies (else by plain loads)
-    int bulk_signs;                 // the sign slab is 16-byte aligned: bulk copy (else plain loads)
+    uint32_t Hmagic;                // ceil(2^32 / (L / 2))
+    int xwords;                     // words of xtab held in shared memory (0: read from global memory)
 };
 
-// ---- mbarrier and bulk-copy primitives (PTX, sm_90 and later) ----
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// Shared state of a block.
+struct PtShared {
+    slab::Planes planes;
+    slab::Geometry geo;
+    uint32_t rthr[32 * kThrRow];  // per rung: its threshold row
+    int E[32];                    // the block's energy sums of a colour-1 half sweep
+    int Epart[2][slab::kMaxC][32];  // by sweep parity: every block's sums
+    uint8_t rung[32];             // slot -> rung
+    uint8_t inverse[kThreads / 32][32];  // a warp's scratch: slot -> rung
+    uint32_t xoff[32], xlen[32], xtail[32];
+    uint64_t bar[2];              // by colour: the neighbours' face words have arrived
+    uint64_t ebar[2];             // by sweep parity: every block's energy sums have arrived
+    int fail[2];                  // by colour: a wait gave up (read one half sweep later)
+};
 
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
-                 : "memory");
-}
-
-// global -> this block's shared memory, completion counted on `bar` (16-byte aligned
-// addresses, size a multiple of 16)
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar)
-{
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_addr(dst)),
-        "l"(src), "r"(bytes), "r"(smem_addr(bar))
-        : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity)
-{
-    uint32_t ok = 0;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_addr(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Waits for phase `parity` of `bar`, giving up after kWaitSpins tries.
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity)
-{
-    for (int it = 0; it < kWaitSpins; ++it)
-        if (mbar_try_wait(bar, parity)) return true;
-    return false;
-}
-
+// S: slab::Sweeper, or slab::Resident when a block has a thread for each of its x pairs.
+template <class S>
 __global__ void __launch_bounds__(kThreads, 1) pt_cluster_kernel(const PtcArgs a)
 {
-    extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ pts::Shared sh;
-    __shared__ int s_Etot[2][32];  // block 0: the cluster's sums, by sweep parity
-    __shared__ int s_fail;
-    __shared__ __align__(8) uint64_t s_bar;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ PtShared sh;
 
     cg::cluster_group cluster = cg::this_cluster();
     const int C = a.C;
-    const int r = (int)cluster.block_rank();
+    const int r = C > 1 ? (int)cluster.block_rank() : 0;
     const int inst = blockIdx.x / C;
-    const int L = a.L, H = L >> 1, LL = L * L, K = a.K;
-    const int zc = L / C, z0 = r * zc;
-    const int slab_words = zc * LL;
-    const int items = zc * L * H;  // sites of one colour in the slab
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int K = a.K;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, threads = blockDim.x, warps = threads >> 5;
     const RunKeys key = a.keys[inst];
-    const uint32_t valid = pts::valid_bits(K);
+    const slab::Geometry& geo = sh.geo;
+    if (tid == 0) sh.geo.init(a.L, C, r, warps, a.Hmagic);
+    __syncthreads();
+    uint32_t* w = reinterpret_cast<uint32_t*>(smem) + geo.LL;
+    uint8_t* sgn = smem + slab::Geometry::words(a.L, C) * 4;
+    uint32_t* g = a.spins + (size_t)inst * geo.LL * a.L;
+    slab::load_slab(geo, g, 1, a.j1_ptrs[inst], w, sgn);
+    uint32_t* xtab_s = reinterpret_cast<uint32_t*>(smem + slab::smem_bytes(a.L, C, threads));
+    for (int q = tid; q < a.xwords; q += threads) xtab_s[q] = a.xtab[q];
+    const uint32_t* xtab = a.xwords ? xtab_s : a.xtab;
 
-    uint32_t* slab = reinterpret_cast<uint32_t*>(smem);
-    uint8_t* sgn = smem + (size_t)slab_words * 4;  // [zc][L][L] sign bytes, logical order
-    uint4* s_ties = reinterpret_cast<uint4*>(smem + (((size_t)slab_words * 5 + 15) & ~(size_t)15));
-    uint32_t* g = a.spins + (size_t)inst * LL * L + (size_t)z0 * LL;
-    const uint8_t* j1 = a.j1_ptrs[inst] + (size_t)z0 * LL;
-
-    // ---- stage the slab and its coupling signs in shared memory ----
-    if (tid == 0) {
-        s_fail = 0;
-        if (a.bulk) {
-            mbar_init(&s_bar, 1);
-            const uint32_t sp_bytes = (uint32_t)slab_words * 4u;
-            const uint32_t sg_bytes = a.bulk_signs ? (uint32_t)slab_words : 0u;
-            mbar_expect_tx(&s_bar, sp_bytes + sg_bytes);
-            bulk_load(slab, g, sp_bytes, &s_bar);
-            if (sg_bytes) bulk_load(sgn, j1, sg_bytes, &s_bar);
-        }
-    }
-    if (!a.bulk)
-        for (int q = tid; q < slab_words; q += kThreads) slab[q] = g[q];
-    if (!a.bulk || !a.bulk_signs)
-        for (int q = tid; q < slab_words; q += kThreads) sgn[q] = j1[q];
-    pts::load_state(sh, a.rung_of_slot + (size_t)inst * 32, a.slot_of_rung + (size_t)inst * K, a.thr, K,
-                    a.minE[inst], tid);
+    // slot maps and thresholds; a lane is a slot or a rung.  slot: this rung's slot, in every
+    // warp's own registers.
+    int slot = lane < K ? a.slot_of_rung[(size_t)inst * K + lane] : lane;
+    int rung = a.rung_of_slot[(size_t)inst * 32 + lane];
+    for (int q = tid; q < K * kThrRow; q += threads) sh.rthr[q] = a.thr[q];
     if (tid < 32) {
-        s_Etot[0][tid] = 0;
-        s_Etot[1][tid] = 0;
+        sh.rung[tid] = (uint8_t)rung;
+        sh.E[tid] = 0;
+        if (tid + 1 < K) {
+            sh.xoff[tid] = a.xoff[tid];
+            sh.xlen[tid] = a.xlen[tid];
+            sh.xtail[tid] = a.xtail[tid];
+        }
     }
-    __syncthreads();  // mbarrier initialised before any thread waits on it
-    if (a.bulk && !mbar_wait_bounded(&s_bar, 0)) s_fail = 1;
-    pts::build_thresholds(sh, warp, lane);
-    // Every block's slab is in place (and every block's failure flag set) before any block
-    // reads a neighbour's slab.
-    cluster.sync();
-    int fail = 0;
-    for (int q = 0; q < C; ++q) fail |= *cluster.map_shared_rank(&s_fail, q);
-    if (fail && tid == 0) atomicExch(a.status, SG_ETIMEOUT);
-
-    // slabs of the blocks above (z0 + zc) and below (z0 - 1), periodic in z
-    const uint32_t* up = cluster.map_shared_rank(slab, (r + 1) % C);
-    const uint32_t* dn = cluster.map_shared_rank(slab, (r + C - 1) % C);
-    int* Etot0 = cluster.map_shared_rank(&s_Etot[0][0], 0);
-    const bool uniform = items % kThreads == 0;  // every lane of a warp has the same item count
-
-    // item q of a colour: its site, its words (z neighbours in another block's slab at the
-    // slab's faces) and its draws
-    auto fetch = [&](int q, int colour, pts::Work& w, const pts::Updater& u) {
-        const int rl = H == 1 ? q : (int)__umulhi((uint32_t)q, a.Hmagic);  // slab row
-        const int j = q - rl * H;
-        const int zl = (int)__umulhi((uint32_t)rl, a.Lmagic), y = rl - zl * L;
-        const int par = (y + z0 + zl + colour) & 1;
-        const int rowoff = rl * L;
-        const int pos = par * H + j;
-        const int is = rowoff + pos;
-        const int ho = rowoff + (1 - par) * H;
-        w.is = is;
-        w.i = (uint32_t)(z0 * LL + rowoff + 2 * j + par);
-        w.self = slab[is];
-        w.n[0] = slab[ho + (j + par == H ? 0 : j + par)];
-        w.n[1] = slab[ho + (j + par == 0 ? H - 1 : j + par - 1)];
-        w.n[2] = slab[is + (y + 1 == L ? -(L - 1) * L : L)];
-        w.n[3] = slab[is + (y == 0 ? (L - 1) * L : -L)];
-        w.n[4] = zl + 1 == zc ? up[y * L + pos] : slab[is + LL];
-        w.n[5] = zl == 0 ? dn[(zc - 1) * LL + y * L + pos] : slab[is - LL];
-        w.sbits = sgn[rowoff + 2 * j + par];
-        u.draws(w);
-    };
-    // one half sweep of `colour` over this block's slab: items q = tid, tid + kThreads, ...
-    auto half = [&](const int colour, uint32_t sweep) {
-        pts::Updater u(sh, slab, s_ties, key, valid, sweep, tid, colour == 1);
-        int m = 0;
-        for (int q = tid; q < items; q += kThreads) {
-            pts::Work w;
-            fetch(q, colour, w, u);
-            u.update(w);
-            if (uniform && ++m == pts::kCheckEvery) {
-                m = 0;
-                u.maybe_resolve();
-            }
-        }
-        u.resolve();
-        if (colour == 1) {
-            u.energy_to_block();
-            __syncthreads();
-            if (tid < 32) {  // the block's sums into block 0's buffer of this sweep's parity
-                atomicAdd(&Etot0[(sweep & 1u) * 32 + tid], sh.E[tid]);
-                sh.E[tid] = 0;
-            }
+    if (tid == 0) {
+        slab::mbar_init(&sh.bar[0]);
+        slab::mbar_init(&sh.bar[1]);
+        slab::mbar_init(&sh.ebar[0]);
+        slab::mbar_init(&sh.ebar[1]);
+        slab::mbar_init_fence();
+        sh.fail[0] = sh.fail[1] = 0;
+    }
+    int minE = a.minE[inst];
+    uint32_t accepted = 0;  // first warp, by the pair's lower rung
+    __syncthreads();
+    // this warp's share of the threshold planes: planes of the slots' leading bytes, then lz
+    auto build_planes = [&]() {
+        const uint32_t* row = sh.rthr + rung * kThrRow;
+        const uint32_t t2 = row[2], t4 = row[4], t6 = row[6];
+        for (int j = warp; j < 9; j += warps) {
+            const uint32_t mask = j < 8 ? 1u << (24 + j) : 0xFFFFFFu;
+            const uint32_t p2 = __ballot_sync(slab::kAll, (t2 & mask) != 0u), p4 = __ballot_sync(slab::kAll, (t4 & mask) != 0u),
+                           p6 = __ballot_sync(slab::kAll, (t6 & mask) != 0u);
+            if (lane == 0) *(j < 8 ? &sh.planes.tp[j] : &sh.planes.lz) = make_uint4(p2, p4, p6, 0u);
         }
     };
+    build_planes();
+
+    __syncthreads();  // the slab is in place
+    S s(geo, w, sgn, reinterpret_cast<const uint4*>(smem + slab::smem_queue_offset(a.L, C)));
+    s.planes = slab::smem_addr(&sh.planes);
+    s.thr = sh.rthr;
+    s.rung = sh.rung;
+    s.E = sh.E;
+    s.draws.k0 = key.k0;
+    s.draws.k1 = key.k1;
+    s.word = 0u;
+    s.valid = K >= 32 ? 0xFFFFFFFFu : (1u << K) - 1u;
+    const uint32_t up = (uint32_t)(r + 1 == C ? 0 : r + 1), dn = (uint32_t)(r == 0 ? C - 1 : r - 1);
+    uint32_t up_w = 0, dn_w = 0, up_bar = 0, dn_bar = 0;
+    if (C > 1) {
+        up_w = slab::cluster_addr(s.w0, up) - s.w0;
+        dn_w = slab::cluster_addr(s.w0, dn) - s.w0;
+        up_bar = slab::cluster_addr(slab::smem_addr(&sh.bar[0]), up);
+        dn_bar = slab::cluster_addr(slab::smem_addr(&sh.bar[0]), dn);
+        // every block has loaded its halos and set up its barriers before a neighbour pushes
+        cluster.sync();
+    } else {
+        __syncthreads();
+    }
 
     // a sweep base in device memory lets a captured graph replay the launch for later sweeps
     const uint32_t sb = a.sweep_base ? *a.sweep_base : 0u;
     const uint32_t s_end = sb + (uint32_t)a.s_end;
-    if (!fail) {
-        for (uint32_t sweep = sb + (uint32_t)a.s_begin; sweep < s_end; ++sweep) {
-            half(0, sweep);
-            cluster.sync();  // colour 0 complete in every slab
-            // block 0 clears the other parity's buffer: every block read it after the
-            // previous sweep, before the barrier above
-            if (r == 0 && tid < 32) s_Etot[(sweep + 1u) & 1u][tid] = 0;
-            half(1, sweep);
-            cluster.sync();  // colour 1 and the energy sums complete
-            // the exchange, decided by every block from the cluster's sums (App. D.2)
-            if (warp == 0) {
-                const int Eq = Etot0[(sweep & 1u) * 32 + lane];
-                pts::exchange(sh, Eq, sweep, K, key, a.xtab, a.xoff, a.xlen, a.xtail, r == 0, lane);
-                if (r == 0 && sweep + 1 == s_end) a.E[(size_t)inst * 32 + lane] = Eq;
+    uint32_t sweep = sb + (uint32_t)a.s_begin;
+    uint32_t phase = 0;  // of bar[0], bar[1]; of ebar: bits 2, 3
+    bool ok = true;
+    uint32_t A[S::kItems][8];
+    s.draws.set_sweep(sweep, 0u);
+    s.first_draws(A);
+    for (; sweep < s_end; ++sweep) {
+        s.sweep = sweep;
+        // colour 0
+        if (C > 1 && tid == 0) slab::mbar_expect(&sh.bar[0], (uint32_t)geo.LL * 4u);
+        if constexpr (S::kResident) {
+            s.template half<0, slab::kCompare, true, false>(A, true);
+            s.template push_faces<0>(C == 1, up_w, dn_w, up_bar, dn_bar);
+        } else {
+            s.template half<slab::kCompare, true, false>(0, A[0]);
+            s.push_faces(0, C == 1, up_w, dn_w, up_bar, dn_bar);
+        }
+        __syncthreads();
+        if (C > 1) {
+            if (sh.fail[1]) {  // set before this barrier, the same for every thread
+                ok = false;
+                break;
             }
-            pts::build_thresholds(sh, warp, lane);
-            __syncthreads();
+            if (!slab::mbar_wait(&sh.bar[0], phase & 1u)) sh.fail[0] = 1;
+            phase ^= 1u;
+        }
+        // colour 1, with the energies
+        const uint32_t par = sweep & 1u;
+        if (C > 1 && tid == 0) {
+            slab::mbar_expect(&sh.bar[1], (uint32_t)geo.LL * 4u);
+            slab::mbar_expect(&sh.ebar[par], (uint32_t)C * 128u);
+        }
+        if constexpr (S::kResident) {
+            s.template half<1, slab::kCompare, true, true>(A, true);
+            s.template push_faces<1>(C == 1, up_w, dn_w, up_bar + 8u, dn_bar + 8u);
+        } else {
+            s.template half<slab::kCompare, true, true>(1, A[0]);
+            s.push_faces(1, C == 1, up_w, dn_w, up_bar + 8u, dn_bar + 8u);
+        }
+        s.energy_to_block();
+        __syncthreads();
+        if (C > 1) {
+            if (sh.fail[0]) {
+                ok = false;
+                break;
+            }
+            // the block's sums to every block, a warp a block
+            for (int q = warp; q < C; q += warps) {
+                const uint32_t base = slab::cluster_addr(slab::smem_addr(&sh.Epart[par][r][lane]), (uint32_t)q);
+                slab::push_word(base, (uint32_t)sh.E[lane], slab::cluster_addr(slab::smem_addr(&sh.ebar[par]), (uint32_t)q));
+            }
+        }
+        // the exchange (App. D.2): pairs (k, k + 1) with k = sweep mod 2, accepted when
+        // d = E_a - E_b <= 0 or the draw u < T_k(d); a lane is a rung of a pair
+        const int k = ((lane - (int)par) & ~1) + (int)par;
+        const bool pair = k >= 0 && k + 1 < K;
+        const int other = (lane == k ? lane + 1 : lane - 1) & 31;
+        const uint32_t u = philox4x32_10((uint32_t)k, sweep, 0u, kDomainExchange, key.k0, key.k1).v[0];
+        int Eq;  // this slot's energy
+        if (C > 1) {
+            if (!slab::mbar_wait(&sh.ebar[par], (phase >> (2 + par)) & 1u)) sh.fail[1] = 1;
+            phase ^= 4u << par;
+            Eq = 0;
+            for (int q = 0; q < C; ++q) Eq += sh.Epart[par][q][lane];
+        } else {
+            Eq = sh.E[lane];
+        }
+        const int E_rung = __shfl_sync(slab::kAll, Eq, slot);  // of the slot at this rung
+        const int E_other = __shfl_sync(slab::kAll, E_rung, other), slot_other = __shfl_sync(slab::kAll, slot, other);
+        const int d = lane == k ? E_rung - E_other : E_other - E_rung;
+        bool accept = pair && d <= 0;
+        if (pair && d > 0) {
+            const uint32_t T = (uint32_t)d <= sh.xlen[k] ? xtab[sh.xoff[k] + (uint32_t)(d - 1)] : sh.xtail[k];
+            accept = u < T;
+        }
+        if (accept) slot = slot_other;
+        if (lane < K) sh.inverse[warp][slot] = (uint8_t)lane;
+        __syncwarp();
+        rung = lane < K ? sh.inverse[warp][lane] : 0;
+        build_planes();
+        if (warp == 0) {
+            sh.rung[lane] = (uint8_t)rung;
+            accepted += accept && lane == k;
+            const int m = __reduce_min_sync(slab::kAll, lane < K ? Eq : 0x7FFFFFFF);
+            minE = min(minE, m);
+            if (r == 0 && sweep + 1 == s_end) a.E[(size_t)inst * 32 + lane] = Eq;
+        }
+        __syncthreads();  // the next sweep's planes are complete, and E has been read
+        if (warp == 0) sh.E[lane] = 0;
+        if (C > 1) {
+            if (!slab::mbar_wait(&sh.bar[1], (phase >> 1) & 1u)) sh.fail[1] = 1;
+            phase ^= 2u;
         }
     }
+    __syncthreads();
+    ok = ok && !sh.fail[0] && !sh.fail[1];
+    if (!ok && tid == 0) atomicExch(a.status, SG_ETIMEOUT);
 
     // ---- write back ----
-    if (!fail)
-        for (int q = tid; q < slab_words; q += kThreads) g[q] = slab[q];
-    if (r == 0 && !fail && warp == 0)
-        pts::store_state(sh, a.rung_of_slot + (size_t)inst * 32, a.slot_of_rung + (size_t)inst * K,
-                         a.accepts + (size_t)inst * (K - 1), a.minE + inst, K, lane);
-    // after a wait that gave up, copies may still be in flight into this block's shared
-    // memory: wait once more (bounded) before the block leaves
-    if (fail && a.bulk) mbar_wait_bounded(&s_bar, 0);
-    cluster.sync();  // no block leaves while another may still read its shared memory
+    if (ok) {
+        const int n = geo.zc * geo.LL;
+        for (int q = tid; q < n; q += threads) g[(size_t)geo.z0 * geo.LL + q] = w[q];
+        if (r == 0 && warp == 0) {
+            a.rung_of_slot[(size_t)inst * 32 + lane] = (uint8_t)rung;
+            if (lane < K) a.slot_of_rung[(size_t)inst * K + lane] = (uint8_t)slot;
+            if (lane + 1 < K) a.accepts[(size_t)inst * (K - 1) + lane] += (unsigned long long)accepted;
+            if (lane == 0) a.minE[inst] = minE;
+        }
+    }
+    __syncthreads();
+    if (C > 1) cluster.sync();  // no block leaves while another may still push to it
 }
 
-size_t dyn_smem(int L, int C)
+int block_threads(int L, int C) { return slab::resident_threads(slab::pairs_of(L, C), kThreads); }
+const void* kernel_of(int L, int C)
 {
-    const size_t slab_words = (size_t)(L / C) * L * L;
-    return ((slab_words * 5 + 15) & ~(size_t)15) + pts::kTieBytes;
+    switch (slab::resident_items(slab::pairs_of(L, C), kThreads)) {
+        case 1: return (const void*)pt_cluster_kernel<slab::Resident<1>>;
+        case 2: return (const void*)pt_cluster_kernel<slab::Resident<2>>;
+        default: return (const void*)pt_cluster_kernel<slab::Sweeper>;
+    }
 }
+size_t dyn_smem(int L, int C) { return slab::smem_bytes(L, C, block_threads(L, C)); }
 
+// (shared memory: without the exchange thresholds, which take what is left)
 cudaLaunchConfig_t cluster_config(int L, int C, int I, cudaLaunchAttribute* attr)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(C * I, 1, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.blockDim = dim3(block_threads(L, C), 1, 1);
     cfg.dynamicSmemBytes = dyn_smem(L, C);
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = C;
@@ -285,51 +304,66 @@ cudaLaunchConfig_t cluster_config(int L, int C, int I, cudaLaunchAttribute* attr
 
 }  // namespace
 
+namespace {
+// The current device's SM clock in Hz (asking the driver costs about 250 us: it is kept).
+double device_hz()
+{
+    static std::atomic<int> khz_of[64];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::atomic<int>* const kept = dev >= 0 && dev < 64 ? &khz_of[dev] : nullptr;
+    int khz = kept ? kept->load() : 0;
+    if (khz == 0) {
+        if (cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev) != cudaSuccess || khz <= 0) {
+            cudaGetLastError();
+            khz = 2070000;
+        }
+        if (kept) kept->store(khz);
+    }
+    return 1e3 * (double)khz;
+}
+
+// Seconds a sweep of one instance takes on a cluster of C blocks, and of I instances through
+// the row kernels on `sms` SMs, fitted to measurements on a GB300 (K = 32): clusters 2.1 us at
+// L = 8 (C = 2), 2.7 at L = 16, 6.1 at L = 24, 9.4 at L = 32, 49.6 at L = 64 (C = 8); row
+// kernels about 10 us of launches and 6.2 attempts per SM clock.
+double cluster_seconds(double work, int C, double hz) { return 3.7e-6 + work / (C * 11.0 * hz); }
+double row_seconds(double work, int I, int sms, double hz) { return 10e-6 + I * work / (sms * 6.2 * hz); }
+}  // namespace
+
 // Blocks per cluster for a PT run of I instances of side L with K <= 32 temperatures and
 // unit couplings, or 0 when the row kernels should run it.  C is the largest divisor
 // C <= 8 of L whose slab fits shared memory and for which all I clusters are resident at
-// once (one wave).  The cluster form is taken when its estimated time per sweep is below
-// the row kernels', from rates measured on a GB300 (K = 32, L = 8 ... 64, I = 1 ... 15):
-// a cluster sweeps about 7.9 attempts per SM clock with about 4 us of fixed cost per sweep
-// (barriers, exchange); the row kernels about 6.2 attempts per SM clock over the whole GPU
-// with about 10 us per sweep of launch cost.  So it wins for small lattices (L <= 24
-// always, L = 32 from a few instances) and, at L = 64, for 15 instances.  Knob
+// once (one wave) -- but no larger than leaves a block 128 pairs of sites, a warp for each
+// partition of its SM (L = 8: 2.11 us a sweep on one or two blocks, 2.45 on eight).  The
+// cluster form is taken when its estimated time per sweep is below the row kernels'.  Knob
 // SG_PT_CLUSTER = 0 turns the form off, = 1 takes it whenever a slab fits.
-int pt_cluster_blocks(int I, int L, int K)
+int pt_cluster_blocks(int I, int L, int K, double* seconds)
 {
+    if (seconds) *seconds = 0;
     const char* e = getenv("SG_PT_CLUSTER");
     const int knob = e ? atoi(e) : -1;
     if (knob == 0 || K > 32 || K < 1 || L < 2 || (L & 1) || I < 1) return 0;
-    int dev = 0, smem = 0, sms = 1, clock_khz = 2070000;
+    int dev = 0, smem = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaDeviceGetAttribute(&clock_khz, cudaDevAttrClockRate, dev);
-    const double hz = 1e3 * (double)clock_khz;
+    const double hz = device_hz();
     const char* fc = getenv("SG_PT_CLUSTER_C");  // tuning knob: force C (when it divides L and fits)
     const int forced = fc ? atoi(fc) : 0;
     for (int C = 8; C >= 1; --C) {
         if (L % C || (forced > 0 && C != forced)) continue;
         const size_t bytes = dyn_smem(L, C);
-        if (bytes + 16 * 1024 > (size_t)smem) continue;
-        if (cudaFuncSetAttribute(pt_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) !=
-            cudaSuccess) {
-            cudaGetLastError();
-            continue;
-        }
+        if (bytes + sizeof(PtShared) > (size_t)smem) continue;
         if (knob == 1 || forced > 0) return C;
-        cudaLaunchAttribute attr[1];
-        cudaLaunchConfig_t cfg = cluster_config(L, C, 1, attr);
-        int active = 0;
-        if (cudaOccupancyMaxActiveClusters(&active, pt_cluster_kernel, &cfg) != cudaSuccess) {
-            cudaGetLastError();
-            continue;
-        }
-        if (active < I) continue;
-        const double work = (double)L * L * L * K;  // attempts per sweep of one instance
-        const double t_cluster = 4e-6 + work / (C * 7.9 * hz);
-        const double t_rows = 10e-6 + I * work / (sms * 6.2 * hz);
-        return t_cluster < 0.95 * t_rows ? C : 0;
+        if (resident_clusters(kernel_of(L, C), C, bytes, block_threads(L, C)) < I) continue;
+        bool smaller = false;  // a smaller cluster with blocks of at most 128 pairs
+        for (int c = C - 1; c >= 1 && !smaller; --c) smaller = L % c == 0 && slab::pairs_of(L, c) <= 128;
+        if (smaller) continue;
+        const double work = (double)L * L * L * 32.0;  // attempts per sweep of one instance (whole words)
+        const double t = cluster_seconds(work, C, hz);
+        if (seconds) *seconds = t;
+        return t < 0.95 * row_seconds(work, I, sms, hz) ? C : 0;
     }
     return 0;
 }
@@ -341,48 +375,35 @@ int pt_cluster_blocks(int I, int L, int K)
 // L = 64 with 16 instances of 32 temperatures: 15 clusters of 8 blocks on 120 SMs, one
 // instance on the other 32.  Knob SG_PT_HYBRID = 0 turns the split off; SG_PT_CLUSTER = 0
 // turns off every cluster form.
-int pt_cluster_split(int I, int L, int K, int* M, int* side_sms)
+int pt_cluster_split(int I, int L, int K, int* M, int* side_sms, double* seconds)
 {
+    *seconds = 0;
     *M = 0;
     *side_sms = 0;
     const char* e = getenv("SG_PT_HYBRID");
     if (e && atoi(e) == 0) return 0;
     const char* c = getenv("SG_PT_CLUSTER");
     if ((c && atoi(c) == 0) || K > 32 || K < 1 || L < 2 || (L & 1) || I < 2) return 0;
-    int dev = 0, smem = 0, sms = 1, clock_khz = 2070000;
+    int dev = 0, smem = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaDeviceGetAttribute(&clock_khz, cudaDevAttrClockRate, dev);
-    const double hz = 1e3 * (double)clock_khz;
-    const double work = (double)L * L * L * K;
-    const double t_rows = 10e-6 + I * work / (sms * 6.2 * hz);
-    double best = 0.95 * t_rows;
+    const double hz = device_hz();
+    const double work = (double)L * L * L * 32.0;  // whole words
+    double best = 0.95 * row_seconds(work, I, sms, hz);
     int bestC = 0;
     for (int C = 8; C >= 1; --C) {
         if (L % C) continue;
         const size_t bytes = dyn_smem(L, C);
-        if (bytes + 16 * 1024 > (size_t)smem) continue;
-        if (cudaFuncSetAttribute(pt_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) !=
-            cudaSuccess) {
-            cudaGetLastError();
-            continue;
-        }
-        cudaLaunchAttribute attr[1];
-        cudaLaunchConfig_t cfg = cluster_config(L, C, 1, attr);
-        int active = 0, per_sm = 0;
-        if (cudaOccupancyMaxActiveClusters(&active, pt_cluster_kernel, &cfg) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pt_cluster_kernel, kThreads, bytes) !=
-                cudaSuccess) {
-            cudaGetLastError();
-            continue;
-        }
-        if (active >= I || active < 1 || per_sm < 1) continue;  // one wave: pt_cluster_blocks decides
-        const double t_cluster = 4e-6 + work / (C * 7.9 * hz);
+        if (bytes + sizeof(PtShared) > (size_t)smem) continue;
+        const int active = resident_clusters(kernel_of(L, C), C, bytes, block_threads(L, C));
+        if (active >= I || active < 1) continue;  // one wave: pt_cluster_blocks decides
+        const int per_sm = std::max(1, (active * C + sms - 1) / sms);  // blocks an SM holds
+        const double t_cluster = cluster_seconds(work, C, hz);
         for (int m = active; m >= 1; --m) {
             const int left = sms - (m * C + per_sm - 1) / per_sm;
             if (left < 1) continue;
-            const double t_side = 10e-6 + (I - m) * work / (left * 6.2 * hz);
+            const double t_side = row_seconds(work, I - m, left, hz);
             const double t = t_cluster > t_side ? t_cluster : t_side;
             if (t < best) {
                 best = t;
@@ -392,13 +413,14 @@ int pt_cluster_split(int I, int L, int K, int* M, int* side_sms)
             }
         }
     }
+    *seconds = best;
     return bestC;
 }
 
 int32_t launch_pt_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const RunKeys* keys, const uint32_t* thr,
                           uint8_t* rung_of_slot, uint8_t* slot_of_rung, int32_t* E, unsigned long long* accepts,
                           int32_t* minE, const ExchangeTablesDev& xt, int* status, int I, int L, int K, int C,
-                          int s_begin, int s_end, bool bulk_signs, cudaStream_t st, const uint32_t* sweep_base)
+                          int s_begin, int s_end, cudaStream_t st, const uint32_t* sweep_base)
 {
     PtcArgs a{};
     a.sweep_base = sweep_base;
@@ -423,27 +445,23 @@ int32_t launch_pt_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const Ru
     a.s_end = s_end;
     const int H = L / 2;
     a.Hmagic = H == 1 ? 0u : (uint32_t)((0x100000000ull + (uint64_t)H - 1) / (uint64_t)H);
-    a.Lmagic = (uint32_t)((0x100000000ull + (uint64_t)L - 1) / (uint64_t)L);
-    // the sign bytes of a slab start at z0 * L^2 bytes into the instance's array: a bulk
-    // copy needs its address and size to be multiples of 16
-    a.bulk_signs = bulk_signs && ((size_t)(L / C) * L * L) % 16 == 0;
-    // knob SG_PT_BULK = 0: plain loads instead of bulk copies (for comparison)
-    static const bool bulk = [] {
-        const char* k = getenv("SG_PT_BULK");
-        return !(k && atoi(k) == 0);
-    }();
-    a.bulk = bulk ? 1 : 0;
-    const size_t smem = dyn_smem(L, C);
-    if (cudaFuncSetAttribute(pt_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess) {
-        cudaGetLastError();
+    int dev = 0, most = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    // the exchange thresholds in shared memory when they fit beside the slab
+    const size_t xbytes = sizeof(uint32_t) * xt.words;
+    a.xwords = dyn_smem(L, C) + xbytes + sizeof(PtShared) <= (size_t)most ? (int)xt.words : 0;
+    const size_t smem = dyn_smem(L, C) + sizeof(uint32_t) * (size_t)a.xwords;
+    if (!allow_shared(kernel_of(L, C))) {
         set_error("pt_cluster_kernel: cannot use %zu bytes of shared memory", smem);
         return SG_ECUDA;
     }
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = cluster_config(L, C, I, attr);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, pt_cluster_kernel, a);
+    void* args[] = {&a};
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, kernel_of(L, C), args);
     if (e != cudaSuccess) {
         cudaGetLastError();
         set_error("pt_cluster_kernel launch failed: %s", cudaGetErrorString(e));

@@ -422,10 +422,9 @@ int32_t capture_chunk(Request* q, int n, cudaGraphExec_t* out)
     SG_TRY_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
     int32_t rc = SG_OK;
     if (q->mode == kPT && q->ptc > 0) {
-        const ExchangeTablesDev xd{xa.xtab, xa.xoff, xa.xlen, xa.xtail};
-        const bool aligned = (reinterpret_cast<uintptr_t>(q->at<uint8_t>(y.j1)) & 15u) == 0;
+        const ExchangeTablesDev xd{xa.xtab, xa.xoff, xa.xlen, xa.xtail, q->xt.tab.size()};
         rc = launch_pt_cluster(spins, j1p, kp, thr, xa.rung_of_slot, xa.slot_of_rung, xa.E, xa.accepts, xa.minE, xd,
-                               status, 1, q->L, q->req.width, q->ptc, 0, n, aligned, st, base);
+                               status, 1, q->L, q->req.width, q->ptc, 0, n, st, base);
     }
     for (int c = 0; c < n && rc == SG_OK && !(q->mode == kPT && q->ptc > 0); ++c) {
         if (q->mode == kRowsSA) {

@@ -223,16 +223,17 @@ int32_t launch_pt_exchange(const ExchangeArgs& x, int I, uint32_t sweep, cudaStr
 // ptcluster.cu: PT with unit couplings and K <= 32, every sweep of [s_begin, s_end) in one
 // launch, one thread-block cluster of C blocks per instance (lattice in shared memory).
 // pt_cluster_blocks gives C, or 0 when the row kernels should run the batch.
-// bulk_signs: every instance's sign array is 16-byte aligned (slabs then come in by bulk copies).
 // sweep_base: if set, the sweeps are *sweep_base + [s_begin, s_end) (graph replays).
 struct ExchangeTablesDev {
     const uint32_t *tab, *off, *len, *tail;
+    size_t words;  // of tab
 };
-int pt_cluster_blocks(int I, int L, int K);
+// *seconds (if given): its estimate of a sweep's time, 0 when the form is forced or off.
+int pt_cluster_blocks(int I, int L, int K, double* seconds = nullptr);
 // A batch too large for one wave of clusters but faster on them: C for the first *M
 // instances on clusters (M < I, all resident at once), the others through the row kernels
-// on the side_sms SMs the clusters leave; or 0.
-int pt_cluster_split(int I, int L, int K, int* M, int* side_sms);
+// on the side_sms SMs the clusters leave, *seconds a sweep by its estimate; or 0.
+int pt_cluster_split(int I, int L, int K, int* M, int* side_sms, double* seconds);
 // ptcoop.cu: the same on one cooperative grid, each instance's rows split into row blocks
 // held in shared memory (one block per SM).  pt_coop_plan gives the per-block plan
 // (instance, rank, first row, rows; then per instance first block and block count; then
@@ -254,8 +255,7 @@ int32_t launch_pt_coop(int8_t* spins, const uint8_t* const* j1_ptrs, const RunKe
 int32_t launch_pt_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const RunKeys* keys, const uint32_t* thr,
                           uint8_t* rung_of_slot, uint8_t* slot_of_rung, int32_t* E, unsigned long long* accepts,
                           int32_t* minE, const ExchangeTablesDev& xt, int* status, int I, int L, int K, int C,
-                          int s_begin, int s_end, bool bulk_signs, cudaStream_t st,
-                          const uint32_t* sweep_base = nullptr);
+                          int s_begin, int s_end, cudaStream_t st, const uint32_t* sweep_base = nullptr);
 int32_t launch_pt_setup(const unsigned long long* E64, int32_t* E, uint8_t* rung_of_slot,
                         uint8_t* slot_of_rung, unsigned long long* accepts, int32_t* minE,
                         int I, int Rp, int K, cudaStream_t st);

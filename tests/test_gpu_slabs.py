@@ -1,0 +1,74 @@
+"""Lattices held in the shared memory of thread-block clusters, against the row kernels, bit
+for bit: every cluster size at the edges of the block forms (one pair of sites a thread, two
+pairs, columns), sides whose columns do not fill a warp, slabs of one plane, and schedules
+through all three ways a sweep's thresholds can decide."""
+import numpy as np
+import pytest
+
+from paper_2501_17267_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sg():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    torch.cuda.init()
+    from paper_2501_17267_gb300 import sg
+    return sg
+
+
+# (L, C): pairs a block = L^3 / 2C, up to 512 one a thread, up to 1024 two, else columns
+SLABS = [(2, 1), (2, 2), (4, 1), (4, 4), (6, 3), (8, 1), (8, 8), (10, 1), (10, 5), (12, 1), (12, 6), (14, 1), (14, 7),
+         (16, 2), (16, 4), (18, 3), (20, 2), (22, 2), (24, 8), (26, 2), (34, 2), (48, 6), (50, 5)]
+BETAS = [(0.1, 3.0, "linear"), (0.5, 30.0, "geometric"), (20.0, 0.1, "linear")]
+
+
+@pytest.mark.parametrize("L,C", SLABS)
+def test_annealing_on_clusters_equals_row_kernel(sg, monkeypatch, L, C):
+    R, S = (40, 12) if L <= 26 else (5, 7)
+    inst = sg.Instance.create(L, 300 + L)
+    for k, (b0, b1, schedule) in enumerate(BETAS):
+        args = dict(replicas=R, sweeps=S, beta0=b0, beta1=b1, schedule=schedule, seed=11 + k, instance_id=3, spins="host")
+        monkeypatch.setenv("SG_SA_CLUSTER", "1")
+        monkeypatch.setenv("SG_SA_CLUSTER_C", str(C))
+        a = sg.sa_run(inst, **args)
+        monkeypatch.delenv("SG_SA_CLUSTER_C")
+        monkeypatch.setenv("SG_SA_CLUSTER", "0")
+        b = sg.sa_run(inst, **args)
+        assert np.array_equal(a["spins"], b["spins"]) and np.array_equal(a["E"], b["E"])
+
+
+@pytest.mark.parametrize("L,C", SLABS + [(60, 6), (64, 8)])
+def test_tempering_on_clusters_equals_row_kernels(sg, monkeypatch, L, C):
+    K, S = (32, 9) if L > 26 else (13 if L % 4 else 32, 20)
+    insts = [sg.Instance.create(L, 500 + 10 * L + k) for k in range(2 if L <= 26 else 1)]
+    ps = [dict(temps=K, sweeps=S, beta_min=0.2, beta_max=3.0, seed=5, instance_id=k) for k in range(len(insts))]
+    monkeypatch.setenv("SG_PT_CLUSTER", "1")
+    monkeypatch.setenv("SG_PT_CLUSTER_C", str(C))
+    a = sg.pt_run_batch(insts, ps, spins="host")
+    monkeypatch.delenv("SG_PT_CLUSTER_C")
+    monkeypatch.setenv("SG_PT_CLUSTER", "0")
+    b = sg.pt_run_batch(insts, ps, spins="host")
+    for x, y in zip(a, b):
+        for key in ("spins", "E", "perm", "accepts"):
+            assert np.array_equal(x[key], y[key]), key
+        assert x["minE"] == y["minE"]
+
+
+@pytest.mark.parametrize("n_small", [40, 200])
+def test_batch_of_small_lattices_on_clusters_and_single_blocks(sg, monkeypatch, tmp_path, n_small):
+    """Few small planes are annealed by whole clusters, enough of them by single blocks."""
+    sides = [24, 20] + [(4, 8, 12, 16)[k % 4] for k in range(n_small)]
+    insts = [sg.Instance.create(L, 900 + k) for k, L in enumerate(sides)]
+    ps = [dict(replicas=40, sweeps=(6, 11)[k % 2], beta0=0.1, beta1=3.0, schedule="linear", seed=2, instance_id=k)
+          for k in range(len(sides))]
+    monkeypatch.setenv("SG_AUTOTUNE_CACHE", str(tmp_path / "tune.json"))
+    runs = []
+    for wg in ("0", "1"):  # clusters; planes of one word, a block each
+        monkeypatch.setenv("SG_BATCH_WG", wg)
+        runs.append(sg.sa_run_batch(insts, ps, spins="host"))
+    for x, y in zip(*runs):
+        assert np.array_equal(x["spins"], y["spins"]) and np.array_equal(x["E"], y["E"])
