@@ -441,7 +441,7 @@ int32_t run_sa_group(const std::vector<int>& members, const sg_instance* const* 
                                                             : 0;
     if (C > 0) {
         SG_RET(log.run(SG_KERNEL_SWEEP_CHUNK, (int64_t)I * N * R * S, st, [&] {
-            return launch_sa_cluster(spins, j1p, kp, d_thr.as<uint32_t>(), d_flag.as<int>() + 1, I, L, Wn, R, S, C,
+            return launch_sa_cluster(spins, j1p, kp, d_thr.as<uint32_t>(), d_flag.as<int>() + 1, I, L, Wn, R, 0, S, C,
                                      threads, st);
         }));
     } else if (S >= kGraphMinSweeps) {

@@ -39,7 +39,9 @@ struct ClusterArgs {
     const RunKeys* keys;            // [I]
     const uint32_t* thr;            // [S][kThrRow]
     int* status;                    // SG_ETIMEOUT when a bounded wait gave up
-    int L, Wn, R, S, C;             // side, words, replicas, sweeps, blocks per cluster
+    int L, Wn, R, C;                // side, words, replicas, blocks per cluster
+    int s_begin, s_end;             // sweeps [s_begin, s_end), from *sweep_base on when that is set
+    const uint32_t* sweep_base;
     uint32_t Hmagic;                // ceil(2^32 / (L / 2))
 };
 
@@ -224,8 +226,9 @@ sa_cluster_kernel(const ClusterArgs a)
     p.L = a.L;
     p.w = w;
     p.R = a.R;
-    p.s_begin = 0;
-    p.s_end = a.S;
+    const int base = a.sweep_base ? (int)*a.sweep_base : 0;  // (a captured graph replays the launch for later sweeps)
+    p.s_begin = base + a.s_begin;
+    p.s_end = base + a.s_end;
     p.Hmagic = a.Hmagic;
     init_shared(sh);
     uint32_t phase = 0;
@@ -378,11 +381,13 @@ int sa_block_threads(int L, int C, int threads)
 //                    one warp 0.53, L = 16 with 1024 replicas on C = 4 blocks of 16 warps 1.2)
 //   other blocks     2000 + 300 per warp of items (20 x L = 50 on C = 5 12.8, L = 64 on C = 8 20.6)
 //   row kernels      6500 + 490 per warp of items over the whole GPU (18.2 and 5.2 for the same)
-// The fewest cycles win, fewer blocks among equals; L = 16 with 1024 replicas takes C = 4 (2.4
+// The fewest cycles win, fewer blocks among equals.  With `busy` runs of the kind sharing the
+// device (a loaded server) a form's time is its own or, if that is longer, busy times its share
+// of the device.  One run alone: L = 16 with 1024 replicas takes C = 4 (2.4
 // ms a run of 1000 sweeps against 5.1 at C = 2), L = 4 one block (1.05 ms against 1.20 at
 // C = 2 and 1.25 at C = 4).  force: a cluster form whatever the row kernel would take.
 // Knobs: SG_SA_CLUSTER_C forces C, SG_SA_CLUSTER_THREADS the threads.
-int sa_cluster_blocks(int I, int L, int Wn, bool force, int* threads)
+int sa_cluster_blocks(int I, int L, int Wn, bool force, int* threads, int busy)
 {
     *threads = slab::kMaxThreads;
     int dev = 0, smem = 0, sms = 1;
@@ -396,7 +401,8 @@ int sa_cluster_blocks(int I, int L, int Wn, bool force, int* threads)
     const int t = et && atoi(et) >= 32 && atoi(et) <= slab::kMaxThreads ? atoi(et) / 32 * 32 : slab::kMaxThreads;
     *threads = t;
     const double row_items = (double)clusters * L * L * (L / 2) / 32.0;  // warps of items a half sweep
-    double best = force || forced ? 1e300 : 0.95 * (6500.0 + 490.0 * row_items / (4.0 * sms));
+    const double row_share = 490.0 * row_items / (4.0 * sms);
+    double best = force || forced ? 1e300 : 0.95 * std::max(6500.0 + row_share, busy * row_share);
     int bestC = 0;
     for (int C = 1; C <= 8; ++C) {
         if (L % C || (forced && C != forced)) continue;
@@ -409,7 +415,8 @@ int sa_cluster_blocks(int I, int L, int Wn, bool force, int* threads)
         const int64_t waves = (clusters + active - 1) / active;
         const int64_t per_sm = (std::min(clusters, active) * C + sms - 1) / sms;  // blocks on the busiest SM
         const double warps = std::max(1.0, (double)per_sm * (double)((pairs + 31) / 32) / 4.0);
-        const double cost = waves * (slab::resident_items(pairs, t) ? 750.0 + 400.0 * warps : 2000.0 + 300.0 * warps);
+        double cost = waves * (slab::resident_items(pairs, t) ? 750.0 + 400.0 * warps : 2000.0 + 300.0 * warps);
+        cost = std::max(cost, cost * busy * (double)(std::min(clusters, active) * C) / sms);
         if (cost < best) {
             best = cost;
             bestC = C;
@@ -473,7 +480,8 @@ int32_t launch_sa_cluster_planes(const Plane* d_planes, const int* d_order, int 
 }
 
 int32_t launch_sa_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const RunKeys* keys, const uint32_t* thr,
-                          int* status, int I, int L, int Wn, int R, int S, int C, int threads, cudaStream_t st)
+                          int* status, int I, int L, int Wn, int R, int s_begin, int s_end, int C, int threads,
+                          cudaStream_t st, const uint32_t* sweep_base)
 {
     if (threads < 32 || threads > slab::kMaxThreads || threads % 32) {
         set_error("sa_cluster_kernel: %d threads a block (a multiple of 32 up to %d)", threads, slab::kMaxThreads);
@@ -488,7 +496,9 @@ int32_t launch_sa_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const Ru
     a.L = L;
     a.Wn = Wn;
     a.R = R;
-    a.S = S;
+    a.s_begin = s_begin;
+    a.s_end = s_end;
+    a.sweep_base = sweep_base;
     a.C = C;
     const int H = L / 2;
     a.Hmagic = H == 1 ? 0u : (uint32_t)((0x100000000ull + (uint64_t)H - 1) / (uint64_t)H);

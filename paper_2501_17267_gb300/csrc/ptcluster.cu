@@ -368,6 +368,35 @@ int pt_cluster_blocks(int I, int L, int K, double* seconds)
     return 0;
 }
 
+// Blocks per cluster for one request of a server with `busy` requests in service (0: row
+// kernels).  A form's time per sweep is its own or, where that is longer, busy times its share
+// of the device: the row kernels spread an instance over every SM and take the least time
+// alone, but at L = 64 a sweep costs them 4.3 us of the whole device and a cluster of eight
+// blocks 2.6; small lattices share the device best on few blocks each.
+int pt_cluster_blocks_shared(int L, int K, int busy)
+{
+    const char* e = getenv("SG_PT_CLUSTER");
+    if (e || busy <= 1) return pt_cluster_blocks(1, L, K);
+    if (K > 32 || K < 1 || L < 2 || (L & 1)) return 0;
+    int dev = 0, smem = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const double hz = device_hz();
+    const double work = (double)L * L * L * 32.0;
+    double best = 0.95 * std::max(row_seconds(work, 1, sms, hz), busy * (row_seconds(work, 1, sms, hz) - 10e-6));
+    int bestC = 0;
+    for (int C = 8; C >= 1; --C) {
+        if (L % C || dyn_smem(L, C) + sizeof(PtShared) > (size_t)smem) continue;
+        const double t = cluster_seconds(work, C, hz), shared = std::max(t, busy * C * t / sms);
+        if (shared < best && resident_clusters(kernel_of(L, C), C, dyn_smem(L, C), block_threads(L, C)) > 0) {
+            best = shared;
+            bestC = C;
+        }
+    }
+    return bestC;
+}
+
 // A batch with more instances than clusters fit at once: the first M instances on clusters
 // (one wave), the other I - M through the row kernels on the SMs the clusters leave, both
 // at the same time.  With the rates above, M minimises the longer of the two parts' times

@@ -7,8 +7,11 @@
 // their state resident in one stream-ordered allocation each, and keeps every admitted
 // request busy, one chunk of sweeps at a time, with no barrier between requests:
 //   - PT requests, and SA requests on lattices too large for one thread block, replay
-//     their own CUDA graph (a chunk of multi-block sweeps whose sweep index lives in
-//     device memory, then the energy check) on their own stream;
+//     their own CUDA graph (a chunk of sweeps whose sweep index lives in device memory, as
+//     one launch of a cluster kernel or as launches of the row kernels, then the energy
+//     check) on their own stream; the form is chosen chunk by chunk by how many requests
+//     share the device -- row kernels finish a lone large lattice first, clusters do the most
+//     sweeps with a full device;
 //   - small SA requests share a persistent plane launch (batch.cu) per plane width,
 //     relaunched with whatever small requests are ready whenever the previous one ends.
 // The worker polls events, so a chunk that ends lets its request check for completion
@@ -100,7 +103,7 @@ struct Request {
     sg_result result{};
     std::unique_ptr<sg_instance, int32_t (*)(sg_instance*)> inst{nullptr, sg_instance_destroy};
     int mode = kPlanes;
-    int ptc = -1;              // PT: blocks per cluster of the cluster kernel, 0: row kernels (-1: not chosen yet)
+    int C = 0;                 // blocks per cluster the chunk in flight runs on (0: the row kernels)
     int L = 0, Wn = 0, Rp = 0, WG = 1;
     int64_t N = 0;
     int64_t target = 0;        // done when min energy <= target
@@ -117,7 +120,7 @@ struct Request {
     Layout lay;
     unsigned char* mem = nullptr;
     Slot* slot = nullptr;
-    std::map<int, cudaGraphExec_t> graphs;  // chunk length -> graph
+    std::map<std::pair<int, int>, cudaGraphExec_t> graphs;  // chunk length, blocks per cluster -> graph
     template <class T>
     T* at(size_t off) const
     {
@@ -219,6 +222,8 @@ int plane_max_L()
 struct sg_server {
     sg_server_config cfg{};
     int device = 0;
+    int sms = 1;
+    size_t turn = 0;  // worker: where the next round over the requests in service starts
     std::mutex mu;
     std::condition_variable cv_work, cv_done;
     std::deque<sg::Request*> queue;
@@ -384,10 +389,21 @@ int32_t admit_request(sg_server* srv, Request* q)
     return rc;
 }
 
-// Captures one chunk of n sweeps of a PT or large-SA request as a graph: the sweeps
+// Blocks per cluster for the next chunk of a PT or large-SA request with `busy` requests in
+// service, 0 for the row kernels.  (A chunk's result does not depend on the form that runs it.)
+int chunk_form(const Request* q, int busy)
+{
+    if (!q->inst->unit_couplings) return 0;
+    if (q->mode == kPT) return q->Wn == 1 ? pt_cluster_blocks_shared(q->L, q->req.width, busy) : 0;
+    int threads = 0;
+    return sa_cluster_blocks(1, q->L, q->Wn, false, &threads, busy);
+}
+
+// Captures one chunk of n sweeps of a PT or large-SA request as a graph (C blocks a cluster,
+// or the row kernels): the sweeps
 // (sweep index = device base + c), the base advanced by n, and the chunk's lowest energy
 // copied to the slot's pinned word.
-int32_t capture_chunk(Request* q, int n, cudaGraphExec_t* out)
+int32_t capture_chunk(Request* q, int n, int C, cudaGraphExec_t* out)
 {
     const Layout& y = q->lay;
     cudaStream_t st = q->slot->st;
@@ -415,18 +431,20 @@ int32_t capture_chunk(Request* q, int n, cudaGraphExec_t* out)
         xa.K = q->req.width;
         xa.sweep_base = base;
     }
-    // PT of a lattice the cluster kernel sweeps faster (its cost model; small L): the
-    // chunk is one launch of it instead of two launches per sweep
-    if (q->mode == kPT && q->ptc < 0)
-        q->ptc = unit && q->Wn == 1 ? pt_cluster_blocks(1, q->L, q->req.width) : 0;
     SG_TRY_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
     int32_t rc = SG_OK;
-    if (q->mode == kPT && q->ptc > 0) {
-        const ExchangeTablesDev xd{xa.xtab, xa.xoff, xa.xlen, xa.xtail, q->xt.tab.size()};
-        rc = launch_pt_cluster(spins, j1p, kp, thr, xa.rung_of_slot, xa.slot_of_rung, xa.E, xa.accepts, xa.minE, xd,
-                               status, 1, q->L, q->req.width, q->ptc, 0, n, st, base);
+    if (C > 0) {  // the chunk is one launch of a cluster kernel instead of two launches per sweep
+        if (q->mode == kPT) {
+            const ExchangeTablesDev xd{xa.xtab, xa.xoff, xa.xlen, xa.xtail, q->xt.tab.size()};
+            rc = launch_pt_cluster(spins, j1p, kp, thr, xa.rung_of_slot, xa.slot_of_rung, xa.E, xa.accepts, xa.minE,
+                                   xd, status, 1, q->L, q->req.width, C, 0, n, st, base);
+        } else {
+            int threads = 0;
+            sa_cluster_blocks(1, q->L, q->Wn, false, &threads);
+            rc = launch_sa_cluster(spins, j1p, kp, thr, status, 1, q->L, q->Wn, q->req.width, 0, n, C, threads, st, base);
+        }
     }
-    for (int c = 0; c < n && rc == SG_OK && !(q->mode == kPT && q->ptc > 0); ++c) {
+    for (int c = 0; c < n && rc == SG_OK && C == 0; ++c) {
         if (q->mode == kRowsSA) {
             for (int colour = 0; colour < 2 && rc == SG_OK; ++colour)
                 rc = launch_sweep_rows_sa(spins, j6p, j1p, kp, thr, unit, 1, q->L, q->Wn, q->req.width,
@@ -510,11 +528,13 @@ void fail_request(Request* q, int32_t code)
     q->done = true;
 }
 
-// Launches the next chunk of a PT or large-SA request on its own stream.
-void launch_own_chunk(Request* q, int chunk)
+// Launches the next chunk of a PT or large-SA request on its own stream, on C blocks a cluster
+// or through the row kernels.
+void launch_own_chunk(Request* q, int chunk, int C)
 {
     cudaStream_t st = q->slot->st;
     const int n = next_step(q, chunk);
+    q->C = C;
     if (q->mode == kRowsSA && q->need_init) {
         const uint32_t k0 = (uint32_t)q->req.seed;
         const uint32_t k1 = (uint32_t)(q->req.seed >> 32) ^ (uint32_t)q->restart;  // restart k = instance id k
@@ -527,11 +547,12 @@ void launch_own_chunk(Request* q, int chunk)
         }
         q->need_init = false;
     }
-    auto it = q->graphs.find(n);
+    const auto key = std::make_pair(n, C);
+    auto it = q->graphs.find(key);
     if (it == q->graphs.end()) {
         cudaGraphExec_t g = nullptr;
-        if (capture_chunk(q, n, &g) != SG_OK) return fail_request(q, SG_ECUDA);
-        it = q->graphs.emplace(n, g).first;
+        if (capture_chunk(q, n, C, &g) != SG_OK) return fail_request(q, SG_ECUDA);
+        it = q->graphs.emplace(key, g).first;
     }
     if (cudaGraphLaunch(it->second, st) != cudaSuccess || cudaEventRecord(q->slot->ev, st) != cudaSuccess) {
         cudaGetLastError();
@@ -708,6 +729,7 @@ void retire(sg_server* srv, Request* q)
 void worker_main(sg_server* srv)
 {
     cudaSetDevice(srv->device);
+    cudaDeviceGetAttribute(&srv->sms, cudaDevAttrMultiProcessorCount, srv->device);
     const int chunk = srv->cfg.chunk_sweeps;
     std::unique_lock<std::mutex> lock(srv->mu);
     for (;;) {
@@ -747,12 +769,36 @@ void worker_main(sg_server* srv)
                 q->result.status = SG_ECANCELED;
                 q->done = true;
             }
-        // next chunks
-        for (Request* q : act)
-            if (!q->done && !q->inflight && q->mode != kPlanes) {
-                launch_own_chunk(q, chunk);
-                progress = true;
+        // Next chunks.  A cluster holds its SMs for a whole chunk while the row kernels need SMs
+        // anew for every half sweep: with requests of both forms in service the clusters leave a
+        // quarter of the device free, and whoever had to wait for that goes first next time.
+        int rows = 0, cluster_blocks = 0;
+        for (Request* q : act) {
+            if (q->mode == kPlanes || q->done) continue;
+            if (q->inflight) {
+                rows += q->C == 0;
+                cluster_blocks += q->C * q->Wn;
             }
+        }
+        const int busy = (int)act.size();
+        const size_t first = act.empty() ? 0 : srv->turn % act.size();
+        bool waited = false;
+        for (size_t a = 0; a < act.size(); ++a) {
+            const size_t at = (first + a) % act.size();
+            Request* q = act[at];
+            if (q->done || q->inflight || q->mode == kPlanes) continue;
+            const int C = chunk_form(q, busy);
+            const int blocks = C * (q->mode == kPT ? 1 : q->Wn);
+            if (C > 0 && rows > 0 && cluster_blocks > 0 && cluster_blocks + blocks > srv->sms - srv->sms / 4) {
+                if (!waited) srv->turn = at;
+                waited = true;
+                continue;
+            }
+            launch_own_chunk(q, chunk, C);
+            rows += C == 0;
+            cluster_blocks += blocks;
+            progress = true;
+        }
         for (PlaneGroup& g : srv->groups)
             if (!g.inflight) {
                 launch_group(g, act, chunk);

@@ -198,12 +198,13 @@ bool allow_shared(const void* fn);
 
 // cluster.cu: SA with all sweeps in one launch, one thread-block cluster of C blocks per
 // (word, instance); sa_cluster_blocks gives C and the threads to plan a block with, or 0 when
-// the row kernel should run instead (its estimate is shorter, unless `force`; slabs too large,
-// or more clusters than fit at once).
-int sa_cluster_blocks(int I, int L, int Wn, bool force, int* threads);
+// the row kernel should run instead (its estimate is shorter, unless `force`, or no slab fits);
+// busy: runs like this one that share the device.  sweep_base: sweeps [s_begin, s_end) are
+// counted from *sweep_base (graph replays).
+int sa_cluster_blocks(int I, int L, int Wn, bool force, int* threads, int busy = 1);
 int32_t launch_sa_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const RunKeys* keys,
-                          const uint32_t* thr /* [S][kThrRow] */, int* status, int I, int L, int Wn, int R, int S,
-                          int C, int threads, cudaStream_t st);
+                          const uint32_t* thr /* [S][kThrRow] */, int* status, int I, int L, int Wn, int R, int s_begin,
+                          int s_end, int C, int threads, cudaStream_t st, const uint32_t* sweep_base = nullptr);
 // The persistent cluster form for batches of one-word planes (batch.cu): C for planes of
 // sides Ls (every side a multiple of C, the slab of the largest fitting), or 0.
 int sa_cluster_list_blocks(const int* Ls, int n, int max_L);
@@ -230,6 +231,8 @@ struct ExchangeTablesDev {
 };
 // *seconds (if given): its estimate of a sweep's time, 0 when the form is forced or off.
 int pt_cluster_blocks(int I, int L, int K, double* seconds = nullptr);
+// The same for one instance on a device it shares with busy - 1 runs like it.
+int pt_cluster_blocks_shared(int L, int K, int busy);
 // A batch too large for one wave of clusters but faster on them: C for the first *M
 // instances on clusters (M < I, all resident at once), the others through the row kernels
 // on the side_sms SMs the clusters leave, *seconds a sweep by its estimate; or 0.

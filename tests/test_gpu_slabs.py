@@ -72,3 +72,21 @@ def test_batch_of_small_lattices_on_clusters_and_single_blocks(sg, monkeypatch, 
         runs.append(sg.sa_run_batch(insts, ps, spins="host"))
     for x, y in zip(*runs):
         assert np.array_equal(x["spins"], y["spins"]) and np.array_equal(x["E"], y["E"])
+
+
+def test_loaded_server_equals_requests_one_at_a_time(sg):
+    """With many requests in service chunks run on clusters of any size, alone through the row
+    kernels: both kinds, one and two words, restarts shorter than the cap, a chunk that does not
+    divide them."""
+    reqs = [sg.request(kind, L, 40 + 7 * L + k, 40 if kind == sg.SG_REQ_SA and k % 2 else 32, 0.1 + 0.1 * kind, 3.0, 0.002,
+                       70, run_seed=k, sweeps_per_restart=50)
+            for k, L in enumerate((24, 32, 40, 20, 64, 48) * 4) for kind in (sg.SG_REQ_SA, sg.SG_REQ_PT)]
+    results = []
+    for active in (64, 1):
+        with sg.Server(4 << 30, max_active=active, chunk_sweeps=15) as srv:
+            tickets = [srv.submit(q) for q in reqs]
+            results.append([srv.poll(t) for t in tickets])
+    for a, b in zip(*results):
+        for key in ("status", "reached", "sweeps", "minE", "e_gs"):
+            assert a[key] == b[key], key
+        assert a["status"] == sg.SG_OK
