@@ -102,29 +102,13 @@ struct PlacedEdge {  // tile-relative lower corner and axis of an image edge
     int dx, dy, dz, axis;
     int8_t J;
 };
+using Placements = std::array<std::array<std::array<PlacedEdge, 12>, 48>, 3>;
 
-}  // namespace
-
-int32_t generate_instance(int L, uint64_t seed, const double class_prob[3], int gauge,
-                          int8_t* J3, int8_t* planted, int64_t* e_gs)
+// All (class, symmetry) placements.
+const Placements& placements()
 {
-    if (L < 2 || L > SG_LMAX || (L & 1)) {
-        set_error("L must be even with 2 <= L <= %d (got %d)", SG_LMAX, L);
-        return SG_EINVAL;
-    }
-    const double w0 = class_prob[0], w1 = class_prob[1], w2 = class_prob[2];
-    if (!(w0 >= 0 && w1 >= 0 && w2 >= 0) || !(w0 + w1 + w2 > 0)) {
-        set_error("class_prob must be non-negative with a positive sum");
-        return SG_EINVAL;
-    }
-    const double total = w0 + w1 + w2;
-    // inverse CDF of a 32-bit uniform word against cumulative weights in 2^32 fixed point
-    const uint64_t cut0 = (uint64_t)floor(ldexp(w0 / total, 32));
-    const uint64_t cut1 = (uint64_t)floor(ldexp((w0 + w1) / total, 32));
-
-    // all (class, symmetry) placements, precomputed
-    static std::array<std::array<std::array<PlacedEdge, 12>, 48>, 3> placed = [] {
-        std::array<std::array<std::array<PlacedEdge, 12>, 48>, 3> P{};
+    static const Placements placed = [] {
+        Placements P{};
         for (int cls = 0; cls < 3; ++cls) {
             auto t = class_template(cls);
             for (int g = 0; g < 48; ++g) {
@@ -145,6 +129,133 @@ int32_t generate_instance(int L, uint64_t seed, const double class_prob[3], int 
         }
         return P;
     }();
+    return placed;
+}
+
+// Inverse CDF of a 32-bit uniform word: the cumulative class weights in 2^32 fixed point.
+struct ClassCuts {
+    uint64_t cut0, cut1;
+};
+ClassCuts class_cuts(const double class_prob[3])
+{
+    const double w0 = class_prob[0], w1 = class_prob[1], total = w0 + w1 + class_prob[2];
+    return ClassCuts{(uint64_t)floor(ldexp(w0 / total, 32)), (uint64_t)floor(ldexp((w0 + w1) / total, 32))};
+}
+
+// ---- the same generator on the device, for instances whose couplings the host never reads ----
+
+// A placed edge in a byte: lower corner (3 bits), axis (2), negative (1).
+struct PackedPlacements {
+    uint8_t e[3][48][12];
+};
+
+// One thread a tile: its class and symmetry, the couplings of its twelve edges (each edge
+// belongs to one tile), the sum of the tiles' minima.
+__global__ void generate_tiles_kernel(const PackedPlacements placed, int L, uint32_t k0, uint32_t k1, uint64_t cut0,
+                                      uint64_t cut1, int8_t* __restrict__ J3, unsigned long long* __restrict__ e_gs)
+{
+    const int H = L >> 1, half = H * H * H;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    int E = 0;
+    if (t < 2 * half) {
+        const Philox4 r = philox4x32_10((uint32_t)t, 0, 0, kDomainGenerate, k0, k1);
+        const int cls = r.v[0] < cut0 ? 0 : r.v[0] < cut1 ? 1 : 2;
+        const int g = (int)__umulhi(r.v[1], 48u);
+        constexpr int m0 = kTemplateMin[0], m1 = kTemplateMin[1], m2 = kTemplateMin[2];
+        E = cls == 0 ? m0 : cls == 1 ? m1 : m2;
+        const int parity = t >= half, q = t - parity * half;
+        const int ox = 2 * (q % H) + parity, oy = 2 * (q / H % H) + parity, oz = 2 * (q / (H * H)) + parity;
+#pragma unroll
+        for (int e = 0; e < 12; ++e) {
+            const int b = placed.e[cls][g][e];
+            int x = ox + (b & 1), y = oy + ((b >> 1) & 1), z = oz + ((b >> 2) & 1);
+            x = x >= L ? x - L : x, y = y >= L ? y - L : y, z = z >= L ? z - L : z;
+            J3[3 * (x + L * (y + L * z)) + ((b >> 3) & 3)] = (b & 32) ? (int8_t)-1 : (int8_t)1;
+        }
+    }
+    E = __reduce_add_sync(0xFFFFFFFFu, E);
+    if ((threadIdx.x & 31) == 0 && E) atomicAdd(e_gs, (unsigned long long)(long long)E);
+}
+
+// Gauge of every site: 1 where tau = -1.
+__global__ void generate_gauge_kernel(int N, int gauge, uint32_t k0, uint32_t k1, uint8_t* __restrict__ tau)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < N) tau[i] = gauge ? (uint8_t)(philox4x32_10((uint32_t)i, 0, 0, kDomainGauge, k0, k1).v[0] >> 31) : (uint8_t)0;
+}
+
+// The per-site records of the gauged couplings J tau tau' (kernels.cu: bytes +x, -x, +y, -y,
+// +z, -z; sign bits).
+__global__ void generate_records_kernel(const int8_t* __restrict__ J3, const uint8_t* __restrict__ tau, int L,
+                                        uint2* __restrict__ j6, uint8_t* __restrict__ j1)
+{
+    const int LL = L * L, i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= LL * L) return;
+    const int x = i % L, y = i / L % L, z = i / LL;
+    const int xp = i + (x + 1 == L ? 1 - L : 1), xm = i + (x == 0 ? L - 1 : -1);
+    const int yp = i + (y + 1 == L ? L - LL : L), ym = i + (y == 0 ? LL - L : -L);
+    const int zp = i + (z + 1 == L ? LL - LL * L : LL), zm = i + (z == 0 ? LL * L - LL : -LL);
+    const uint32_t t = tau[i];
+    const uint32_t n = ((uint32_t)(J3[3 * i] < 0) ^ t ^ tau[xp]) | ((uint32_t)(J3[3 * xm] < 0) ^ t ^ tau[xm]) << 1 |
+                       ((uint32_t)(J3[3 * i + 1] < 0) ^ t ^ tau[yp]) << 2 | ((uint32_t)(J3[3 * ym + 1] < 0) ^ t ^ tau[ym]) << 3 |
+                       ((uint32_t)(J3[3 * i + 2] < 0) ^ t ^ tau[zp]) << 4 | ((uint32_t)(J3[3 * zm + 2] < 0) ^ t ^ tau[zm]) << 5;
+    auto coupling = [&](int q) { return (n >> q) & 1u ? 0xFFu : 0x01u; };
+    j6[i] = make_uint2(coupling(0) | coupling(1) << 8 | coupling(2) << 16 | coupling(3) << 24, coupling(4) | coupling(5) << 8);
+    j1[i] = (uint8_t)n;
+}
+
+}  // namespace
+
+int32_t launch_generate_instance(const sg_instance_desc& d, int8_t* J3, uint8_t* tau, unsigned long long* e_gs,
+                                 uint2* j6, uint8_t* j1, cudaStream_t st)
+{
+    PackedPlacements packed;
+    const Placements& P = placements();
+    for (int c = 0; c < 3; ++c)
+        for (int g = 0; g < 48; ++g)
+            for (int e = 0; e < 12; ++e) {
+                const PlacedEdge& q = P[c][g][e];
+                packed.e[c][g][e] = (uint8_t)(q.dx | q.dy << 1 | q.dz << 2 | q.axis << 3 | (q.J < 0 ? 32 : 0));
+            }
+    const ClassCuts cuts = class_cuts(d.class_prob);
+    const uint32_t k0 = (uint32_t)d.seed, k1 = (uint32_t)(d.seed >> 32);
+    const int L = d.L, N = L * L * L, threads = 256;
+    SG_TRY_CUDA(cudaMemsetAsync(e_gs, 0, sizeof(*e_gs), st));
+    generate_tiles_kernel<<<(N / 4 + threads - 1) / threads, threads, 0, st>>>(packed, L, k0, k1, cuts.cut0, cuts.cut1,
+                                                                              J3, e_gs);
+    generate_gauge_kernel<<<(N + threads - 1) / threads, threads, 0, st>>>(N, d.gauge, k0, k1, tau);
+    generate_records_kernel<<<(N + threads - 1) / threads, threads, 0, st>>>(J3, tau, L, j6, j1);
+    SG_TRY_CUDA(cudaGetLastError());
+    return SG_OK;
+}
+
+int64_t planted_energy(const sg_instance_desc& d)
+{
+    const ClassCuts cuts = class_cuts(d.class_prob);
+    const uint32_t k0 = (uint32_t)d.seed, k1 = (uint32_t)(d.seed >> 32);
+    const int64_t tiles = (int64_t)d.L * d.L * d.L / 4;
+    int64_t E = 0;
+    for (int64_t t = 0; t < tiles; ++t) {
+        const uint32_t r = philox4x32_10((uint32_t)t, 0, 0, kDomainGenerate, k0, k1).v[0];
+        E += kTemplateMin[r < cuts.cut0 ? 0 : r < cuts.cut1 ? 1 : 2];
+    }
+    return E;
+}
+
+int32_t generate_instance(int L, uint64_t seed, const double class_prob[3], int gauge,
+                          int8_t* J3, int8_t* planted, int64_t* e_gs)
+{
+    if (L < 2 || L > SG_LMAX || (L & 1)) {
+        set_error("L must be even with 2 <= L <= %d (got %d)", SG_LMAX, L);
+        return SG_EINVAL;
+    }
+    const double w0 = class_prob[0], w1 = class_prob[1], w2 = class_prob[2];
+    if (!(w0 >= 0 && w1 >= 0 && w2 >= 0) || !(w0 + w1 + w2 > 0)) {
+        set_error("class_prob must be non-negative with a positive sum");
+        return SG_EINVAL;
+    }
+    const auto [cut0, cut1] = class_cuts(class_prob);
+    const Placements& placed = placements();
 
     const int64_t N = (int64_t)L * L * L;
     const int H = L / 2;

@@ -1,8 +1,8 @@
 // server.cu -- continuously batched solve server: requests run until their lowest energy
 // reaches a target gap (time to target, TT-eps, Eq. 2) or a sweep cap.
 //
-// sg_submit generates the request's instance and host tables in the caller's thread and
-// queues it.  One worker thread per server owns the device work: it admits queued
+// sg_submit makes the request's host tables in the caller's thread (tables of one schedule or
+// ladder are shared) and queues it; its instance is generated on the device when it is admitted.  One worker thread per server owns the device work: it admits queued
 // requests (FIFO) while their device memory fits the budget and a slot is free, keeps
 // their state resident in one stream-ordered allocation each, and keeps every admitted
 // request busy, one chunk of sweeps at a time, with no barrier between requests:
@@ -76,7 +76,7 @@ enum Mode { kPlanes = 0, kRowsSA = 1, kPT = 2 };
 struct Slot {
     cudaStream_t st = nullptr;
     cudaEvent_t ev = nullptr;
-    long long* h_out = nullptr;  // pinned: [0] min energy of the last chunk, [1] its status word
+    long long* h_out = nullptr;  // pinned: [0] min energy of the last chunk, [1] its status word, [2] E_gs
 };
 
 size_t align_up(size_t v) { return (v + 255) & ~(size_t)255; }
@@ -101,7 +101,7 @@ struct Request {
     bool done = false;       // retire
     bool inflight = false;   // a chunk (own stream or plane launch) is running
     sg_result result{};
-    std::unique_ptr<sg_instance, int32_t (*)(sg_instance*)> inst{nullptr, sg_instance_destroy};
+    bool known = false;        // result.e_gs and target are set (read back with the first chunk)
     int mode = kPlanes;
     int C = 0;                 // blocks per cluster the chunk in flight runs on (0: the row kernels)
     int L = 0, Wn = 0, Rp = 0, WG = 1;
@@ -112,7 +112,7 @@ struct Request {
     int step = 0;              // sweeps of the chunk in flight
     // host tables made at submit
     std::shared_ptr<const std::vector<uint32_t>> thr;  // SA: [S][kThrRow]; PT: [K][kThrRow]
-    ExchangeTables xt;
+    std::shared_ptr<const ExchangeTables> xt;          // PT
     // SA
     int restart = 0, in_restart = 0;
     bool need_init = true;
@@ -165,10 +165,10 @@ Layout layout_of(const Request& q)
         y.acc = take(8 * Kp);
         y.minE = take(4);
         y.done = take(4);
-        y.xtab = take(4 * q.xt.tab.size());
-        y.xoff = take(4 * q.xt.off.size());
-        y.xlen = take(4 * q.xt.len.size());
-        y.xtail = take(4 * q.xt.tail.size());
+        y.xtab = take(4 * q.xt->tab.size());
+        y.xoff = take(4 * q.xt->off.size());
+        y.xlen = take(4 * q.xt->len.size());
+        y.xtail = take(4 * q.xt->tail.size());
         y.out = take(8);
         y.status = take(4);
     }
@@ -191,10 +191,14 @@ struct PlaneGroup {
     std::vector<int> first;
 };
 
-// Host schedule tables shared by requests with the same SA schedule.
-struct ScheduleCache {
+// Host tables shared by requests with the same SA schedule or PT ladder (and lattice size, which
+// bounds the exchange tables); dropped when many different ones have come.
+struct TableCache {
+    using Words = std::shared_ptr<const std::vector<uint32_t>>;
+    static constexpr size_t kMost = 64;
     std::mutex mu;
-    std::map<std::tuple<int, double, double, int>, std::shared_ptr<const std::vector<uint32_t>>> tables;
+    std::map<std::tuple<int, double, double, int>, Words> schedules;
+    std::map<std::tuple<int, double, double, int64_t>, std::pair<Words, std::shared_ptr<const ExchangeTables>>> ladders;
 };
 
 int largest_wg(int Wn)
@@ -233,7 +237,7 @@ struct sg_server {
     size_t in_use = 0;
     bool stop = false;
     std::thread worker;
-    sg::ScheduleCache schedules;  // used by the submitting threads
+    sg::TableCache tables;  // used by the submitting threads
     // device resources of the worker
     cudaMemPool_t pool = nullptr;
     std::vector<std::unique_ptr<sg::Slot>> slots;  // all slots made
@@ -287,47 +291,50 @@ Slot* take_slot(sg_server* srv)
     return srv->slots.back().get();
 }
 
-// Host part of a request, in the submitting thread: the instance, its target and the
-// acceptance tables.  SG_OK or SG_EINVAL.
-int32_t prepare_request(ScheduleCache& cache, Request* q)
+// Host part of a request, in the submitting thread: its acceptance tables.  SG_OK or SG_EINVAL.
+int32_t prepare_request(TableCache& cache, Request* q)
 {
     const sg_request& r = q->req;
-    sg_instance* inst = nullptr;
-    int32_t rc = sg_instance_create(&r.instance, &inst);
-    if (rc != SG_OK) return rc;
-    q->inst.reset(inst);
-    q->L = inst->L;
-    q->N = inst->N;
+    q->L = r.instance.L;
+    q->N = (int64_t)q->L * q->L * q->L;
     q->Wn = words_for(r.width);
     q->Rp = 32 * q->Wn;
     q->WG = largest_wg(q->Wn);
-    q->result.e_gs = inst->e_gs;
-    const int64_t abs_gs = inst->e_gs < 0 ? -inst->e_gs : inst->e_gs;
-    q->target = inst->e_gs + (int64_t)floor(r.eps_target * (double)abs_gs);
+    std::lock_guard<std::mutex> lock(cache.mu);
     if (r.kind == SG_REQ_SA) {
         q->mode = q->L <= plane_max_L() ? kPlanes : kRowsSA;
         const auto key = std::make_tuple(r.sweeps_per_restart, r.beta0, r.beta1, r.schedule);
-        std::lock_guard<std::mutex> lock(cache.mu);
-        auto it = cache.tables.find(key);
-        if (it == cache.tables.end()) {
+        auto it = cache.schedules.find(key);
+        if (it == cache.schedules.end()) {
             const int S = r.sweeps_per_restart;
             std::vector<double> beta(S);
             beta_schedule(S, r.beta0, r.beta1, r.schedule == SG_SCHEDULE_GEOMETRIC, beta.data());
             auto t = std::make_shared<std::vector<uint32_t>>((size_t)S * kThrRow);
             for (int s = 0; s < S; ++s) metropolis_row(beta[s], t->data() + (size_t)s * kThrRow);
-            it = cache.tables.emplace(key, std::move(t)).first;
+            if (cache.schedules.size() >= TableCache::kMost) cache.schedules.clear();
+            it = cache.schedules.emplace(key, std::move(t)).first;
         }
         q->thr = it->second;
     } else {
         q->mode = kPT;
         const int K = r.width;
-        std::vector<double> ladder(K);
-        beta_schedule(K, r.beta0, r.beta1, 1, ladder.data());
-        auto t = std::make_shared<std::vector<uint32_t>>((size_t)K * kThrRow);
-        for (int k = 0; k < K; ++k) metropolis_row(ladder[k], t->data() + (size_t)k * kThrRow);
-        q->thr = t;
-        rc = build_exchange_tables(ladder, 4 * (int64_t)inst->abs_sum, &q->xt);
-        if (rc != SG_OK) return rc;
+        const int64_t dmax = 12 * q->N;  // four times the sum of |J| over the 3N edges, all 1
+        const auto key = std::make_tuple(K, r.beta0, r.beta1, dmax);
+        auto it = cache.ladders.find(key);
+        if (it == cache.ladders.end()) {
+            std::vector<double> ladder(K);
+            beta_schedule(K, r.beta0, r.beta1, 1, ladder.data());
+            auto t = std::make_shared<std::vector<uint32_t>>((size_t)K * kThrRow);
+            for (int k = 0; k < K; ++k) metropolis_row(ladder[k], t->data() + (size_t)k * kThrRow);
+            auto x = std::make_shared<ExchangeTables>();
+            const int32_t rc = build_exchange_tables(ladder, dmax, x.get());
+            if (rc != SG_OK) return rc;
+            if (cache.ladders.size() >= TableCache::kMost) cache.ladders.clear();
+            it = cache.ladders.emplace(key, std::make_pair(TableCache::Words(std::move(t)),
+                                                           std::shared_ptr<const ExchangeTables>(std::move(x)))).first;
+        }
+        q->thr = it->second.first;
+        q->xt = it->second.second;
     }
     q->lay = layout_of(*q);
     q->bytes = q->lay.total;
@@ -350,11 +357,15 @@ int32_t admit_request(sg_server* srv, Request* q)
     }
     q->mem = static_cast<unsigned char*>(p);
     const Layout& y = q->lay;
-    const sg_instance* inst = q->inst.get();
+    // the instance, its spins' memory serving as scratch (N gauge bytes, then E_gs: a site has a
+    // word of spins at least)
     const size_t N = (size_t)q->N;
-    SG_TRY_CUDA(cudaMemcpyAsync(q->at<void>(y.J3), inst->J3.data(), 3 * N, cudaMemcpyHostToDevice, st));
-    int32_t rc = launch_prepare_j6(q->at<int8_t>(y.J3), q->at<uint2>(y.j6), q->at<uint8_t>(y.j1), q->L, st);
+    unsigned char* scratch = q->at<unsigned char>(y.spins);
+    unsigned long long* e_gs = reinterpret_cast<unsigned long long*>(scratch + (N + 7) / 8 * 8);
+    int32_t rc = launch_generate_instance(q->req.instance, q->at<int8_t>(y.J3), scratch, e_gs, q->at<uint2>(y.j6),
+                                          q->at<uint8_t>(y.j1), st);
     if (rc != SG_OK) return rc;
+    SG_TRY_CUDA(cudaMemcpyAsync(q->slot->h_out + 2, e_gs, 8, cudaMemcpyDeviceToHost, st));
     SG_TRY_CUDA(cudaMemcpyAsync(q->at<void>(y.thr), q->thr->data(), 4 * q->thr->size(), cudaMemcpyHostToDevice, st));
     if (q->mode == kPlanes) {  // the shared plane launch waits for these uploads
         SG_TRY_CUDA(cudaEventRecord(q->slot->ev, st));
@@ -368,7 +379,7 @@ int32_t admit_request(sg_server* srv, Request* q)
     // PT: keys, exchange tables, initial spins and energies, the identity permutation
     const RunKeys key{(uint32_t)q->req.seed, (uint32_t)(q->req.seed >> 32)};
     SG_TRY_CUDA(cudaMemcpyAsync(q->at<void>(y.keys), &key, sizeof(key), cudaMemcpyHostToDevice, st));
-    const ExchangeTables& xt = q->xt;
+    const ExchangeTables& xt = *q->xt;
     SG_TRY_CUDA(cudaMemcpyAsync(q->at<void>(y.xtab), xt.tab.data(), 4 * xt.tab.size(), cudaMemcpyHostToDevice, st));
     SG_TRY_CUDA(cudaMemcpyAsync(q->at<void>(y.xoff), xt.off.data(), 4 * xt.off.size(), cudaMemcpyHostToDevice, st));
     SG_TRY_CUDA(cudaMemcpyAsync(q->at<void>(y.xlen), xt.len.data(), 4 * xt.len.size(), cudaMemcpyHostToDevice, st));
@@ -381,7 +392,7 @@ int32_t admit_request(sg_server* srv, Request* q)
     rc = launch_init_spins(q->at<int8_t>(y.spins), kp, 1, q->L, q->Wn, q->req.width, st);
     if (rc == SG_OK)
         rc = launch_energy(q->at<int8_t>(y.spins), j6p, 1, q->L, q->Wn, q->at<unsigned long long>(y.E64), st,
-                           q->inst->unit_couplings ? j1p : nullptr);
+                           j1p);
     if (rc == SG_OK)
         rc = launch_pt_setup(q->at<unsigned long long>(y.E64), q->at<int32_t>(y.E), q->at<uint8_t>(y.perm),
                              q->at<uint8_t>(y.inv), q->at<unsigned long long>(y.acc), q->at<int32_t>(y.minE), 1,
@@ -393,7 +404,6 @@ int32_t admit_request(sg_server* srv, Request* q)
 // service, 0 for the row kernels.  (A chunk's result does not depend on the form that runs it.)
 int chunk_form(const Request* q, int busy)
 {
-    if (!q->inst->unit_couplings) return 0;
     if (q->mode == kPT) return q->Wn == 1 ? pt_cluster_blocks_shared(q->L, q->req.width, busy) : 0;
     int threads = 0;
     return sa_cluster_blocks(1, q->L, q->Wn, false, &threads, busy);
@@ -413,7 +423,7 @@ int32_t capture_chunk(Request* q, int n, int C, cudaGraphExec_t* out)
     const RunKeys* kp = q->at<RunKeys>(y.keys);
     uint32_t* base = q->at<uint32_t>(y.base);
     const uint32_t* thr = q->at<uint32_t>(y.thr);
-    const bool unit = q->inst->unit_couplings;
+    const bool unit = true;  // tile-planted
     int* status = q->at<int>(y.status);
     ExchangeArgs xa{};
     if (q->mode == kPT) {
@@ -435,7 +445,7 @@ int32_t capture_chunk(Request* q, int n, int C, cudaGraphExec_t* out)
     int32_t rc = SG_OK;
     if (C > 0) {  // the chunk is one launch of a cluster kernel instead of two launches per sweep
         if (q->mode == kPT) {
-            const ExchangeTablesDev xd{xa.xtab, xa.xoff, xa.xlen, xa.xtail, q->xt.tab.size()};
+            const ExchangeTablesDev xd{xa.xtab, xa.xoff, xa.xlen, xa.xtail, q->xt->tab.size()};
             rc = launch_pt_cluster(spins, j1p, kp, thr, xa.rung_of_slot, xa.slot_of_rung, xa.E, xa.accepts, xa.minE,
                                    xd, status, 1, q->L, q->req.width, C, 0, n, st, base);
         } else {
@@ -497,10 +507,19 @@ int next_step(const Request* q, int chunk)
                                    q->req.sweep_cap - q->sweeps});
 }
 
+// The planted energy and the energy that ends the request.
+void learn_target(Request* q, int64_t e_gs)
+{
+    q->known = true;
+    q->result.e_gs = e_gs;
+    q->target = e_gs + (int64_t)floor(q->req.eps_target * (double)(e_gs < 0 ? -e_gs : e_gs));
+}
+
 // Folds a finished chunk into the request: lowest energy, sweep counts, restart end,
 // and the completion test.
 void finish_chunk(Request* q, int64_t chunk_min)
 {
+    if (!q->known) learn_target(q, q->slot->h_out[2]);
     q->minE = std::min(q->minE, chunk_min);
     q->sweeps += q->step;
     if (q->mode != kPT) {
@@ -610,8 +629,7 @@ void launch_group(PlaneGroup& g, const std::vector<Request*>& act, int chunk)
     g.planes.clear();
     g.init_planes.clear();
     g.first.assign(1, 0);
-    bool unit = true;
-    for (Request* q : g.reqs) unit &= q->inst->unit_couplings;
+    const bool unit = true;  // tile-planted
     for (Request* q : g.reqs) {
         q->step = next_step(q, chunk);
         for (int w0 = 0; w0 < q->Wn; w0 += g.WG) {
@@ -718,9 +736,8 @@ void retire(sg_server* srv, Request* q)
     if (q->slot) srv->free_slots.push_back(q->slot);
     q->slot = nullptr;
     cudaGetLastError();
-    q->inst.reset();
     q->thr.reset();
-    q->xt = ExchangeTables();
+    q->xt.reset();
     q->t_done = Clock::now();
     q->finished = true;
     if (q->admitted) srv->in_use -= q->bytes;
@@ -834,6 +851,7 @@ void worker_main(sg_server* srv)
 
 void finish_result(Request* q)
 {
+    if (!q->known) learn_target(q, planted_energy(q->req.instance));  // no chunk of it has run
     sg_result& r = q->result;
     r.sweeps = q->sweeps;
     const bool ran = q->minE != INT64_MAX;
@@ -927,7 +945,7 @@ extern "C" int32_t sg_submit(sg_server* srv, const sg_request* req, uint64_t* ti
     q->t_submit = Clock::now();
     q->req = *req;
     q->result.status = SG_OK;
-    int32_t rc = prepare_request(srv->schedules, q.get());
+    int32_t rc = prepare_request(srv->tables, q.get());
     if (rc != SG_OK) return rc;
     if (q->bytes > srv->cfg.hbm_budget_bytes) {
         set_error("request needs %zu bytes of device memory, more than the server budget", q->bytes);
@@ -1031,7 +1049,7 @@ extern "C" int32_t sg_request_bytes(const sg_request* req, uint64_t* bytes)
         set_error("bad request");
         return SG_EINVAL;
     }
-    ScheduleCache cache;
+    TableCache cache;
     Request q;
     q.req = *req;
     const int32_t rc = prepare_request(cache, &q);

@@ -59,6 +59,12 @@ namespace sg {
 int32_t generate_instance(int L, uint64_t seed, const double class_prob[3], int gauge,
                           int8_t* J3, int8_t* planted, int64_t* e_gs);
 
+// The same instance made on the device (no host couplings): records and sign bytes as
+// launch_prepare_j6 makes them, E_gs in *e_gs.  Scratch: J3 [3N], tau [N].  d has been checked.
+int32_t launch_generate_instance(const sg_instance_desc& d, int8_t* J3, uint8_t* tau, unsigned long long* e_gs,
+                                 uint2* j6, uint8_t* j1, cudaStream_t st);
+int64_t planted_energy(const sg_instance_desc& d);  // its E_gs alone (host)
+
 // ---- schedules and acceptance tables (host) ----
 // Metropolis thresholds for one beta: thr[k] = min(floor(2^32 exp(-beta*2k)), 2^32-1),
 // k = 0..kMaxK (the accepted energy increase is dE = 2k; entry 0 is unused).

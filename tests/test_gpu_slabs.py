@@ -90,3 +90,19 @@ def test_loaded_server_equals_requests_one_at_a_time(sg):
         for key in ("status", "reached", "sweeps", "minE", "e_gs"):
             assert a[key] == b[key], key
         assert a["status"] == sg.SG_OK
+
+
+@pytest.mark.parametrize("L,probs,gauge", [(2, wl.UNIFORM, True), (4, (0, 0, 1), False), (6, (0.3, 0.7, 0), True),
+                                           (12, (1, 0, 0), True), (40, wl.UNIFORM, True)])
+def test_server_generates_the_host_generators_instance(sg, L, probs, gauge):
+    """E_gs and the lowest energies of requests, whose instances are made on the device, against
+    runs of the instances that the host generator makes."""
+    reqs = [sg.request(kind, L, 2 ** 33 + 17 * L, 32, 0.3, 3.0, 0.0, 20, run_seed=9, sweeps_per_restart=20,
+                       class_prob=probs, gauge=gauge) for kind in (sg.SG_REQ_SA, sg.SG_REQ_PT)]
+    with sg.Server(1 << 30, max_active=4, chunk_sweeps=20) as srv:
+        tickets = [srv.submit(q) for q in reqs]
+        sa, pt = [srv.poll(t) for t in tickets]
+    inst = sg.Instance.create(L, 2 ** 33 + 17 * L, probs, gauge)
+    assert sa["e_gs"] == pt["e_gs"] == inst.e_gs
+    assert sa["minE"] == sg.sa_run(inst, 32, 20, 0.3, 3.0, seed=9)["E"].min()
+    assert pt["minE"] == sg.pt_run(inst, 32, 20, 0.3, 3.0, seed=9)["minE"]
