@@ -42,6 +42,7 @@ struct ClusterArgs {
     int L, Wn, R, C;                // side, words, replicas, blocks per cluster
     int s_begin, s_end;             // sweeps [s_begin, s_end), from *sweep_base on when that is set
     const uint32_t* sweep_base;
+    ChunkReport report;             // of a run of one instance and word
     uint32_t Hmagic;                // ceil(2^32 / (L / 2))
 };
 
@@ -71,6 +72,8 @@ struct Shared {
     int mode[2];
     uint64_t bar[2];  // by colour: the neighbours' face words of that colour have arrived
     int fail[2];      // by colour: a wait for that barrier gave up (read one half sweep later)
+    int E[32];        // report: the block's energies, and in block 0 the cluster's
+    int E_cluster[32];
 };
 
 // Called by every thread of every block of the cluster once the barriers are initialised;
@@ -78,7 +81,7 @@ struct Shared {
 // back.  Returns false when a wait gave up.
 template <class S>
 __device__ __forceinline__ bool anneal_plane(const PlaneRun& p, const int C, unsigned char* smem, Shared& sh,
-                                             uint32_t& phase)
+                                             uint32_t& phase, bool energies = false)
 {
     cg::cluster_group cluster = cg::this_cluster();
     const int r = C > 1 ? (int)cluster.block_rank() : 0;
@@ -193,6 +196,17 @@ __device__ __forceinline__ bool anneal_plane(const PlaneRun& p, const int C, uns
     uint32_t* dst = p.g + (size_t)geo.z0 * geo.LL * p.stride;
     if (ok)
         for (int q = tid; q < n; q += blockDim.x) dst[(size_t)q * p.stride] = w[q];
+    if (energies) {  // of the words as they are (each bond joins a colour-0 and a colour-1 site), in block 0
+        if (tid < 32) sh.E[tid] = sh.E_cluster[tid] = 0;
+        __syncthreads();
+        s.E = sh.E;
+        if constexpr (S::kResident) s.template half<1, slab::kCountOnly, false, true>(A, false);
+        else s.template half<slab::kCountOnly, false, true>(1, A[0]);
+        s.energy_to_block();
+        __syncthreads();
+        if (C > 1) cluster.sync();  // block 0's sums are cleared
+        if (warp == 0) atomicAdd(C > 1 ? cluster.map_shared_rank(&sh.E_cluster[lane], 0) : &sh.E_cluster[lane], sh.E[lane]);
+    }
     __syncthreads();
     return ok;
 }
@@ -232,8 +246,16 @@ sa_cluster_kernel(const ClusterArgs a)
     p.Hmagic = a.Hmagic;
     init_shared(sh);
     uint32_t phase = 0;
-    if (!anneal_plane<S>(p, a.C, smem, sh, phase) && threadIdx.x == 0) atomicExch(a.status, SG_ETIMEOUT);
-    if (a.C > 1) cg::this_cluster().sync();  // no block leaves while another may still push to it
+    if (!anneal_plane<S>(p, a.C, smem, sh, phase, a.report.out != nullptr) && threadIdx.x == 0)
+        atomicExch(a.status, SG_ETIMEOUT);
+    // no block leaves while another may still push to it; energies and status are complete
+    if (a.C > 1) cg::this_cluster().sync();
+    else __syncthreads();
+    if (a.report.out && (a.C == 1 || cg::this_cluster().block_rank() == 0) && threadIdx.x < 32) {
+        const int left = a.R - 32 * w, lane = threadIdx.x;
+        const int least = __reduce_min_sync(slab::kAll, lane < left ? sh.E_cluster[lane] : 0x7FFFFFFF);
+        if (lane == 0) a.report.write(least, *static_cast<volatile int*>(a.status));
+    }
 }
 
 // Persistent form for batches (batch.cu's planes of one word, [N][1]).  Clusters take planes
@@ -481,7 +503,7 @@ int32_t launch_sa_cluster_planes(const Plane* d_planes, const int* d_order, int 
 
 int32_t launch_sa_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const RunKeys* keys, const uint32_t* thr,
                           int* status, int I, int L, int Wn, int R, int s_begin, int s_end, int C, int threads,
-                          cudaStream_t st, const uint32_t* sweep_base)
+                          cudaStream_t st, const uint32_t* sweep_base, const ChunkReport& report)
 {
     if (threads < 32 || threads > slab::kMaxThreads || threads % 32) {
         set_error("sa_cluster_kernel: %d threads a block (a multiple of 32 up to %d)", threads, slab::kMaxThreads);
@@ -499,6 +521,7 @@ int32_t launch_sa_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const Ru
     a.s_begin = s_begin;
     a.s_end = s_end;
     a.sweep_base = sweep_base;
+    a.report = report;
     a.C = C;
     const int H = L / 2;
     a.Hmagic = H == 1 ? 0u : (uint32_t)((0x100000000ull + (uint64_t)H - 1) / (uint64_t)H);

@@ -54,6 +54,7 @@ struct PtcArgs {
     int* status;                    // SG_ETIMEOUT when a bounded wait gave up
     int L, K, C, s_begin, s_end;
     const uint32_t* sweep_base;     // if set, sweeps run from *sweep_base + s_begin to *sweep_base + s_end
+    ChunkReport report;             // of a run of one instance
     uint32_t Hmagic;                // ceil(2^32 / (L / 2))
     int xwords;                     // words of xtab held in shared memory (0: read from global memory)
 };
@@ -272,7 +273,8 @@ __global__ void __launch_bounds__(kThreads, 1) pt_cluster_kernel(const PtcArgs a
         }
     }
     __syncthreads();
-    if (C > 1) cluster.sync();  // no block leaves while another may still push to it
+    if (C > 1) cluster.sync();  // no block leaves while another may still push to it; the status is complete
+    if (a.report.out && r == 0 && tid == 0) a.report.write(minE, *static_cast<volatile int*>(a.status));
 }
 
 int block_threads(int L, int C) { return slab::resident_threads(slab::pairs_of(L, C), kThreads); }
@@ -449,10 +451,12 @@ int pt_cluster_split(int I, int L, int K, int* M, int* side_sms, double* seconds
 int32_t launch_pt_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const RunKeys* keys, const uint32_t* thr,
                           uint8_t* rung_of_slot, uint8_t* slot_of_rung, int32_t* E, unsigned long long* accepts,
                           int32_t* minE, const ExchangeTablesDev& xt, int* status, int I, int L, int K, int C,
-                          int s_begin, int s_end, cudaStream_t st, const uint32_t* sweep_base)
+                          int s_begin, int s_end, cudaStream_t st, const uint32_t* sweep_base,
+                          const ChunkReport& report)
 {
     PtcArgs a{};
     a.sweep_base = sweep_base;
+    a.report = report;
     a.spins = reinterpret_cast<uint32_t*>(spins);
     a.j1_ptrs = j1_ptrs;
     a.keys = keys;

@@ -2,20 +2,20 @@
 // reaches a target gap (time to target, TT-eps, Eq. 2) or a sweep cap.
 //
 // sg_submit makes the request's host tables in the caller's thread (tables of one schedule or
-// ladder are shared) and queues it; its instance is generated on the device when it is admitted.  One worker thread per server owns the device work: it admits queued
-// requests (FIFO) while their device memory fits the budget and a slot is free, keeps
-// their state resident in one stream-ordered allocation each, and keeps every admitted
-// request busy, one chunk of sweeps at a time, with no barrier between requests:
-//   - PT requests, and SA requests on lattices too large for one thread block, replay
-//     their own CUDA graph (a chunk of sweeps whose sweep index lives in device memory, as
-//     one launch of a cluster kernel or as launches of the row kernels, then the energy
-//     check) on their own stream; the form is chosen chunk by chunk by how many requests
-//     share the device -- row kernels finish a lone large lattice first, clusters do the most
-//     sweeps with a full device;
+// ladder are shared) and queues it; its instance is generated on the device when it is
+// admitted.  One worker thread per server owns the device work: it admits queued requests
+// (FIFO) while their device memory fits the budget and a slot is free, keeps their state
+// resident in one stream-ordered allocation each, and keeps every admitted request busy, one
+// chunk of sweeps at a time, with no barrier between requests:
+//   - PT requests, and SA requests on lattices too large for one thread block, run their
+//     chunks on their own stream: as one launch of a cluster kernel, which reports the chunk
+//     itself, or as a CUDA graph of the row kernels' launches and the energy check.  The form
+//     is chosen chunk by chunk by how many requests share the device -- row kernels finish a
+//     lone large lattice first, clusters do the most sweeps with a full device;
 //   - small SA requests share a persistent plane launch (batch.cu) per plane width,
 //     relaunched with whatever small requests are ready whenever the previous one ends.
-// The worker polls events, so a chunk that ends lets its request check for completion
-// and start the next chunk at once, and arrivals join as soon as they are admitted.
+// The worker polls reports and events, so a chunk that ends lets its request check for
+// completion and start the next chunk at once, and arrivals join as soon as they are admitted.
 // Completion is checked only at chunk ends, at sweep counts fixed by the request alone,
 // so each result is the same alone and in any mix.
 #include <limits.h>
@@ -24,6 +24,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <condition_variable>
 #include <deque>
@@ -42,7 +43,7 @@ namespace {
 
 using Clock = std::chrono::steady_clock;
 
-__global__ void advance_kernel(uint32_t* base, uint32_t by) { *base += by; }
+__global__ void set_base_kernel(uint32_t* base, uint32_t sweep) { *base = sweep; }
 
 // Start of an SA restart: key (k0, k1) and sweep index 0.
 __global__ void restart_kernel(RunKeys* keys, uint32_t k0, uint32_t k1, uint32_t* base)
@@ -76,7 +77,7 @@ enum Mode { kPlanes = 0, kRowsSA = 1, kPT = 2 };
 struct Slot {
     cudaStream_t st = nullptr;
     cudaEvent_t ev = nullptr;
-    long long* h_out = nullptr;  // pinned: [0] min energy of the last chunk, [1] its status word, [2] E_gs
+    long long* h_out = nullptr;  // pinned: [0] min energy of the last chunk, [1] its status word, [2] E_gs, [3] its token
 };
 
 size_t align_up(size_t v) { return (v + 255) & ~(size_t)255; }
@@ -104,6 +105,8 @@ struct Request {
     bool known = false;        // result.e_gs and target are set (read back with the first chunk)
     int mode = kPlanes;
     int C = 0;                 // blocks per cluster the chunk in flight runs on (0: the row kernels)
+    long long token = 0;       // the chunk in flight reports itself with this token (0: the slot's event)
+    int polls = 0;             // looks at that report
     int L = 0, Wn = 0, Rp = 0, WG = 1;
     int64_t N = 0;
     int64_t target = 0;        // done when min energy <= target
@@ -120,7 +123,7 @@ struct Request {
     Layout lay;
     unsigned char* mem = nullptr;
     Slot* slot = nullptr;
-    std::map<std::pair<int, int>, cudaGraphExec_t> graphs;  // chunk length, blocks per cluster -> graph
+    std::map<int, cudaGraphExec_t> graphs;  // chunk length -> graph (row kernels)
     template <class T>
     T* at(size_t off) const
     {
@@ -406,14 +409,37 @@ int chunk_form(const Request* q, int busy)
 {
     if (q->mode == kPT) return q->Wn == 1 ? pt_cluster_blocks_shared(q->L, q->req.width, busy) : 0;
     int threads = 0;
-    return sa_cluster_blocks(1, q->L, q->Wn, false, &threads, busy);
+    return q->Wn == 1 ? sa_cluster_blocks(1, q->L, 1, false, &threads, busy) : 0;  // (a report is one word's)
 }
 
-// Captures one chunk of n sweeps of a PT or large-SA request as a graph (C blocks a cluster,
-// or the row kernels): the sweeps
-// (sweep index = device base + c), the base advanced by n, and the chunk's lowest energy
-// copied to the slot's pinned word.
-int32_t capture_chunk(Request* q, int n, int C, cudaGraphExec_t* out)
+// One chunk of n sweeps on clusters of C blocks: a single launch, which reports the chunk's
+// lowest energy itself.  Nothing that waits for it follows on its stream: the device has fewer
+// hardware queues than a loaded server has streams, and a dependent operation at the head of
+// one keeps the launches of other streams behind it.
+int32_t launch_cluster_chunk(Request* q, int n, int C, long long token)
+{
+    const Layout& y = q->lay;
+    const uint8_t* const* j1p = reinterpret_cast<const uint8_t* const*>(q->at<const void*>(y.jp) + 1);
+    const ChunkReport report{q->slot->h_out, token};
+    if (q->mode == kPT) {
+        const ExchangeTablesDev xd{q->at<uint32_t>(y.xtab), q->at<uint32_t>(y.xoff), q->at<uint32_t>(y.xlen),
+                                   q->at<uint32_t>(y.xtail), q->xt->tab.size()};
+        return launch_pt_cluster(q->at<int8_t>(y.spins), j1p, q->at<RunKeys>(y.keys), q->at<uint32_t>(y.thr),
+                                 q->at<uint8_t>(y.perm), q->at<uint8_t>(y.inv), q->at<int32_t>(y.E),
+                                 q->at<unsigned long long>(y.acc), q->at<int32_t>(y.minE), xd, q->at<int>(y.status), 1,
+                                 q->L, q->req.width, C, (int)q->sweeps, (int)q->sweeps + n, q->slot->st, nullptr, report);
+    }
+    int threads = 0;
+    sa_cluster_blocks(1, q->L, q->Wn, false, &threads);
+    return launch_sa_cluster(q->at<int8_t>(y.spins), j1p, q->at<RunKeys>(y.keys), q->at<uint32_t>(y.thr),
+                             q->at<int>(y.status), 1, q->L, q->Wn, q->req.width, q->in_restart, q->in_restart + n, C,
+                             threads, q->slot->st, nullptr, report);
+}
+
+// Captures one chunk of n sweeps of a PT or large-SA request through the row kernels as a
+// graph: the sweeps (sweep index = device base + c), and the chunk's lowest energy copied to
+// the slot's pinned word.
+int32_t capture_chunk(Request* q, int n, cudaGraphExec_t* out)
 {
     const Layout& y = q->lay;
     cudaStream_t st = q->slot->st;
@@ -443,18 +469,7 @@ int32_t capture_chunk(Request* q, int n, int C, cudaGraphExec_t* out)
     }
     SG_TRY_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
     int32_t rc = SG_OK;
-    if (C > 0) {  // the chunk is one launch of a cluster kernel instead of two launches per sweep
-        if (q->mode == kPT) {
-            const ExchangeTablesDev xd{xa.xtab, xa.xoff, xa.xlen, xa.xtail, q->xt->tab.size()};
-            rc = launch_pt_cluster(spins, j1p, kp, thr, xa.rung_of_slot, xa.slot_of_rung, xa.E, xa.accepts, xa.minE,
-                                   xd, status, 1, q->L, q->req.width, C, 0, n, st, base);
-        } else {
-            int threads = 0;
-            sa_cluster_blocks(1, q->L, q->Wn, false, &threads);
-            rc = launch_sa_cluster(spins, j1p, kp, thr, status, 1, q->L, q->Wn, q->req.width, 0, n, C, threads, st, base);
-        }
-    }
-    for (int c = 0; c < n && rc == SG_OK && C == 0; ++c) {
+    for (int c = 0; c < n && rc == SG_OK; ++c) {
         if (q->mode == kRowsSA) {
             for (int colour = 0; colour < 2 && rc == SG_OK; ++colour)
                 rc = launch_sweep_rows_sa(spins, j6p, j1p, kp, thr, unit, 1, q->L, q->Wn, q->req.width,
@@ -472,7 +487,6 @@ int32_t capture_chunk(Request* q, int n, int C, cudaGraphExec_t* out)
         }
     }
     if (rc == SG_OK) {
-        advance_kernel<<<1, 1, 0, st>>>(base, (uint32_t)n);
         if (q->mode == kRowsSA) {
             cudaMemsetAsync(q->at<void>(y.E64), 0, 8 * (size_t)q->Rp, st);
             rc = launch_energy(spins, j6p, 1, q->L, q->Wn, q->at<unsigned long long>(y.E64), st, unit ? j1p : nullptr);
@@ -566,13 +580,24 @@ void launch_own_chunk(Request* q, int chunk, int C)
         }
         q->need_init = false;
     }
-    const auto key = std::make_pair(n, C);
-    auto it = q->graphs.find(key);
+    if (C > 0) {
+        static std::atomic<long long> tokens{0};
+        q->token = ++tokens;
+        q->polls = 0;
+        if (launch_cluster_chunk(q, n, C, q->token) != SG_OK) return fail_request(q, SG_ECUDA);
+        q->step = n;
+        q->inflight = true;
+        return;
+    }
+    q->token = 0;
+    auto it = q->graphs.find(n);
     if (it == q->graphs.end()) {
         cudaGraphExec_t g = nullptr;
-        if (capture_chunk(q, n, C, &g) != SG_OK) return fail_request(q, SG_ECUDA);
-        it = q->graphs.emplace(key, g).first;
+        if (capture_chunk(q, n, &g) != SG_OK) return fail_request(q, SG_ECUDA);
+        it = q->graphs.emplace(n, g).first;
     }
+    set_base_kernel<<<1, 1, 0, st>>>(q->at<uint32_t>(q->lay.base),
+                                     (uint32_t)(q->mode == kPT ? q->sweeps : (int64_t)q->in_restart));
     if (cudaGraphLaunch(it->second, st) != cudaSuccess || cudaEventRecord(q->slot->ev, st) != cudaSuccess) {
         cudaGetLastError();
         return fail_request(q, SG_ECUDA);
@@ -584,12 +609,24 @@ void launch_own_chunk(Request* q, int chunk, int C)
 // True once the request's chunk has ended (and then folds it in).
 bool poll_own_chunk(Request* q)
 {
-    const cudaError_t e = cudaEventQuery(q->slot->ev);
-    if (e == cudaErrorNotReady) return false;
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        fail_request(q, SG_ECUDA);
-        return true;
+    if (q->token != 0) {
+        if (*static_cast<volatile long long*>(q->slot->h_out + 3) != q->token) {
+            // (now and then: has the device failed?)
+            const cudaError_t e = ++q->polls % 1024 ? cudaErrorNotReady : cudaStreamQuery(q->slot->st);
+            if (e == cudaErrorNotReady || e == cudaSuccess) return false;
+            cudaGetLastError();
+            fail_request(q, SG_ECUDA);
+            return true;
+        }
+        std::atomic_thread_fence(std::memory_order_acquire);
+    } else {
+        const cudaError_t e = cudaEventQuery(q->slot->ev);
+        if (e == cudaErrorNotReady) return false;
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            fail_request(q, SG_ECUDA);
+            return true;
+        }
     }
     if (*reinterpret_cast<const int*>(q->slot->h_out + 1) != 0) {  // a bounded device wait gave up
         fail_request(q, SG_ETIMEOUT);
@@ -794,7 +831,7 @@ void worker_main(sg_server* srv)
             if (q->mode == kPlanes || q->done) continue;
             if (q->inflight) {
                 rows += q->C == 0;
-                cluster_blocks += q->C * q->Wn;
+                cluster_blocks += q->C;
             }
         }
         const int busy = (int)act.size();
@@ -805,7 +842,7 @@ void worker_main(sg_server* srv)
             Request* q = act[at];
             if (q->done || q->inflight || q->mode == kPlanes) continue;
             const int C = chunk_form(q, busy);
-            const int blocks = C * (q->mode == kPT ? 1 : q->Wn);
+            const int blocks = C;
             if (C > 0 && rows > 0 && cluster_blocks > 0 && cluster_blocks + blocks > srv->sms - srv->sms / 4) {
                 if (!waited) srv->turn = at;
                 waited = true;

@@ -196,6 +196,23 @@ int32_t launch_sweep_rows_pt(int8_t* spins, const uint2* const* j6_ptrs,
                              bool unit_j, int I, int L, int Wn, int K, uint32_t sweep, int colour,
                              const ExchangeArgs* xch, unsigned* done, bool* fused, cudaStream_t st,
                              const uint32_t* sweep_base = nullptr, int* status = nullptr, int sms = 0);
+// Where a cluster kernel reports a chunk of one request (pinned host memory), so that nothing
+// has to follow it on its stream: the lowest energy, the status, then the token.
+struct ChunkReport {
+    long long* out = nullptr;  // [0] lowest energy, [1] status, [3] token; null: no report
+    long long token = 0;
+#if defined(__CUDACC__)
+    __device__ __forceinline__ void write(long long energy, int status) const
+    {
+        volatile long long* o = out;
+        o[0] = energy;
+        o[1] = status;
+        __threadfence_system();
+        o[3] = token;
+    }
+#endif
+};
+
 // Clusters of C blocks with `smem` bytes of dynamic shared memory each that the device keeps
 // resident at once for kernel `fn` (0: none, or the shape is refused); allow_shared raises the
 // kernel's limit of dynamic shared memory to the most a block can have.
@@ -210,7 +227,8 @@ bool allow_shared(const void* fn);
 int sa_cluster_blocks(int I, int L, int Wn, bool force, int* threads, int busy = 1);
 int32_t launch_sa_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const RunKeys* keys,
                           const uint32_t* thr /* [S][kThrRow] */, int* status, int I, int L, int Wn, int R, int s_begin,
-                          int s_end, int C, int threads, cudaStream_t st, const uint32_t* sweep_base = nullptr);
+                          int s_end, int C, int threads, cudaStream_t st, const uint32_t* sweep_base = nullptr,
+                          const ChunkReport& report = ChunkReport{});
 // The persistent cluster form for batches of one-word planes (batch.cu): C for planes of
 // sides Ls (every side a multiple of C, the slab of the largest fitting), or 0.
 int sa_cluster_list_blocks(const int* Ls, int n, int max_L);
@@ -264,7 +282,8 @@ int32_t launch_pt_coop(int8_t* spins, const uint8_t* const* j1_ptrs, const RunKe
 int32_t launch_pt_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const RunKeys* keys, const uint32_t* thr,
                           uint8_t* rung_of_slot, uint8_t* slot_of_rung, int32_t* E, unsigned long long* accepts,
                           int32_t* minE, const ExchangeTablesDev& xt, int* status, int I, int L, int K, int C,
-                          int s_begin, int s_end, cudaStream_t st, const uint32_t* sweep_base = nullptr);
+                          int s_begin, int s_end, cudaStream_t st, const uint32_t* sweep_base = nullptr,
+                          const ChunkReport& report = ChunkReport{});
 int32_t launch_pt_setup(const unsigned long long* E64, int32_t* E, uint8_t* rung_of_slot,
                         uint8_t* slot_of_rung, unsigned long long* accepts, int32_t* minE,
                         int I, int Rp, int K, cudaStream_t st);

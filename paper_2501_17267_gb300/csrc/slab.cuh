@@ -319,7 +319,8 @@ __device__ __forceinline__ void load_slab(const Geometry& g, const uint32_t* __r
 
 // How a half sweep's thresholds can accept: not at all (all zero), only where the leading
 // byte is 0 (every threshold below 2^24), or by a full compare.
-enum Mode { kNoDraws = 0, kTailOnly = 1, kCompare = 2 };
+// (kCountOnly: no update, for the energies of the words as they are.)
+enum Mode { kNoDraws = 0, kTailOnly = 1, kCompare = 2, kCountOnly = 3 };
 
 // Thresholds of a word: plane j of k = 2, 4, 6 in tp[j] (bit b: replica b), and the
 // replicas whose threshold has nonzero low 24 bits -- only those can accept on a tie.
@@ -464,7 +465,8 @@ struct Sweeper {
                 if (colour == 1) draws.set_sweep(sweep + 1u, word);
             }
         }
-        if (MODE != kNoDraws) draws.planes((uint32_t)c.site, B);
+        constexpr bool kDraws = MODE == kCompare || MODE == kTailOnly;
+        if (kDraws) draws.planes((uint32_t)c.site, B);
         // masks of negative couplings: six sign bits spread to the tops of bytes
         const uint32_t m1 = sb * 0x10204080u, m2 = sb * 0x408u;
         const uint32_t a0 = logic<kXor3>(self, near, sign_bytes(m1, 0x8888u));
@@ -492,9 +494,9 @@ struct Sweeper {
             const uint32_t any = (A[0] | A[1] | A[2]) | (A[3] | A[4] | A[5]) | (A[6] | A[7]);
             tie = alive & c2 & ~any;
         }
-        const uint32_t flip = (~c2 | lt) & alive;
-        st_word_if(alive, is, self ^ flip);
-        if (MODE != kNoDraws) {
+        const uint32_t flip = MODE == kCountOnly ? 0u : (~c2 | lt) & alive;
+        if (MODE != kCountOnly) st_word_if(alive, is, self ^ flip);
+        if (kDraws) {
             const uint4 lz = ld_quad(planes + 128u);
             tie &= logic<kSelect>(c1, lz.z, logic<kSelect>(c0, lz.y, lz.x));
             const unsigned who = __ballot_sync(kAll, tie != 0u);
@@ -562,8 +564,7 @@ struct Sweeper {
                 }
                 if (!step<MODE, TEMPERING, ENERGY, 1>(c, colour, H4, LL4, B, A)) break;
             }
-            if (MODE != kNoDraws)
-                while (c.qn) decide<TEMPERING, ENERGY>(c.qn);
+            while ((MODE == kCompare || MODE == kTailOnly) && c.qn) decide<TEMPERING, ENERGY>(c.qn);
         }
         __syncwarp();
     }
@@ -731,10 +732,10 @@ struct Resident {
                 const uint32_t any = (A[r][0] | A[r][1] | A[r][2]) | (A[r][3] | A[r][4] | A[r][5]) | (A[r][6] | A[r][7]);
                 tie[r] = alive & c2 & ~any;
             }
-            flip[r] = (~c2 | lt) & alive;
+            flip[r] = MODE == kCountOnly ? 0u : (~c2 | lt) & alive;
         }
         if (C == 1) draws.set_sweep(sweep + 1u, word);
-        if (MODE != kNoDraws) {
+        if (MODE == kCompare || MODE == kTailOnly) {
             const uint4 lz = ld_quad(planes + 128u);
             uint32_t low[R], tail[R], bit[R], more = 0;
 #pragma unroll
