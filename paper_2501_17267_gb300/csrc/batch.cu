@@ -80,6 +80,7 @@ __global__ void __launch_bounds__(256) sa_planes_kernel(const Plane* __restrict_
     extern __shared__ __align__(16) uint32_t s_plane[];
     __shared__ int s_item;
     __shared__ uint32_t s_thr[kThrRow];
+    __shared__ __align__(16) uint32_t s_gp[UNITJ ? 4 : mp::kGeneralPlanes];
     __shared__ uint4 s_ties[8 * kTieCap * 2];  // per warp: {site, storage, word index, tie}, {c0, c1, stored word, -}
     __shared__ int s_tie_n[8];
     const int tid = threadIdx.x, nthreads = blockDim.x;
@@ -118,6 +119,9 @@ __global__ void __launch_bounds__(256) sa_planes_kernel(const Plane* __restrict_
                 for (int m = 0; m < 24; ++m) tp[m] = mp::threshold_plane_bit(s_thr[2 + 2 * (m / 8)], m % 8) ? ~0u : 0u;
 #pragma unroll
                 for (int m = 0; m < 3; ++m) lz[m] = (s_thr[2 + 2 * m] & 0xFFFFFFu) ? ~0u : 0u;
+            } else {
+                for (int q = tid; q < mp::kGeneralPlanes; q += nthreads) s_gp[q] = mp::general_plane_of(q, s_thr);
+                __syncthreads();
             }
             // Deferred ties of this warp, decided by all its lanes together (every lane
             // runs the same iterations of the site loop below).
@@ -205,8 +209,10 @@ __global__ void __launch_bounds__(256) sa_planes_kernel(const Plane* __restrict_
                                     }
                                 }
                             } else {
-                                flip = mp::update_word_general(self[u][wi], nw, J[u], valid, s_thr, 0, A,
-                                                               (uint32_t)i_[u], (uint32_t)sw, w, key);
+                                uint32_t c[4];
+                                int M;
+                                flip = mp::update_word_general(self[u][wi], nw, J[u], valid, s_gp, s_thr, 0, A,
+                                                               (uint32_t)i_[u], (uint32_t)sw, w, key, c, &M);
                             }
                             out[wi] = self[u][wi] ^ flip;
                             any |= flip != 0u;

@@ -142,24 +142,13 @@ __device__ __forceinline__ void xor_word(uint32_t addr, uint32_t v)
     asm volatile("red.shared.xor.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
-__device__ __forceinline__ uint32_t sign_bytes(uint32_t x, uint32_t sel)
-{
-    uint32_t d;
-    asm("prmt.b32 %0, %1, %1, %2;" : "=r"(d) : "r"(x), "r"(sel));
-    return d;
-}
-
-// Three-input logic of the updates, spelled out: left to the compiler a word costs about
-// eight operations more.
-template <int TABLE>
-__device__ __forceinline__ uint32_t logic(uint32_t a, uint32_t b, uint32_t c)
-{
-    uint32_t d;
-    asm("lop3.b32 %0, %1, %2, %3, %4;" : "=r"(d) : "r"(a), "r"(b), "r"(c), "n"(TABLE));
-    return d;
-}
-constexpr int kXor3 = 0x96, kMaj = 0xE8, kSelect = 0xCA /* a ? b : c */, kBorrow = 0x8E /* majority of ~a, b, c */,
-              kAndEqual = 0x90 /* a where b = c */;
+using mp::kAndEqual;
+using mp::kBorrow;
+using mp::kMaj;
+using mp::kSelect;
+using mp::kXor3;
+using mp::logic;
+using mp::sign_bytes;
 
 // ---------------------------------------------------------------- draws
 
@@ -317,10 +306,9 @@ __device__ __forceinline__ void load_slab(const Geometry& g, const uint32_t* __r
 
 // ---------------------------------------------------------------- updates
 
-// How a half sweep's thresholds can accept: not at all (all zero), only where the leading
-// byte is 0 (every threshold below 2^24), or by a full compare.
-// (kCountOnly: no update, for the energies of the words as they are.)
-enum Mode { kNoDraws = 0, kTailOnly = 1, kCompare = 2, kCountOnly = 3 };
+// What a half sweep does: mp::Mode by its thresholds, or no update at all, for the energies of
+// the words as they are.
+constexpr int kNoDraws = mp::kNoDraws, kTailOnly = mp::kTailOnly, kCompare = mp::kCompare, kCountOnly = 3;
 
 // Thresholds of a word: plane j of k = 2, 4, 6 in tp[j] (bit b: replica b), and the
 // replicas whose threshold has nonzero low 24 bits -- only those can accept on a tie.

@@ -60,6 +60,7 @@ constexpr int kTieResolvePipe = kTieCap - 4;
 constexpr int kVBits = 10;      // planes of the per-thread energy counters
 constexpr int kPlanes = 28;     // threshold planes kept per word
 constexpr int kVItems = ((1 << kVBits) - 1) / 6;  // items a counter holds before a fold
+constexpr int kVItemsGeneral = ((1 << kVBits) - 1) / (6 * SG_JMAX);
 
 struct SweepArgs {
     uint32_t* spins;                 // [I][N][Wn] words, storage order
@@ -99,7 +100,7 @@ __global__ void __launch_bounds__(256, PT && !ENERGY ? SG_SWEEP_MINB : SG_SWEEP_
 {
     __shared__ uint32_t s_thr[PT ? 256 * kThrStride : kThrRow];
     // per word: 24 threshold-byte planes, 3 planes "threshold has low bits" (k = 2, 4, 6), 1 spare
-    __shared__ __align__(16) uint32_t s_tp[(PT ? 8 : 1) * kPlanes];
+    __shared__ __align__(16) uint32_t s_tp[(PT ? 8 : 1) * (UNITJ ? kPlanes : mp::kGeneralPlanes)];
     __shared__ int s_E[PT ? 256 : 1];
     __shared__ uint4 s_ties[8 * kTieCap * 2];      // per warp: {site, storage, word index, tie}, {c0, c1, stored word, -}
     __shared__ int s_tie_n[8];
@@ -157,6 +158,19 @@ __global__ void __launch_bounds__(256, PT && !ENERGY ? SG_SWEEP_MINB : SG_SWEEP_
             s_tp[q] = plane;
         }
         __syncthreads();
+    } else {
+        if constexpr (PT) {
+            mp::general_planes(s_tp, s_thr, kThrStride, Wn, tid, nthreads);
+        } else {
+            for (int q = tid; q < mp::kGeneralPlanes; q += nthreads) s_tp[q] = mp::general_plane_of(q, s_thr);
+        }
+        __syncthreads();
+    }
+    // SA: one row serves every replica, and says how much a word has to do
+    int mode = mp::kCompare;
+    if (!PT && UNITJ) {
+        const uint32_t any = s_thr[2] | s_thr[4] | s_thr[6];
+        mode = any == 0u ? mp::kNoDraws : (any >> 24) == 0u ? mp::kTailOnly : mp::kCompare;
     }
     if constexpr (ENERGY) {
         wait_for_predecessor();
@@ -236,15 +250,15 @@ __global__ void __launch_bounds__(256, PT && !ENERGY ? SG_SWEEP_MINB : SG_SWEEP_
     uint32_t V[kVBits];
 #pragma unroll
     for (int j = 0; j < kVBits; ++j) V[j] = 0;
-    int nitems = 0;
+    int nitems = 0, weight = 0;  // items, and the weight of all their bonds (unit couplings: 6 each)
     auto fold_thread = [&]() {  // this thread's counters into the block sums (any time)
         for (int b = 0; b < 32; ++b) {
-            const int e = 6 * nitems - 2 * mp::vcount(V, b);
+            const int e = weight - 2 * mp::vcount(V, b);
             if (e) atomicAdd(&s_E[32 * g + b], e);
         }
 #pragma unroll
         for (int j = 0; j < kVBits; ++j) V[j] = 0;
-        nitems = 0;
+        nitems = weight = 0;
     };
 
     // one word of one site with unit couplings: update, store, queue ties, count energy
@@ -255,15 +269,24 @@ __global__ void __launch_bounds__(256, PT && !ENERGY ? SG_SWEEP_MINB : SG_SWEEP_
         uint32_t S[6];
         mp::unit_signs(sbits, S);
         const uint32_t valid = valid_bits(a.Rvalid, w);
-        uint32_t tp[24];
-        load_tp(w, tp);
+        if (!PT && mode == mp::kNoDraws) {
+            *wp = self ^ mp::update_word_free(self, n, S, valid);
+            return;
+        }
         uint32_t flip, tie, c0, c1, c2;
-        mp::update_word_unit(self, n, S, valid, tp, A, &flip, &tie, &c0, &c1, &c2);
+        if (!PT && mode == mp::kTailOnly) {
+            mp::update_word_tail(self, n, S, valid, A, &flip, &tie, &c0, &c1, &c2);
+        } else {
+            uint32_t tp[24];
+            load_tp(w, tp);
+            mp::update_word_unit(self, n, S, valid, tp, A, &flip, &tie, &c0, &c1, &c2);
+        }
         tie &= tie_can_accept(w, c0, c1);  // the others reject whatever the low bits
         if (tie) flip |= queue_tie((uint32_t)i, (uint32_t)is, (uint32_t)w, tie, c0, c1, self ^ flip);
         if (energy) {
             mp::count_after_flip(flip, c0, c1, c2);
             mp::vadd3(V, c0, c1, c2);
+            weight += 6;
             if (++nitems == kVItems) fold_thread();
         }
         if (flip) *wp = self ^ flip;
@@ -298,7 +321,7 @@ __global__ void __launch_bounds__(256, PT && !ENERGY ? SG_SWEEP_MINB : SG_SWEEP_
             it.self = sw[(uint32_t)(it.is * Wn)];
 #pragma unroll
             for (int q = 0; q < 6; ++q) it.n[q] = sw[(uint32_t)(nb[q] * Wn)];
-            mp::lead_planes((uint32_t)it.i, sweep, (uint32_t)w, key, it.A);
+            if (PT || mode != mp::kNoDraws) mp::lead_planes((uint32_t)it.i, sweep, (uint32_t)w, key, it.A);
         };
         const int rstride = gridDim.x * blockDim.y;
         int row = blockIdx.x * blockDim.y + threadIdx.y;
@@ -363,18 +386,16 @@ __global__ void __launch_bounds__(256, PT && !ENERGY ? SG_SWEEP_MINB : SG_SWEEP_
                         continue;
                     }
                     const uint32_t valid = valid_bits(a.Rvalid, w);
-                    const uint32_t flip = mp::update_word_general(self, n, J, valid, thr_row((uint32_t)w),
-                                                                  PT ? kThrStride : 0, A, (uint32_t)i, sweep,
-                                                                  (uint32_t)w, key);
-                    if (energy) {  // slow path: each replica's s_i sum_q J_q s_q after the update
-                        const uint32_t after = self ^ flip;
-                        for (int b = 0; b < 32; ++b) {
-                            int h = 0;
-#pragma unroll
-                            for (int q = 0; q < 6; ++q) h += J[q] * (((n[q] >> b) & 1u) ? -1 : 1);
-                            const int e = ((after >> b) & 1u) ? -h : h;
-                            if (e) atomicAdd(&s_E[32 * w + b], e);
-                        }
+                    uint32_t c[4];
+                    int M;
+                    const uint32_t flip = mp::update_word_general(
+                        self, n, J, valid, s_tp + (PT ? w : 0) * mp::kGeneralPlanes, thr_row((uint32_t)w),
+                        PT ? kThrStride : 0, A, (uint32_t)i, sweep, (uint32_t)w, key, c, &M);
+                    if (energy) {  // each replica's s_i sum_q J_q s_q after the update: M - 2c
+                        mp::weight_after_flip(flip, M, c);
+                        mp::vadd4(V, c);
+                        weight += M;
+                        if (++nitems == kVItemsGeneral) fold_thread();
                     }
                     if (flip) s[(size_t)is * Wn + w] = self ^ flip;
                 }
@@ -388,25 +409,23 @@ __global__ void __launch_bounds__(256, PT && !ENERGY ? SG_SWEEP_MINB : SG_SWEEP_
     resolve_list();
 
     if (energy) {
-        if (UNITJ) {
-            if (warp_lanes == 32) {
-                // lane r collects replica r of every lane through a bit transpose per plane
-                uint32_t T[kVBits];
+        if (warp_lanes == 32) {
+            // lane r collects replica r of every lane through a bit transpose per plane
+            uint32_t T[kVBits];
 #pragma unroll
-                for (int jb = 0; jb < kVBits; ++jb) T[jb] = mp::warp_transpose(V[jb], lane);
-                for (int w = 0; w < Wn; ++w) {
-                    const unsigned m = __ballot_sync(0xFFFFFFFFu, g == w);
-                    if (!m) continue;
-                    const int items = __reduce_add_sync(0xFFFFFFFFu, g == w ? nitems : 0);
-                    int cnt = 0;
+            for (int jb = 0; jb < kVBits; ++jb) T[jb] = mp::warp_transpose(V[jb], lane);
+            for (int w = 0; w < Wn; ++w) {
+                const unsigned m = __ballot_sync(0xFFFFFFFFu, g == w);
+                if (!m) continue;
+                const int total = __reduce_add_sync(0xFFFFFFFFu, g == w ? weight : 0);
+                int cnt = 0;
 #pragma unroll
-                    for (int jb = 0; jb < kVBits; ++jb) cnt += __popc(T[jb] & m) << jb;
-                    const int e = 6 * items - 2 * cnt;
-                    if (e) atomicAdd(&s_E[32 * w + lane], e);
-                }
-            } else {
-                fold_thread();
+                for (int jb = 0; jb < kVBits; ++jb) cnt += __popc(T[jb] & m) << jb;
+                const int e = total - 2 * cnt;
+                if (e) atomicAdd(&s_E[32 * w + lane], e);
             }
+        } else {
+            fold_thread();
         }
         __syncthreads();
         int32_t* Ei = a.E + (size_t)inst * Rp;
