@@ -619,9 +619,13 @@ int32_t run_sa_planes(const std::vector<int>& members, const sg_instance* const*
     // (cluster.cu), so that a large plane is not one block's work alone.
     int Ccl = 0;
     if (unit) {
-        std::vector<int> Ls(I);
-        for (int a = 0; a < I; ++a) Ls[a] = insts[members[a]]->L;
-        Ccl = sa_cluster_list_blocks(Ls.data(), I, max_L);
+        std::vector<int> Ls(I), sweeps(I), Wns(I);
+        for (int a = 0; a < I; ++a) {
+            Ls[a] = insts[members[a]]->L;
+            sweeps[a] = ps[members[a]].sweeps;
+            Wns[a] = words_for(ps[members[a]].replicas);
+        }
+        Ccl = sa_cluster_list_blocks(Ls.data(), sweeps.data(), Wns.data(), I);
     }
     auto width = [](int wg) { return wg == 0 ? 1 : wg; };  // words per plane in memory
     // planes running at once: blocks, or clusters (one block per SM)
@@ -647,7 +651,7 @@ int32_t run_sa_planes(const std::vector<int>& members, const sg_instance* const*
         cudaGetDeviceProperties(&prop, dev);
         std::ostringstream ks;
         ks << prop.name << "/" << sms << "/" << (unit ? "u" : "g") << "/smem" << smem_for(1) / 1024 << "/c" << Ccl
-           << "/t5";
+           << "/t6";
         for (auto& m : mix)
             ks << "/" << std::get<0>(m.first) << "x" << std::get<1>(m.first) << "x" << std::get<2>(m.first) << "x" << m.second;
         key = ks.str();

@@ -3,7 +3,7 @@
 //
 // A half sweep of a small lattice is too little work to pay for a launch, and a whole
 // lattice per block (batch.cu) leaves most SMs idle when an instance has few words.
-// Here cluster (word, instance) of C blocks splits the lattice into C slabs of L / C
+// Here cluster (word, instance) of C blocks splits the lattice into C slabs of about L / C
 // z-planes, block r keeping slab r of the word in its shared memory for the whole run
 // (slab.cuh: the updates, and how the blocks exchange their faces).  Every attempt draws
 // the same counters as the row kernel (site, sweep, word), so the results are
@@ -259,8 +259,7 @@ sa_cluster_kernel(const ClusterArgs a)
 }
 
 // Persistent form for batches (batch.cu's planes of one word, [N][1]).  Clusters take planes
-// order[0 .. n_cluster) through the counter next[0] until none is left (every side a multiple
-// of C), then each block by itself planes order[n_cluster .. n) through next[1]: a small
+// order[0 .. n_cluster) through the counter next[0] until none is left (no side below C), then each block by itself planes order[n_cluster .. n) through next[1]: a small
 // lattice does not fill a cluster, its half sweep being a chain of latencies, and four of them
 // side by side take little longer than one.  next[2]: status word.
 __global__ void __launch_bounds__(kListBlock, 1) sa_cluster_list_kernel(const Plane* __restrict__ planes,
@@ -392,16 +391,24 @@ int sa_block_threads(int L, int C, int threads)
     const int64_t pairs = slab::pairs_of(L, C);
     return slab::resident_threads(pairs, threads) + (slab::resident_items(pairs, threads) ? 32 : 0);
 }
+// Cycles of a half sweep with `per_sm` blocks of at most `threads` threads on an SM (see below).
+double half_sweep_cycles(int L, int C, int threads, int per_sm)
+{
+    const int64_t pairs = slab::pairs_of(L, C);
+    const double warps = std::max(1.0, (double)per_sm * (double)((pairs + 31) / 32) / 4.0);
+    return slab::resident_items(pairs, threads) ? 750.0 + 400.0 * warps : 2000.0 + 300.0 * warps;
+}
 }  // namespace
 
 // Blocks per cluster (and the threads to plan a block with) for an SA run of I instances of
-// side L with Wn words, or 0 when the row kernel should run it.  Candidates are the divisors
-// C <= 8 of L whose slab fits shared memory; clusters that are not resident at once (as the
-// driver reports for the kernel) run in waves.  A half sweep's cycles, fitted to measurements
+// side L with Wn words, or 0 when the row kernel should run it.  Candidates are the
+// C <= 8 whose largest slab fits shared memory and is thinner than with fewer blocks; clusters
+// that are not resident at once (as the driver reports for the kernel) run in waves.  A half sweep's cycles, fitted to measurements
 // on a GB300 (us at 2.07 GHz), times the waves:
 //   resident blocks  750 + 400 per warp of pairs an SM partition holds (L = 4 on one block of
 //                    one warp 0.53, L = 16 with 1024 replicas on C = 4 blocks of 16 warps 1.2)
-//   other blocks     2000 + 300 per warp of items (20 x L = 50 on C = 5 12.8, L = 64 on C = 8 20.6)
+//   other blocks     2000 + 300 per warp of items (20 x L = 50 on C = 5 12.8, L = 64 on C = 8 20.6;
+//                    clusters of 7 or 8 blocks would take 20 x L = 50 in two waves, C = 6 in one)
 //   row kernels      6500 + 490 per warp of items over the whole GPU (18.2 and 5.2 for the same)
 // The fewest cycles win, fewer blocks among equals.  With `busy` runs of the kind sharing the
 // device (a loaded server) a form's time is its own or, if that is longer, busy times its share
@@ -427,17 +434,15 @@ int sa_cluster_blocks(int I, int L, int Wn, bool force, int* threads, int busy)
     double best = force || forced ? 1e300 : 0.95 * std::max(6500.0 + row_share, busy * row_share);
     int bestC = 0;
     for (int C = 1; C <= 8; ++C) {
-        if (L % C || (forced && C != forced)) continue;
+        if (forced ? C != forced || C > L : !slab::worth(L, C)) continue;
         const int bt = sa_block_threads(L, C, t);
         const size_t bytes = slab::smem_bytes(L, C, bt);
         if (bytes + 2048 > (size_t)smem) continue;
         const int64_t active = resident_clusters(sa_cluster_fn(L, C, t), C, bytes, bt);
         if (active < 1) continue;
-        const int64_t pairs = slab::pairs_of(L, C);
         const int64_t waves = (clusters + active - 1) / active;
         const int64_t per_sm = (std::min(clusters, active) * C + sms - 1) / sms;  // blocks on the busiest SM
-        const double warps = std::max(1.0, (double)per_sm * (double)((pairs + 31) / 32) / 4.0);
-        double cost = waves * (slab::resident_items(pairs, t) ? 750.0 + 400.0 * warps : 2000.0 + 300.0 * warps);
+        double cost = waves * half_sweep_cycles(L, C, t, (int)per_sm);
         cost = std::max(cost, cost * busy * (double)(std::min(clusters, active) * C) / sms);
         if (cost < best) {
             best = cost;
@@ -455,20 +460,40 @@ size_t sa_list_smem(int max_L, int C)
 }
 }  // namespace
 
-int sa_cluster_list_blocks(const int* Ls, int n, int max_L)
+// Blocks per cluster for a batch: the C with the least estimated time, max(all work over the
+// clusters, the longest member on one).  14 lattices of sides 22, 40 and 44, 12 replicas: 1.0 ms
+// a call; 7.4 where clusters had to divide every side, which left planes of one block each.
+int sa_cluster_list_blocks(const int* Ls, const int* sweeps, const int* words, int n)
 {
-    int dev = 0, smem = 0;
+    int dev = 0, smem = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    for (int C = 8; C >= 2; --C) {
-        bool ok = true;
-        for (int k = 0; k < n && ok; ++k) ok = Ls[k] % C == 0;
-        if (!ok) continue;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int max_L = *std::max_element(Ls, Ls + n), min_L = *std::min_element(Ls, Ls + n);
+    int64_t small = 0;
+    for (int k = 0; k < n; ++k) small += Ls[k] <= kListAloneL ? words[k] : 0;
+    const bool alone = small >= sms;  // those run on single blocks
+    double best = 1e300;
+    int bestC = 0;
+    for (int C = 1; C <= std::min(slab::kMaxC, min_L); ++C) {
         const size_t bytes = sa_list_smem(max_L, C);
         if (bytes + 2048 > (size_t)smem) continue;
-        if (resident_clusters((const void*)sa_cluster_list_kernel, C, bytes, kListBlock) > 0) return C;
+        const int clusters = resident_clusters((const void*)sa_cluster_list_kernel, C, bytes, kListBlock);
+        if (clusters < 1) continue;
+        double total = 0, longest = 0;
+        for (int k = 0; k < n; ++k) {
+            const bool one = alone && Ls[k] <= kListAloneL;
+            const double t = sweeps[k] * half_sweep_cycles(Ls[k], one ? 1 : C, kListBlock, 1);
+            total += words[k] * (one ? t / C : t);
+            longest = std::max(longest, t);
+        }
+        const double t = std::max(total / clusters, longest);
+        if (t < best) {
+            best = t;
+            bestC = C;
+        }
     }
-    return 0;
+    return bestC;
 }
 
 int32_t launch_sa_cluster_planes(const Plane* d_planes, const int* d_order, int n_cluster, int n, unsigned* d_next,

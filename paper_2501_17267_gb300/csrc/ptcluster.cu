@@ -3,7 +3,7 @@
 // shared memory for the whole chunk.
 //
 // Cluster `inst` of C blocks splits the L^3 lattice of its instance into C z-slabs of
-// L / C planes, one 32-bit word of 32 slots per site (slab.cuh: the updates, and how the
+// about L / C planes, one 32-bit word of 32 slots per site (slab.cuh: the updates, and how the
 // blocks exchange their faces); the spins are written back at the end.
 //
 // Energies and the exchange.  Each bond joins a colour-0 and a colour-1 site, so the
@@ -329,14 +329,14 @@ double device_hz()
 // the row kernels on `sms` SMs, fitted to measurements on a GB300 (K = 32): clusters 2.1 us at
 // L = 8 (C = 2), 2.7 at L = 16, 6.1 at L = 24, 9.4 at L = 32, 49.6 at L = 64 (C = 8); row
 // kernels about 10 us of launches and 6.2 attempts per SM clock.
-double cluster_seconds(double work, int C, double hz) { return 3.7e-6 + work / (C * 11.0 * hz); }
+double cluster_seconds(int L, int C, double hz) { return 3.7e-6 + 64.0 * slab::pairs_of(L, C) / (11.0 * hz); }
 double row_seconds(double work, int I, int sms, double hz) { return 10e-6 + I * work / (sms * 6.2 * hz); }
 }  // namespace
 
 // Blocks per cluster for a PT run of I instances of side L with K <= 32 temperatures and
-// unit couplings, or 0 when the row kernels should run it.  C is the largest divisor
-// C <= 8 of L whose slab fits shared memory and for which all I clusters are resident at
-// once (one wave) -- but no larger than leaves a block 128 pairs of sites, a warp for each
+// unit couplings, or 0 when the row kernels should run it.  C is the largest up to 8 that
+// makes the slabs thinner, whose largest slab fits shared memory and for which all I clusters
+// are resident at once (one wave) -- but no larger than leaves a block 128 pairs of sites, a warp for each
 // partition of its SM (L = 8: 2.11 us a sweep on one or two blocks, 2.45 on eight).  The
 // cluster form is taken when its estimated time per sweep is below the row kernels'.  Knob
 // SG_PT_CLUSTER = 0 turns the form off, = 1 takes it whenever a slab fits.
@@ -354,16 +354,16 @@ int pt_cluster_blocks(int I, int L, int K, double* seconds)
     const char* fc = getenv("SG_PT_CLUSTER_C");  // tuning knob: force C (when it divides L and fits)
     const int forced = fc ? atoi(fc) : 0;
     for (int C = 8; C >= 1; --C) {
-        if (L % C || (forced > 0 && C != forced)) continue;
+        if (forced > 0 ? C != forced || C > L : !slab::worth(L, C)) continue;
         const size_t bytes = dyn_smem(L, C);
         if (bytes + sizeof(PtShared) > (size_t)smem) continue;
         if (knob == 1 || forced > 0) return C;
         if (resident_clusters(kernel_of(L, C), C, bytes, block_threads(L, C)) < I) continue;
         bool smaller = false;  // a smaller cluster with blocks of at most 128 pairs
-        for (int c = C - 1; c >= 1 && !smaller; --c) smaller = L % c == 0 && slab::pairs_of(L, c) <= 128;
+        for (int c = C - 1; c >= 1 && !smaller; --c) smaller = slab::pairs_of(L, c) <= 128;
         if (smaller) continue;
         const double work = (double)L * L * L * 32.0;  // attempts per sweep of one instance (whole words)
-        const double t = cluster_seconds(work, C, hz);
+        const double t = cluster_seconds(L, C, hz);
         if (seconds) *seconds = t;
         return t < 0.95 * row_seconds(work, I, sms, hz) ? C : 0;
     }
@@ -389,8 +389,8 @@ int pt_cluster_blocks_shared(int L, int K, int busy)
     double best = 0.95 * std::max(row_seconds(work, 1, sms, hz), busy * (row_seconds(work, 1, sms, hz) - 10e-6));
     int bestC = 0;
     for (int C = 8; C >= 1; --C) {
-        if (L % C || dyn_smem(L, C) + sizeof(PtShared) > (size_t)smem) continue;
-        const double t = cluster_seconds(work, C, hz), shared = std::max(t, busy * C * t / sms);
+        if (!slab::worth(L, C) || dyn_smem(L, C) + sizeof(PtShared) > (size_t)smem) continue;
+        const double t = cluster_seconds(L, C, hz), shared = std::max(t, busy * C * t / sms);
         if (shared < best && resident_clusters(kernel_of(L, C), C, dyn_smem(L, C), block_threads(L, C)) > 0) {
             best = shared;
             bestC = C;
@@ -424,13 +424,13 @@ int pt_cluster_split(int I, int L, int K, int* M, int* side_sms, double* seconds
     double best = 0.95 * row_seconds(work, I, sms, hz);
     int bestC = 0;
     for (int C = 8; C >= 1; --C) {
-        if (L % C) continue;
+        if (!slab::worth(L, C)) continue;
         const size_t bytes = dyn_smem(L, C);
         if (bytes + sizeof(PtShared) > (size_t)smem) continue;
         const int active = resident_clusters(kernel_of(L, C), C, bytes, block_threads(L, C));
         if (active >= I || active < 1) continue;  // one wave: pt_cluster_blocks decides
         const int per_sm = std::max(1, (active * C + sms - 1) / sms);  // blocks an SM holds
-        const double t_cluster = cluster_seconds(work, C, hz);
+        const double t_cluster = cluster_seconds(L, C, hz);
         for (int m = active; m >= 1; --m) {
             const int left = sms - (m * C + per_sm - 1) / per_sm;
             if (left < 1) continue;

@@ -230,8 +230,8 @@ int32_t launch_sa_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const Ru
                           int s_end, int C, int threads, cudaStream_t st, const uint32_t* sweep_base = nullptr,
                           const ChunkReport& report = ChunkReport{});
 // The persistent cluster form for batches of one-word planes (batch.cu): C for planes of
-// sides Ls (every side a multiple of C, the slab of the largest fitting), or 0.
-int sa_cluster_list_blocks(const int* Ls, int n, int max_L);
+// sides Ls, each of words[k] planes and sweeps[k] sweeps, or 0 when the largest does not fit.
+int sa_cluster_list_blocks(const int* Ls, const int* sweeps, const int* words, int n);
 // Planes order[0 .. n_cluster) go to clusters, the others, of sides up to kListAloneL, to
 // single blocks; d_next: two zeroed counters and the status word.
 constexpr int kListAloneL = 16;

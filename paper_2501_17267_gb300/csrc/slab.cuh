@@ -2,9 +2,11 @@
 // (App. D.1 / D.2, unit couplings): the machinery shared by the annealing kernels
 // (cluster.cu) and the tempering kernel (ptcluster.cu).
 //
-// Block r of a cluster of C blocks holds z-planes [r zc, (r + 1) zc) of one 32-bit word a
-// site (zc = L / C), between two halo planes: a copy of the plane below its slab and of the
-// plane above it.  A half sweep updates the sites of one colour from the words of the other.
+// Block r of a cluster of C blocks holds z-planes [r L / C, (r + 1) L / C) of one 32-bit word a
+// site, between two halo planes: a copy of the plane below its slab and of the plane above it.
+// (C need not divide L; slabs then differ by a plane, and the largest one counts: 20 L = 50
+// lattices take C = 7, slabs of at most 8 planes, instead of C = 5.)  A half sweep updates the
+// sites of one colour from the words of the other.
 //
 // Columns.  A lane owns a column (y, j): the colour's site of x pair j in row y of every
 // plane of its segment, walked upwards.  With M(z) the other word of the pair in plane z --
@@ -201,7 +203,7 @@ struct Draws {
 
 // (Kept in shared memory: most of it is read once a unit.)
 struct Geometry {
-    int L, H, LL, zc, z0;         // side, half, plane, planes of the slab, first of them
+    int L, H, LL, zc, z0, zdn;    // side, half, plane, planes of the slab, first of them, planes of the slab below
     int cols, chunks;             // columns of a colour, warps of columns
     int segments, seglen, units;  // z segments of a column, their planes, (segment, chunk) pairs
     uint32_t Hmagic, Lmagic;      // ceil(2^32 / H), ceil(2^32 / L)
@@ -213,8 +215,9 @@ struct Geometry {
         L = L_;
         H = L >> 1;
         LL = L * L;
-        zc = L / C;
-        z0 = r * zc;
+        z0 = first(L, C, r);
+        zc = first(L, C, r + 1) - z0;
+        zdn = r == 0 ? L - first(L, C, C - 1) : z0 - first(L, C, r - 1);
         cols = L * H;
         chunks = (cols + 31) / 32;
         Hmagic = Hmagic_;
@@ -234,9 +237,16 @@ struct Geometry {
         }
         units = chunks * segments;
     }
-    __host__ __device__ static size_t words(int L, int C) { return (size_t)(L / C + 2) * L * L; }
-    __host__ __device__ static size_t sites(int L, int C) { return (size_t)(L / C) * L * L; }
+    __host__ __device__ static int first(int L, int C, int r) { return r * L / C; }  // block r's first plane
+    // of the largest slab: its planes, its words with both halos, its sites
+    __host__ __device__ static int planes(int L, int C) { return (L + C - 1) / C; }
+    __host__ __device__ static size_t words(int L, int C) { return (size_t)(planes(L, C) + 2) * L * L; }
+    __host__ __device__ static size_t sites(int L, int C) { return (size_t)planes(L, C) * L * L; }
 };
+
+// Whether clusters of C blocks can hold side L: C of them have a plane, and fewer would not do
+// with slabs as thin.
+inline bool worth(int L, int C) { return C <= L && (C == 1 || Geometry::planes(L, C) < Geometry::planes(L, C - 1)); }
 
 // Dynamic shared memory of a block: halo, slab and halo words, the slab's sign bytes in
 // storage order, the warps' tie queues.
@@ -563,14 +573,15 @@ struct Sweeper {
     __device__ __forceinline__ void push_faces(const int colour, bool alone, uint32_t up, uint32_t dn, uint32_t up_bar,
                                                uint32_t dn_bar)
     {
-        const uint32_t LL4 = 4u * (uint32_t)g.LL, H4 = 4u * (uint32_t)g.H, slab = (uint32_t)g.zc * LL4;
+        const uint32_t LL4 = 4u * (uint32_t)g.LL, H4 = 4u * (uint32_t)g.H, slab = (uint32_t)g.zc * LL4,
+                       slab_dn = (uint32_t)g.zdn * LL4;
         Unit v = u;
         for (int q = warp; q < g.units;) {
             const uint32_t odd = v.flags ^ (uint32_t)colour;
             if ((v.flags & (kBottom | kLive)) == (kBottom | kLive)) {  // to the upper halo of the block below
                 const uint32_t is = v.base + ((odd & kOdd) ? H4 : 0u);
                 if (alone) st_word_if(1u, is + slab, ld_word(is));
-                else push_word(dn + is + slab, ld_word(is), dn_bar);
+                else push_word(dn + is + slab_dn, ld_word(is), dn_bar);
             }
             if ((v.flags & (kTop | kLive)) == (kTop | kLive)) {  // to the lower halo of the block above
                 const uint32_t is = v.base + (uint32_t)(v.n - 1) * LL4 + (((odd ^ (uint32_t)(v.n - 1)) & kOdd) ? H4 : 0u);
@@ -618,7 +629,7 @@ struct Resident {
     uint32_t word, valid, sweep;
     int warp, lane;
     int LL4;
-    uint32_t slab;            // bytes of the slab
+    uint32_t slab, slab_dn;   // bytes of the slab, and of the one below
     bool idle;                // a warp beyond the pairs (uniform)
     struct Pair {
         // of its site of colour 0 and of colour 1
@@ -635,6 +646,7 @@ struct Resident {
         const int L = g.L, H = g.H, LL = g.LL;
         LL4 = 4 * LL;
         slab = (uint32_t)(g.zc * LL4);
+        slab_dn = (uint32_t)(g.zdn * LL4);
         idle = warp * 32 >= g.zc * g.cols;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
@@ -786,7 +798,7 @@ struct Resident {
             const Pair& q = pair[r];
             if (q.flags & kBottom) {
                 if (alone) st_word_if(1u, q.at[C] + slab, q.value[C]);
-                else push_word(dn + q.at[C] + slab, q.value[C], dn_bar);
+                else push_word(dn + q.at[C] + slab_dn, q.value[C], dn_bar);
             }
             if (q.flags & kTop) {
                 if (alone) st_word_if(1u, q.at[C] - slab, q.value[C]);
@@ -821,7 +833,7 @@ inline int resident_threads(int64_t pairs, int threads)
     const int r = resident_items(pairs, threads);
     return r == 0 ? threads : (int)((pairs + 32 * r - 1) / (32 * r)) * 32;
 }
-__host__ __device__ inline int64_t pairs_of(int L, int C) { return (int64_t)(L / C) * L * (L / 2); }
+__host__ __device__ inline int64_t pairs_of(int L, int C) { return (int64_t)Geometry::planes(L, C) * L * (L / 2); }
 
 }  // namespace slab
 }  // namespace sg

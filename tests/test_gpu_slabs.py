@@ -58,6 +58,27 @@ def test_tempering_on_clusters_equals_row_kernels(sg, monkeypatch, L, C):
         assert x["minE"] == y["minE"]
 
 
+# C that does not divide L: slabs differ by a plane
+@pytest.mark.parametrize("L,C", [(4, 3), (6, 4), (8, 5), (10, 7), (14, 4), (18, 5), (22, 3), (26, 8), (34, 7), (50, 7)])
+def test_slabs_of_unequal_height(sg, monkeypatch, L, C):
+    test_annealing_on_clusters_equals_row_kernel(sg, monkeypatch, L, C)
+    test_tempering_on_clusters_equals_row_kernels(sg, monkeypatch, L, C)
+
+
+def test_batch_whose_sides_share_no_divisor(sg, monkeypatch, tmp_path):
+    sides = [22, 40, 44, 10, 26]
+    insts = [sg.Instance.create(L, 700 + k) for k, L in enumerate(sides)]
+    ps = [dict(replicas=40, sweeps=(6, 11)[k % 2], beta0=0.1, beta1=3.0, schedule="linear", seed=2, instance_id=k)
+          for k in range(len(sides))]
+    monkeypatch.setenv("SG_AUTOTUNE_CACHE", str(tmp_path / "tune.json"))
+    runs = []
+    for wg in ("0", "1"):  # clusters; planes of one word, a block each
+        monkeypatch.setenv("SG_BATCH_WG", wg)
+        runs.append(sg.sa_run_batch(insts, ps, spins="host"))
+    for x, y in zip(*runs):
+        assert np.array_equal(x["spins"], y["spins"]) and np.array_equal(x["E"], y["E"])
+
+
 @pytest.mark.parametrize("n_small", [40, 200])
 def test_batch_of_small_lattices_on_clusters_and_single_blocks(sg, monkeypatch, tmp_path, n_small):
     """Few small planes are annealed by whole clusters, enough of them by single blocks."""
