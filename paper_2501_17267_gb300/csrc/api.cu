@@ -948,11 +948,13 @@ int32_t fragment_batch(const sg_instance* const* insts, const sg_fragment_params
     for (int s = 0; s < S; ++s) metropolis_row(beta[s], &thr[(size_t)s * kThrRow]);
     std::vector<RunKeys> keys(I);
     std::vector<const void*> jp((size_t)I);
+    bool unit = true;
     for (int a = 0; a < I; ++a) {
         keys[a] = make_key(ps[a].seed, ps[a].instance_id);
         const uint2* j6 = nullptr;
         SG_RET(instance_device_j6(const_cast<sg_instance*>(insts[a]), st, &j6, nullptr));
         jp[a] = j6;
+        unit &= insts[a]->unit_couplings;
     }
     DevBuf d_spins, d_thr, d_keys, d_j6, d_E64, d_bad;
     SG_RET(d_spins.alloc((size_t)I * N, st));
@@ -979,7 +981,7 @@ int32_t fragment_batch(const sg_instance* const* insts, const sg_fragment_params
     SG_RET(log.run(SG_KERNEL_SWEEP, units, st, [&] {
         if (tropical) return launch_fragment_tropical_waves(d_spins.as<int8_t>(), d_j6.as<const uint2*>(), I, L, l, st);
         return launch_fragment_waves(d_spins.as<int8_t>(), d_j6.as<const uint2*>(), d_keys.as<RunKeys>(),
-                                     d_thr.as<uint32_t>(), I, L, l, S, st);
+                                     d_thr.as<uint32_t>(), I, L, l, S, unit, st);
     }, V));
     // energies (Eq. 1) of the int8 configurations
     for (int a = 0; a < I; a += (int)kMaxGroup) {

@@ -5,19 +5,28 @@
 // mod l.  The fragment of such a spin is the cube of side l centred on it; with L a
 // multiple of l the fragments of one wave are disjoint, so one launch anneals all of
 // them.  A warp owns one fragment: its 32 reads are the 32 bits of one word per cube
-// site, kept in shared memory for the whole anneal, beside the site's couplings (those
-// of bonds leaving the cube cleared) and a list of the free sites of each colour.  Sites
-// fixed by earlier waves hold all-equal words and are never updated.  Bonds may have
-// |J| = 2 or 0: a site's positive bond terms are counted for all 32 reads at once in bit
-// planes weighted by |J|, which gives x = s_i h_i of every read; only the reads with
-// x < 0 take their draw and threshold one by one.  The read of lowest cube energy fixes
-// the centre spin in global memory.
+// site, kept in shared memory for the whole anneal, beside a word of the site's couplings
+// and a list of the free sites of each colour.  Sites fixed by earlier waves hold all-equal
+// words and are never updated.  The read of lowest cube energy fixes the centre spin in
+// global memory.
+//
+// A half sweep takes the colour's free sites 32 at a time, in two steps.  First a lane has
+// a site: for all reads at once it counts P, the weight of the positive bond terms
+// J s_i s_k, and keeps d = ceil(M / 2) - P as bit planes, M the weight of all the site's
+// bonds.  x = s_i h_i = 2P - M is negative exactly where d > 0 (the others accept), and the
+// threshold is then that of k = 2d, or 2d - 1 when M is odd.  Then a lane has a site and
+// four of its reads, the reads one Philox block draws for: 32-bit draws leave no other way
+// than a block for each four reads, and they are most of the work.  The second step runs
+// with all lanes busy however few sites are free, where a lane that stayed with its site
+// through its eight blocks left two thirds of them idle on average (the free sites shrink
+// from l^3 to one over the waves) and followed branches for each read.
 #include <stdint.h>
 #include <stdio.h>
 
 #include <algorithm>
 #include <vector>
 
+#include "metropolis.cuh"
 #include "philox.cuh"
 #include "sg_internal.h"
 
@@ -34,6 +43,7 @@ struct FragArgs {
     const RunKeys* keys;           // [I]
     const uint32_t* thr;           // [S][kThrRow]
     int L, l, S;
+    uint32_t lmagic;               // ceil(2^32 / l) (0 for l = 1)
 };
 
 __device__ __forceinline__ int coupling(uint2 r, int q)
@@ -41,174 +51,254 @@ __device__ __forceinline__ int coupling(uint2 r, int q)
     return (int)(int8_t)(((q < 4 ? r.x : r.y) >> (8 * (q & 3))) & 0xFFu);
 }
 
-__global__ void __launch_bounds__(kWarps * 32) fragment_wave_kernel(const FragArgs a, int wave)
+// The draws of one fragment: Philox counters (centre, sweep, item, domain), whose first two
+// rounds share two of their four multiplies (one of each round's pair sees the centre alone).
+struct FragDraws {
+    RunKeys key;
+    uint32_t sx, sy, sl;
+    __device__ __forceinline__ FragDraws(uint32_t centre, const RunKeys& k) : key(k)
+    {
+        uint32_t hi, lo, h2;
+        philox_mulhilo(kPhiloxMulA, centre, &hi, &lo);
+        philox_mulhilo(kPhiloxMulB, hi ^ kDomainFragment ^ key.k1, &h2, &sl);
+        sx = h2 ^ (key.k0 + kPhiloxWeylA);
+        sy = lo ^ (key.k1 + kPhiloxWeylB);
+    }
+    __device__ __forceinline__ void draw(uint32_t sweep, uint32_t item, uint32_t (&c)[4]) const
+    {
+        uint32_t hi, lo, h2, l2;
+        philox_mulhilo(kPhiloxMulB, item, &hi, &lo);
+        philox_mulhilo(kPhiloxMulA, hi ^ sweep ^ key.k0, &h2, &l2);
+        c[0] = lo ^ sx, c[1] = sl, c[2] = h2 ^ sy, c[3] = l2;
+#pragma unroll
+        for (int r = 2; r < 10; ++r) {
+            philox_mulhilo(kPhiloxMulA, c[0], &hi, &lo);
+            philox_mulhilo(kPhiloxMulB, c[2], &h2, &l2);
+            c[0] = mp::logic<mp::kXor3>(h2, c[1], key.k0 + (uint32_t)r * kPhiloxWeylA);
+            c[1] = l2;
+            c[2] = mp::logic<mp::kXor3>(hi, c[3], key.k1 + (uint32_t)r * kPhiloxWeylB);
+            c[3] = lo;
+        }
+    }
+};
+
+// Reads: bit 8m + g of a word is read 4g + m, so that the reads of one Philox block (a g) are
+// the same bit of the word's four bytes, and a ballot over (site, g) lanes is a byte a site.
+//
+// Records: site q of the cube (9 bits), M (4), then six bits each (order +x, -x, +y, -y, +z,
+// -z): bonds inside the cube that are positive, of weight 1, of weight 2.
+constexpr int kOrAnd = 0xF8;  // (mp::logic) a | (b & c)
+constexpr int kRecM = 9, kRecPos = 13, kRecOne = 19, kRecTwo = 25;
+
+__device__ __forceinline__ uint32_t rotate_right(uint32_t x, int n) { return __funnelshift_r(x, x, n); }
+
+// UNITJ: all |J| = 1 (no record has bonds of weight 2).
+template <bool UNITJ>
+__global__ void __launch_bounds__(kWarps * 32, 8) fragment_wave_kernel(const FragArgs a, int wave)
 {
-    __shared__ uint32_t s_words[kWarps][kVMax];  // bit r: read r's spin is -1
-    __shared__ uint2 s_rec[kWarps][kVMax];       // couplings of the bonds inside the cube (others 0)
+    constexpr unsigned kAll = 0xFFFFFFFFu;
+    constexpr int kPad = kLMax * kLMax;  // a bond that leaves the cube still loads a word
+    __shared__ uint32_t s_words[kWarps][kVMax + 2 * kPad];
+    __shared__ uint32_t s_rec[kWarps][kVMax];
     __shared__ uint16_t s_free[kWarps][2][(kVMax + 1) / 2];  // free sites of each colour
+    __shared__ __align__(16) uint4 s_item[kWarps][32];       // of a lane's site: the planes of d, then 8q | odd M << 31
+    __shared__ __align__(64) uint32_t s_thr[kWarps][16];     // the sweep's thresholds, [M odd][d]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int inst = blockIdx.y;
-    const int L = a.L, l = a.l, h = (l - 1) / 2, V = l * l * l;
+    const int L = a.L, l = a.l, h = (l - 1) / 2, ll = l * l, V = ll * l;
     const int per = L / l;
     const int frag = blockIdx.x * kWarps + warp;
     if (frag >= per * per * per) return;  // the whole warp
-    const int ca = wave % l, cb = (wave / l) % l, cc = wave / (l * l);
+    const int ca = wave % l, cb = (wave / l) % l, cc = wave / ll;
     const int cx = ca + l * (frag % per), cy = cb + l * ((frag / per) % per), cz = cc + l * (frag / (per * per));
-    const uint32_t centre = (uint32_t)(cx + L * (cy + L * cz));
-    const RunKeys key = a.keys[inst];
+    const int centre = cx + L * (cy + L * cz);
+    const FragDraws draws((uint32_t)centre, a.keys[inst]);
     const uint2* __restrict__ j6 = a.j6_ptrs[inst];
     int8_t* __restrict__ sp = a.spins + (size_t)inst * L * L * L;
-    uint32_t* words = s_words[warp];
-    uint2* recs = s_rec[warp];
+    uint32_t* const words = s_words[warp] + kPad;
+    uint32_t* const recs = s_rec[warp];
+    uint4* const items = s_item[warp];
+    uint32_t* const thr = s_thr[warp];
 
-    auto site_of = [&](int q, int* x, int* y, int* z) {
-        const int dx = q % l, dy = (q / l) % l, dz = q / (l * l);
-        *x = (cx + dx - h + L) % L;
-        *y = (cy + dy - h + L) % L;
-        *z = (cz + dz - h + L) % L;
-    };
-    // fixed by an earlier wave: its residue class precedes this wave's
-    auto fixed = [&](int x, int y, int z) { return (x % l) + l * ((y % l) + l * (z % l)) < wave; };
-
-    // cube sites: couplings of the bonds inside the cube, initial words, and the list of
-    // the free sites of each colour (compacted by ballot, warp-uniform counts)
+    // cube sites: records, the words of fixed sites, and the lists of the free sites of each
+    // colour (compacted by ballot, warp-uniform counts)
     int nfree[2] = {0, 0};
     for (int base = 0; base < V; base += 32) {
         const int q = base + lane;
         bool free_site = false;
         int colour = 0;
         if (q < V) {
-            int x, y, z;
-            site_of(q, &x, &y, &z);
+            const int row = l == 1 ? q : (int)__umulhi((uint32_t)q, a.lmagic), dx = q - row * l;
+            const int dz = l == 1 ? row : (int)__umulhi((uint32_t)row, a.lmagic), dy = row - dz * l;
+            auto wrap = [](int v, int n) { return v < 0 ? v + n : v >= n ? v - n : v; };
+            const int x = wrap(cx + dx - h, L), y = wrap(cy + dy - h, L), z = wrap(cz + dz - h, L);
             const int i = x + L * (y + L * z);
-            const int dd[3] = {q % l, (q / l) % l, q / (l * l)};
-            uint2 r = j6[i];
+            const uint2 r = j6[i];
+            const int d[3] = {dx, dy, dz};
+            uint32_t M = 0, pos = 0, one = 0, two = 0;
 #pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                const int up = 2 * d, dn = 2 * d + 1;  // record bytes of the +d and -d bonds
-                if (dd[d] + 1 >= l) (up < 4 ? r.x : r.y) &= ~(0xFFu << (8 * (up & 3)));
-                if (dd[d] == 0) (dn < 4 ? r.x : r.y) &= ~(0xFFu << (8 * (dn & 3)));
+            for (int k = 0; k < 6; ++k) {
+                const int J = (k & 1 ? d[k / 2] > 0 : d[k / 2] + 1 < l) ? coupling(r, k) : 0;
+                const int weight = J < 0 ? -J : J;
+                pos |= (J > 0 ? 1u : 0u) << k;
+                one |= (weight == 1 ? 1u : 0u) << k;
+                two |= (weight == 2 ? 1u : 0u) << k;
+                M += (uint32_t)weight;
             }
-            recs[q] = r;
-            uint32_t word = 0;
-            if (fixed(x, y, z)) {
-                word = sp[i] < 0 ? 0xFFFFFFFFu : 0u;
+            recs[q] = (uint32_t)q | M << kRecM | pos << kRecPos | one << kRecOne | two << kRecTwo;
+            // fixed by an earlier wave: its residue class precedes this wave's
+            if (wrap(ca + dx - h, l) + l * (wrap(cb + dy - h, l) + l * wrap(cc + dz - h, l)) < wave) {
+                words[q] = sp[i] < 0 ? kAll : 0u;
             } else {
                 free_site = true;
                 colour = (x + y + z) & 1;
-                for (int g = 0; g < 8; ++g) {
-                    const Philox4 u = philox4x32_10(centre, kSweepInit, (uint32_t)(8 * q + g), kDomainFragment,
-                                                    key.k0, key.k1);
-#pragma unroll
-                    for (int m = 0; m < 4; ++m) word |= (u.v[m] >> 31) << (4 * g + m);
-                }
             }
-            words[q] = word;
         }
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
             const bool mine = free_site && colour == c;
-            const unsigned bal = __ballot_sync(0xFFFFFFFFu, mine);
+            const unsigned bal = __ballot_sync(kAll, mine);
             if (mine) s_free[warp][c][nfree[c] + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)q;
             nfree[c] += __popc(bal);
         }
     }
     __syncwarp();
 
-    // One site, all 32 reads: with p_k the reads whose bond term J_k s_i s_k is positive,
-    // x = s_i h_i = 2P - M for P = sum |J_k| p_k (kept as bit planes P0..P3) and
-    // M = sum |J_k|.  x >= 0 accepts; the others compare their draw with thr[-x].
+    const int g = lane & 7;                                   // second steps: the lane's Philox block
+    const uint32_t byte = (uint32_t)(lane & 3) * 0x11u + 0x40u;  // (prmt) bytes lane % 4 of two words
+    // Of up to 32 sites, four at a time: bit(e, m) decides read 4g + m of site e; returns the
+    // word of the lane's site.
+    auto rounds = [&](int n, auto&& prepare, auto&& bit) {
+        uint32_t word = 0;
+#pragma unroll 2
+        for (int r = 0; 4 * r < n; ++r) {
+            uint32_t v[4], ctx[2];
+            prepare(4 * r + (lane >> 3), v, ctx);
+            unsigned b[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) b[m] = __ballot_sync(kAll, bit(m, v, ctx));
+            const uint32_t mine = __byte_perm(__byte_perm(b[0], b[1], byte), __byte_perm(b[2], b[3], byte), 0x5410);
+            if ((lane >> 2) == r) word = mine;
+        }
+        return word;
+    };
+
+    // initial words
+    for (int c = 0; c < 2; ++c) {
+        for (int base = 0; base < nfree[c]; base += 32) {
+            const int n = min(32, nfree[c] - base);
+            const uint16_t* list = s_free[warp][c] + base;
+            const uint32_t word = rounds(
+                n,
+                [&](int e, uint32_t (&v)[4], uint32_t (&)[2]) {
+                    draws.draw(kSweepInit, 8u * list[min(e, n - 1)] + (uint32_t)g, v);
+                },
+                [](int m, const uint32_t (&v)[4], const uint32_t (&)[2]) { return v[m] >> 31; });
+            if (lane < n) words[list[lane]] = word;
+        }
+    }
+    __syncwarp();
+
+    const int entry_k = 2 * (lane & 7) - ((lane >> 3) & 1);  // thr[lane], lane < 16
+    auto entry_of = [&](int sw) {
+        return lane < 16 && entry_k >= 1 && entry_k < kThrRow && sw < a.S ? a.thr[(size_t)sw * kThrRow + entry_k] : 0u;
+    };
+    uint32_t entry = entry_of(0);
     for (int sw = 0; sw < a.S; ++sw) {
-        const uint32_t* thr = a.thr + (size_t)sw * kThrRow;
-        for (int colour = 0; colour < 2; ++colour) {
-            for (int e = lane; e < nfree[colour]; e += 32) {
-                const int q = s_free[warp][colour][e];
-                const uint2 rec = recs[q];
+        if (lane < 16) thr[lane] = entry;
+        entry = entry_of(sw + 1);
+        for (int c = 0; c < 2; ++c) {
+            for (int base = 0; base < nfree[c]; base += 32) {
+                const int n = min(32, nfree[c] - base);
+                const int q = s_free[warp][c][base + min(lane, n - 1)];
+                const uint32_t rec = recs[q];
                 const uint32_t self = words[q];
-                uint32_t P0 = 0, P1 = 0, P2 = 0, P3 = 0;
-                int M = 0;
+                const uint32_t nb[6] = {words[q + 1],  words[q - 1],  words[q + l],
+                                        words[q - l], words[q + ll], words[q - ll]};
+                uint32_t pos[6], mask[6], p[6];
+                mp::unit_signs((rec >> kRecPos) & 63u, pos);
+                mp::unit_signs((rec >> kRecOne) & 63u, mask);
 #pragma unroll
-                for (int k = 0; k < 6; ++k) {
-                    const int J = coupling(rec, k);
-                    if (J == 0) continue;  // no bond (or one leaving the cube)
-                    const int step = k < 2 ? 1 : k < 4 ? l : l * l;
-                    const uint32_t eq = ~(self ^ words[(k & 1) ? q - step : q + step]);
-                    const uint32_t p = J > 0 ? eq : ~eq;
-                    if (J == 1 || J == -1) {  // add p at weight 1
-                        const uint32_t c1 = P0 & p;
-                        P0 ^= p;
-                        const uint32_t c2 = P1 & c1;
-                        P1 ^= c1;
-                        P3 ^= P2 & c2;
-                        P2 ^= c2;
-                        M += 1;
-                    } else {  // |J| = 2: add p at weight 2
-                        const uint32_t c2 = P1 & p;
-                        P1 ^= p;
-                        P3 ^= P2 & c2;
-                        P2 ^= c2;
-                        M += 2;
-                    }
-                }
-                // need: x < 0, i.e. P < T = ceil(M / 2) (borrow of P - T, LSB first)
-                const int T = (M + 1) >> 1;
-                uint32_t need = 0;
-                {
-                    const uint32_t Pj[4] = {P0, P1, P2, P3};
+                for (int k = 0; k < 6; ++k) p[k] = mp::logic<mp::kXor3>(self, nb[k], pos[k]);
+                uint32_t P[4], term[6];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const uint32_t tm = ((T >> j) & 1) ? 0xFFFFFFFFu : 0u;
-                        need = (~Pj[j] & tm) | (~(Pj[j] ^ tm) & need);
-                    }
-                }
-                uint32_t flip = ~need;
-                for (int g = 0; g < 8; ++g) {  // reads 4g .. 4g + 3
-                    const uint32_t nm = (need >> (4 * g)) & 0xFu;
-                    if (!nm) continue;
-                    const Philox4 u =
-                        philox4x32_10(centre, (uint32_t)sw, (uint32_t)(8 * q + g), kDomainFragment, key.k0, key.k1);
+                for (int k = 0; k < 6; ++k) term[k] = p[k] & mask[k];
+                mp::count_six(term, P[0], P[1], P[2]);
+                P[3] = 0;
+                if constexpr (!UNITJ) {
+                    mp::unit_signs((rec >> kRecTwo) & 63u, mask);
 #pragma unroll
-                    for (int m = 0; m < 4; ++m) {
-                        if (!((nm >> m) & 1u)) continue;
-                        const int b = 4 * g + m;
-                        const int Pb = (int)(((P0 >> b) & 1u) | (((P1 >> b) & 1u) << 1) | (((P2 >> b) & 1u) << 2) |
-                                             (((P3 >> b) & 1u) << 3));
-                        if (u.v[m] < thr[M - 2 * Pb]) flip |= 1u << b;
-                    }
+                    for (int k = 0; k < 6; ++k) term[k] = p[k] & mask[k];
+                    uint32_t t0, t1, t2;
+                    mp::count_six(term, t0, t1, t2);
+                    const uint32_t k1 = P[1] & t0, k2 = mp::maj3(P[2], t1, k1);
+                    P[1] ^= t0;
+                    P[2] = mp::logic<mp::kXor3>(P[2], t1, k1);
+                    P[3] = t2 ^ k2;
                 }
-                words[q] = self ^ flip;
+                // d = T - P, its borrow marks P > T
+                const int M = (int)(rec >> kRecM) & 15, T = (M + 1) >> 1;
+                const uint32_t T0 = mp::plane_mask(T, 0), T1 = mp::plane_mask(T, 1), T2 = mp::plane_mask(T, 2);
+                const uint32_t d0 = T0 ^ P[0], b0 = ~T0 & P[0];
+                const uint32_t d1 = mp::logic<mp::kXor3>(T1, P[1], b0), b1 = mp::logic<mp::kBorrow>(T1, P[1], b0);
+                const uint32_t d2 = mp::logic<mp::kXor3>(T2, P[2], b1), b2 = mp::logic<mp::kBorrow>(T2, P[2], b1);
+                const uint32_t need = (d0 | d1 | d2) & ~(b2 | P[3]);
+                // the planes where the second step shifts them to: bits 2, 3 and 4 of a byte
+                items[lane] = make_uint4(rotate_right(d0, 30), rotate_right(d1, 29), rotate_right(d2, 28),
+                                         8u * (uint32_t)q | (uint32_t)M << 31);
+                __syncwarp();
+                const uint32_t lt = rounds(
+                    n,
+                    [&](int e, uint32_t (&v)[4], uint32_t (&ctx)[2]) {
+                        const uint4 it = items[e];
+                        draws.draw((uint32_t)sw, (it.w & 0x7FFFFFFFu) + (uint32_t)g, v);
+                        // byte m: offset of read 4g + m's threshold, d * 4 + (M odd) * 32
+                        const uint32_t odd = (uint32_t)((int)it.w >> 31) & 0x20202020u;
+                        ctx[0] = mp::logic<kOrAnd>(odd, rotate_right(it.x, g), 0x04040404u);
+                        ctx[0] = mp::logic<kOrAnd>(ctx[0], rotate_right(it.y, g), 0x08080808u);
+                        ctx[0] = mp::logic<kOrAnd>(ctx[0], rotate_right(it.z, g), 0x10101010u);
+                    },
+                    [&](int m, const uint32_t (&v)[4], const uint32_t (&ctx)[2]) {
+                        const uint32_t at = __byte_perm(ctx[0], 0u, 0x4440u + (uint32_t)m);
+                        return (uint32_t)(v[m] < *reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(thr) + at));
+                    });
+                if (lane < n) words[q] = self ^ (~need | lt);
+                __syncwarp();
             }
-            __syncwarp();
         }
     }
 
-    // lane r: the cube energy of read r (bonds inside the cube, each once)
-    long long e = 0;
-    for (int q = 0; q < V; ++q) {
-        int x, y, z;
-        site_of(q, &x, &y, &z);
-        const uint2 rec = recs[q];
-        const int dd[3] = {q % l, (q / l) % l, q / (l * l)};
-        const int sq = ((words[q] >> lane) & 1u) ? -1 : 1;
+    // lane b: the weight of the positive terms of read b, each bond of the cube once, through
+    // vertical counters over the lane's sites and a bit transpose a plane
+    constexpr int kPlanesE = UNITJ ? 6 : 7;  // at most 11 sites a lane of weight 3 (6)
+    uint32_t C[kPlanesE];
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const int step = d == 0 ? 1 : d == 1 ? l : l * l;
-            if (dd[d] + 1 < l) e += (long long)coupling(rec, 2 * d) * sq * (((words[q + step] >> lane) & 1u) ? -1 : 1);
+    for (int j = 0; j < kPlanesE; ++j) C[j] = 0;
+    for (int q = lane; q < V; q += 32) {
+        const uint32_t rec = recs[q], self = words[q];
+        const uint32_t nb[3] = {words[q + 1], words[q + l], words[q + ll]};
+        uint32_t one[3], two[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const uint32_t p = mp::logic<mp::kXor3>(self, nb[k], mp::plane_mask((int)rec, kRecPos + 2 * k));
+            one[k] = p & mp::plane_mask((int)rec, kRecOne + 2 * k);
+            two[k] = UNITJ ? 0u : p & mp::plane_mask((int)rec, kRecTwo + 2 * k);
         }
+        uint32_t w[4] = {mp::logic<mp::kXor3>(one[0], one[1], one[2]), mp::maj3(one[0], one[1], one[2]), 0u, 0u};
+        if constexpr (!UNITJ) {
+            const uint32_t t0 = mp::logic<mp::kXor3>(two[0], two[1], two[2]), t1 = mp::maj3(two[0], two[1], two[2]);
+            w[2] = t1 ^ (w[1] & t0);
+            w[1] ^= t0;
+        }
+        mp::vadd4(C, w);
     }
+    int weight = 0;
+#pragma unroll
+    for (int j = 0; j < kPlanesE; ++j) weight += __popc(mp::warp_transpose(C[j], lane)) << j;
     // the first read of lowest energy
-    long long be = e;
-    int br = lane;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const long long oe = __shfl_xor_sync(0xFFFFFFFFu, be, o);
-        const int orr = __shfl_xor_sync(0xFFFFFFFFu, br, o);
-        if (oe < be || (oe == be && orr < br)) {
-            be = oe;
-            br = orr;
-        }
-    }
-    if (lane == 0) sp[centre] = ((words[h + l * (h + l * h)] >> br) & 1u) ? (int8_t)-1 : (int8_t)1;
+    const unsigned rank = (unsigned)weight * 32u + (unsigned)(4 * (lane & 7) + (lane >> 3));
+    const unsigned least = __reduce_min_sync(kAll, rank);
+    if (rank == least) sp[centre] = ((words[h + l * (h + l * h)] >> lane) & 1u) ? (int8_t)-1 : (int8_t)1;
 }
 
 // Exact zero-temperature fragment marginals (l = 1 or 3): the centre spin of each fragment
@@ -334,7 +424,7 @@ int32_t check(const char* what)
 }  // namespace
 
 int32_t launch_fragment_waves(int8_t* spins, const uint2* const* j6_ptrs, const RunKeys* keys, const uint32_t* thr,
-                              int I, int L, int l, int S, cudaStream_t st)
+                              int I, int L, int l, int S, bool unit, cudaStream_t st)
 {
     FragArgs a{};
     a.spins = spins;
@@ -344,11 +434,13 @@ int32_t launch_fragment_waves(int8_t* spins, const uint2* const* j6_ptrs, const 
     a.L = L;
     a.l = l;
     a.S = S;
+    a.lmagic = l == 1 ? 0u : (uint32_t)((0x100000000ull + (uint64_t)l - 1) / (uint64_t)l);
     const int per = L / l;
     const int frags = per * per * per;
     const dim3 grid((frags + kWarps - 1) / kWarps, I);
     for (int w = 0; w < l * l * l; ++w) {
-        fragment_wave_kernel<<<grid, kWarps * 32, 0, st>>>(a, w);
+        if (unit) fragment_wave_kernel<true><<<grid, kWarps * 32, 0, st>>>(a, w);
+        else fragment_wave_kernel<false><<<grid, kWarps * 32, 0, st>>>(a, w);
         const int32_t rc = check("fragment_wave_kernel");
         if (rc != SG_OK) return rc;
     }

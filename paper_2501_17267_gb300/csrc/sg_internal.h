@@ -240,7 +240,7 @@ int32_t launch_sa_cluster_planes(const Plane* d_planes, const int* d_order, int 
 // fragment.cu: the fragment meta-heuristic's waves (one launch per wave) on [I][N] int8 spins
 // (0 = not fixed yet; all fixed on return), thr: [S][kThrRow] geometric schedule.
 int32_t launch_fragment_waves(int8_t* spins, const uint2* const* j6_ptrs, const RunKeys* keys, const uint32_t* thr,
-                              int I, int L, int l, int S, cudaStream_t st);
+                              int I, int L, int l, int S, bool unit, cudaStream_t st);
 // the same waves with exact zero-temperature fragment marginals (l <= 3)
 int32_t launch_fragment_tropical_waves(int8_t* spins, const uint2* const* j6_ptrs, int I, int L, int l,
                                        cudaStream_t st);

@@ -129,6 +129,22 @@ def test_fragment_run_general_couplings(sg):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("L,l,S,kind", [(6, 1, 2, "mixed"), (12, 3, 9, "mixed"), (10, 5, 4, "mixed"), (14, 7, 2, "mixed"),
+                                        (10, 5, 3, "double"), (20, 5, 0, "mixed")])
+def test_fragment_weights_and_parities(sg, L, l, S, kind):
+    """Bonds of weight 0, 1 and 2 (fields of both parities, up to 12) in cubes of every side;
+    cold schedules, whose larger fields have thresholds of zero."""
+    J3 = wl.random_couplings(43 + L, L, jmax=2, allow_zero=True)
+    if kind == "double":
+        J3 = np.where(J3 < 0, -2, 2).astype(np.int8)
+    inst = sg.Instance.from_couplings(L, J3, e_gs=-1)
+    for b0, b1 in [(0.2, 2.0), (2.0, 40.0)]:
+        res = sg.fragment_run(inst, l, S, b0, b1, seed=8, instance_id=4, spins="host")
+        ospins, oE = o.fragment_run(L, J3, l, S, b0, b1, 8, 4)
+        assert np.array_equal(res["spins"], ospins) and res["E"] == oE
+
+
+@pytest.mark.gpu
 def test_fragment_batch_equals_separate_runs(sg):
     insts = [sg.Instance.create(10, 3200 + k, (0, 0, 1), True) for k in range(3)]
     params = [dict(l=5, sweeps=4, beta0=0.5, beta1=6.0, seed=1, instance_id=k) for k in range(3)]
