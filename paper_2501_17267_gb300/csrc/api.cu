@@ -613,11 +613,11 @@ int32_t run_pt_group(const std::vector<int>& members, const sg_instance* const* 
     std::vector<int> cplan;
     if (unit_j && Wn == 1 && S > 0 && pt_coop_wanted(I, L, K)) cplan = pt_coop_plan(I, L, K, &coop_blocks, &coop_smem);
     double t_wave = 0, t_split = 0;
-    int Ccl = cplan.empty() && unit_j && Wn == 1 && S > 0 ? pt_cluster_blocks(I, L, K, &t_wave) : 0;
+    int Ccl = cplan.empty() && unit_j && S > 0 ? pt_cluster_blocks(I, L, K, &t_wave) : 0;
     int Mh = 0, side_sms = 0, Chy = 0;
     // (a split may beat one wave of smaller clusters: 16 instances at L = 48 take 8 blocks each
     // for 15 of them rather than 6 for all)
-    if (cplan.empty() && unit_j && Wn == 1 && S >= kGraphMinSweeps && (Ccl == 0 || t_wave > 0))
+    if (cplan.empty() && unit_j && S >= kGraphMinSweeps && (Ccl == 0 || t_wave > 0))
         Chy = pt_cluster_split(I, L, K, &Mh, &side_sms, &t_split);
     if (Ccl > 0 && Chy > 0) (t_split < t_wave ? Ccl : Chy) = 0;
     if (!cplan.empty()) {

@@ -46,12 +46,6 @@ struct ClusterArgs {
     uint32_t Hmagic;                // ceil(2^32 / (L / 2))
 };
 
-__device__ __forceinline__ uint32_t word_valid_bits(int R, int w)
-{
-    const int left = R - 32 * w;
-    return left >= 32 ? 0xFFFFFFFFu : left <= 0 ? 0u : (1u << left) - 1u;
-}
-
 // One word of one lattice, annealed by a cluster of C blocks (block r: z-slab r): the
 // plane's word of site s is g[s * stride]; the draws use word index w of the instance.
 struct PlaneRun {
@@ -120,7 +114,7 @@ __device__ __forceinline__ bool anneal_plane(const PlaneRun& p, const int C, uns
     s.draws.k0 = p.key.k0;
     s.draws.k1 = p.key.k1;
     s.word = (uint32_t)p.w;
-    s.valid = word_valid_bits(p.R, p.w);
+    s.valid = slab::word_valid_bits(p.R, p.w);
     const uint32_t up = (uint32_t)(r + 1 == C ? 0 : r + 1), dn = (uint32_t)(r == 0 ? C - 1 : r - 1);
     uint32_t up_w = 0, dn_w = 0, up_bar = 0, dn_bar = 0;
     if (C > 1) {
@@ -358,7 +352,8 @@ int resident_clusters(const void* fn, int C, size_t smem, int threads)
     return active;
 }
 
-// Lets `fn` use as much dynamic shared memory as a block can have beside its static one.  (The
+// Lets `fn` use clusters of up to 16 blocks, and as much dynamic shared memory as a block can
+// have beside its static one.  (The
 // limit is always the same one, so that launches from several threads do not lower it under one
 // another.)
 bool allow_shared(const void* fn)
@@ -367,6 +362,7 @@ bool allow_shared(const void* fn)
     cudaFuncAttributes at{};
     if (cudaGetDevice(&dev) != cudaSuccess || cudaFuncGetAttributes(&at, fn) != cudaSuccess ||
         cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)at.sharedSizeBytes) !=
             cudaSuccess) {
         cudaGetLastError();
@@ -402,7 +398,7 @@ double half_sweep_cycles(int L, int C, int threads, int per_sm)
 
 // Blocks per cluster (and the threads to plan a block with) for an SA run of I instances of
 // side L with Wn words, or 0 when the row kernel should run it.  Candidates are the
-// C <= 8 whose largest slab fits shared memory and is thinner than with fewer blocks; clusters
+// C <= 16 (8 in a loaded server) whose largest slab fits shared memory and is thinner than with fewer blocks; clusters
 // that are not resident at once (as the driver reports for the kernel) run in waves.  A half sweep's cycles, fitted to measurements
 // on a GB300 (us at 2.07 GHz), times the waves:
 //   resident blocks  750 + 400 per warp of pairs an SM partition holds (L = 4 on one block of
@@ -433,7 +429,7 @@ int sa_cluster_blocks(int I, int L, int Wn, bool force, int* threads, int busy)
     const double row_share = 490.0 * row_items / (4.0 * sms);
     double best = force || forced ? 1e300 : 0.95 * std::max(6500.0 + row_share, busy * row_share);
     int bestC = 0;
-    for (int C = 1; C <= 8; ++C) {
+    for (int C = 1; C <= (busy > 1 ? 8 : slab::kMaxC); ++C) {
         if (forced ? C != forced || C > L : !slab::worth(L, C)) continue;
         const int bt = sa_block_threads(L, C, t);
         const size_t bytes = slab::smem_bytes(L, C, bt);

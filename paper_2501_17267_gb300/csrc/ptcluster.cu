@@ -38,13 +38,13 @@ namespace {
 constexpr int kThreads = slab::kMaxThreads;
 
 struct PtcArgs {
-    uint32_t* spins;                // [I][N] words (slots 0..31 of a site), storage order
+    uint32_t* spins;                // [I][N][words] (32 slots of a site a word), storage order
     const uint8_t* const* j1_ptrs;  // per instance: [N] coupling sign bits (all |J| = 1)
     const RunKeys* keys;            // [I]
     const uint32_t* thr;            // [K][kThrRow] thresholds by rung
-    uint8_t* rung_of_slot;          // [I][32]
+    uint8_t* rung_of_slot;          // [I][32 words]
     uint8_t* slot_of_rung;          // [I][K]
-    int32_t* E;                     // [I][32] out: slot energies after the last sweep
+    int32_t* E;                     // [I][32 words] out: slot energies after the last sweep
     unsigned long long* accepts;    // [I][K-1]
     int32_t* minE;                  // [I]
     const uint32_t* xtab;           // exchange thresholds (exchange.cuh)
@@ -59,32 +59,35 @@ struct PtcArgs {
     int xwords;                     // words of xtab held in shared memory (0: read from global memory)
 };
 
-// Shared state of a block.
+// Shared state of a block, WN words an instance.
+template <int WN>
 struct PtShared {
     slab::Planes planes;
     slab::Geometry geo;
-    uint32_t rthr[32 * kThrRow];  // per rung: its threshold row
+    uint32_t rthr[32 * WN * kThrRow];  // per rung: its threshold row
     int E[32];                    // the block's energy sums of a colour-1 half sweep
     int Epart[2][slab::kMaxC][32];  // by sweep parity: every block's sums
-    uint8_t rung[32];             // slot -> rung
-    uint8_t inverse[kThreads / 32][32];  // a warp's scratch: slot -> rung
-    uint32_t xoff[32], xlen[32], xtail[32];
+    uint8_t rung[32];             // slot of the block's word -> rung
+    uint8_t inverse[kThreads / 32][32 * WN];  // a warp's scratch: slot -> rung
+    uint32_t xoff[32 * WN], xlen[32 * WN], xtail[32 * WN];
     uint64_t bar[2];              // by colour: the neighbours' face words have arrived
     uint64_t ebar[2];             // by sweep parity: every block's energy sums have arrived
     int fail[2];                  // by colour: a wait gave up (read one half sweep later)
 };
 
-// S: slab::Sweeper, or slab::Resident when a block has a thread for each of its x pairs.
-template <class S>
+// S: slab::Sweeper, or slab::Resident when a block has a thread for each of its x pairs.  WN: words
+// an instance (K <= 32 WN); a cluster has C blocks for each, which share nothing but the energies.
+template <class S, int WN>
 __global__ void __launch_bounds__(kThreads, 1) pt_cluster_kernel(const PtcArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ PtShared sh;
+    __shared__ PtShared<WN> sh;
 
     cg::cluster_group cluster = cg::this_cluster();
-    const int C = a.C;
-    const int r = C > 1 ? (int)cluster.block_rank() : 0;
-    const int inst = blockIdx.x / C;
+    const int C = a.C, blocks = WN * C;  // of a word, of the cluster
+    const int rank = blocks > 1 ? (int)cluster.block_rank() : 0;
+    const int word = WN == 1 ? 0 : rank / C, r = rank - word * C;
+    const int inst = blockIdx.x / blocks;
     const int K = a.K;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, threads = blockDim.x, warps = threads >> 5;
     const RunKeys key = a.keys[inst];
@@ -93,24 +96,26 @@ __global__ void __launch_bounds__(kThreads, 1) pt_cluster_kernel(const PtcArgs a
     __syncthreads();
     uint32_t* w = reinterpret_cast<uint32_t*>(smem) + geo.LL;
     uint8_t* sgn = smem + slab::Geometry::words(a.L, C) * 4;
-    uint32_t* g = a.spins + (size_t)inst * geo.LL * a.L;
-    slab::load_slab(geo, g, 1, a.j1_ptrs[inst], w, sgn);
+    uint32_t* g = a.spins + (size_t)inst * geo.LL * a.L * WN + word;
+    slab::load_slab(geo, g, WN, a.j1_ptrs[inst], w, sgn);
     uint32_t* xtab_s = reinterpret_cast<uint32_t*>(smem + slab::smem_bytes(a.L, C, threads));
     for (int q = tid; q < a.xwords; q += threads) xtab_s[q] = a.xtab[q];
     const uint32_t* xtab = a.xwords ? xtab_s : a.xtab;
 
-    // slot maps and thresholds; a lane is a slot or a rung.  slot: this rung's slot, in every
-    // warp's own registers.
-    int slot = lane < K ? a.slot_of_rung[(size_t)inst * K + lane] : lane;
-    int rung = a.rung_of_slot[(size_t)inst * 32 + lane];
+    // slot maps and thresholds; a lane is slots or rungs 32 i + lane.  slot[i]: the rung's slot, in
+    // every warp's own registers; rung: of slot `lane` of the block's word.
+    int slot[WN];
+#pragma unroll
+    for (int i = 0; i < WN; ++i) slot[i] = 32 * i + lane < K ? a.slot_of_rung[(size_t)inst * K + 32 * i + lane] : 32 * i + lane;
+    int rung = a.rung_of_slot[((size_t)inst * WN + word) * 32 + lane];
     for (int q = tid; q < K * kThrRow; q += threads) sh.rthr[q] = a.thr[q];
     if (tid < 32) {
         sh.rung[tid] = (uint8_t)rung;
         sh.E[tid] = 0;
-        if (tid + 1 < K) {
-            sh.xoff[tid] = a.xoff[tid];
-            sh.xlen[tid] = a.xlen[tid];
-            sh.xtail[tid] = a.xtail[tid];
+        for (int k = tid; k + 1 < K; k += 32) {
+            sh.xoff[k] = a.xoff[k];
+            sh.xlen[k] = a.xlen[k];
+            sh.xtail[k] = a.xtail[k];
         }
     }
     if (tid == 0) {
@@ -122,7 +127,7 @@ __global__ void __launch_bounds__(kThreads, 1) pt_cluster_kernel(const PtcArgs a
         sh.fail[0] = sh.fail[1] = 0;
     }
     int minE = a.minE[inst];
-    uint32_t accepted = 0;  // first warp, by the pair's lower rung
+    uint32_t accepted[WN] = {};  // first warp, by the pair's lower rung
     __syncthreads();
     // this warp's share of the threshold planes: planes of the slots' leading bytes, then lz
     auto build_planes = [&]() {
@@ -145,20 +150,20 @@ __global__ void __launch_bounds__(kThreads, 1) pt_cluster_kernel(const PtcArgs a
     s.E = sh.E;
     s.draws.k0 = key.k0;
     s.draws.k1 = key.k1;
-    s.word = 0u;
-    s.valid = K >= 32 ? 0xFFFFFFFFu : (1u << K) - 1u;
-    const uint32_t up = (uint32_t)(r + 1 == C ? 0 : r + 1), dn = (uint32_t)(r == 0 ? C - 1 : r - 1);
+    s.word = (uint32_t)word;
+    s.valid = slab::word_valid_bits(K, word);
+    const uint32_t first = (uint32_t)(word * C);
+    const uint32_t up = first + (uint32_t)(r + 1 == C ? 0 : r + 1), dn = first + (uint32_t)(r == 0 ? C - 1 : r - 1);
     uint32_t up_w = 0, dn_w = 0, up_bar = 0, dn_bar = 0;
     if (C > 1) {
         up_w = slab::cluster_addr(s.w0, up) - s.w0;
         dn_w = slab::cluster_addr(s.w0, dn) - s.w0;
         up_bar = slab::cluster_addr(slab::smem_addr(&sh.bar[0]), up);
         dn_bar = slab::cluster_addr(slab::smem_addr(&sh.bar[0]), dn);
-        // every block has loaded its halos and set up its barriers before a neighbour pushes
-        cluster.sync();
-    } else {
-        __syncthreads();
     }
+    // every block has loaded its halos and set up its barriers before another pushes
+    if (blocks > 1) cluster.sync();
+    else __syncthreads();
 
     // a sweep base in device memory lets a captured graph replay the launch for later sweeps
     const uint32_t sb = a.sweep_base ? *a.sweep_base : 0u;
@@ -167,7 +172,7 @@ __global__ void __launch_bounds__(kThreads, 1) pt_cluster_kernel(const PtcArgs a
     uint32_t phase = 0;  // of bar[0], bar[1]; of ebar: bits 2, 3
     bool ok = true;
     uint32_t A[S::kItems][8];
-    s.draws.set_sweep(sweep, 0u);
+    s.draws.set_sweep(sweep, s.word);
     s.first_draws(A);
     for (; sweep < s_end; ++sweep) {
         s.sweep = sweep;
@@ -181,19 +186,21 @@ __global__ void __launch_bounds__(kThreads, 1) pt_cluster_kernel(const PtcArgs a
             s.push_faces(0, C == 1, up_w, dn_w, up_bar, dn_bar);
         }
         __syncthreads();
-        if (C > 1) {
+        if (blocks > 1) {
             if (sh.fail[1]) {  // set before this barrier, the same for every thread
                 ok = false;
                 break;
             }
-            if (!slab::mbar_wait(&sh.bar[0], phase & 1u)) sh.fail[0] = 1;
-            phase ^= 1u;
+            if (C > 1) {
+                if (!slab::mbar_wait(&sh.bar[0], phase & 1u)) sh.fail[0] = 1;
+                phase ^= 1u;
+            }
         }
         // colour 1, with the energies
         const uint32_t par = sweep & 1u;
-        if (C > 1 && tid == 0) {
-            slab::mbar_expect(&sh.bar[1], (uint32_t)geo.LL * 4u);
-            slab::mbar_expect(&sh.ebar[par], (uint32_t)C * 128u);
+        if (blocks > 1 && tid == 0) {
+            if (C > 1) slab::mbar_expect(&sh.bar[1], (uint32_t)geo.LL * 4u);
+            slab::mbar_expect(&sh.ebar[par], (uint32_t)blocks * 128u);
         }
         if constexpr (S::kResident) {
             s.template half<1, slab::kCompare, true, true>(A, true);
@@ -204,51 +211,84 @@ __global__ void __launch_bounds__(kThreads, 1) pt_cluster_kernel(const PtcArgs a
         }
         s.energy_to_block();
         __syncthreads();
-        if (C > 1) {
+        if (blocks > 1) {
             if (sh.fail[0]) {
                 ok = false;
                 break;
             }
             // the block's sums to every block, a warp a block
-            for (int q = warp; q < C; q += warps) {
-                const uint32_t base = slab::cluster_addr(slab::smem_addr(&sh.Epart[par][r][lane]), (uint32_t)q);
+            for (int q = warp; q < blocks; q += warps) {
+                const uint32_t base = slab::cluster_addr(slab::smem_addr(&sh.Epart[par][rank][lane]), (uint32_t)q);
                 slab::push_word(base, (uint32_t)sh.E[lane], slab::cluster_addr(slab::smem_addr(&sh.ebar[par]), (uint32_t)q));
             }
         }
         // the exchange (App. D.2): pairs (k, k + 1) with k = sweep mod 2, accepted when
-        // d = E_a - E_b <= 0 or the draw u < T_k(d); a lane is a rung of a pair
-        const int k = ((lane - (int)par) & ~1) + (int)par;
-        const bool pair = k >= 0 && k + 1 < K;
-        const int other = (lane == k ? lane + 1 : lane - 1) & 31;
-        const uint32_t u = philox4x32_10((uint32_t)k, sweep, 0u, kDomainExchange, key.k0, key.k1).v[0];
-        int Eq;  // this slot's energy
-        if (C > 1) {
+        // d = E_a - E_b <= 0 or the draw u < T_k(d); a lane is a rung of a pair (WN of them)
+        int k[WN];
+        uint32_t u[WN];
+#pragma unroll
+        for (int i = 0; i < WN; ++i) {
+            k[i] = ((32 * i + lane - (int)par) & ~1) + (int)par;
+            u[i] = philox4x32_10((uint32_t)k[i], sweep, 0u, kDomainExchange, key.k0, key.k1).v[0];
+        }
+        int Eq[WN];  // of slots 32 i + lane
+        if (blocks > 1) {
             if (!slab::mbar_wait(&sh.ebar[par], (phase >> (2 + par)) & 1u)) sh.fail[1] = 1;
             phase ^= 4u << par;
-            Eq = 0;
-            for (int q = 0; q < C; ++q) Eq += sh.Epart[par][q][lane];
+#pragma unroll
+            for (int i = 0; i < WN; ++i) {
+                Eq[i] = 0;
+                for (int q = 0; q < C; ++q) Eq[i] += sh.Epart[par][i * C + q][lane];
+            }
         } else {
-            Eq = sh.E[lane];
+            Eq[0] = sh.E[lane];
         }
-        const int E_rung = __shfl_sync(slab::kAll, Eq, slot);  // of the slot at this rung
-        const int E_other = __shfl_sync(slab::kAll, E_rung, other), slot_other = __shfl_sync(slab::kAll, slot, other);
-        const int d = lane == k ? E_rung - E_other : E_other - E_rung;
-        bool accept = pair && d <= 0;
-        if (pair && d > 0) {
-            const uint32_t T = (uint32_t)d <= sh.xlen[k] ? xtab[sh.xoff[k] + (uint32_t)(d - 1)] : sh.xtail[k];
-            accept = u < T;
+        // v[at], at = 32 i + lane of a lane's array
+        auto gather = [&](const int (&v)[WN], int at) {
+            int x = __shfl_sync(slab::kAll, v[0], at & 31);
+#pragma unroll
+            for (int i = 1; i < WN; ++i) {
+                const int y = __shfl_sync(slab::kAll, v[i], at & 31);
+                if (at >> 5 == i) x = y;
+            }
+            return x;
+        };
+        int E_rung[WN], slot_now[WN];  // of the slot at this rung
+        bool swapped[WN];
+#pragma unroll
+        for (int i = 0; i < WN; ++i) {
+            E_rung[i] = gather(Eq, slot[i]);
+            slot_now[i] = slot[i];
         }
-        if (accept) slot = slot_other;
-        if (lane < K) sh.inverse[warp][slot] = (uint8_t)lane;
+#pragma unroll
+        for (int i = 0; i < WN; ++i) {
+            const int at = 32 * i + lane, other = (at == k[i] ? at + 1 : at - 1) & (32 * WN - 1);
+            const bool pair = k[i] >= 0 && k[i] + 1 < K;
+            const int E_other = gather(E_rung, other), slot_other = gather(slot_now, other);
+            const int d = at == k[i] ? E_rung[i] - E_other : E_other - E_rung[i];
+            bool accept = pair && d <= 0;
+            if (pair && d > 0) {
+                const uint32_t T =
+                    (uint32_t)d <= sh.xlen[k[i]] ? xtab[sh.xoff[k[i]] + (uint32_t)(d - 1)] : sh.xtail[k[i]];
+                accept = u[i] < T;
+            }
+            if (accept) slot[i] = slot_other;
+            if (at < K) sh.inverse[warp][slot[i]] = (uint8_t)at;
+            swapped[i] = accept && at == k[i];
+        }
         __syncwarp();
-        rung = lane < K ? sh.inverse[warp][lane] : 0;
+        rung = 32 * word + lane < K ? sh.inverse[warp][32 * word + lane] : 0;
         build_planes();
         if (warp == 0) {
             sh.rung[lane] = (uint8_t)rung;
-            accepted += accept && lane == k;
-            const int m = __reduce_min_sync(slab::kAll, lane < K ? Eq : 0x7FFFFFFF);
-            minE = min(minE, m);
-            if (r == 0 && sweep + 1 == s_end) a.E[(size_t)inst * 32 + lane] = Eq;
+            int least = 0x7FFFFFFF;
+#pragma unroll
+            for (int i = 0; i < WN; ++i) {
+                accepted[i] += swapped[i];
+                if (32 * i + lane < K) least = min(least, Eq[i]);
+                if (rank == 0 && sweep + 1 == s_end) a.E[((size_t)inst * WN + i) * 32 + lane] = Eq[i];
+            }
+            minE = min(minE, __reduce_min_sync(slab::kAll, least));
         }
         __syncthreads();  // the next sweep's planes are complete, and E has been read
         if (warp == 0) sh.E[lane] = 0;
@@ -264,45 +304,47 @@ __global__ void __launch_bounds__(kThreads, 1) pt_cluster_kernel(const PtcArgs a
     // ---- write back ----
     if (ok) {
         const int n = geo.zc * geo.LL;
-        for (int q = tid; q < n; q += threads) g[(size_t)geo.z0 * geo.LL + q] = w[q];
-        if (r == 0 && warp == 0) {
-            a.rung_of_slot[(size_t)inst * 32 + lane] = (uint8_t)rung;
-            if (lane < K) a.slot_of_rung[(size_t)inst * K + lane] = (uint8_t)slot;
-            if (lane + 1 < K) a.accepts[(size_t)inst * (K - 1) + lane] += (unsigned long long)accepted;
+        for (int q = tid; q < n; q += threads) g[((size_t)geo.z0 * geo.LL + q) * WN] = w[q];
+        if (r == 0 && warp == 0) a.rung_of_slot[((size_t)inst * WN + word) * 32 + lane] = (uint8_t)rung;
+        if (rank == 0 && warp == 0) {
+#pragma unroll
+            for (int i = 0; i < WN; ++i) {
+                const int k = 32 * i + lane;
+                if (k < K) a.slot_of_rung[(size_t)inst * K + k] = (uint8_t)slot[i];
+                if (k + 1 < K) a.accepts[(size_t)inst * (K - 1) + k] += (unsigned long long)accepted[i];
+            }
             if (lane == 0) a.minE[inst] = minE;
         }
     }
     __syncthreads();
-    if (C > 1) cluster.sync();  // no block leaves while another may still push to it; the status is complete
-    if (a.report.out && r == 0 && tid == 0) a.report.write(minE, *static_cast<volatile int*>(a.status));
+    if (blocks > 1) cluster.sync();  // no block leaves while another may still push to it; the status is complete
+    if (a.report.out && rank == 0 && tid == 0) a.report.write(minE, *static_cast<volatile int*>(a.status));
 }
 
 int block_threads(int L, int C) { return slab::resident_threads(slab::pairs_of(L, C), kThreads); }
+template <int WN>
 const void* kernel_of(int L, int C)
 {
     switch (slab::resident_items(slab::pairs_of(L, C), kThreads)) {
-        case 1: return (const void*)pt_cluster_kernel<slab::Resident<1>>;
-        case 2: return (const void*)pt_cluster_kernel<slab::Resident<2>>;
-        default: return (const void*)pt_cluster_kernel<slab::Sweeper>;
+        case 1: return (const void*)pt_cluster_kernel<slab::Resident<1>, WN>;
+        case 2: return (const void*)pt_cluster_kernel<slab::Resident<2>, WN>;
+        default: return (const void*)pt_cluster_kernel<slab::Sweeper, WN>;
     }
 }
+constexpr int kMaxWords = 2;
+const void* kernel_of(int L, int C, int words) { return words == 1 ? kernel_of<1>(L, C) : kernel_of<2>(L, C); }
 size_t dyn_smem(int L, int C) { return slab::smem_bytes(L, C, block_threads(L, C)); }
-
-// (shared memory: without the exchange thresholds, which take what is left)
-cudaLaunchConfig_t cluster_config(int L, int C, int I, cudaLaunchAttribute* attr)
+// (with the static part, without the exchange thresholds, which take what is left)
+size_t all_smem(int L, int C, int words)
 {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(C * I, 1, 1);
-    cfg.blockDim = dim3(block_threads(L, C), 1, 1);
-    cfg.dynamicSmemBytes = dyn_smem(L, C);
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = C;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cfg;
+    return dyn_smem(L, C) + (words == 1 ? sizeof(PtShared<1>) : sizeof(PtShared<2>));
 }
+// Clusters of side L, C blocks for each of `words` words, that fit the device at once.
+int resident(int L, int C, int words)
+{
+    return resident_clusters(kernel_of(L, C, words), C * words, dyn_smem(L, C), block_threads(L, C));
+}
+bool runs(int L, int K) { return K >= 1 && K <= 32 * kMaxWords && L >= 2 && !(L & 1); }
 
 }  // namespace
 
@@ -333,36 +375,37 @@ double cluster_seconds(int L, int C, double hz) { return 3.7e-6 + 64.0 * slab::p
 double row_seconds(double work, int I, int sms, double hz) { return 10e-6 + I * work / (sms * 6.2 * hz); }
 }  // namespace
 
-// Blocks per cluster for a PT run of I instances of side L with K <= 32 temperatures and
-// unit couplings, or 0 when the row kernels should run it.  C is the largest up to 8 that
-// makes the slabs thinner, whose largest slab fits shared memory and for which all I clusters
-// are resident at once (one wave) -- but no larger than leaves a block 128 pairs of sites, a warp for each
-// partition of its SM (L = 8: 2.11 us a sweep on one or two blocks, 2.45 on eight).  The
-// cluster form is taken when its estimated time per sweep is below the row kernels'.  Knob
-// SG_PT_CLUSTER = 0 turns the form off, = 1 takes it whenever a slab fits.
+// Blocks per word for a PT run of I instances of side L with K <= 64 temperatures and
+// unit couplings, or 0 when the row kernels should run it.  C is the largest, up to 16 blocks a
+// cluster, that makes the slabs thinner, whose largest slab fits shared memory and for which
+// all I clusters are resident at once (one wave) -- but no larger than leaves a block 128 pairs
+// of sites, a warp for each partition of its SM (L = 8: 2.11 us a sweep on one or two blocks,
+// 2.45 on eight).  The cluster form is taken when its estimated time per sweep is below the row
+// kernels'.  Knob SG_PT_CLUSTER = 0 turns the form off, = 1 takes it whenever a slab fits.
 int pt_cluster_blocks(int I, int L, int K, double* seconds)
 {
     if (seconds) *seconds = 0;
     const char* e = getenv("SG_PT_CLUSTER");
     const int knob = e ? atoi(e) : -1;
-    if (knob == 0 || K > 32 || K < 1 || L < 2 || (L & 1) || I < 1) return 0;
+    if (knob == 0 || !runs(L, K) || I < 1) return 0;
     int dev = 0, smem = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const double hz = device_hz();
-    const char* fc = getenv("SG_PT_CLUSTER_C");  // tuning knob: force C (when it divides L and fits)
+    const int words = words_for(K);
+    const char* fc = getenv("SG_PT_CLUSTER_C");  // tuning knob: force C (when it fits)
     const int forced = fc ? atoi(fc) : 0;
-    for (int C = 8; C >= 1; --C) {
+    for (int C = slab::kMaxC / words; C >= 1; --C) {
         if (forced > 0 ? C != forced || C > L : !slab::worth(L, C)) continue;
-        const size_t bytes = dyn_smem(L, C);
-        if (bytes + sizeof(PtShared) > (size_t)smem) continue;
-        if (knob == 1 || forced > 0) return C;
-        if (resident_clusters(kernel_of(L, C), C, bytes, block_threads(L, C)) < I) continue;
+        if (all_smem(L, C, words) > (size_t)smem) continue;
+        const int fit = resident(L, C, words);
+        if ((knob == 1 || forced > 0) && fit > 0) return C;
+        if (fit < I) continue;
         bool smaller = false;  // a smaller cluster with blocks of at most 128 pairs
         for (int c = C - 1; c >= 1 && !smaller; --c) smaller = slab::pairs_of(L, c) <= 128;
         if (smaller) continue;
-        const double work = (double)L * L * L * 32.0;  // attempts per sweep of one instance (whole words)
+        const double work = (double)L * L * L * 32.0 * words;  // attempts per sweep of one instance (whole words)
         const double t = cluster_seconds(L, C, hz);
         if (seconds) *seconds = t;
         return t < 0.95 * row_seconds(work, I, sms, hz) ? C : 0;
@@ -379,7 +422,7 @@ int pt_cluster_blocks_shared(int L, int K, int busy)
 {
     const char* e = getenv("SG_PT_CLUSTER");
     if (e || busy <= 1) return pt_cluster_blocks(1, L, K);
-    if (K > 32 || K < 1 || L < 2 || (L & 1)) return 0;
+    if (!runs(L, K) || words_for(K) > 1) return 0;
     int dev = 0, smem = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -389,9 +432,9 @@ int pt_cluster_blocks_shared(int L, int K, int busy)
     double best = 0.95 * std::max(row_seconds(work, 1, sms, hz), busy * (row_seconds(work, 1, sms, hz) - 10e-6));
     int bestC = 0;
     for (int C = 8; C >= 1; --C) {
-        if (!slab::worth(L, C) || dyn_smem(L, C) + sizeof(PtShared) > (size_t)smem) continue;
+        if (!slab::worth(L, C) || all_smem(L, C, 1) > (size_t)smem) continue;
         const double t = cluster_seconds(L, C, hz), shared = std::max(t, busy * C * t / sms);
-        if (shared < best && resident_clusters(kernel_of(L, C), C, dyn_smem(L, C), block_threads(L, C)) > 0) {
+        if (shared < best && resident(L, C, 1) > 0) {
             best = shared;
             bestC = C;
         }
@@ -414,25 +457,24 @@ int pt_cluster_split(int I, int L, int K, int* M, int* side_sms, double* seconds
     const char* e = getenv("SG_PT_HYBRID");
     if (e && atoi(e) == 0) return 0;
     const char* c = getenv("SG_PT_CLUSTER");
-    if ((c && atoi(c) == 0) || K > 32 || K < 1 || L < 2 || (L & 1) || I < 2) return 0;
+    if ((c && atoi(c) == 0) || !runs(L, K) || I < 2) return 0;
     int dev = 0, smem = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const double hz = device_hz();
-    const double work = (double)L * L * L * 32.0;  // whole words
+    const int words = words_for(K);
+    const double work = (double)L * L * L * 32.0 * words;  // whole words
     double best = 0.95 * row_seconds(work, I, sms, hz);
     int bestC = 0;
-    for (int C = 8; C >= 1; --C) {
-        if (!slab::worth(L, C)) continue;
-        const size_t bytes = dyn_smem(L, C);
-        if (bytes + sizeof(PtShared) > (size_t)smem) continue;
-        const int active = resident_clusters(kernel_of(L, C), C, bytes, block_threads(L, C));
+    for (int C = slab::kMaxC / words; C >= 1; --C) {
+        if (!slab::worth(L, C) || all_smem(L, C, words) > (size_t)smem) continue;
+        const int active = resident(L, C, words);
         if (active >= I || active < 1) continue;  // one wave: pt_cluster_blocks decides
-        const int per_sm = std::max(1, (active * C + sms - 1) / sms);  // blocks an SM holds
+        const int per_sm = std::max(1, (active * C * words + sms - 1) / sms);  // blocks an SM holds
         const double t_cluster = cluster_seconds(L, C, hz);
         for (int m = active; m >= 1; --m) {
-            const int left = sms - (m * C + per_sm - 1) / per_sm;
+            const int left = sms - (m * C * words + per_sm - 1) / per_sm;
             if (left < 1) continue;
             const double t_side = row_seconds(work, I - m, left, hz);
             const double t = t_cluster > t_side ? t_cluster : t_side;
@@ -483,18 +525,28 @@ int32_t launch_pt_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const Ru
     cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     // the exchange thresholds in shared memory when they fit beside the slab
     const size_t xbytes = sizeof(uint32_t) * xt.words;
-    a.xwords = dyn_smem(L, C) + xbytes + sizeof(PtShared) <= (size_t)most ? (int)xt.words : 0;
+    const int words = words_for(K);
+    const void* const fn = kernel_of(L, C, words);
+    a.xwords = all_smem(L, C, words) + xbytes <= (size_t)most ? (int)xt.words : 0;
     const size_t smem = dyn_smem(L, C) + sizeof(uint32_t) * (size_t)a.xwords;
-    if (!allow_shared(kernel_of(L, C))) {
+    if (!allow_shared(fn)) {
         set_error("pt_cluster_kernel: cannot use %zu bytes of shared memory", smem);
         return SG_ECUDA;
     }
     cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = cluster_config(L, C, I, attr);
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C * words;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(C * words * I, 1, 1);
+    cfg.blockDim = dim3(block_threads(L, C), 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
     void* args[] = {&a};
-    const cudaError_t e = cudaLaunchKernelExC(&cfg, kernel_of(L, C), args);
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
     if (e != cudaSuccess) {
         cudaGetLastError();
         set_error("pt_cluster_kernel launch failed: %s", cudaGetErrorString(e));

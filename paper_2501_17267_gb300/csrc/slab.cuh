@@ -42,7 +42,7 @@ namespace sg {
 namespace slab {
 
 constexpr int kMaxThreads = 512;
-constexpr int kMaxC = 8;        // blocks a cluster
+constexpr int kMaxC = 16;       // blocks a cluster (more than 8: the kernels ask for it, allow_shared)
 constexpr int kTieCap = 64;     // queue entries a warp: decided from 32, an item adds at most 32
 constexpr unsigned kAll = 0xFFFFFFFFu;
 constexpr long long kWaitCycles = 1ll << 33;  // a bounded wait gives up after about 4 s
@@ -312,6 +312,12 @@ __device__ __forceinline__ void load_slab(const Geometry& g, const uint32_t* __r
         w[q - g.LL] = src[(size_t)(below + q) * stride];
         w[slab + q] = src[(size_t)(above + q) * stride];
     }
+}
+
+__device__ __forceinline__ uint32_t word_valid_bits(int R, int w)
+{
+    const int left = R - 32 * w;
+    return left >= 32 ? 0xFFFFFFFFu : left <= 0 ? 0u : (1u << left) - 1u;
 }
 
 // ---------------------------------------------------------------- updates

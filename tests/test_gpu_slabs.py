@@ -65,6 +65,32 @@ def test_slabs_of_unequal_height(sg, monkeypatch, L, C):
     test_tempering_on_clusters_equals_row_kernels(sg, monkeypatch, L, C)
 
 
+# more blocks than a portable cluster has
+@pytest.mark.parametrize("L,C", [(16, 16), (24, 12), (26, 13), (32, 11), (32, 16), (50, 10)])
+def test_clusters_of_more_than_eight_blocks(sg, monkeypatch, L, C):
+    test_annealing_on_clusters_equals_row_kernel(sg, monkeypatch, L, C)
+    test_tempering_on_clusters_equals_row_kernels(sg, monkeypatch, L, C)
+
+
+# two words of slots, each on C blocks of the cluster: word edges, every block form, C = 1
+@pytest.mark.parametrize("L,C,K", [(4, 1, 33), (8, 1, 64), (8, 4, 40), (10, 3, 63), (16, 4, 48), (16, 2, 33), (22, 7, 64),
+                                   (32, 8, 48), (40, 8, 50)])
+def test_tempering_with_two_words_of_slots(sg, monkeypatch, L, C, K):
+    S = 20 if L <= 26 else 7
+    insts = [sg.Instance.create(L, 500 + 10 * L + k) for k in range(2)]
+    ps = [dict(temps=K, sweeps=S, beta_min=0.2, beta_max=3.0, seed=5, instance_id=k) for k in range(2)]
+    monkeypatch.setenv("SG_PT_CLUSTER", "1")
+    monkeypatch.setenv("SG_PT_CLUSTER_C", str(C))
+    a = sg.pt_run_batch(insts, ps, spins="host")
+    monkeypatch.delenv("SG_PT_CLUSTER_C")
+    monkeypatch.setenv("SG_PT_CLUSTER", "0")
+    b = sg.pt_run_batch(insts, ps, spins="host")
+    for x, y in zip(a, b):
+        for key in ("spins", "E", "perm", "accepts"):
+            assert np.array_equal(x[key], y[key]), key
+        assert x["minE"] == y["minE"]
+
+
 def test_batch_whose_sides_share_no_divisor(sg, monkeypatch, tmp_path):
     sides = [22, 40, 44, 10, 26]
     insts = [sg.Instance.create(L, 700 + k) for k, L in enumerate(sides)]
