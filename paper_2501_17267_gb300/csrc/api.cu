@@ -433,16 +433,20 @@ int32_t run_sa_group(const std::vector<int>& members, const sg_instance* const* 
     // SA keeps no per-sweep energies: the energy of every replica is computed once,
     // from the final spins.
     SG_RET(log.run(SG_KERNEL_INIT, cells, st, [&] { return launch_init_spins(spins, kp, I, L, Wn, R, st); }));
-    // Unit couplings, where it is faster: every sweep in one launch, a word per thread-block
-    // cluster (cluster.cu).  Knob SG_SA_CLUSTER = 0 / 1 disables or forces it.
+    // Where it is faster: every sweep in one launch, a word per thread-block cluster (cluster.cu;
+    // cluster_general.cu).  Knob SG_SA_CLUSTER = 0 / 1 disables or forces it.
     const char* ck = getenv("SG_SA_CLUSTER");
+    const bool force = ck && atoi(ck) == 1;
     int threads = 0;
-    const int C = unit_j && S > 0 && !(ck && atoi(ck) == 0) ? sa_cluster_blocks(I, L, Wn, ck && atoi(ck) == 1, &threads)
-                                                            : 0;
+    const int C = S < 1 || (ck && atoi(ck) == 0) ? 0
+                  : unit_j                       ? sa_cluster_blocks(I, L, Wn, force, &threads)
+                                                 : sa_general_cluster_blocks(I, L, Wn, force);
     if (C > 0) {
         SG_RET(log.run(SG_KERNEL_SWEEP_CHUNK, (int64_t)I * N * R * S, st, [&] {
-            return launch_sa_cluster(spins, j1p, kp, d_thr.as<uint32_t>(), d_flag.as<int>() + 1, I, L, Wn, R, 0, S, C,
-                                     threads, st);
+            int* const status = d_flag.as<int>() + 1;
+            if (!unit_j)
+                return launch_sa_general_cluster(spins, j6p, kp, d_thr.as<uint32_t>(), status, I, L, Wn, R, S, C, st);
+            return launch_sa_cluster(spins, j1p, kp, d_thr.as<uint32_t>(), status, I, L, Wn, R, 0, S, C, threads, st);
         }));
     } else if (S >= kGraphMinSweeps) {
         // the kernel reads row *base + c of the whole [S][kThrRow] table

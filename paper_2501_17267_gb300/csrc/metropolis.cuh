@@ -242,7 +242,7 @@ static __device__ __noinline__ uint32_t resolve_tie_bits(uint32_t tie, uint32_t 
 // where k > 0, and then k = 2u, or 2u - 1 when M is odd: six thresholds a parity, picked by the
 // three planes of u.  Replica by replica, as it was, a warp followed its slowest replica through
 // 32 branches (19 lanes of 32 active, 30 % of the issue slots): a half sweep of 100 replicas of
-// an L = 24 lattice took 8.4 us, and takes 3.6 in planes, about what its launch takes; tempering
+// an L = 24 lattice took 8.4 us a launch, and takes 3.6 in planes (2.5 on clusters, which need none); tempering
 // 48 slots sums its energies in the same counters as unit couplings.
 //
 // Threshold planes of a word: gp[general_plane(odd, j, u)] has bit b equal to bit 24 + j of
@@ -305,26 +305,9 @@ __device__ __forceinline__ void count_six(const uint32_t (&a)[6], uint32_t& c0, 
 
 __device__ __forceinline__ uint32_t plane_mask(int v, int bit) { return 0u - ((uint32_t)(v >> bit) & 1u); }
 
-// One word.  J[q] are the six couplings, gp its threshold planes, row[b * stride + k] the
-// threshold of replica b (read for ties alone).  Returns the flips; c: the planes of the
-// satisfied weight before them, *M the weight of all bonds.
-__device__ __forceinline__ uint32_t update_word_general(uint32_t self, const uint32_t (&n)[6], const int (&J)[6],
-                                                        uint32_t valid, const uint32_t* __restrict__ gp,
-                                                        const uint32_t* __restrict__ row, int stride,
-                                                        const uint32_t (&A)[8], uint32_t site, uint32_t sweep,
-                                                        uint32_t w, const RunKeys& key, uint32_t (&c)[4], int* M)
+// The satisfied weight from the satisfied bonds of weight 1 and of weight 2.
+__device__ __forceinline__ void satisfied_weight(const uint32_t (&one)[6], const uint32_t (&two)[6], uint32_t (&c)[4])
 {
-    uint32_t one[6], two[6];
-    int m = 0;
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-        const uint32_t satisfied = logic<kXor3>(self, n[q], J[q] < 0 ? ~0u : 0u);
-        const int weight = J[q] < 0 ? -J[q] : J[q];
-        one[q] = weight == 1 ? satisfied : 0u;
-        two[q] = weight == 2 ? satisfied : 0u;
-        m += weight;
-    }
-    *M = m;
     uint32_t o0, o1, o2, t0, t1, t2;
     count_six(one, o0, o1, o2);
     count_six(two, t0, t1, t2);
@@ -333,14 +316,26 @@ __device__ __forceinline__ uint32_t update_word_general(uint32_t self, const uin
     const uint32_t k1 = o1 & t0;
     c[2] = logic<kXor3>(o2, t1, k1);
     c[3] = t2 ^ maj3(o2, t1, k1);
+}
+
+// The replicas of a word that flip.  c: planes of the satisfied weight, M the weight of all
+// bonds, gp the word's threshold planes, row[b * stride + k] the threshold of replica b (read
+// for ties alone).  Without DRAWS all thresholds are zero.
+template <bool DRAWS>
+__device__ __forceinline__ uint32_t flips_general(const uint32_t (&c)[4], int M, uint32_t valid,
+                                                  const uint32_t* __restrict__ gp, const uint32_t* __restrict__ row,
+                                                  int stride, const uint32_t (&A)[8], uint32_t site, uint32_t sweep,
+                                                  uint32_t w, const RunKeys& key)
+{
     // u = c - h, four planes; its borrow marks c < h
-    const int h = m >> 1, odd = m & 1;
+    const int h = M >> 1, odd = M & 1;
     const uint32_t h0 = plane_mask(h, 0), h1 = plane_mask(h, 1), h2 = plane_mask(h, 2);
     const uint32_t u0 = c[0] ^ h0, b0 = ~c[0] & h0;
     const uint32_t u1 = logic<kXor3>(c[1], h1, b0), b1 = logic<kBorrow>(c[1], h1, b0);
     const uint32_t u2 = logic<kXor3>(c[2], h2, b1), b2 = logic<kBorrow>(c[2], h2, b1);
     const uint32_t u3 = c[3] ^ b2, b3 = ~c[3] & b2;
     const uint32_t need = ~b3 & (u0 | u1 | u2 | u3);
+    if (!DRAWS) return ~need & valid;
     auto pick = [&](int j) {  // each replica's plane j
         const uint4 x = *reinterpret_cast<const uint4*>(gp + general_plane(odd, j, 1));
         const uint2 y = *reinterpret_cast<const uint2*>(gp + general_plane(odd, j, 5));
@@ -369,6 +364,29 @@ __device__ __forceinline__ uint32_t update_word_general(uint32_t self, const uin
         if ((word >> 8) < low) flip |= 1u << b;
     }
     return flip;
+}
+
+// One word of a site with couplings J[q].  Returns the flips; c: the planes of the satisfied
+// weight before them, *M the weight of all bonds.
+__device__ __forceinline__ uint32_t update_word_general(uint32_t self, const uint32_t (&n)[6], const int (&J)[6],
+                                                        uint32_t valid, const uint32_t* __restrict__ gp,
+                                                        const uint32_t* __restrict__ row, int stride,
+                                                        const uint32_t (&A)[8], uint32_t site, uint32_t sweep,
+                                                        uint32_t w, const RunKeys& key, uint32_t (&c)[4], int* M)
+{
+    uint32_t one[6], two[6];
+    int m = 0;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+        const uint32_t satisfied = logic<kXor3>(self, n[q], J[q] < 0 ? ~0u : 0u);
+        const int weight = J[q] < 0 ? -J[q] : J[q];
+        one[q] = weight == 1 ? satisfied : 0u;
+        two[q] = weight == 2 ? satisfied : 0u;
+        m += weight;
+    }
+    *M = m;
+    satisfied_weight(one, two, c);
+    return flips_general<true>(c, m, valid, gp, row, stride, A, site, sweep, w, key);
 }
 
 // Planes of the satisfied weight after the flips (a flip turns c into M - c).

@@ -229,6 +229,10 @@ int32_t launch_sa_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const Ru
                           const uint32_t* thr /* [S][kThrRow] */, int* status, int I, int L, int Wn, int R, int s_begin,
                           int s_end, int C, int threads, cudaStream_t st, const uint32_t* sweep_base = nullptr,
                           const ChunkReport& report = ChunkReport{});
+// cluster_general.cu: the same for couplings that are not all +-1
+int sa_general_cluster_blocks(int I, int L, int Wn, bool force);
+int32_t launch_sa_general_cluster(int8_t* spins, const uint2* const* j6_ptrs, const RunKeys* keys, const uint32_t* thr,
+                                  int* status, int I, int L, int Wn, int R, int S, int C, cudaStream_t st);
 // The persistent cluster form for batches of one-word planes (batch.cu): C for planes of
 // sides Ls, each of words[k] planes and sweeps[k] sweeps, or 0 when the largest does not fit.
 int sa_cluster_list_blocks(const int* Ls, const int* sweeps, const int* words, int n);

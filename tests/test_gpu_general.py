@@ -49,3 +49,20 @@ def test_general_couplings_match_oracle(sg, L, n, kind):
     for k in ("spins", "E", "perm", "accepts"):
         assert np.array_equal(res[k], ref[k]), k
     assert res["minE"] == ref["minE"]
+
+
+# (L, C): one pair a thread and several, slabs of one plane, of unequal height, a block alone
+@pytest.mark.parametrize("L,C", [(2, 1), (2, 2), (4, 3), (6, 1), (10, 5), (12, 12), (16, 2), (16, 16), (22, 4), (24, 7),
+                                 (32, 2)])
+def test_general_couplings_on_clusters_equal_row_kernel(sg, monkeypatch, L, C):
+    for kind, n, (b0, b1, schedule) in [("mixed", 40, (0.1, 3.0, "linear")), ("double", 3, (0.5, 30.0, "geometric")),
+                                        ("sparse", 65, (20.0, 0.1, "linear"))]:
+        inst = sg.Instance.from_couplings(L, _couplings(L, kind), e_gs=-1)
+        args = dict(replicas=n, sweeps=9, beta0=b0, beta1=b1, schedule=schedule, seed=5, instance_id=2, spins="host")
+        monkeypatch.setenv("SG_SA_CLUSTER", "1")
+        monkeypatch.setenv("SG_SA_CLUSTER_C", str(C))
+        a = sg.sa_run(inst, **args)
+        monkeypatch.delenv("SG_SA_CLUSTER_C")
+        monkeypatch.setenv("SG_SA_CLUSTER", "0")
+        b = sg.sa_run(inst, **args)
+        assert np.array_equal(a["spins"], b["spins"]) and np.array_equal(a["E"], b["E"])
