@@ -123,6 +123,7 @@ __global__ void __launch_bounds__(kWarps * 32, 8) fragment_wave_kernel(const Fra
     // cube sites: records, the words of fixed sites, and the lists of the free sites of each
     // colour (compacted by ballot, warp-uniform counts)
     int nfree[2] = {0, 0};
+    uint32_t fixed = 0;  // of the lane's sites lane, 32 + lane, ...
     for (int base = 0; base < V; base += 32) {
         const int q = base + lane;
         bool free_site = false;
@@ -146,9 +147,10 @@ __global__ void __launch_bounds__(kWarps * 32, 8) fragment_wave_kernel(const Fra
                 M += (uint32_t)weight;
             }
             recs[q] = (uint32_t)q | M << kRecM | pos << kRecPos | one << kRecOne | two << kRecTwo;
-            // fixed by an earlier wave: its residue class precedes this wave's
+            // fixed by an earlier wave: its residue class precedes this wave's (its spin is read below)
             if (wrap(ca + dx - h, l) + l * (wrap(cb + dy - h, l) + l * wrap(cc + dz - h, l)) < wave) {
-                words[q] = sp[i] < 0 ? kAll : 0u;
+                words[q] = (uint32_t)i;
+                fixed |= 1u << (base / 32);
             } else {
                 free_site = true;
                 colour = (x + y + z) & 1;
@@ -183,7 +185,7 @@ __global__ void __launch_bounds__(kWarps * 32, 8) fragment_wave_kernel(const Fra
         return word;
     };
 
-    // initial words
+    // initial words: of the free sites, and, once the wave before is done, of the fixed ones
     for (int c = 0; c < 2; ++c) {
         for (int base = 0; base < nfree[c]; base += 32) {
             const int n = min(32, nfree[c] - base);
@@ -197,6 +199,10 @@ __global__ void __launch_bounds__(kWarps * 32, 8) fragment_wave_kernel(const Fra
             if (lane < n) words[list[lane]] = word;
         }
     }
+    mp::wait_for_predecessor();
+    mp::allow_successor();
+    for (int q = lane; q < V; q += 32)
+        if ((fixed >> (q / 32)) & 1u) words[q] = sp[words[q]] < 0 ? kAll : 0u;
     __syncwarp();
 
     const int entry_k = 2 * (lane & 7) - ((lane >> 3) & 1);  // thr[lane], lane < 16
@@ -313,8 +319,8 @@ __global__ void __launch_bounds__(kWarps * 32, 8) fragment_wave_kernel(const Fra
 // a min-plus butterfly over bit q of the 512 states (s_q is plane 0's spin before the step
 // and plane 1's after it).  Plane 2 likewise from above, and the two tables plus plane 1's
 // own energy give the two minima.  A state that contradicts a fixed spin starts at kBarred.
-// About 28 K additions and minima a cube instead of 2^27 energies: 232.4 ms -> 0.23 ms for
-// four L = 12 lattices (27 launches of 4.7 us and the energies).
+// About 28 K additions and minima a cube instead of 2^27 energies: 232.4 ms -> 0.18 ms a
+// call for four L = 12 lattices (27 launches of 2.4 us, the rest the energies and the host).
 //
 // A warp owns a fragment: lane holds bits 4 .. 8 of a state (spin q of a plane is bit q,
 // q = dx + 3 dy, set meaning -1), its 16 registers bits 0 .. 3, so four butterflies stay in
@@ -339,18 +345,21 @@ __global__ void __launch_bounds__(kTropWarps * 32) fragment_tropical_kernel(int8
         return;
     }
     // lane q < 27: cube site q, its value (0 = free) and its three forward bonds
-    int value = 0, Jx = 0, Jy = 0, Jz = 0;
+    int value = 0, Jx = 0, Jy = 0, Jz = 0, at = 0;
     if (lane < 27) {
         const int dx = lane % 3, dy = (lane / 3) % 3, dz = lane / 9;
         const int x = cx + dx - 1, y = cy + dy - 1, z = cz + dz - 1;
         const int i = (x < 0 ? x + L : x >= L ? x - L : x) +
                       L * ((y < 0 ? y + L : y >= L ? y - L : y) + L * (z < 0 ? z + L : z >= L ? z - L : z));
-        value = sp[i];
+        at = i;
         const uint2 rec = j6_ptrs[inst][i];
         Jx = coupling(rec, 0);
         Jy = coupling(rec, 2);
         Jz = coupling(rec, 4);
     }
+    mp::wait_for_predecessor();  // the wave before: the only writer of spins
+    mp::allow_successor();
+    if (lane < 27) value = sp[at];
     const uint32_t fixed = __ballot_sync(kAll, value != 0), minus = __ballot_sync(kAll, value < 0);
     auto sign = [&](int bit) { return ((lane >> (bit - 4)) & 1) ? -1 : 1; };  // of a spin held by the lane
     // plane dz's own energy of the lane's 16 states (kBarred where a fixed spin disagrees)
@@ -411,12 +420,29 @@ __global__ void __launch_bounds__(kTropWarps * 32) fragment_tropical_kernel(int8
     if (lane == 0) sp[centre] = m <= mm ? (int8_t)1 : (int8_t)-1;
 }
 
-int32_t check(const char* what)
+// A launch a wave.  Every wave after the first may start while its predecessor still runs: it
+// reads couplings and keys, and draws its first words, before it waits for the predecessor's
+// spins (the first one starts when everything before it on the stream is done).  Four L = 12
+// lattices, exact: 0.23 -> 0.18 ms a call; one L = 10, annealed in cubes of 5: 6.2 -> 6.0.
+template <class F>
+int32_t launch_waves(int waves, dim3 grid, int threads, cudaStream_t st, const char* what, F&& launch)
 {
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) {
-        set_error("%s: %s", what, cudaGetErrorString(e));
-        return SG_ECUDA;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    for (int w = 0; w < waves; ++w) {
+        cfg.numAttrs = w > 0 ? 1 : 0;
+        const cudaError_t e = launch(&cfg, w);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            set_error("%s: %s", what, cudaGetErrorString(e));
+            return SG_ECUDA;
+        }
     }
     return SG_OK;
 }
@@ -438,13 +464,9 @@ int32_t launch_fragment_waves(int8_t* spins, const uint2* const* j6_ptrs, const 
     const int per = L / l;
     const int frags = per * per * per;
     const dim3 grid((frags + kWarps - 1) / kWarps, I);
-    for (int w = 0; w < l * l * l; ++w) {
-        if (unit) fragment_wave_kernel<true><<<grid, kWarps * 32, 0, st>>>(a, w);
-        else fragment_wave_kernel<false><<<grid, kWarps * 32, 0, st>>>(a, w);
-        const int32_t rc = check("fragment_wave_kernel");
-        if (rc != SG_OK) return rc;
-    }
-    return SG_OK;
+    return launch_waves(l * l * l, grid, kWarps * 32, st, "fragment_wave_kernel", [&](const cudaLaunchConfig_t* cfg, int w) {
+        return cudaLaunchKernelEx(cfg, unit ? fragment_wave_kernel<true> : fragment_wave_kernel<false>, a, w);
+    });
 }
 
 int32_t launch_fragment_tropical_waves(int8_t* spins, const uint2* const* j6_ptrs, int I, int L, int l,
@@ -452,12 +474,10 @@ int32_t launch_fragment_tropical_waves(int8_t* spins, const uint2* const* j6_ptr
 {
     const int per = L / l;
     const dim3 grid((per * per * per + kTropWarps - 1) / kTropWarps, I);
-    for (int w = 0; w < l * l * l; ++w) {
-        fragment_tropical_kernel<<<grid, kTropWarps * 32, 0, st>>>(spins, j6_ptrs, L, l, w);
-        const int32_t rc = check("fragment_tropical_kernel");
-        if (rc != SG_OK) return rc;
-    }
-    return SG_OK;
+    return launch_waves(l * l * l, grid, kTropWarps * 32, st, "fragment_tropical_kernel",
+                        [&](const cudaLaunchConfig_t* cfg, int w) {
+                            return cudaLaunchKernelEx(cfg, fragment_tropical_kernel, spins, j6_ptrs, L, l, w);
+                        });
 }
 
 }  // namespace sg

@@ -28,6 +28,11 @@ namespace mp {
 
 constexpr int kRep = 32;  // replicas per spin word
 
+// Programmatic dependent launch (PTX griddepcontrol, sm_90 and later).  Both are no-ops
+// in a launch made without the programmatic-serialization attribute.
+__device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void allow_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Three-input logic of the updates, spelled out: left to the compiler a word costs about
 // eight operations more.
 template <int TABLE>

@@ -79,10 +79,8 @@ struct SweepArgs {
     const uint32_t* sweep_base;   // if set, the sweep index is *sweep_base + sweep
 };
 
-// Programmatic dependent launch (PTX griddepcontrol, sm_90 and later).  Both are no-ops
-// in a launch made without the programmatic-serialization attribute.
-__device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void allow_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+using mp::allow_successor;
+using mp::wait_for_predecessor;
 
 __device__ __forceinline__ uint32_t valid_bits(int Rvalid, int w)
 {
