@@ -130,7 +130,12 @@ __device__ __forceinline__ bool anneal_plane(const PlaneRun& p, const int C, uns
     uint32_t A[S::kItems][8];
     bool ok = true;
     s.draws.set_sweep((uint32_t)p.s_begin, s.word);
-    s.first_draws(A);
+    if constexpr (S::kAssisted) {
+        if (s.drawer) s.template hand_over<0>();
+        __syncthreads();
+    } else {
+        s.first_draws(A);
+    }
     for (int sw = p.s_begin; sw < p.s_end && ok; ++sw) {
         const int b = sw & 1;
         const int mode = sh.mode[b];
@@ -154,6 +159,16 @@ __device__ __forceinline__ bool anneal_plane(const PlaneRun& p, const int C, uns
         auto expect = [&](int colour) {
             if (C > 1 && tid == 0) slab::mbar_expect(&sh.bar[colour], (uint32_t)geo.LL * 4u);
         };
+        if constexpr (S::kAssisted) {
+            if (s.drawer) {
+                if (mode != slab::kNoDraws) s.template hand_over<1>();
+                if (!(ok = finish(0))) break;
+                s.draws.set_sweep((uint32_t)sw + 1u, s.word);
+                if (sh.mode[b ^ 1] != slab::kNoDraws) s.template hand_over<0>();
+                ok = finish(1);
+                continue;
+            }
+        }
         if constexpr (S::kResident) {
             expect(0);
             if (mode == slab::kCompare) s.template half<0, slab::kCompare, false, false>(A, true);
@@ -219,7 +234,10 @@ __device__ __forceinline__ void init_shared(Shared& sh)
 // S: slab::Sweeper, or slab::Resident when a block has a thread for each of its x pairs and a
 // warp to spare for the tables.
 template <class S>
-__global__ void __launch_bounds__(S::kResident ? slab::kMaxThreads + 32 : slab::kMaxThreads, 1)
+__global__ void __launch_bounds__(S::kAssisted   ? 2 * slab::kAssistedPairs + 32
+                                  : S::kResident ? slab::kMaxThreads + 32
+                                                 : slab::kMaxThreads,
+                                  1)
 sa_cluster_kernel(const ClusterArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -373,10 +391,12 @@ bool allow_shared(const void* fn)
 
 namespace {
 // The kernel for a block of at most `threads` threads, and its threads: the resident forms get
-// a warp more, for the tables.
+// a warp more, for the tables, and the assisted form another set for the draws.
 const void* sa_cluster_fn(int L, int C, int threads)
 {
-    switch (slab::resident_items(slab::pairs_of(L, C), threads)) {
+    const int64_t pairs = slab::pairs_of(L, C);
+    if (slab::assisted(pairs, threads)) return (const void*)sa_cluster_kernel<slab::Resident<1, true>>;
+    switch (slab::resident_items(pairs, threads)) {
         case 1: return (const void*)sa_cluster_kernel<slab::Resident<1>>;
         case 2: return (const void*)sa_cluster_kernel<slab::Resident<2>>;
         default: return (const void*)sa_cluster_kernel<slab::Sweeper>;
@@ -385,14 +405,17 @@ const void* sa_cluster_fn(int L, int C, int threads)
 int sa_block_threads(int L, int C, int threads)
 {
     const int64_t pairs = slab::pairs_of(L, C);
-    return slab::resident_threads(pairs, threads) + (slab::resident_items(pairs, threads) ? 32 : 0);
+    return slab::resident_threads(pairs, threads) * (slab::assisted(pairs, threads) ? 2 : 1) +
+           (slab::resident_items(pairs, threads) ? 32 : 0);
 }
 // Cycles of a half sweep with `per_sm` blocks of at most `threads` threads on an SM (see below).
 double half_sweep_cycles(int L, int C, int threads, int per_sm)
 {
     const int64_t pairs = slab::pairs_of(L, C);
     const double warps = std::max(1.0, (double)per_sm * (double)((pairs + 31) / 32) / 4.0);
-    return slab::resident_items(pairs, threads) ? 750.0 + 400.0 * warps : 2000.0 + 300.0 * warps;
+    return slab::assisted(pairs, threads)         ? 500.0 + 400.0 * warps
+           : slab::resident_items(pairs, threads) ? 750.0 + 400.0 * warps
+                                                  : 2000.0 + 300.0 * warps;
 }
 }  // namespace
 
@@ -401,16 +424,17 @@ double half_sweep_cycles(int L, int C, int threads, int per_sm)
 // C <= 16 (8 in a loaded server) whose largest slab fits shared memory and is thinner than with fewer blocks; clusters
 // that are not resident at once (as the driver reports for the kernel) run in waves.  A half sweep's cycles, fitted to measurements
 // on a GB300 (us at 2.07 GHz), times the waves:
-//   resident blocks  750 + 400 per warp of pairs an SM partition holds (L = 4 on one block of
-//                    one warp 0.53, L = 16 with 1024 replicas on C = 4 blocks of 16 warps 1.2)
+//   resident blocks  750 + 400 per warp of pairs an SM partition holds (L = 16 with 1024
+//                    replicas on C = 4 blocks of 16 warps 1.2), 500 + 400 where a second set of
+//                    warps draws (L = 4 on one block of one warp 0.41)
 //   other blocks     2000 + 300 per warp of items (20 x L = 50 on C = 5 12.8, L = 64 on C = 8 20.6;
 //                    clusters of 7 or 8 blocks would take 20 x L = 50 in two waves, C = 6 in one)
 //   row kernels      6500 + 490 per warp of items over the whole GPU (18.2 and 5.2 for the same)
 // The fewest cycles win, fewer blocks among equals.  With `busy` runs of the kind sharing the
 // device (a loaded server) a form's time is its own or, if that is longer, busy times its share
 // of the device.  One run alone: L = 16 with 1024 replicas takes C = 4 (2.4
-// ms a run of 1000 sweeps against 5.1 at C = 2), L = 4 one block (1.05 ms against 1.20 at
-// C = 2 and 1.25 at C = 4).  force: a cluster form whatever the row kernel would take.
+// ms a run of 1000 sweeps against 5.1 at C = 2), L = 4 one block (0.82 ms;
+// in line 1.05, 1.20 at C = 2 and 1.25 at C = 4).  force: a cluster form whatever the row kernel would take.
 // Knobs: SG_SA_CLUSTER_C forces C, SG_SA_CLUSTER_THREADS the threads.
 int sa_cluster_blocks(int I, int L, int Wn, bool force, int* threads, int busy)
 {

@@ -78,7 +78,7 @@ struct PtShared {
 // S: slab::Sweeper, or slab::Resident when a block has a thread for each of its x pairs.  WN: words
 // an instance (K <= 32 WN); a cluster has C blocks for each, which share nothing but the energies.
 template <class S, int WN>
-__global__ void __launch_bounds__(kThreads, 1) pt_cluster_kernel(const PtcArgs a)
+__global__ void __launch_bounds__(S::kAssisted ? 2 * slab::kAssistedPairs : kThreads, 1) pt_cluster_kernel(const PtcArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ PtShared<WN> sh;
@@ -173,14 +173,23 @@ __global__ void __launch_bounds__(kThreads, 1) pt_cluster_kernel(const PtcArgs a
     bool ok = true;
     uint32_t A[S::kItems][8];
     s.draws.set_sweep(sweep, s.word);
-    s.first_draws(A);
+    if constexpr (S::kAssisted) {
+        if (s.drawer) s.template hand_over<0>();
+        __syncthreads();
+    } else {
+        s.first_draws(A);
+    }
     for (; sweep < s_end; ++sweep) {
         s.sweep = sweep;
         // colour 0
         if (C > 1 && tid == 0) slab::mbar_expect(&sh.bar[0], (uint32_t)geo.LL * 4u);
         if constexpr (S::kResident) {
-            s.template half<0, slab::kCompare, true, false>(A, true);
-            s.template push_faces<0>(C == 1, up_w, dn_w, up_bar, dn_bar);
+            if (S::kAssisted && s.drawer) {
+                s.template hand_over<1>();
+            } else {
+                s.template half<0, slab::kCompare, true, false>(A, true);
+                s.template push_faces<0>(C == 1, up_w, dn_w, up_bar, dn_bar);
+            }
         } else {
             s.template half<slab::kCompare, true, false>(0, A[0]);
             s.push_faces(0, C == 1, up_w, dn_w, up_bar, dn_bar);
@@ -203,13 +212,19 @@ __global__ void __launch_bounds__(kThreads, 1) pt_cluster_kernel(const PtcArgs a
             slab::mbar_expect(&sh.ebar[par], (uint32_t)blocks * 128u);
         }
         if constexpr (S::kResident) {
-            s.template half<1, slab::kCompare, true, true>(A, true);
-            s.template push_faces<1>(C == 1, up_w, dn_w, up_bar + 8u, dn_bar + 8u);
+            if (S::kAssisted && s.drawer) {
+                s.draws.set_sweep(sweep + 1u, s.word);
+                s.template hand_over<0>();
+            } else {
+                s.template half<1, slab::kCompare, true, true>(A, true);
+                s.template push_faces<1>(C == 1, up_w, dn_w, up_bar + 8u, dn_bar + 8u);
+                s.energy_to_block();
+            }
         } else {
             s.template half<slab::kCompare, true, true>(1, A[0]);
             s.push_faces(1, C == 1, up_w, dn_w, up_bar + 8u, dn_bar + 8u);
+            s.energy_to_block();
         }
-        s.energy_to_block();
         __syncthreads();
         if (blocks > 1) {
             if (sh.fail[0]) {
@@ -321,10 +336,15 @@ __global__ void __launch_bounds__(kThreads, 1) pt_cluster_kernel(const PtcArgs a
     if (a.report.out && rank == 0 && tid == 0) a.report.write(minE, *static_cast<volatile int*>(a.status));
 }
 
-int block_threads(int L, int C) { return slab::resident_threads(slab::pairs_of(L, C), kThreads); }
+int block_threads(int L, int C)
+{
+    const int64_t pairs = slab::pairs_of(L, C);
+    return slab::resident_threads(pairs, kThreads) * (slab::assisted(pairs, kThreads) ? 2 : 1);
+}
 template <int WN>
 const void* kernel_of(int L, int C)
 {
+    if (slab::assisted(slab::pairs_of(L, C), kThreads)) return (const void*)pt_cluster_kernel<slab::Resident<1, true>, WN>;
     switch (slab::resident_items(slab::pairs_of(L, C), kThreads)) {
         case 1: return (const void*)pt_cluster_kernel<slab::Resident<1>, WN>;
         case 2: return (const void*)pt_cluster_kernel<slab::Resident<2>, WN>;

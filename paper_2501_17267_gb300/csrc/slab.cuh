@@ -339,7 +339,7 @@ constexpr int kVBits = 9;
 
 // A warp's share of the half sweeps of a launch.
 struct Sweeper {
-    static constexpr bool kResident = false;
+    static constexpr bool kResident = false, kAssisted = false;
     static constexpr int kItems = 1;
     const Geometry& g;
     uint32_t w0, s0;          // addresses of the slab's first word and of its sign byte, less a quarter of w0
@@ -621,9 +621,17 @@ struct Sweeper {
 // words a site; its ties are decided on the spot -- the tail draw of every lane's first tie
 // runs beside the draws of the next half sweep -- and its face words go to the neighbours
 // straight from registers.
-template <int R>
+//
+// ASSISTED (R = 1): a second set of warps makes the draws, a half sweep ahead, and hands them over
+// through shared memory (where the queues would be), two buffers by colour; the block barrier
+// that ends a half sweep orders both sides.  For blocks of so few pairs that each partition of
+// the SM has one warp to run: L = 4 with 8 replicas takes 0.41 us a half sweep (0.53 with the
+// draws in line), tempering 20 lattices of L = 4 1.6 us a sweep (1.9), of L = 8 2.06 (2.15).
+// (Leaving out the tail draws where no lane has a tie: 0.38 with 8 replicas, but 0.55 instead of
+// 0.52 with 20 at L = 8; not kept.)
+template <int R, bool ASSISTED = false>
 struct Resident {
-    static constexpr bool kResident = true;
+    static constexpr bool kResident = true, kAssisted = ASSISTED;
     static constexpr int kItems = R;
     const Geometry& g;
     uint32_t w0;
@@ -637,6 +645,8 @@ struct Resident {
     int LL4;
     uint32_t slab, slab_dn;   // bytes of the slab, and of the one below
     bool idle;                // a warp beyond the pairs (uniform)
+    bool drawer;              // of the second set of warps (uniform)
+    uint32_t mail, mail_step; // the lane's draws: address of four planes of colour 0, bytes to the next four
     struct Pair {
         // of its site of colour 0 and of colour 1
         uint32_t at[2], value[2], mask[2][R == 1 ? 6 : 1];  // (R = 2: masks are spread from the sign bits)
@@ -646,25 +656,31 @@ struct Resident {
         uint32_t c0, c1, c2;  // counts after a colour-1 half sweep (energies)
     } pair[R];
 
-    __device__ __forceinline__ Resident(const Geometry& geo, const uint32_t* words, const uint8_t* signs, const uint4*)
+    __device__ __forceinline__ Resident(const Geometry& geo, const uint32_t* words, const uint8_t* signs,
+                                        const uint4* letters)
         : g(geo), w0(smem_addr(words)), rung(nullptr), E(nullptr), warp(threadIdx.x >> 5), lane(threadIdx.x & 31)
     {
         const int L = g.L, H = g.H, LL = g.LL;
         LL4 = 4 * LL;
         slab = (uint32_t)(g.zc * LL4);
         slab_dn = (uint32_t)(g.zdn * LL4);
-        idle = warp * 32 >= g.zc * g.cols;
+        const int set = ASSISTED ? (int)blockDim.x / 64 * 32 : (int)blockDim.x;  // threads with pairs
+        const bool second = ASSISTED && (int)threadIdx.x >= set;
+        drawer = second && (int)threadIdx.x < 2 * set;
+        idle = second || warp * 32 >= g.zc * g.cols;
+        mail_step = 16u * (uint32_t)set;
+        mail = smem_addr(letters) + 16u * (uint32_t)((int)threadIdx.x - (second ? set : 0));
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             Pair& q = pair[r];
-            const int n = (int)threadIdx.x + r * (int)blockDim.x;
+            const int n = (int)threadIdx.x + r * (int)blockDim.x - (second ? set : 0);
             const bool live = n < g.zc * g.cols;
             const int p = live ? n : 0;
             const int row = H == 1 ? p : (int)__umulhi((uint32_t)p, g.Hmagic), j = p - row * H;
             const int zl = (int)__umulhi((uint32_t)row, g.Lmagic), y = row - zl * L;
             q.yp = 4 * (y + 1 == L ? L - LL : L);
             q.ym = 4 * (y == 0 ? LL - L : -L);
-            q.flags = live ? kLive | (zl == 0 ? kBottom : 0u) | (zl + 1 == g.zc ? kTop : 0u) : 0u;
+            q.flags = live && !second ? kLive | (zl == 0 ? kBottom : 0u) | (zl + 1 == g.zc ? kTop : 0u) : 0u;
             q.c0 = q.c1 = q.c2 = 0u;
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
@@ -691,12 +707,29 @@ struct Resident {
         for (int r = 0; r < R; ++r) draws.planes((uint32_t)pair[r].site[0], A[r]);
     }
 
+    // (ASSISTED, second set) Hands over the draws of the lane's site of colour C.
+    template <int C>
+    __device__ __forceinline__ void hand_over() const
+    {
+        uint32_t A[8];
+        draws.planes((uint32_t)pair[0].site[C], A);
+        const uint32_t to = mail + (C ? 2u * mail_step : 0u);
+        st_quad_if(1u, to, A[0], A[1], A[2], A[3]);
+        st_quad_if(1u, to + mail_step, A[4], A[5], A[6], A[7]);
+    }
+
     // A: the draws of the lane's sites of colour C; on return, when `next`, those of its other
-    // sites in the half sweep that follows.
+    // sites in the half sweep that follows.  (ASSISTED: they come from the second set.)
     template <int C, int MODE, bool TEMPERING, bool ENERGY>
     __device__ __forceinline__ void half(uint32_t (&A)[R][8], bool next)
     {
         if (idle) return;
+        if constexpr (ASSISTED && (MODE == kCompare || MODE == kTailOnly)) {
+            const uint32_t from = mail + (C ? 2u * mail_step : 0u);
+            const uint4 lo = ld_quad(from), hi = ld_quad(from + mail_step);
+            A[0][0] = lo.x, A[0][1] = lo.y, A[0][2] = lo.z, A[0][3] = lo.w;
+            A[0][4] = hi.x, A[0][5] = hi.y, A[0][6] = hi.z, A[0][7] = hi.w;
+        }
         uint32_t flip[R], tie[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
@@ -740,7 +773,7 @@ struct Resident {
             }
             flip[r] = MODE == kCountOnly ? 0u : (~c2 | lt) & alive;
         }
-        if (C == 1) draws.set_sweep(sweep + 1u, word);
+        if (C == 1 && !ASSISTED) draws.set_sweep(sweep + 1u, word);
         if (MODE == kCompare || MODE == kTailOnly) {
             const uint4 lz = ld_quad(planes + 128u);
             uint32_t low[R], tail[R], bit[R], more = 0;
@@ -752,7 +785,7 @@ struct Resident {
                 bit[r] = 1u << b;
                 low[r] = low_of<TEMPERING>(q, b);
                 tail[r] = tail_of(q.site[C], b);
-                draws.planes((uint32_t)q.site[C ^ 1], A[r]);
+                if (!ASSISTED) draws.planes((uint32_t)q.site[C ^ 1], A[r]);
             }
 #pragma unroll
             for (int r = 0; r < R; ++r) {
@@ -770,7 +803,7 @@ struct Resident {
                     more |= tie[r];
                 }
             }
-        } else if (next) {
+        } else if (next && !ASSISTED) {
 #pragma unroll
             for (int r = 0; r < R; ++r) draws.planes((uint32_t)pair[r].site[C ^ 1], A[r]);
         }
@@ -834,6 +867,9 @@ __host__ __device__ inline int resident_items(int64_t pairs, int threads)
 {
     return pairs <= threads ? 1 : pairs <= 2 * threads ? 2 : 0;
 }
+// ASSISTED up to so many pairs a block.
+constexpr int kAssistedPairs = 128;
+inline bool assisted(int64_t pairs, int threads) { return pairs <= (threads < kAssistedPairs ? threads : kAssistedPairs); }
 inline int resident_threads(int64_t pairs, int threads)
 {
     const int r = resident_items(pairs, threads);
