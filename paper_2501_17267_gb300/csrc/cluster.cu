@@ -415,7 +415,7 @@ double half_sweep_cycles(int L, int C, int threads, int per_sm)
     const double warps = std::max(1.0, (double)per_sm * (double)((pairs + 31) / 32) / 4.0);
     return slab::assisted(pairs, threads)         ? 500.0 + 400.0 * warps
            : slab::resident_items(pairs, threads) ? 750.0 + 400.0 * warps
-                                                  : 2000.0 + 300.0 * warps;
+                                                  : 2000.0 + 350.0 * warps;
 }
 }  // namespace
 
@@ -427,9 +427,11 @@ double half_sweep_cycles(int L, int C, int threads, int per_sm)
 //   resident blocks  750 + 400 per warp of pairs an SM partition holds (L = 16 with 1024
 //                    replicas on C = 4 blocks of 16 warps 1.2), 500 + 400 where a second set of
 //                    warps draws (L = 4 on one block of one warp 0.41)
-//   other blocks     2000 + 300 per warp of items (20 x L = 50 on C = 5 12.8, L = 64 on C = 8 20.6;
-//                    clusters of 7 or 8 blocks would take 20 x L = 50 in two waves, C = 6 in one)
-//   row kernels      6500 + 490 per warp of items over the whole GPU (18.2 and 5.2 for the same)
+//   other blocks     2000 + 350 per warp of items (hot schedules: 20 x L = 50 on C = 6, one wave,
+//                    16.2, 4 x L = 64 on C = 16 11.9, 32 words of L = 64 on C = 8, three waves,
+//                    59.8; cold ones, which seldom compare, down to 300)
+//   row kernels      6500 + 520 per warp of items over the whole GPU (17.7, 10.0 and 54.5 for the
+//                    same)
 // The fewest cycles win, fewer blocks among equals.  With `busy` runs of the kind sharing the
 // device (a loaded server) a form's time is its own or, if that is longer, busy times its share
 // of the device.  One run alone: L = 16 with 1024 replicas takes C = 4 (2.4
@@ -450,7 +452,7 @@ int sa_cluster_blocks(int I, int L, int Wn, bool force, int* threads, int busy)
     const int t = et && atoi(et) >= 32 && atoi(et) <= slab::kMaxThreads ? atoi(et) / 32 * 32 : slab::kMaxThreads;
     *threads = t;
     const double row_items = (double)clusters * L * L * (L / 2) / 32.0;  // warps of items a half sweep
-    const double row_share = 490.0 * row_items / (4.0 * sms);
+    const double row_share = 520.0 * row_items / (4.0 * sms);
     double best = force || forced ? 1e300 : 0.95 * std::max(6500.0 + row_share, busy * row_share);
     int bestC = 0;
     for (int C = 1; C <= (busy > 1 ? 8 : slab::kMaxC); ++C) {
@@ -461,6 +463,7 @@ int sa_cluster_blocks(int I, int L, int Wn, bool force, int* threads, int busy)
         const int64_t active = resident_clusters(sa_cluster_fn(L, C, t), C, bytes, bt);
         if (active < 1) continue;
         const int64_t waves = (clusters + active - 1) / active;
+        if (C > 8 && waves > 1 && !forced) continue;  // (a wave of these follows another slowly)
         const int64_t per_sm = (std::min(clusters, active) * C + sms - 1) / sms;  // blocks on the busiest SM
         double cost = waves * half_sweep_cycles(L, C, t, (int)per_sm);
         cost = std::max(cost, cost * busy * (double)(std::min(clusters, active) * C) / sms);
