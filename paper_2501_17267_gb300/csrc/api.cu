@@ -609,9 +609,9 @@ int32_t run_pt_group(const std::vector<int>& members, const sg_instance* const* 
     xa.K = K;
     xa.sweep_base = nullptr;
     unsigned* done = d_done.as<unsigned>();
-    // K <= 32 with unit couplings: chunks of sweeps in one cooperative launch holding the
-    // batch in shared memory (ptcoop.cu), or on thread-block clusters, one per instance
-    // (ptcluster.cu)
+    // Unit couplings: chunks of sweeps in one cooperative launch holding the batch in shared
+    // memory (ptcoop.cu, K <= 32), or on thread-block clusters, one per instance (ptcluster.cu,
+    // K <= 64)
     int coop_blocks = 0;
     size_t coop_smem = 0;
     std::vector<int> cplan;
@@ -976,7 +976,7 @@ int32_t fragment_batch(const sg_instance* const* insts, const sg_fragment_params
     LaunchLog log;
     const int64_t V = (int64_t)l * l * l;
     // attempts: wave w anneals V - w free sites of each of N / V fragments, 32 reads, S sweeps;
-    // tropical: wave w enumerates 2^(V - w) states of each of N / V fragments
+    // tropical: wave w decides among 2^(V - w) states of each of N / V fragments
     int64_t units = (int64_t)I * N * 32 * S * (V + 1) / 2;
     if (tropical) {
         units = 0;

@@ -1,13 +1,12 @@
-// ptslab.cuh -- the per-block machinery of the parallel-tempering kernels that keep part
-// of a lattice in shared memory for many sweeps (App. D.2): ptcluster.cu (z-slabs of a
-// thread-block cluster) and ptcoop.cu (row blocks of a cooperative grid).  K <= 32: one
-// 32-bit word of 32 slots per site, all couplings +-1.
+// ptslab.cuh -- the per-block machinery of the cooperative parallel-tempering kernel
+// (ptcoop.cu), which keeps row blocks of a lattice in shared memory for many sweeps
+// (App. D.2).  K <= 32: one 32-bit word of 32 slots per site, all couplings +-1.
 //
 // A block holds its slots' thresholds (per slot rows for ties, and the bit planes of the
 // word the bit-sliced compare reads), updates words (metropolis.cuh) with a per-warp queue
 // of tied draws decided later, and, in a colour-1 half sweep, sums every slot's energy
 // (6 - 2c per site, c the satisfied count after the update) in bit-sliced counters.  The
-// kernels supply the geometry: which words a thread updates and where their neighbours lie.
+// kernel supplies the geometry: which words a thread updates and where their neighbours lie.
 #pragma once
 #include <stdint.h>
 

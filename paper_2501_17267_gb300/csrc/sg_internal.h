@@ -249,9 +249,9 @@ int32_t launch_fragment_waves(int8_t* spins, const uint2* const* j6_ptrs, const 
 int32_t launch_fragment_tropical_waves(int8_t* spins, const uint2* const* j6_ptrs, int I, int L, int l,
                                        cudaStream_t st);
 int32_t launch_pt_exchange(const ExchangeArgs& x, int I, uint32_t sweep, cudaStream_t st);
-// ptcluster.cu: PT with unit couplings and K <= 32, every sweep of [s_begin, s_end) in one
-// launch, one thread-block cluster of C blocks per instance (lattice in shared memory).
-// pt_cluster_blocks gives C, or 0 when the row kernels should run the batch.
+// ptcluster.cu: PT with unit couplings and K <= 64, every sweep of [s_begin, s_end) in one
+// launch, one thread-block cluster per instance (lattice in shared memory), of C blocks for
+// each word of slots.  pt_cluster_blocks gives C, or 0 when the row kernels should run the batch.
 // sweep_base: if set, the sweeps are *sweep_base + [s_begin, s_end) (graph replays).
 struct ExchangeTablesDev {
     const uint32_t *tab, *off, *len, *tail;

@@ -26,7 +26,7 @@ def gap_vs_L(sg, Ls, l: int = 5, sweeps: int = 20, beta0: float = 0.5, beta1: fl
              instances: int = 20, seed_base: int = 9 * 10 ** 6, tropical: bool = False):
     """Mean gap and throughput at each L, and the a / L + b fit.  tropical: exact
     zero-temperature cube marginals (l <= 3) instead of SA anneals; the rate is then in
-    enumerated cube states per second."""
+    cube states decided per second (2^F for F free spins)."""
     rows = []
     for L in Ls:
         insts = [sg.Instance.create(L, seed_base + 1000 * L + k, F6, True) for k in range(instances)]
