@@ -17,6 +17,9 @@
 // thresholds are kept in shared memory where they fit, since a lookup of them lies on the
 // path of every sweep.
 //
+// 33 to 64 temperatures are two words a site, each on C blocks of the cluster (4 lattices of
+// L = 32, 48 temperatures: 10.3 us a sweep, 15.6 through the row kernels).
+//
 // Every attempt draws the same counters as the row kernel (site, sweep, word) and the
 // exchange the same counters as the stand-alone exchange (pair, sweep), so results are
 // bit-identical to the row kernel and to the oracle.
@@ -390,7 +393,8 @@ double device_hz()
 // Seconds a sweep of one instance takes on a cluster of C blocks, and of I instances through
 // the row kernels on `sms` SMs, fitted to measurements on a GB300 (K = 32): clusters 2.1 us at
 // L = 8 (C = 2), 2.7 at L = 16, 6.1 at L = 24, 9.4 at L = 32, 49.6 at L = 64 (C = 8); row
-// kernels about 10 us of launches and 6.2 attempts per SM clock.
+// kernels about 10 us of launches and 6.2 attempts per SM clock.  On C = 16: 2.4 us at L = 16, 5.1
+// at 24, 6.5 at 32, 12.5 at 40 (the row kernels 11.9).
 double cluster_seconds(int L, int C, double hz) { return 3.7e-6 + 64.0 * slab::pairs_of(L, C) / (11.0 * hz); }
 double row_seconds(double work, int I, int sms, double hz) { return 10e-6 + I * work / (sms * 6.2 * hz); }
 }  // namespace
