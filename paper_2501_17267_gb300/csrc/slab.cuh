@@ -333,9 +333,12 @@ struct Planes {
     uint4 lz;
 };
 
-// Planes of the energy counters: a lane has fewer than 85 items of at most 6 (a slab that
-// fits shared memory has at most 38 K sites, 19 K a colour, over 512 threads).
+// Planes of the energy counters: they hold kFoldPairs pairs of items of at most 6 each.  A lane
+// of 512 threads has at most 42 items (a slab that fits shared memory has at most 38 K sites,
+// 19 K a colour), half of what fits; blocks of fewer threads may have more, which only counts
+// (kCountOnly), and folds its counters into the block's sums before they run over.
 constexpr int kVBits = 9;
+constexpr int kFoldPairs = ((1 << kVBits) - 1) / 12;
 
 // A warp's share of the half sweeps of a launch.
 struct Sweeper {
@@ -542,16 +545,19 @@ struct Sweeper {
         }
     }
 
+    __device__ __forceinline__ void clear_counters()
+    {
+#pragma unroll
+        for (int j = 0; j < kVBits; ++j) V[j] = 0;
+        nitems = 0;
+    }
+
     // This warp's columns of a half sweep.  A: the draws of its first item, on return those of
     // its first item of the next half sweep.
     template <int MODE, bool TEMPERING, bool ENERGY>
     __device__ __forceinline__ void half(const int colour, uint32_t (&A)[8])
     {
-        if (ENERGY) {
-#pragma unroll
-            for (int j = 0; j < kVBits; ++j) V[j] = 0;
-            nitems = 0;
-        }
+        if (ENERGY) clear_counters();
         if (warp < g.units) {
             const int H4 = 4 * g.H, LL4 = 4 * g.LL;
             Cursor c;
@@ -559,7 +565,7 @@ struct Sweeper {
             c.qn = 0;
             enter<0>(c, colour, H4, LL4);
             uint32_t B[8];
-            for (;;) {
+            for (int pairs = 1;; ++pairs) {
                 if (!step<MODE, TEMPERING, ENERGY, 0>(c, colour, H4, LL4, A, B)) {
 #pragma unroll
                     for (int j = 0; j < 8; ++j) A[j] = B[j];
@@ -567,6 +573,11 @@ struct Sweeper {
                     break;
                 }
                 if (!step<MODE, TEMPERING, ENERGY, 1>(c, colour, H4, LL4, B, A)) break;
+                if (MODE == kCountOnly && pairs == kFoldPairs) {  // (a warp's lanes are at the same item)
+                    energy_to_block();
+                    clear_counters();
+                    pairs = 0;
+                }
             }
             while ((MODE == kCompare || MODE == kTailOnly) && c.qn) decide<TEMPERING, ENERGY>(c.qn);
         }

@@ -1,0 +1,35 @@
+"""The forms a server's chunks take, and its host side."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sg():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    torch.cuda.init()
+    from paper_2501_17267_gb300 import sg
+    return sg
+
+
+def _one(sg, req, chunk):
+    with sg.Server(4 << 30, chunk_sweeps=chunk) as srv:
+        return srv.poll(srv.submit(req))
+
+
+# Items a lane of a block with so many threads sums in its nine-bit counters: 175, 128, 85 and 42.
+@pytest.mark.parametrize("L,C,threads", [(56, 8, 64), (64, 8, 128), (34, 1, 256), (64, 8, 512)])
+def test_chunk_energies_with_any_number_of_threads(sg, monkeypatch, L, C, threads):
+    """A chunk on clusters reports the lowest energy sg_sa_run gives, however many items a thread
+    of its blocks has: of a hot lattice (about half the bonds satisfied) and of a cold one."""
+    for beta in (0.01, 3.0):
+        req = sg.request(sg.SG_REQ_SA, L, 60 + L, 32, 0.01, beta, 0.0, 12, run_seed=5, sweeps_per_restart=12)
+        want = sg.sa_run(sg.Instance.create(L, 60 + L), 32, 12, 0.01, beta, seed=5)["E"].min()
+        monkeypatch.setenv("SG_SA_CLUSTER_C", str(C))
+        monkeypatch.setenv("SG_SA_CLUSTER_THREADS", str(threads))
+        got = _one(sg, req, 12)
+        monkeypatch.delenv("SG_SA_CLUSTER_C")
+        monkeypatch.delenv("SG_SA_CLUSTER_THREADS")
+        assert got["status"] == sg.SG_OK and got["minE"] == want
