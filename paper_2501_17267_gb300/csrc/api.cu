@@ -49,6 +49,20 @@ bool stats_timing()
     return stats().timing;
 }
 
+// Polls a bounded wait of the cooperative PT kernel makes before it gives up (each a read
+// through L2, about 500 cycles, so several seconds in all); SG_WAIT_LIMIT overrides it (a test
+// sets 0 to make every wait give up on purpose).  The cluster kernels wait as long in cycles.
+long long wait_limit()
+{
+    const char* e = getenv("SG_WAIT_LIMIT");
+    if (e && *e) {
+        const long long v = atoll(e);
+        if (v >= 0) return v;
+    }
+    return 1ll << 24;
+}
+long long wait_limit_cycles() { return 512 * std::min(wait_limit(), 1ll << 50); }
+
 void stats_add(int kind, int64_t launches, int64_t units, double device_ms)
 {
     std::lock_guard<std::mutex> g(stats().mu);
@@ -255,19 +269,6 @@ constexpr int kGraphMinSweeps = 16;
 // Sweeps per launch of the thread-block-cluster and cooperative PT kernels (state carried
 // in device memory between launches).
 constexpr int kClusterChunkSweeps = 2000;
-
-// Polls a bounded wait of the cooperative PT kernel makes before it gives up (each a read
-// through L2, well under a microsecond, so several seconds in all); SG_WAIT_LIMIT
-// overrides it (a test sets 0 to make a wait give up on purpose).
-long long wait_limit()
-{
-    const char* e = getenv("SG_WAIT_LIMIT");
-    if (e && *e) {
-        const long long v = atoll(e);
-        if (v >= 0) return v;
-    }
-    return 1ll << 24;
-}
 
 // Whether a PT batch goes to the cooperative kernel.  Knob SG_PT_COOP = 0 / 1 turns it
 // off / on; otherwise it is off.

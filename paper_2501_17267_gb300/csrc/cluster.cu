@@ -43,6 +43,7 @@ struct ClusterArgs {
     int s_begin, s_end;             // sweeps [s_begin, s_end), from *sweep_base on when that is set
     const uint32_t* sweep_base;
     ChunkReport report;             // of a run of one instance and word
+    long long wait_limit;           // cycles a wait for the neighbours lasts at most
     uint32_t Hmagic;                // ceil(2^32 / (L / 2))
 };
 
@@ -72,10 +73,10 @@ struct Shared {
 
 // Called by every thread of every block of the cluster once the barriers are initialised;
 // phase: the barriers' phase bits, kept from plane to plane.  Ends with the plane written
-// back.  Returns false when a wait gave up.
+// back.  Returns false when a wait gave up (after `limit` cycles).
 template <class S>
 __device__ __forceinline__ bool anneal_plane(const PlaneRun& p, const int C, unsigned char* smem, Shared& sh,
-                                             uint32_t& phase, bool energies = false)
+                                             uint32_t& phase, const long long limit, bool energies = false)
 {
     cg::cluster_group cluster = cg::this_cluster();
     const int r = C > 1 ? (int)cluster.block_rank() : 0;
@@ -146,13 +147,17 @@ __device__ __forceinline__ bool anneal_plane(const PlaneRun& p, const int C, uns
             set_tables(sw + 1, entry);
             entry = entry_of(sw + 2);
         }
-        // the end of a half sweep: the faces pushed, the block met, the neighbours' faces here
+        // The end of a half sweep: the faces pushed, the block met, the neighbours' faces here.
+        // False when the wait of the half sweep before gave up (its flag was set before this
+        // barrier and is the same for every thread); this one's faces are waited for first, so
+        // that none is on its way when the block leaves.
         auto finish = [&](int colour) {
             __syncthreads();
             if (C > 1) {
-                if (sh.fail[colour ^ 1]) return false;  // set before this barrier, the same for every thread
-                if (!slab::mbar_wait(&sh.bar[colour], (phase >> colour) & 1u)) sh.fail[colour] = 1;
+                const bool lost = sh.fail[colour ^ 1] != 0;
+                if (!slab::mbar_wait<S::kResident>(&sh.bar[colour], (phase >> colour) & 1u, limit)) sh.fail[colour] = 1;
                 phase ^= 1u << colour;
+                if (lost) return false;
             }
             return true;
         };
@@ -258,7 +263,7 @@ sa_cluster_kernel(const ClusterArgs a)
     p.Hmagic = a.Hmagic;
     init_shared(sh);
     uint32_t phase = 0;
-    if (!anneal_plane<S>(p, a.C, smem, sh, phase, a.report.out != nullptr) && threadIdx.x == 0)
+    if (!anneal_plane<S>(p, a.C, smem, sh, phase, a.wait_limit, a.report.out != nullptr) && threadIdx.x == 0)
         atomicExch(a.status, SG_ETIMEOUT);
     // no block leaves while another may still push to it; energies and status are complete
     if (a.C > 1) cg::this_cluster().sync();
@@ -276,7 +281,8 @@ sa_cluster_kernel(const ClusterArgs a)
 // side by side take little longer than one.  next[2]: status word.
 __global__ void __launch_bounds__(kListBlock, 1) sa_cluster_list_kernel(const Plane* __restrict__ planes,
                                                                         const int* __restrict__ order, int n_cluster,
-                                                                        int n, unsigned* __restrict__ next, int C)
+                                                                        int n, unsigned* __restrict__ next, int C,
+                                                                        long long wait_limit)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ Shared sh;
@@ -302,9 +308,9 @@ __global__ void __launch_bounds__(kListBlock, 1) sa_cluster_list_kernel(const Pl
         p.Hmagic = q.Hmagic;
         bool done;
         switch (slab::resident_items(slab::pairs_of(q.L, blocks), kListBlock)) {
-            case 1: done = anneal_plane<slab::Resident<1>>(p, blocks, smem, sh, phase); break;
-            case 2: done = anneal_plane<slab::Resident<2>>(p, blocks, smem, sh, phase); break;
-            default: done = anneal_plane<slab::Sweeper>(p, blocks, smem, sh, phase); break;
+            case 1: done = anneal_plane<slab::Resident<1>>(p, blocks, smem, sh, phase, wait_limit); break;
+            case 2: done = anneal_plane<slab::Resident<2>>(p, blocks, smem, sh, phase, wait_limit); break;
+            default: done = anneal_plane<slab::Sweeper>(p, blocks, smem, sh, phase, wait_limit); break;
         }
         if (!done) {
             ok = false;
@@ -540,7 +546,8 @@ int32_t launch_sa_cluster_planes(const Plane* d_planes, const int* d_order, int 
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, sa_cluster_list_kernel, d_planes, d_order, n_cluster, n, d_next, C);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, sa_cluster_list_kernel, d_planes, d_order, n_cluster, n, d_next, C,
+                                             wait_limit_cycles());
     if (e != cudaSuccess) {
         cudaGetLastError();
         set_error("sa_cluster_list_kernel launch failed: %s", cudaGetErrorString(e));
@@ -570,6 +577,7 @@ int32_t launch_sa_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const Ru
     a.s_end = s_end;
     a.sweep_base = sweep_base;
     a.report = report;
+    a.wait_limit = wait_limit_cycles();
     a.C = C;
     const int H = L / 2;
     a.Hmagic = H == 1 ? 0u : (uint32_t)((0x100000000ull + (uint64_t)H - 1) / (uint64_t)H);

@@ -38,6 +38,7 @@ struct GeneralArgs {
     const uint32_t* thr;           // [S][kThrRow]
     int* status;                   // SG_ETIMEOUT when a bounded wait gave up
     int L, Wn, R, C, S;            // side, words, replicas, blocks per cluster, sweeps
+    long long wait_limit;          // cycles a wait for the neighbours lasts at most
     uint32_t Hmagic;               // ceil(2^32 / (L / 2))
 };
 
@@ -208,12 +209,13 @@ __global__ void __launch_bounds__(kThreads, 1) sa_general_cluster_kernel(const G
             if (tid < pairs) draws.planes(site_of(item(tid, colour ^ 1)), A);
             __syncthreads();
             if (C > 1) {
-                if (sh.fail[colour ^ 1]) {  // set before this barrier, the same for every thread
+                const bool lost = sh.fail[colour ^ 1] != 0;  // set before this barrier, the same for every thread
+                if (!slab::mbar_wait<false>(&sh.bar[colour], (phase >> colour) & 1u, a.wait_limit)) sh.fail[colour] = 1;
+                phase ^= 1u << colour;
+                if (lost) {  // (only now: no face may be on its way when the block leaves)
                     ok = false;
                     break;
                 }
-                if (!slab::mbar_wait(&sh.bar[colour], (phase >> colour) & 1u)) sh.fail[colour] = 1;
-                phase ^= 1u << colour;
             }
         }
     }
@@ -283,6 +285,7 @@ int32_t launch_sa_general_cluster(int8_t* spins, const uint2* const* j6_ptrs, co
     a.R = R;
     a.C = C;
     a.S = S;
+    a.wait_limit = wait_limit_cycles();
     const int H = L / 2;
     a.Hmagic = H == 1 ? 0u : (uint32_t)((0x100000000ull + (uint64_t)H - 1) / (uint64_t)H);
     const void* const fn = (const void*)sa_general_cluster_kernel;

@@ -58,6 +58,7 @@ struct PtcArgs {
     int L, K, C, s_begin, s_end;
     const uint32_t* sweep_base;     // if set, sweeps run from *sweep_base + s_begin to *sweep_base + s_end
     ChunkReport report;             // of a run of one instance
+    long long wait_limit;           // cycles a wait for other blocks lasts at most
     uint32_t Hmagic;                // ceil(2^32 / (L / 2))
     int xwords;                     // words of xtab held in shared memory (0: read from global memory)
 };
@@ -75,7 +76,7 @@ struct PtShared {
     uint32_t xoff[32 * WN], xlen[32 * WN], xtail[32 * WN];
     uint64_t bar[2];              // by colour: the neighbours' face words have arrived
     uint64_t ebar[2];             // by sweep parity: every block's energy sums have arrived
-    int fail[2];                  // by colour: a wait gave up (read one half sweep later)
+    int fail[2];                  // a wait gave up: before the exchange, after it (read after the next block barrier)
 };
 
 // S: slab::Sweeper, or slab::Resident when a block has a thread for each of its x pairs.  WN: words
@@ -198,15 +199,13 @@ __global__ void __launch_bounds__(S::kAssisted ? 2 * slab::kAssistedPairs : kThr
             s.push_faces(0, C == 1, up_w, dn_w, up_bar, dn_bar);
         }
         __syncthreads();
-        if (blocks > 1) {
-            if (sh.fail[1]) {  // set before this barrier, the same for every thread
-                ok = false;
-                break;
-            }
-            if (C > 1) {
-                if (!slab::mbar_wait(&sh.bar[0], phase & 1u)) sh.fail[0] = 1;
-                phase ^= 1u;
-            }
+        // Flags are set before a block barrier and read after it, the same for every thread.  A
+        // block that lost a wait leaves at the end of the sweep, when nothing is on its way to it.
+        bool lost = false;
+        if (blocks > 1) lost = sh.fail[1] != 0;
+        if (C > 1) {
+            if (!slab::mbar_wait<S::kResident>(&sh.bar[0], phase & 1u, a.wait_limit)) sh.fail[0] = 1;
+            phase ^= 1u;
         }
         // colour 1, with the energies
         const uint32_t par = sweep & 1u;
@@ -230,10 +229,6 @@ __global__ void __launch_bounds__(S::kAssisted ? 2 * slab::kAssistedPairs : kThr
         }
         __syncthreads();
         if (blocks > 1) {
-            if (sh.fail[0]) {
-                ok = false;
-                break;
-            }
             // the block's sums to every block, a warp a block
             for (int q = warp; q < blocks; q += warps) {
                 const uint32_t base = slab::cluster_addr(slab::smem_addr(&sh.Epart[par][rank][lane]), (uint32_t)q);
@@ -251,7 +246,7 @@ __global__ void __launch_bounds__(S::kAssisted ? 2 * slab::kAssistedPairs : kThr
         }
         int Eq[WN];  // of slots 32 i + lane
         if (blocks > 1) {
-            if (!slab::mbar_wait(&sh.ebar[par], (phase >> (2 + par)) & 1u)) sh.fail[1] = 1;
+            if (!slab::mbar_wait<S::kResident>(&sh.ebar[par], (phase >> (2 + par)) & 1u, a.wait_limit)) sh.fail[0] = 1;
             phase ^= 4u << par;
 #pragma unroll
             for (int i = 0; i < WN; ++i) {
@@ -310,9 +305,14 @@ __global__ void __launch_bounds__(S::kAssisted ? 2 * slab::kAssistedPairs : kThr
         }
         __syncthreads();  // the next sweep's planes are complete, and E has been read
         if (warp == 0) sh.E[lane] = 0;
+        if (blocks > 1) lost |= sh.fail[0] != 0;
         if (C > 1) {
-            if (!slab::mbar_wait(&sh.bar[1], (phase >> 1) & 1u)) sh.fail[1] = 1;
+            if (!slab::mbar_wait<S::kResident>(&sh.bar[1], (phase >> 1) & 1u, a.wait_limit)) sh.fail[1] = 1;
             phase ^= 2u;
+        }
+        if (lost) {
+            ok = false;
+            break;
         }
     }
     __syncthreads();
@@ -523,6 +523,7 @@ int32_t launch_pt_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const Ru
     PtcArgs a{};
     a.sweep_base = sweep_base;
     a.report = report;
+    a.wait_limit = wait_limit_cycles();
     a.spins = reinterpret_cast<uint32_t*>(spins);
     a.j1_ptrs = j1_ptrs;
     a.keys = keys;

@@ -196,6 +196,11 @@ int32_t launch_sweep_rows_pt(int8_t* spins, const uint2* const* j6_ptrs,
                              bool unit_j, int I, int L, int Wn, int K, uint32_t sweep, int colour,
                              const ExchangeArgs* xch, unsigned* done, bool* fused, cudaStream_t st,
                              const uint32_t* sweep_base = nullptr, int* status = nullptr, int sms = 0);
+// Limit of the kernels' waits for other blocks: polls (ptcoop.cu), and the cycles they take (the
+// cluster kernels).  api.cu.
+long long wait_limit();
+long long wait_limit_cycles();
+
 // Where a cluster kernel reports a chunk of one request (pinned host memory), so that nothing
 // has to follow it on its stream: the lowest energy, the status, then the token.
 struct ChunkReport {

@@ -45,7 +45,7 @@ constexpr int kMaxThreads = 512;
 constexpr int kMaxC = 16;       // blocks a cluster (more than 8: the kernels ask for it, allow_shared)
 constexpr int kTieCap = 64;     // queue entries a warp: decided from 32, an item adds at most 32
 constexpr unsigned kAll = 0xFFFFFFFFu;
-constexpr long long kWaitCycles = 1ll << 33;  // a bounded wait gives up after about 4 s
+constexpr long long kDrainCycles = 1ll << 31;  // what a wait that gave up still allows (about a second)
 
 // ---------------------------------------------------------------- PTX primitives
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -85,14 +85,33 @@ __device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity)
     return ok != 0;
 }
 
-// Waits for phase `parity`; false when it gave up.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity)
+// Polls for phase `parity`; false when it came after `limit` cycles or not at all.  The words on
+// their way are waited for beyond the limit too, again with a limit: the block must not leave, nor
+// its shared memory serve something else, while they can still arrive.
+__device__ __forceinline__ bool mbar_poll(uint64_t* bar, uint32_t parity, long long limit)
 {
-    if (mbar_try(bar, parity)) return true;
     const long long t0 = clock64();
-    while (clock64() - t0 < kWaitCycles)
-        if (mbar_try(bar, parity)) return true;
-    return false;
+    long long t;
+    bool here;
+    do {
+        here = mbar_try(bar, parity);
+        t = clock64() - t0;
+    } while (!here && t < limit + kDrainCycles);
+    return here && t < limit;
+}
+static __device__ __noinline__ bool mbar_poll_apart(uint64_t* bar, uint32_t parity, long long limit)
+{
+    return mbar_poll(bar, parity, limit);
+}
+// Waits for phase `parity`, for `limit` cycles (0: not at all); false when it gave up.  APART: the
+// polling out of line, where it takes registers from a half sweep that has none to spare (resident
+// blocks: 1.00 ms against 1.04 at L = 4 with 8 replicas and 1000 sweeps; elsewhere the call costs
+// more: 48 temperatures at L = 32 3.66 ms in line, 3.72 apart).
+template <bool APART>
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long long limit)
+{
+    if (limit > 0 && mbar_try(bar, parity)) return true;
+    return APART ? mbar_poll_apart(bar, parity, limit) : mbar_poll(bar, parity, limit);
 }
 
 // one word into another block's shared memory, its four bytes counted on that block's `bar`
