@@ -704,6 +704,7 @@ int32_t run_sa_planes(const std::vector<int>& members, const sg_instance* const*
                 SG_B(launch_planes_init(width(wg), static_cast<Plane*>(d_pl.p), (int)planes.size(), st));
                 const int conc = concurrency(wg);
                 double t_best = 1e300;
+                int gave_up = 0;  // the cluster form's status: a trial cut short measures nothing
                 for (int rep = 0; rep < 2; ++rep) {
                     SG_TRY_CUDA(cudaMemsetAsync(d_next.p, 0, 3 * sizeof(unsigned), st));
                     SG_TRY_CUDA(cudaStreamSynchronize(st));
@@ -712,7 +713,12 @@ int32_t run_sa_planes(const std::vector<int>& members, const sg_instance* const*
                                       (int)planes.size(), static_cast<unsigned*>(d_next.p), st));
                     SG_TRY_CUDA(cudaStreamSynchronize(st));
                     t_best = std::min(t_best, std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count());
+                    SG_TRY_CUDA(cudaMemcpyAsync(&gave_up, static_cast<unsigned*>(d_next.p) + 2, sizeof(int),
+                                                cudaMemcpyDeviceToHost, st));
+                    SG_TRY_CUDA(cudaStreamSynchronize(st));
+                    if (gave_up) break;
                 }
+                if (gave_up) continue;
                 const double rate = trial_work / t_best;  // attempts per second, whole GPU
                 double total = 0, biggest = 0;
                 for (double w : work) {

@@ -67,6 +67,21 @@ def test_batch_on_clusters(sg, monkeypatch, n_small):
     _gives_up_then_runs(sg, monkeypatch, lambda: sg.sa_run_batch(insts, ps, spins="host"), want)
 
 
+def test_trial_that_gives_up_is_not_chosen(sg, monkeypatch, tmp_path):
+    """The batch's tuner times its forms; one whose waits gave up is no candidate, nor kept as one."""
+    sides = [48] * 12 + [24, 40]
+    insts = [sg.Instance.create(L, 400 + k) for k, L in enumerate(sides)]
+    ps = [dict(replicas=64, sweeps=(40, 60)[k % 2], beta0=0.1, beta1=3.0, schedule="linear", seed=2, instance_id=k)
+          for k in range(len(sides))]
+    monkeypatch.setenv("SG_BATCH_WG", "1")
+    want = sg.sa_run_batch(insts, ps, spins="host")
+    monkeypatch.delenv("SG_BATCH_WG")
+    monkeypatch.setenv("SG_AUTOTUNE_CACHE", str(tmp_path / "tune.json"))
+    monkeypatch.setenv("SG_WAIT_LIMIT", "0")
+    for a, b in zip(sg.sa_run_batch(insts, ps, spins="host"), want):
+        assert np.array_equal(a["E"], b["E"]) and np.array_equal(a["spins"], b["spins"])
+
+
 def test_served_chunks(sg, monkeypatch):
     """A chunk whose waits gave up ends its request; the server serves the next one."""
     reqs = [sg.request(sg.SG_REQ_SA, 32, 4, 32, 0.1, 3.0, 0.0, 40, sweeps_per_restart=40),
