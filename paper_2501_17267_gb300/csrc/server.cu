@@ -405,11 +405,16 @@ int32_t admit_request(sg_server* srv, Request* q)
 
 // Blocks per cluster for the next chunk of a PT or large-SA request with `busy` requests in
 // service, 0 for the row kernels.  (A chunk's result does not depend on the form that runs it.)
+// Knobs as for the runs of their own: SG_PT_CLUSTER, and SG_SA_CLUSTER = 0 / 1, which turns the
+// cluster kernel off or takes it whenever a slab fits.
 int chunk_form(const Request* q, int busy)
 {
-    if (q->mode == kPT) return q->Wn == 1 ? pt_cluster_blocks_shared(q->L, q->req.width, busy) : 0;
+    if (q->Wn != 1) return 0;  // (a report is one word's)
+    if (q->mode == kPT) return pt_cluster_blocks_shared(q->L, q->req.width, busy);
+    const char* e = getenv("SG_SA_CLUSTER");
+    if (e && atoi(e) == 0) return 0;
     int threads = 0;
-    return q->Wn == 1 ? sa_cluster_blocks(1, q->L, 1, false, &threads, busy) : 0;  // (a report is one word's)
+    return sa_cluster_blocks(1, q->L, 1, e && atoi(e) == 1, &threads, busy);
 }
 
 // One chunk of n sweeps on clusters of C blocks: a single launch, which reports the chunk's

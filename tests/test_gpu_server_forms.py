@@ -33,3 +33,20 @@ def test_chunk_energies_with_any_number_of_threads(sg, monkeypatch, L, C, thread
         monkeypatch.delenv("SG_SA_CLUSTER_C")
         monkeypatch.delenv("SG_SA_CLUSTER_THREADS")
         assert got["status"] == sg.SG_OK and got["minE"] == want
+
+
+# the cost model takes clusters for a lone L = 32 and row kernels for a lone L = 64
+@pytest.mark.parametrize("L,clusters", [(32, True), (64, False)])
+def test_annealing_knob_reaches_the_server(sg, monkeypatch, L, clusters):
+    """SG_SA_CLUSTER turns the cluster kernel off, or takes it, for chunks too: with waits that give
+    up at once a chunk on clusters times out, one through the row kernels does not."""
+    req = sg.request(sg.SG_REQ_SA, L, 4, 32, 0.1, 3.0, 0.0, 40, sweeps_per_restart=40)
+    want = _one(sg, req, 20)
+    assert want["status"] == sg.SG_OK
+    monkeypatch.setenv("SG_WAIT_LIMIT", "0")
+    assert (_one(sg, req, 20)["status"] == sg.SG_ETIMEOUT) == clusters
+    monkeypatch.setenv("SG_SA_CLUSTER", "1")
+    assert _one(sg, req, 20)["status"] == sg.SG_ETIMEOUT
+    monkeypatch.setenv("SG_SA_CLUSTER", "0")
+    got = _one(sg, req, 20)
+    assert got["status"] == sg.SG_OK and got["minE"] == want["minE"]
