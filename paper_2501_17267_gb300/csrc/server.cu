@@ -290,6 +290,7 @@ Slot* take_slot(sg_server* srv)
         if (s->st) cudaStreamDestroy(s->st);
         return nullptr;
     }
+    memset(s->h_out, 0, 64);  // (no chunk has token 0)
     srv->slots.push_back(std::move(s));
     return srv->slots.back().get();
 }

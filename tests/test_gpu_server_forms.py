@@ -1,7 +1,13 @@
 """The forms a server's chunks take, and its host side."""
+import os
+import subprocess
+import sys
+
 import pytest
 
 pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.fixture(scope="module")
@@ -50,3 +56,45 @@ def test_annealing_knob_reaches_the_server(sg, monkeypatch, L, clusters):
     monkeypatch.setenv("SG_SA_CLUSTER", "0")
     got = _one(sg, req, 20)
     assert got["status"] == sg.SG_OK and got["minE"] == want["minE"]
+
+
+# Pinned memory comes with whatever it held; here an energy, a status, a ground state and the first
+# token a server writes.
+_PINNED = """
+#define _GNU_SOURCE
+#include <dlfcn.h>
+#include <stddef.h>
+int cudaHostAlloc(void** p, size_t n, unsigned flags)
+{
+    static int (*real)(void**, size_t, unsigned);
+    if (!real) {
+        void* lib = dlopen("libcudart.so.13", RTLD_NOW | RTLD_NOLOAD);
+        *(void**)&real = dlsym(lib ? lib : RTLD_NEXT, "cudaHostAlloc");
+    }
+    const int rc = real ? real(p, n, flags) : 1;
+    if (rc == 0 && n == 64) {
+        long long* w = (long long*)*p;
+        w[0] = -1000000000, w[1] = 0, w[2] = -1, w[3] = 1;
+    }
+    return rc;
+}
+"""
+_SOLVE = """
+from paper_2501_17267_gb300 import sg
+inst = sg.Instance.create(40, 7)
+want = int(sg.sa_run(inst, 32, 400, 0.1, 3.0, seed=5)["E"].min())
+req = sg.request(sg.SG_REQ_SA, 40, 7, 32, 0.1, 3.0, 0.0, 400, run_seed=5, sweeps_per_restart=400)
+with sg.Server(1 << 30, chunk_sweeps=400) as srv:
+    got = srv.poll(srv.submit(req))
+assert got["e_gs"] == inst.e_gs and got["minE"] == want, (got, want)
+"""
+
+
+def test_report_words_start_clean(tmp_path):
+    """What the words of a chunk's report held before is no report (in a process of its own)."""
+    (tmp_path / "pinned.c").write_text(_PINNED)
+    lib = str(tmp_path / "pinned.so")
+    subprocess.run(["gcc", "-shared", "-fPIC", str(tmp_path / "pinned.c"), "-o", lib, "-ldl"], check=True)
+    env = dict(os.environ, LD_PRELOAD=lib, SG_SA_CLUSTER_C="8")
+    r = subprocess.run([sys.executable, "-c", _SOLVE], cwd=ROOT, env=env, capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stderr[-2000:]
