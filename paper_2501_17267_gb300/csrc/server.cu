@@ -199,9 +199,31 @@ struct PlaneGroup {
 struct TableCache {
     using Words = std::shared_ptr<const std::vector<uint32_t>>;
     static constexpr size_t kMost = 64;
+    using Ladder = std::pair<Words, std::shared_ptr<const ExchangeTables>>;
     std::mutex mu;
     std::map<std::tuple<int, double, double, int>, Words> schedules;
-    std::map<std::tuple<int, double, double, int64_t>, std::pair<Words, std::shared_ptr<const ExchangeTables>>> ladders;
+    std::map<std::tuple<int, double, double, int64_t>, Ladder> ladders;
+
+    // The tables of `key`, made by `make` where they are not there yet.  They are made without the
+    // lock, so that nobody waits for another caller's (two may make the same ones: the first stay).
+    template <class Key, class Tables, class F>
+    int32_t get(std::map<Key, Tables>& all, const Key& key, Tables* out, F&& make)
+    {
+        {
+            std::lock_guard<std::mutex> lock(mu);
+            const auto it = all.find(key);
+            if (it != all.end()) {
+                *out = it->second;
+                return SG_OK;
+            }
+        }
+        const int32_t rc = make(out);
+        if (rc != SG_OK) return rc;
+        std::lock_guard<std::mutex> lock(mu);
+        if (all.size() >= kMost) all.clear();
+        *out = all.emplace(key, *out).first->second;
+        return SG_OK;
+    }
 };
 
 int largest_wg(int Wn)
@@ -304,41 +326,38 @@ int32_t prepare_request(TableCache& cache, Request* q)
     q->Wn = words_for(r.width);
     q->Rp = 32 * q->Wn;
     q->WG = largest_wg(q->Wn);
-    std::lock_guard<std::mutex> lock(cache.mu);
     if (r.kind == SG_REQ_SA) {
         q->mode = q->L <= plane_max_L() ? kPlanes : kRowsSA;
         const auto key = std::make_tuple(r.sweeps_per_restart, r.beta0, r.beta1, r.schedule);
-        auto it = cache.schedules.find(key);
-        if (it == cache.schedules.end()) {
+        const int32_t rc = cache.get(cache.schedules, key, &q->thr, [&](TableCache::Words* out) {
             const int S = r.sweeps_per_restart;
             std::vector<double> beta(S);
             beta_schedule(S, r.beta0, r.beta1, r.schedule == SG_SCHEDULE_GEOMETRIC, beta.data());
             auto t = std::make_shared<std::vector<uint32_t>>((size_t)S * kThrRow);
             for (int s = 0; s < S; ++s) metropolis_row(beta[s], t->data() + (size_t)s * kThrRow);
-            if (cache.schedules.size() >= TableCache::kMost) cache.schedules.clear();
-            it = cache.schedules.emplace(key, std::move(t)).first;
-        }
-        q->thr = it->second;
+            *out = std::move(t);
+            return (int32_t)SG_OK;
+        });
+        if (rc != SG_OK) return rc;
     } else {
         q->mode = kPT;
         const int K = r.width;
         const int64_t dmax = 12 * q->N;  // four times the sum of |J| over the 3N edges, all 1
         const auto key = std::make_tuple(K, r.beta0, r.beta1, dmax);
-        auto it = cache.ladders.find(key);
-        if (it == cache.ladders.end()) {
+        TableCache::Ladder tables;
+        const int32_t rc = cache.get(cache.ladders, key, &tables, [&](TableCache::Ladder* out) {
             std::vector<double> ladder(K);
             beta_schedule(K, r.beta0, r.beta1, 1, ladder.data());
             auto t = std::make_shared<std::vector<uint32_t>>((size_t)K * kThrRow);
             for (int k = 0; k < K; ++k) metropolis_row(ladder[k], t->data() + (size_t)k * kThrRow);
             auto x = std::make_shared<ExchangeTables>();
             const int32_t rc = build_exchange_tables(ladder, dmax, x.get());
-            if (rc != SG_OK) return rc;
-            if (cache.ladders.size() >= TableCache::kMost) cache.ladders.clear();
-            it = cache.ladders.emplace(key, std::make_pair(TableCache::Words(std::move(t)),
-                                                           std::shared_ptr<const ExchangeTables>(std::move(x)))).first;
-        }
-        q->thr = it->second.first;
-        q->xt = it->second.second;
+            if (rc == SG_OK) *out = TableCache::Ladder(std::move(t), std::move(x));
+            return rc;
+        });
+        if (rc != SG_OK) return rc;
+        q->thr = tables.first;
+        q->xt = tables.second;
     }
     q->lay = layout_of(*q);
     q->bytes = q->lay.total;

@@ -2,6 +2,8 @@
 import os
 import subprocess
 import sys
+import threading
+import time
 
 import pytest
 
@@ -98,3 +100,31 @@ def test_report_words_start_clean(tmp_path):
     env = dict(os.environ, LD_PRELOAD=lib, SG_SA_CLUSTER_C="8")
     r = subprocess.run([sys.executable, "-c", _SOLVE], cwd=ROOT, env=env, capture_output=True, text=True, timeout=600)
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+def _fine_ladder(sg, beta):
+    """A request whose exchange tables have some 70 million entries (half a second of host work) and
+    whose device memory no small budget covers."""
+    return sg.request(sg.SG_REQ_PT, 128, 1, 64, beta, beta * (1.0 + 63 * 2e-5), 0.0, 10)
+
+
+def test_submit_does_not_wait_for_another_callers_tables(sg):
+    with sg.Server(16 << 20) as srv:
+        spent = []
+
+        def submit():
+            t0 = time.perf_counter()
+            with pytest.raises(sg.SGError):
+                srv.submit(_fine_ladder(sg, 1.0))
+            spent.append(time.perf_counter() - t0)
+
+        other = threading.Thread(target=submit)
+        other.start()
+        time.sleep(0.05)
+        t0 = time.perf_counter()
+        ticket = srv.submit(sg.request(sg.SG_REQ_PT, 4, 2, 8, 0.3, 2.0, 0.0, 10))
+        took = time.perf_counter() - t0
+        other.join()
+        assert spent[0] > 0.2  # long enough to tell
+        assert took < spent[0] / 4
+        srv.poll(ticket)
