@@ -195,10 +195,15 @@ struct PlaneGroup {
 };
 
 // Host tables shared by requests with the same SA schedule or PT ladder (and lattice size, which
-// bounds the exchange tables); dropped when many different ones have come.
+// bounds the exchange tables), as long as all of them together stay small (32 temperatures from
+// 0.2 to 3.0 have some ten thousand words, a schedule of 10^4 sweeps 160 thousand, but a ladder of
+// close rungs can have up to 2^22 a rung): the shared ones are dropped when another would not fit,
+// and tables too large to share live as long as their request.
 struct TableCache {
     using Words = std::shared_ptr<const std::vector<uint32_t>>;
-    static constexpr size_t kMost = 64;
+    static constexpr size_t kMost = 64;                     // entries of each kind
+    static constexpr size_t kMostWords = (size_t)1 << 25;   // words of all of them
+    size_t words = 0;
     using Ladder = std::pair<Words, std::shared_ptr<const ExchangeTables>>;
     std::mutex mu;
     std::map<std::tuple<int, double, double, int>, Words> schedules;
@@ -219,11 +224,21 @@ struct TableCache {
         }
         const int32_t rc = make(out);
         if (rc != SG_OK) return rc;
+        const size_t n = size_of(*out);
+        if (n > kMostWords) return SG_OK;
         std::lock_guard<std::mutex> lock(mu);
-        if (all.size() >= kMost) all.clear();
-        *out = all.emplace(key, *out).first->second;
+        if (schedules.size() >= kMost || ladders.size() >= kMost || words + n > kMostWords) {
+            schedules.clear();
+            ladders.clear();
+            words = 0;
+        }
+        const auto entry = all.emplace(key, *out);
+        if (entry.second) words += n;
+        *out = entry.first->second;
         return SG_OK;
     }
+    static size_t size_of(const Words& t) { return t->size(); }
+    static size_t size_of(const Ladder& t) { return t.first->size() + t.second->tab.size(); }
 };
 
 int largest_wg(int Wn)

@@ -128,3 +128,19 @@ def test_submit_does_not_wait_for_another_callers_tables(sg):
         assert spent[0] > 0.2  # long enough to tell
         assert took < spent[0] / 4
         srv.poll(ticket)
+
+
+def test_tables_kept_between_requests_are_bounded(sg):
+    """Requests that are gone leave no unbounded tables behind."""
+    def resident():
+        with open("/proc/self/statm") as f:
+            return int(f.read().split()[1]) * os.sysconf("SC_PAGE_SIZE")
+
+    with sg.Server(16 << 20) as srv:
+        sizes = []
+        for k in range(5):
+            with pytest.raises(sg.SGError) as e:
+                srv.submit(_fine_ladder(sg, 1.0 + 0.01 * k))
+            assert e.value.code == sg.SG_ENOMEM
+            sizes.append(resident())
+    assert sizes[-1] - sizes[0] < 100 << 20  # one table set is about 280 MB
