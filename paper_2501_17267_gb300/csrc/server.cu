@@ -1065,9 +1065,12 @@ extern "C" int32_t sg_poll(sg_server* srv, uint64_t ticket, int32_t timeout_ms, 
     else if (timeout_ms > 0)
         srv->cv_done.wait_for(lock, std::chrono::milliseconds(timeout_ms), is_done);
     if (!q->finished) return SG_PENDING;
-    finish_result(q);
-    *out = q->result;
+    // (out of the map, so that the planted energy of a request that never ran is the caller's work alone)
+    const std::unique_ptr<Request> own = std::move(it->second);
     srv->all.erase(it);
+    lock.unlock();
+    finish_result(own.get());
+    *out = own->result;
     return SG_OK;
 }
 

@@ -144,3 +144,36 @@ def test_tables_kept_between_requests_are_bounded(sg):
             assert e.value.code == sg.SG_ENOMEM
             sizes.append(resident())
     assert sizes[-1] - sizes[0] < 100 << 20  # one table set is about 280 MB
+
+
+def test_poll_of_a_request_that_never_ran_holds_nobody_up(sg):
+    """The planted energy of a large request cancelled in the queue is host work of the caller
+    that asks for it, not of everybody."""
+    busy = sg.request(sg.SG_REQ_PT, 16, 1, 16, 0.02, 0.1, 0.0, 10 ** 9)  # (too hot to reach anything)
+    large = sg.request(sg.SG_REQ_SA, 256, 3, 1, 0.1, 3.0, 0.0, 10, sweeps_per_restart=10)
+    with sg.Server(8 << 30, max_active=1, chunk_sweeps=10) as srv:
+        running = srv.submit(busy)
+        tickets = [srv.submit(large) for _ in range(4)]
+        for t in tickets:
+            srv.cancel(t)
+        spent, got = [], []
+
+        def ask():
+            for t in tickets:
+                t0 = time.perf_counter()
+                got.append(srv.poll(t))
+                spent.append(time.perf_counter() - t0)
+
+        other = threading.Thread(target=ask)
+        other.start()
+        waits = []
+        while other.is_alive():
+            t0 = time.perf_counter()
+            assert srv.poll(running, timeout_ms=0) is None
+            waits.append(time.perf_counter() - t0)
+            time.sleep(1e-3)
+        other.join()
+        srv.cancel(running)
+        assert all(r["status"] == sg.SG_ECANCELED and r["e_gs"] == got[0]["e_gs"] for r in got)
+    assert min(spent) > 0.01  # long enough to tell
+    assert sorted(waits)[len(waits) // 2] < min(spent) / 3
