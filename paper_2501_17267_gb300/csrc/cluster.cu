@@ -40,8 +40,7 @@ struct ClusterArgs {
     const uint32_t* thr;            // [S][kThrRow]
     int* status;                    // SG_ETIMEOUT when a bounded wait gave up
     int L, Wn, R, C;                // side, words, replicas, blocks per cluster
-    int s_begin, s_end;             // sweeps [s_begin, s_end), from *sweep_base on when that is set
-    const uint32_t* sweep_base;
+    int s_begin, s_end;             // sweeps [s_begin, s_end)
     ChunkReport report;             // of a run of one instance and word
     long long wait_limit;           // cycles a wait for the neighbours lasts at most
     uint32_t Hmagic;                // ceil(2^32 / (L / 2))
@@ -257,9 +256,8 @@ sa_cluster_kernel(const ClusterArgs a)
     p.L = a.L;
     p.w = w;
     p.R = a.R;
-    const int base = a.sweep_base ? (int)*a.sweep_base : 0;  // (a captured graph replays the launch for later sweeps)
-    p.s_begin = base + a.s_begin;
-    p.s_end = base + a.s_end;
+    p.s_begin = a.s_begin;
+    p.s_end = a.s_end;
     p.Hmagic = a.Hmagic;
     init_shared(sh);
     uint32_t phase = 0;
@@ -558,7 +556,7 @@ int32_t launch_sa_cluster_planes(const Plane* d_planes, const int* d_order, int 
 
 int32_t launch_sa_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const RunKeys* keys, const uint32_t* thr,
                           int* status, int I, int L, int Wn, int R, int s_begin, int s_end, int C, int threads,
-                          cudaStream_t st, const uint32_t* sweep_base, const ChunkReport& report)
+                          cudaStream_t st, const ChunkReport& report)
 {
     if (threads < 32 || threads > slab::kMaxThreads || threads % 32) {
         set_error("sa_cluster_kernel: %d threads a block (a multiple of 32 up to %d)", threads, slab::kMaxThreads);
@@ -575,7 +573,6 @@ int32_t launch_sa_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const Ru
     a.R = R;
     a.s_begin = s_begin;
     a.s_end = s_end;
-    a.sweep_base = sweep_base;
     a.report = report;
     a.wait_limit = wait_limit_cycles();
     a.C = C;

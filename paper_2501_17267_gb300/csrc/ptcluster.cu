@@ -56,7 +56,6 @@ struct PtcArgs {
     const uint32_t* xtail;
     int* status;                    // SG_ETIMEOUT when a bounded wait gave up
     int L, K, C, s_begin, s_end;
-    const uint32_t* sweep_base;     // if set, sweeps run from *sweep_base + s_begin to *sweep_base + s_end
     ChunkReport report;             // of a run of one instance
     long long wait_limit;           // cycles a wait for other blocks lasts at most
     uint32_t Hmagic;                // ceil(2^32 / (L / 2))
@@ -169,10 +168,8 @@ __global__ void __launch_bounds__(S::kAssisted ? 2 * slab::kAssistedPairs : kThr
     if (blocks > 1) cluster.sync();
     else __syncthreads();
 
-    // a sweep base in device memory lets a captured graph replay the launch for later sweeps
-    const uint32_t sb = a.sweep_base ? *a.sweep_base : 0u;
-    const uint32_t s_end = sb + (uint32_t)a.s_end;
-    uint32_t sweep = sb + (uint32_t)a.s_begin;
+    const uint32_t s_end = (uint32_t)a.s_end;
+    uint32_t sweep = (uint32_t)a.s_begin;
     uint32_t phase = 0;  // of bar[0], bar[1]; of ebar: bits 2, 3
     bool ok = true;
     uint32_t A[S::kItems][8];
@@ -517,11 +514,9 @@ int pt_cluster_split(int I, int L, int K, int* M, int* side_sms, double* seconds
 int32_t launch_pt_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const RunKeys* keys, const uint32_t* thr,
                           uint8_t* rung_of_slot, uint8_t* slot_of_rung, int32_t* E, unsigned long long* accepts,
                           int32_t* minE, const ExchangeTablesDev& xt, int* status, int I, int L, int K, int C,
-                          int s_begin, int s_end, cudaStream_t st, const uint32_t* sweep_base,
-                          const ChunkReport& report)
+                          int s_begin, int s_end, cudaStream_t st, const ChunkReport& report)
 {
     PtcArgs a{};
-    a.sweep_base = sweep_base;
     a.report = report;
     a.wait_limit = wait_limit_cycles();
     a.spins = reinterpret_cast<uint32_t*>(spins);

@@ -467,13 +467,13 @@ int32_t launch_cluster_chunk(Request* q, int n, int C, long long token)
         return launch_pt_cluster(q->at<int8_t>(y.spins), j1p, q->at<RunKeys>(y.keys), q->at<uint32_t>(y.thr),
                                  q->at<uint8_t>(y.perm), q->at<uint8_t>(y.inv), q->at<int32_t>(y.E),
                                  q->at<unsigned long long>(y.acc), q->at<int32_t>(y.minE), xd, q->at<int>(y.status), 1,
-                                 q->L, q->req.width, C, (int)q->sweeps, (int)q->sweeps + n, q->slot->st, nullptr, report);
+                                 q->L, q->req.width, C, (int)q->sweeps, (int)q->sweeps + n, q->slot->st, report);
     }
     int threads = 0;
     sa_cluster_blocks(1, q->L, q->Wn, false, &threads);
     return launch_sa_cluster(q->at<int8_t>(y.spins), j1p, q->at<RunKeys>(y.keys), q->at<uint32_t>(y.thr),
                              q->at<int>(y.status), 1, q->L, q->Wn, q->req.width, q->in_restart, q->in_restart + n, C,
-                             threads, q->slot->st, nullptr, report);
+                             threads, q->slot->st, report);
 }
 
 // Captures one chunk of n sweeps of a PT or large-SA request through the row kernels as a

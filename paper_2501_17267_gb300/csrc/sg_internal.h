@@ -227,13 +227,11 @@ bool allow_shared(const void* fn);
 // cluster.cu: SA with all sweeps in one launch, one thread-block cluster of C blocks per
 // (word, instance); sa_cluster_blocks gives C and the threads to plan a block with, or 0 when
 // the row kernel should run instead (its estimate is shorter, unless `force`, or no slab fits);
-// busy: runs like this one that share the device.  sweep_base: sweeps [s_begin, s_end) are
-// counted from *sweep_base (graph replays).
+// busy: runs like this one that share the device.
 int sa_cluster_blocks(int I, int L, int Wn, bool force, int* threads, int busy = 1);
 int32_t launch_sa_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const RunKeys* keys,
                           const uint32_t* thr /* [S][kThrRow] */, int* status, int I, int L, int Wn, int R, int s_begin,
-                          int s_end, int C, int threads, cudaStream_t st, const uint32_t* sweep_base = nullptr,
-                          const ChunkReport& report = ChunkReport{});
+                          int s_end, int C, int threads, cudaStream_t st, const ChunkReport& report = ChunkReport{});
 // cluster_general.cu: the same for couplings that are not all +-1
 int sa_general_cluster_blocks(int I, int L, int Wn, bool force);
 int32_t launch_sa_general_cluster(int8_t* spins, const uint2* const* j6_ptrs, const RunKeys* keys, const uint32_t* thr,
@@ -257,7 +255,6 @@ int32_t launch_pt_exchange(const ExchangeArgs& x, int I, uint32_t sweep, cudaStr
 // ptcluster.cu: PT with unit couplings and K <= 64, every sweep of [s_begin, s_end) in one
 // launch, one thread-block cluster per instance (lattice in shared memory), of C blocks for
 // each word of slots.  pt_cluster_blocks gives C, or 0 when the row kernels should run the batch.
-// sweep_base: if set, the sweeps are *sweep_base + [s_begin, s_end) (graph replays).
 struct ExchangeTablesDev {
     const uint32_t *tab, *off, *len, *tail;
     size_t words;  // of tab
@@ -291,8 +288,7 @@ int32_t launch_pt_coop(int8_t* spins, const uint8_t* const* j1_ptrs, const RunKe
 int32_t launch_pt_cluster(int8_t* spins, const uint8_t* const* j1_ptrs, const RunKeys* keys, const uint32_t* thr,
                           uint8_t* rung_of_slot, uint8_t* slot_of_rung, int32_t* E, unsigned long long* accepts,
                           int32_t* minE, const ExchangeTablesDev& xt, int* status, int I, int L, int K, int C,
-                          int s_begin, int s_end, cudaStream_t st, const uint32_t* sweep_base = nullptr,
-                          const ChunkReport& report = ChunkReport{});
+                          int s_begin, int s_end, cudaStream_t st, const ChunkReport& report = ChunkReport{});
 int32_t launch_pt_setup(const unsigned long long* E64, int32_t* E, uint8_t* rung_of_slot,
                         uint8_t* slot_of_rung, unsigned long long* accepts, int32_t* minE,
                         int I, int Rp, int K, cudaStream_t st);
