@@ -52,3 +52,11 @@ def test_every_value_that_is_no_spin_is_counted(sg, L, values):
         spins[k % 3, (7 * k * L + 5) % L ** 3] = v
     with pytest.raises(sg.SGError, match=f"{len(values)} spin values"):
         sg.energy(inst, torch.from_numpy(spins).cuda())
+
+
+# (16, 4, 2 and 1 bytes a load) n such that a block walks over several configurations (3, 7, 7 and
+# 14 with 152 SMs) and the last one over fewer; then more than 128 a block could have
+@pytest.mark.parametrize("L,n,offset", [(64, 103, 0), (36, 320, 0), (34, 200, 0), (34, 200, 1), (2, 128 * 8 * 152 + 77, 0),
+                                        (2, 128 * 8 * 152 + 77, 1)])
+def test_energies_of_many_configurations_a_block(sg, L, n, offset):
+    test_energies_at_every_load_width(sg, L, n, offset)
