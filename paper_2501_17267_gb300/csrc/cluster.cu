@@ -235,8 +235,9 @@ __device__ __forceinline__ void init_shared(Shared& sh)
     __syncthreads();
 }
 
-// S: slab::Sweeper, or slab::Resident when a block has a thread for each of its x pairs and a
-// warp to spare for the tables.
+// S: slab::Sweeper, or slab::Resident when a block has a thread for each of its x pairs, or for
+// every two.  A resident block has a warp more than that takes, whose first work is the tables
+// (with one pair a thread it has no other).
 template <class S>
 __global__ void __launch_bounds__(S::kAssisted   ? 2 * slab::kAssistedPairs + 32
                                   : S::kResident ? slab::kMaxThreads + 32
@@ -274,9 +275,10 @@ sa_cluster_kernel(const ClusterArgs a)
 }
 
 // Persistent form for batches (batch.cu's planes of one word, [N][1]).  Clusters take planes
-// order[0 .. n_cluster) through the counter next[0] until none is left (no side below C), then each block by itself planes order[n_cluster .. n) through next[1]: a small
-// lattice does not fill a cluster, its half sweep being a chain of latencies, and four of them
-// side by side take little longer than one.  next[2]: status word.
+// order[0 .. n_cluster) through the counter next[0] until none is left (no side below C), then each
+// block by itself planes order[n_cluster .. n) through next[1]: a small lattice does not fill a
+// cluster, its half sweep being a chain of latencies, and four of them side by side take little
+// longer than one.  next[2]: status word.
 __global__ void __launch_bounds__(kListBlock, 1) sa_cluster_list_kernel(const Plane* __restrict__ planes,
                                                                         const int* __restrict__ order, int n_cluster,
                                                                         int n, unsigned* __restrict__ next, int C,
@@ -375,9 +377,8 @@ int resident_clusters(const void* fn, int C, size_t smem, int threads)
 }
 
 // Lets `fn` use clusters of up to 16 blocks, and as much dynamic shared memory as a block can
-// have beside its static one.  (The
-// limit is always the same one, so that launches from several threads do not lower it under one
-// another.)
+// have beside its static one.  (The limit is always the same one, so that launches from several
+// threads do not lower it under one another.)
 bool allow_shared(const void* fn)
 {
     int dev = 0, most = 0;
@@ -424,10 +425,10 @@ double half_sweep_cycles(int L, int C, int threads, int per_sm)
 }  // namespace
 
 // Blocks per cluster (and the threads to plan a block with) for an SA run of I instances of
-// side L with Wn words, or 0 when the row kernel should run it.  Candidates are the
-// C <= 16 (8 in a loaded server) whose largest slab fits shared memory and is thinner than with fewer blocks; clusters
-// that are not resident at once (as the driver reports for the kernel) run in waves.  A half sweep's cycles, fitted to measurements
-// on a GB300 (us at 2.07 GHz), times the waves:
+// side L with Wn words, or 0 when the row kernel should run it.  Candidates are the C <= 16 (8 in
+// a loaded server) whose largest slab fits shared memory and is thinner than with fewer blocks;
+// clusters that are not resident at once (as the driver reports for the kernel) run in waves.  A
+// half sweep's cycles, fitted to measurements on a GB300 (us at 2.07 GHz), times the waves:
 //   resident blocks  750 + 400 per warp of pairs an SM partition holds (L = 16 with 1024
 //                    replicas on C = 4 blocks of 16 warps 1.2), 500 + 400 where a second set of
 //                    warps draws (L = 4 on one block of one warp 0.41)
@@ -438,10 +439,10 @@ double half_sweep_cycles(int L, int C, int threads, int per_sm)
 //                    same)
 // The fewest cycles win, fewer blocks among equals.  With `busy` runs of the kind sharing the
 // device (a loaded server) a form's time is its own or, if that is longer, busy times its share
-// of the device.  One run alone: L = 16 with 1024 replicas takes C = 4 (2.4
-// ms a run of 1000 sweeps against 5.1 at C = 2), L = 4 one block (0.82 ms;
-// in line 1.05, 1.20 at C = 2 and 1.25 at C = 4).  force: a cluster form whatever the row kernel would take.
-// Knobs: SG_SA_CLUSTER_C forces C, SG_SA_CLUSTER_THREADS the threads.
+// of the device.  One run alone: L = 16 with 1024 replicas takes C = 4 (2.4 ms a run of 1000
+// sweeps against 5.1 at C = 2), L = 4 one block (0.82 ms; in line 1.05, 1.20 at C = 2 and 1.25 at
+// C = 4).  force: a cluster form whatever the row kernel would take.  Knobs: SG_SA_CLUSTER_C
+// forces C, SG_SA_CLUSTER_THREADS the threads.
 int sa_cluster_blocks(int I, int L, int Wn, bool force, int* threads, int busy)
 {
     *threads = slab::kMaxThreads;

@@ -246,9 +246,10 @@ static __device__ __noinline__ uint32_t resolve_tie_bits(uint32_t tie, uint32_t 
 // a flip costs dE = 2k, k = 2c - M.  With h = M / 2 rounded down, u = c - h is at least 1 exactly
 // where k > 0, and then k = 2u, or 2u - 1 when M is odd: six thresholds a parity, picked by the
 // three planes of u.  Replica by replica, as it was, a warp followed its slowest replica through
-// 32 branches (19 lanes of 32 active, 30 % of the issue slots): a half sweep of 100 replicas of
-// an L = 24 lattice took 8.4 us a launch, and takes 3.6 in planes (2.5 on clusters, which need none); tempering
-// 48 slots sums its energies in the same counters as unit couplings.
+// 32 branches (19 lanes of 32 active, 30 % of the issue slots): a half sweep of 100 replicas of an
+// L = 24 lattice took 8.4 us, one launch of the row kernel.  In planes it takes 3.6, and 2.5 on
+// clusters, which need no launch for it.  Tempering sums its energies in the same counters as for
+// unit couplings.
 //
 // Threshold planes of a word: gp[general_plane(odd, j, u)] has bit b equal to bit 24 + j of
 // replica b's threshold of k = 2u - odd; j = 8: whether its low 24 bits are nonzero.

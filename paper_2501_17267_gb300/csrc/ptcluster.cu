@@ -391,7 +391,9 @@ double device_hz()
 // the row kernels on `sms` SMs, fitted to measurements on a GB300 (K = 32): clusters 2.1 us at
 // L = 8 (C = 2), 2.7 at L = 16, 6.1 at L = 24, 9.4 at L = 32, 49.6 at L = 64 (C = 8); row
 // kernels about 10 us of launches and 6.2 attempts per SM clock.  On C = 16: 2.4 us at L = 16, 5.1
-// at 24, 6.5 at 32, 12.5 at 40 (the row kernels 11.9).
+// at 24, 6.5 at 32, 12.5 at 40 (the row kernels 11.9).  The line fits from L = 24 on.  Smaller
+// lattices sit in resident blocks, for which it gives about 4 us where 2.1 to 2.7 were measured;
+// that is far enough below the row kernels' 10 us for the choice to be the same.
 double cluster_seconds(int L, int C, double hz) { return 3.7e-6 + 64.0 * slab::pairs_of(L, C) / (11.0 * hz); }
 double row_seconds(double work, int I, int sms, double hz) { return 10e-6 + I * work / (sms * 6.2 * hz); }
 }  // namespace

@@ -27,7 +27,8 @@
 // which the next half sweep's first draws hide.  Nothing else orders the blocks, and
 // nothing has to: a face word is pushed only after its warp has read the halo words the
 // neighbour is going to overwrite, and the neighbour overwrites them only after all of this
-// block's face words have arrived there.
+// block's face words have arrived there.  Waits are bounded; a block whose wait gave up still
+// waits (bounded too) for the words of the half sweep it is in before it leaves.
 //
 // Ties (draws whose leading byte equals the threshold's, about 1.5 a warp and item) go to a
 // queue of the warp, by ballot, and are decided 32 at a time.
