@@ -14,7 +14,7 @@
 // M(z + 1), so an item loads five words instead of seven and its addresses follow from the
 // previous item's by a few additions.  The draws of an item are made while the one before it
 // is decided, so that multiplies and logic share the pipes.  A word of 32 attempts in tempering
-// at L = 64 costs 248 warp instructions, 130 of them on the logic pipe, and 409 cycles of a
+// at L = 64 costs 243 warp instructions, 130 of them on the logic pipe, and 403 cycles of a
 // partition (289, 155 and 491 when every item worked out its own geometry and drew for
 // itself); on this GPU a three-input logic operation takes 2 cycles of that and a widening
 // multiply beside it 2.1, 335 for what is left.
