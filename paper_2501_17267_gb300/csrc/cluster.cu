@@ -224,13 +224,14 @@ __device__ __forceinline__ bool anneal_plane(const PlaneRun& p, const int C, uns
     return ok;
 }
 
-__device__ __forceinline__ void init_shared(Shared& sh)
+// given_up: every wait counts as one that gave up.
+__device__ __forceinline__ void init_shared(Shared& sh, bool given_up)
 {
     if (threadIdx.x == 0) {
         slab::mbar_init(&sh.bar[0]);
         slab::mbar_init(&sh.bar[1]);
         slab::mbar_init_fence();
-        sh.fail[0] = sh.fail[1] = 0;
+        sh.fail[0] = sh.fail[1] = given_up;
     }
     __syncthreads();
 }
@@ -260,7 +261,7 @@ sa_cluster_kernel(const ClusterArgs a)
     p.s_begin = a.s_begin;
     p.s_end = a.s_end;
     p.Hmagic = a.Hmagic;
-    init_shared(sh);
+    init_shared(sh, a.C > 1 && a.wait_limit == 0);
     uint32_t phase = 0;
     if (!anneal_plane<S>(p, a.C, smem, sh, phase, a.wait_limit, a.report.out != nullptr) && threadIdx.x == 0)
         atomicExch(a.status, SG_ETIMEOUT);
@@ -289,7 +290,7 @@ __global__ void __launch_bounds__(kListBlock, 1) sa_cluster_list_kernel(const Pl
     __shared__ int s_item;
     cg::cluster_group cluster = cg::this_cluster();
     const int r = (int)cluster.block_rank();
-    init_shared(sh);
+    init_shared(sh, C > 1 && wait_limit == 0);
     uint32_t phase = 0;
     bool ok = true;
     auto run = [&](int it, int blocks) {

@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kThreads, 1) sa_general_cluster_kernel(const G
         slab::mbar_init(&sh.bar[0]);
         slab::mbar_init(&sh.bar[1]);
         slab::mbar_init_fence();
-        sh.fail[0] = sh.fail[1] = 0;
+        sh.fail[0] = sh.fail[1] = C > 1 && a.wait_limit == 0;
     }
     __syncthreads();
     const int zc = geo.zc, z0 = geo.z0, sites = zc * LL;

@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(S::kAssisted ? 2 * slab::kAssistedPairs : kThr
         slab::mbar_init(&sh.ebar[0]);
         slab::mbar_init(&sh.ebar[1]);
         slab::mbar_init_fence();
-        sh.fail[0] = sh.fail[1] = 0;
+        sh.fail[0] = sh.fail[1] = blocks > 1 && a.wait_limit == 0;
     }
     int minE = a.minE[inst];
     uint32_t accepted[WN] = {};  // first warp, by the pair's lower rung

@@ -104,14 +104,17 @@ static __device__ __noinline__ bool mbar_poll_apart(uint64_t* bar, uint32_t pari
 {
     return mbar_poll(bar, parity, limit);
 }
-// Waits for phase `parity`, for `limit` cycles (0: not at all); false when it gave up.  APART: the
-// polling out of line, where it takes registers from a half sweep that has none to spare (resident
-// blocks: 1.00 ms against 1.04 at L = 4 with 8 replicas and 1000 sweeps; elsewhere the call costs
-// more: 48 temperatures at L = 32 3.66 ms in line, 3.72 apart).
+
+// Waits for phase `parity`, for `limit` cycles; false when it gave up.  (With a limit of 0 the
+// kernels start with their flags set, as if every wait had given up: asking for that here, before
+// the first try, cost 40 temperatures at L = 16 3 %.)  APART: the polling out of line, where it
+// takes registers from a half sweep that has none to spare (resident blocks: 1.00 ms against 1.04
+// at L = 4 with 8 replicas and 1000 sweeps; elsewhere the call costs more: 48 temperatures at
+// L = 32 3.66 ms in line, 3.72 apart).
 template <bool APART>
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long long limit)
 {
-    if (limit > 0 && mbar_try(bar, parity)) return true;
+    if (mbar_try(bar, parity)) return true;
     return APART ? mbar_poll_apart(bar, parity, limit) : mbar_poll(bar, parity, limit);
 }
 
